@@ -81,6 +81,75 @@ __device__ __forceinline__ dfl df_mul(dfl a, dfl b) {
     return {s, t};
 }
 
+// Two double-float values side by side in 64-bit register pairs, for the
+// paired FP32 instructions of sm_100 and later: each half rounds as the
+// scalar instruction does, and one issue does the work of two.
+typedef unsigned long long f32x2;
+
+struct df2 {
+    f32x2 hi, lo;
+};
+
+__device__ __forceinline__ f32x2 f2_pack(float a, float b) {
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ float f2_first(f32x2 v) {
+    float a, b;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+    return a;
+}
+__device__ __forceinline__ float f2_second(f32x2 v) {
+    float a, b;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+    return b;
+}
+__device__ __forceinline__ f32x2 f2_add(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 f2_sub(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 f2_mul(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 f2_fma(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ f32x2 f2_neg(f32x2 a) { return a ^ 0x8000000080000000ull; }
+
+// c - a b, half by half the bits of df_fma(df_neg(a), b, c) and of
+// df_fma(a, df_neg(b), c): p = -(a.hi b.hi), which the caller forms with
+// whichever negated factor it shares between calls, and the product's error
+// and cross terms with the opposite sign (every step rounds symmetrically).
+__device__ __forceinline__ df2 df2_fnma(f32x2 p, df2 a, df2 b, df2 c) {
+    f32x2 en = f2_fma(a.hi, b.hi, p);
+    en = f2_fma(a.hi, b.lo, en);
+    en = f2_fma(a.lo, b.hi, en);
+    const f32x2 s = f2_add(c.hi, p);
+    const f32x2 bb = f2_sub(s, c.hi);
+    f32x2 t = f2_add(f2_sub(c.hi, f2_sub(s, bb)), f2_sub(p, bb));
+    t = f2_add(t, f2_sub(c.lo, en));
+    df2 r;
+    r.hi = f2_add(s, t);
+    r.lo = f2_sub(t, f2_sub(r.hi, s));
+    return r;
+}
+
+__device__ __forceinline__ dfl df2_first(df2 v) { return {f2_first(v.hi), f2_first(v.lo)}; }
+__device__ __forceinline__ dfl df2_second(df2 v) { return {f2_second(v.hi), f2_second(v.lo)}; }
+__device__ __forceinline__ df2 df2_pack(dfl a, dfl b) { return {f2_pack(a.hi, b.hi), f2_pack(a.lo, b.lo)}; }
+__device__ __forceinline__ df2 df2_dup(dfl a) { return {f2_pack(a.hi, a.hi), f2_pack(a.lo, a.lo)}; }
+
 // a / b to about 46 bits: one Newton correction of the float quotient
 __device__ __forceinline__ dfl df_div(dfl a, dfl b) {
     const float q1 = __fdiv_rn(a.hi, b.hi);

@@ -36,39 +36,373 @@ namespace {
 // Diagonal block of column J in double-float on the FP32 pipes (an FP64
 // instruction costs about 64 FP32 ones here): L_JJ = chol(A_JJ), log-det,
 // the reciprocal diagonal, and W = L_JJ^-1 with the slices of W's rows.
-// The block lives in shared memory as a packed lower triangle (row-major,
-// P[r(r+1)/2 + c]), 66 KB; two 512-thread CTAs share an SM.
 //
-// Factor and inverse run in one right-looking sweep over c = 0 .. 127.  At
-// step c, position (i, p) of the triangle holds, for rows i > c,
+// Factor and inverse run in one right-looking sweep over c = 0 .. 127.
+// Before step c, position (i, p) of the lower triangle holds, for rows i >= c,
 //   p <  c:  acc_ip = sum_{k<c} L_ik W_kp   (the inverse's partial sums)
-//   p >= c:  a_ip, the Cholesky trailing matrix,
-// and row c holds acc_c. below the diagonal and a_cc on it.  Phase 1 (one
-// thread per row p) finishes column c of L (L_pc = a_pc / L_cc, written out)
-// and row c of W (W_cp = -acc_cp / L_cc, W_cc = 1 / L_cc), and builds
-//   V_p = W_cp (p <= c),   V_p = -L_pc (p > c).
-// Phase 2 applies one rank-1 step to every row i > c, a warp per row:
-//   X_ip += L_ic V_p for p <= i   (X_ic = L_ic V_c: the first term of acc_ic),
-// which is the Cholesky update a_ip -= L_ic L_pc for p > c and the inverse's
-// acc_ip += L_ic W_cp for p <= c.  The lane that finishes a_{c+1,c+1} takes
-// the next pivot (1 / sqrt from a float seed, refined on the FP32 pipes; see
-// take_pivot).
-// After step 127 the triangle holds W.
-constexpr int kDiagThreads = 512;
+//   p >= c:  a_ip, the Cholesky trailing matrix.
+// Step c finishes row c of W (W_cp = -acc_cp / L_cc, W_cc = 1 / L_cc) and
+// column c of L (L_pc = a_pc / L_cc), giving
+//   V_p = W_cp (p <= c),   V_p = -L_pc (p > c),
+// and adds L_ic V_p to every position of the rows i > c: the Cholesky update
+// for p > c, the inverse's for p < c, and at p = c acc_ic = L_ic V_c restarts
+// the position from zero.
+//
+// The steps are taken kDiagB = 8 at a time, every position receiving its
+// terms in the order of c (so the block size does not show in the results):
+//   diag   one warp factors the 8 x 8 block, rows across lanes, the pivots
+//          passed by shuffles;
+//   panel  one thread per column p <= c0 + 7 finishes the 8 rows of W, one
+//          thread per row i > c0 + 7 the 8 columns of L (28 multiply-adds
+//          each), giving the 8 vectors V in shared memory;
+//   update the rows below take the 8 terms.
+// The triangle lives in the registers of 16 warps: lane l of warp w holds
+// columns l + 32 j of rows w + 16 k (j <= k / 2: 20 double-float values a
+// thread), rows k = 2 m and 2 m + 1 as pairs, so that one paired FP32
+// instruction serves both: the update is 15 of them per pair and term, and
+// little else (per term and warp four loads of V shared by its rows, one
+// load per pair of rows).  It first reaches the next block's columns and
+// rows, which go to shared memory; a 17th warp then factors the next 8 x 8
+// block while the others finish the update, and writes the finished rows and
+// columns out while they begin the next.  Three barriers per eight columns.
+//
+// Bound by FP32 issue: the 128^3 / 3 multiply-adds of 15 instructions are
+// 0.10 M cycles on an SM's four schedulers at the measured 1.04 cycles each;
+// the sweep takes 0.21 M, the rest being the panels and the 8 x 8 blocks of
+// the last columns, and the kernel 131 us for up to 152 candidates (254 us
+// with the triangle in shared memory and two barriers a column, where the
+// loads, stores and index arithmetic took three of four issue slots; 160 us
+// with registers but a barrier pair per column, 850 of whose 2000 cycles were
+// the pivot's dependent chain).  n = 1024, T = 100: 4.46 -> 3.50 ms a batch;
+// n = 64, T = 100: 0.363 -> 0.260 ms; n = 4000, T = 256: 130.0 -> 128.2 ms.
+constexpr int kDiagWarps = 16;                         // warps that hold the triangle, plus one
+constexpr int kDiagThreads = 32 * (kDiagWarps + 1);
+constexpr int kDiagRows = GP_NB / kDiagWarps;          // rows per warp
+constexpr int kDiagB = 8;
+constexpr int kDiagBlocks = GP_NB / kDiagB;
+static_assert(kDiagWarps == 16, "the row-to-warp map assumes two row groups per 32-column block");
 constexpr int kPacked = GP_NB * (GP_NB + 1) / 2;
 
 __device__ __forceinline__ int prow(int r) { return r * (r + 1) / 2; }
 
-__global__ void __launch_bounds__(kDiagThreads) k_diag_mixed(MixedBatch b, int J) {
-    extern __shared__ dfl P[];             // kPacked double-float values
-    __shared__ dfl V[GP_NB];
-    __shared__ dfl dinv[GP_NB];            // 1 / L_cc
-    __shared__ dfl lcc[GP_NB];             // L_cc
+struct DiagShared {
+    // the block's vectors V (zero at p > c inside the block): each value
+    // twice (hi, hi, lo, lo), and the rows below in pairs (hi of rows w + 32 m
+    // and w + 32 m + 16, then their lo)
+    float4 vdup[kDiagB][GP_NB];
+    float4 vrow[kDiagB][kDiagWarps][kDiagRows / 2];
+    dfl col[kDiagB][GP_NB];     // the block's columns of the trailing matrix
+    dfl row[kDiagB][GP_NB];     // the block's rows of the inverse's sums
+    float4 ld[kDiagB][kDiagB / 2];   // the block's L: column c, rows 2 u and 2 u + 1 in pairs
+    dfl dinv[GP_NB];            // 1 / L_cc
+    dfl lcc[GP_NB];             // L_cc
+    int failed;
+};
+
+__device__ __forceinline__ df2 df2_load(const float4* p) {
+    const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(p);
+    return {v.x, v.y};
+}
+
+__device__ __forceinline__ void ld_store(DiagShared& sh, int r, int c, dfl v) {
+    float* p = reinterpret_cast<float*>(&sh.ld[c][r >> 1]) + (r & 1);
+    p[0] = v.hi;
+    p[2] = v.lo;
+}
+
+__device__ __forceinline__ dfl df_shfl(dfl a, int src) {
+    return {__shfl_sync(0xffffffffu, a.hi, src), __shfl_sync(0xffffffffu, a.lo, src)};
+}
+
+// Pivots in [2^-100, 2^100] (the float seed's comfortable range): 1 / sqrt(a)
+// from the hardware seed (about 22 correct bits), one float Newton step to y1
+// (about 24 bits), then y = y1 (1 + e/2 + 3 e^2/8) with e = 1 - a y1^2:
+// Newton's step with its second-order term, the next term (5 e^3 / 16) being
+// below 2^-65.  e is about 2^-23 and needed to float precision only, so it
+// comes from the exact products a.hi y1 and (a.hi y1) y1 (1 - q_h is exact,
+// q_h lying within 2^-22 of 1), and y is the exact sum y1 + corr: about 2^-46
+// relative, as two double-float Newton steps give, in a quarter of their
+// dependent chain.
+__device__ __forceinline__ bool pivot_in_range(dfl a) { return a.hi > 7.9e-31f && a.hi < 1.26e30f; }
+
+__device__ __forceinline__ dfl pivot_rsqrt(dfl a) {
+    float y0;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y0) : "f"(a.hi));
+    const float p0 = __fmul_rn(a.hi, y0);
+    const float y1 = __fmaf_rn(__fmul_rn(y0, 0.5f), __fmaf_rn(-p0, y0, 1.f), y0);
+    const float ph = __fmul_rn(a.hi, y1);
+    const float pl = __fmaf_rn(a.hi, y1, -ph);
+    const float qh = __fmul_rn(ph, y1);
+    const float ql = __fmaf_rn(pl, y1, __fmaf_rn(ph, y1, -qh));
+    const float rl = __fmul_rn(__fmul_rn(a.lo, y1), y1);
+    const float e = __fsub_rn(__fsub_rn(__fsub_rn(1.f, qh), ql), rl);
+    const float h = __fmul_rn(y1, 0.5f);
+    const float corr = __fmaf_rn(h, e, __fmul_rn(__fmul_rn(h, __fmul_rn(e, e)), 0.75f));
+    dfl y;
+    fast_two_sum(y1, corr, y.hi, y.lo);
+    return y;
+}
+
+// The 8 x 8 block at c0 with a pivot outside pivot_in_range: those take the
+// double square root; the first that is not positive and finite is recorded
+// in sh.failed.
+__device__ __noinline__ void diag_block8_slow(DiagShared& sh, int c0, int lane) {
+    const int r = lane & 7;
+    dfl a[kDiagB];
+#pragma unroll
+    for (int q = 0; q < kDiagB; ++q) a[q] = sh.col[q][c0 + r];
+    bool ok = true;
+#pragma unroll
+    for (int cc = 0; cc < kDiagB; ++cc) {
+        const dfl piv = df_shfl(a[cc], cc);
+        const bool good = piv.hi > 0.f && isfinite(piv.hi);
+        dfl y = {1.f, 0.f}, d = {1.f, 0.f};
+        if (pivot_in_range(piv)) {
+            y = pivot_rsqrt(piv);
+            d = df_mul(piv, y);
+        } else if (good) {
+            const double ld = sqrt(df_to_double(piv));
+            y = df_from_double(1.0 / ld);
+            d = df_from_double(ld);
+        }
+        if (ok && !good && lane == 0) sh.failed = c0 + cc;
+        ok = ok && good;
+        const dfl l = df_mul(a[cc], y);
+        if (lane == cc) {
+            sh.dinv[c0 + cc] = y;
+            sh.lcc[c0 + cc] = d;
+        }
+        if (lane < kDiagB) ld_store(sh, lane, cc, lane == cc ? d : l);
+#pragma unroll
+        for (int q = cc + 1; q < kDiagB; ++q) a[q] = df_fma(l, df_neg(df_shfl(l, q)), a[q]);
+    }
+}
+
+// The 8 x 8 block at c0 (one warp): lane r < 8 holds its row r.  Every lane
+// takes each pivot and the results go out at the end, so the eight columns
+// are one straight-line chain: a pivot, the column, a shuffle and the next
+// pivot's last term, the other terms beside it.
+__device__ __forceinline__ void diag_block8(DiagShared& sh, int c0, int lane) {
+    const int r = lane & 7;
+    df2 a[kDiagB / 2];
+    dfl l[kDiagB], y[kDiagB];
+#pragma unroll
+    for (int u = 0; u < kDiagB / 2; ++u) a[u] = df2_pack(sh.col[2 * u][c0 + r], sh.col[2 * u + 1][c0 + r]);
+    bool ok = true;
+#pragma unroll
+    for (int cc = 0; cc < kDiagB; ++cc) {
+        const dfl acc = (cc & 1) ? df2_second(a[cc / 2]) : df2_first(a[cc / 2]);
+        const dfl piv = df_shfl(acc, cc);
+        ok = ok && pivot_in_range(piv);
+        y[cc] = pivot_rsqrt(piv);
+        l[cc] = df_mul(acc, y[cc]);        // on lane cc: a y, the pivot's square root
+        const df2 la = df2_dup(l[cc]);
+        const f32x2 nl = f2_neg(la.hi);
+#pragma unroll
+        for (int u = (cc + 1) / 2; u < kDiagB / 2; ++u) {
+            const df2 lq = df2_pack(df_shfl(l[cc], 2 * u), df_shfl(l[cc], 2 * u + 1));
+            a[u] = df2_fnma(f2_mul(nl, lq.hi), la, lq, a[u]);
+        }
+    }
+    if (ok) {
+        if (lane < kDiagB) {
+#pragma unroll
+            for (int cc = 0; cc < kDiagB; ++cc) {
+                ld_store(sh, lane, cc, l[cc]);
+                if (lane == cc) {
+                    sh.dinv[c0 + cc] = y[cc];
+                    sh.lcc[c0 + cc] = l[cc];
+                }
+            }
+        }
+    } else {
+        diag_block8_slow(sh, c0, lane);
+    }
+}
+
+// The panels of block c0: thread p <= c0 + 7 finishes column p of W's eight
+// rows, thread i > c0 + 7 row i of L's eight columns.
+__device__ __forceinline__ void diag_panels(DiagShared& sh, int c0, int warp, int lane) {
+    df2 v[kDiagB / 2];
+    if (warp < 4) {
+        const int p = 32 * warp + lane, q0 = p - c0;       // q0 >= 0: a column of the block
+        if (p >= c0 + kDiagB) return;
+#pragma unroll
+        for (int u = 0; u < kDiagB / 2; ++u)
+            v[u] = q0 < 0 ? df2_pack(sh.row[2 * u][p], sh.row[2 * u + 1][p]) : df2{0, 0};
+#pragma unroll
+        for (int cc = 0; cc < kDiagB; ++cc) {
+            const dfl di = sh.dinv[c0 + cc];
+            const dfl m = df_mul(di, (cc & 1) ? df2_second(v[cc / 2]) : df2_first(v[cc / 2]));
+            dfl w = df_neg(m);
+            if (q0 == cc) w = di;
+            if (q0 > cc) w = dfl{0.f, 0.f};
+            sh.vdup[cc][p] = make_float4(w.hi, w.hi, w.lo, w.lo);
+            const df2 wn = df2_dup(df_neg(w));
+            const f32x2 wh = f2_pack(w.hi, w.hi);
+#pragma unroll
+            for (int u = (cc + 1) / 2; u < kDiagB / 2; ++u) {
+                const df2 ld = df2_load(&sh.ld[cc][u]);
+                v[u] = df2_fnma(f2_mul(ld.hi, wh), ld, wn, v[u]);
+            }
+        }
+    } else if (warp < 8) {
+        const int i = 32 * (warp - 4) + lane;
+        if (i < c0 + kDiagB) return;
+#pragma unroll
+        for (int u = 0; u < kDiagB / 2; ++u) v[u] = df2_pack(sh.col[2 * u][i], sh.col[2 * u + 1][i]);
+#pragma unroll
+        for (int cc = 0; cc < kDiagB; ++cc) {
+            const dfl l = df_mul((cc & 1) ? df2_second(v[cc / 2]) : df2_first(v[cc / 2]), sh.dinv[c0 + cc]);
+            sh.vdup[cc][i] = make_float4(-l.hi, -l.hi, -l.lo, -l.lo);
+            float* vr = reinterpret_cast<float*>(&sh.vrow[cc][i & 15][i >> 5]) + ((i >> 4) & 1);
+            vr[0] = -l.hi;
+            vr[2] = -l.lo;
+            const df2 la = df2_dup(l);
+            const f32x2 nl = f2_neg(la.hi);
+#pragma unroll
+            for (int u = (cc + 1) / 2; u < kDiagB / 2; ++u) {
+                const df2 ld = df2_load(&sh.ld[cc][u]);
+                v[u] = df2_fnma(f2_mul(nl, ld.hi), la, ld, v[u]);
+            }
+        }
+    }
+}
+
+// Block c0's columns of L into the tile T and its rows of W into the packed
+// triangle P, from the vectors V (one warp).
+__device__ __forceinline__ void diag_write(const DiagShared& sh, int c0, float2* T, dfl* P, int lane) {
+    if (lane < kDiagB) {
+#pragma unroll
+        for (int cc = 0; cc < kDiagB; ++cc) {
+            const float* p = reinterpret_cast<const float*>(&sh.ld[cc][lane >> 1]) + (lane & 1);
+            if (lane >= cc) T[(size_t)(c0 + cc) * GP_NB + c0 + lane] = make_float2(p[0], p[2]);
+        }
+    }
+#pragma unroll 2
+    for (int cc = 0; cc < kDiagB; ++cc)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int p = lane + 32 * j;
+            const float4 v = sh.vdup[cc][p];
+            if (p <= c0 + cc)
+                P[prow(c0 + cc) + p] = dfl{v.x, v.z};
+            else if (p >= c0 + kDiagB)
+                T[(size_t)(c0 + cc) * GP_NB + p] = make_float2(-v.x, -v.z);
+        }
+}
+
+// A thread's part of the triangle: rows 2 m and 2 m + 1 of its warp in column
+// block j <= m.
+struct DiagRegs {
+    df2 x[kDiagRows / 2][4];
+};
+
+// Term cc of the block's update for rows k >= K0 of the warp: in column block
+// JN (REST: in all the others), row K0 of an owner in every one.
+template <int JN, int K0, bool OWNER, bool REST>
+__device__ __forceinline__ void diag_term(const DiagShared& sh, DiagRegs& R, int cc, int warp, int lane) {
+    constexpr int M0 = K0 / 2;                 // pair of row K0
+    df2 b[4];
+    f32x2 nb[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+        if (REST ? j != JN : (j == JN || (OWNER && j <= M0))) {
+            b[j] = df2_load(&sh.vdup[cc][lane + 32 * j]);
+            nb[j] = f2_neg(b[j].hi);
+        }
+#pragma unroll
+    for (int m = M0; m < kDiagRows / 2; ++m) {
+        const df2 a = df2_load(&sh.vrow[cc][warp][m]);
+#pragma unroll
+        for (int j = 0; j <= m; ++j) {
+            const bool mine = REST ? j != JN : j == JN;
+            const bool own = OWNER && m == M0 && !mine;      // row K0 alone
+            if (mine && !((K0 & 1) && m == M0)) {
+                R.x[m][j] = df2_fnma(f2_mul(a.hi, nb[j]), a, b[j], R.x[m][j]);
+            } else if (mine || own) {
+                // one row of the pair, on the scalar instructions
+                const dfl bs = df2_first(b[j]);
+                if (K0 & 1)
+                    R.x[m][j] = df2_pack(df2_first(R.x[m][j]),
+                                         df_fma(df_neg(df2_second(a)), bs, df2_second(R.x[m][j])));
+                else
+                    R.x[m][j] = df2_pack(df_fma(df_neg(df2_first(a)), bs, df2_first(R.x[m][j])),
+                                         df2_second(R.x[m][j]));
+            }
+        }
+    }
+}
+
+// The update by the block in sh.V, first part, and the export of block c0's
+// columns (in column block JN, lanes q = 0 .. 7) and rows (owner: row K0 of
+// this warp): rows k >= K0 take the eight terms in column block JN, and row
+// K0 of an owner in the others too.  The exported columns restart at zero.
+template <int JN, int K0, bool OWNER>
+__device__ __forceinline__ void diag_update_first(DiagShared& sh, DiagRegs& R, int c0, int warp, int lane) {
+    if constexpr (K0 < kDiagRows) {
+#pragma unroll 1
+        for (int cc = 0; cc < kDiagB; ++cc) diag_term<JN, K0, OWNER, false>(sh, R, cc, warp, lane);
+        const int q = lane - (c0 & 31);
+#pragma unroll
+        for (int k = K0; k < kDiagRows; ++k)
+            if (q >= 0 && q < kDiagB) {
+                df2& v = R.x[k / 2][JN];
+                sh.col[q][warp + kDiagWarps * k] = (k & 1) ? df2_second(v) : df2_first(v);
+                if (k & 1) v = df2{0, 0};
+            }
+        if (OWNER) {
+#pragma unroll
+            for (int j = 0; j <= K0 / 2; ++j)
+                if (lane + 32 * j < c0)
+                    sh.row[warp + kDiagWarps * K0 - c0][lane + 32 * j] =
+                        (K0 & 1) ? df2_second(R.x[K0 / 2][j]) : df2_first(R.x[K0 / 2][j]);
+        }
+    }
+}
+
+// Second part: rows k >= K0 in every column block but JN.
+template <int JN, int K0>
+__device__ __forceinline__ void diag_update_rest(const DiagShared& sh, DiagRegs& R, int warp, int lane) {
+    if constexpr (K0 < kDiagRows) {
+#pragma unroll 1
+        for (int cc = 0; cc < kDiagB; ++cc) diag_term<JN, K0, false, true>(sh, R, cc, warp, lane);
+    }
+}
+
+// The instance of diag_update_first / diag_update_rest for block nb = 4 JN ..
+// 4 JN + 3 and a warp whose rows reach from k0 on.
+template <int JN>
+__device__ __forceinline__ void diag_dispatch_first(DiagShared& sh, DiagRegs& R, int c0, int k0, bool owner,
+                                                    int warp, int lane) {
+    if (owner) {
+        if (k0 == 2 * JN) diag_update_first<JN, 2 * JN, true>(sh, R, c0, warp, lane);
+        else              diag_update_first<JN, 2 * JN + 1, true>(sh, R, c0, warp, lane);
+    } else {
+        if (k0 == 2 * JN)          diag_update_first<JN, 2 * JN, false>(sh, R, c0, warp, lane);
+        else if (k0 == 2 * JN + 1) diag_update_first<JN, 2 * JN + 1, false>(sh, R, c0, warp, lane);
+        else                       diag_update_first<JN, 2 * JN + 2, false>(sh, R, c0, warp, lane);
+    }
+}
+
+template <int JN>
+__device__ __forceinline__ void diag_dispatch_rest(const DiagShared& sh, DiagRegs& R, int k0, int warp,
+                                                   int lane) {
+    if (k0 == 2 * JN)          diag_update_rest<JN, 2 * JN>(sh, R, warp, lane);
+    else if (k0 == 2 * JN + 1) diag_update_rest<JN, 2 * JN + 1>(sh, R, warp, lane);
+    else                       diag_update_rest<JN, 2 * JN + 2>(sh, R, warp, lane);
+}
+
+__global__ void __launch_bounds__(kDiagThreads, 1) k_diag_mixed(MixedBatch b, int J) {
+    extern __shared__ dfl P[];             // kPacked double-float values: A_JJ in, W out
+    __shared__ DiagShared sh;
     __shared__ dfl bj[2][GP_NB];
     __shared__ dfl xpart[2][GP_NB];
     __shared__ double lsum[GP_NB / 32];
     __shared__ double psum[GP_NB / 32];
-    __shared__ int failed;
+    dfl (&dinv)[GP_NB] = sh.dinv;
+    dfl (&lcc)[GP_NB] = sh.lcc;
+    int& failed = sh.failed;
     const int t = blockIdx.x;
     if (b.st[t].status != GP_OK) return;
     float2* T = df_tile(b, b.A, t, J, J);
@@ -80,121 +414,59 @@ __global__ void __launch_bounds__(kDiagThreads) k_diag_mixed(MixedBatch b, int J
     cp_async_wait_all();
     __syncthreads();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    constexpr int kWarps = kDiagThreads / 32;
-    // pivot c: 1 / sqrt(a) from rsqrtf's seed (about 22 correct bits), one
-    // float Newton step to y1 (about 24 bits), then y = y1 (1 + e/2 + 3 e^2/8)
-    // with e = 1 - a y1^2: Newton's step with its second-order term, the next
-    // term (5 e^3 / 16) being below 2^-65.  e is about 2^-23 and needed to
-    // float precision only, so it comes from the exact products a.hi y1 and
-    // (a.hi y1) y1 (1 - q_h is exact, q_h lying within 2^-22 of 1), and y is
-    // the exact sum y1 + corr: about 2^-46 relative, as two double-float
-    // Newton steps give, in a quarter of their dependent chain, which matters
-    // since the pivot is the sweep's critical path.  Pivots outside
-    // [2^-100, 2^100] (the float seed's comfortable range) take the double
-    // route.
-    auto take_pivot = [&](int c, dfl a) {
-        dfl y, l;
-        if (!(a.hi > 0.f) || !isfinite(a.hi)) {
-            failed = c;
-            y = dfl{1.f, 0.f};
-            l = y;
-        } else if (a.hi > 7.9e-31f && a.hi < 1.26e30f) {
-            const float y0 = rsqrtf(a.hi);
-            const float p0 = __fmul_rn(a.hi, y0);
-            const float y1 = __fmaf_rn(__fmul_rn(y0, 0.5f), __fmaf_rn(-p0, y0, 1.f), y0);
-            const float ph = __fmul_rn(a.hi, y1);
-            const float pl = __fmaf_rn(a.hi, y1, -ph);
-            const float qh = __fmul_rn(ph, y1);
-            const float ql = __fmaf_rn(pl, y1, __fmaf_rn(ph, y1, -qh));
-            const float rl = __fmul_rn(__fmul_rn(a.lo, y1), y1);
-            const float e = __fsub_rn(__fsub_rn(__fsub_rn(1.f, qh), ql), rl);
-            const float h = __fmul_rn(y1, 0.5f);
-            const float corr = __fmaf_rn(h, e, __fmul_rn(__fmul_rn(h, __fmul_rn(e, e)), 0.75f));
-            fast_two_sum(y1, corr, y.hi, y.lo);
-            l = df_mul(a, y);
-        } else {
-            const double piv = df_to_double(a);
-            const double ld = sqrt(piv);
-            y = df_from_double(1.0 / ld);
-            l = df_from_double(ld);
+    constexpr int kWarps = kDiagWarps;
+    DiagRegs R;
+#pragma unroll
+    for (int m = 0; m < kDiagRows / 2; ++m)
+#pragma unroll
+        for (int j = 0; j <= m; ++j) {
+            const int i = warp + 32 * m, p = lane + 32 * j;
+            const dfl u = (warp < kWarps && p <= i) ? P[prow(i) + p] : dfl{0.f, 0.f};
+            const dfl v = (warp < kWarps && p <= i + 16) ? P[prow(i + 16) + p] : dfl{0.f, 0.f};
+            R.x[m][j] = df2_pack(u, v);
         }
-        lcc[c] = l;
-        dinv[c] = y;
-    };
-    if (threadIdx.x == 0) take_pivot(0, P[0]);
+    // block 0's columns (no rows: it has no columns before it)
+    if (lane < kDiagB && warp < kWarps)
+#pragma unroll
+        for (int m = 0; m < kDiagRows / 2; ++m) {
+            sh.col[lane][warp + 32 * m] = df2_first(R.x[m][0]);
+            sh.col[lane][warp + 32 * m + 16] = df2_second(R.x[m][0]);
+            R.x[m][0] = df2{0, 0};
+        }
     __syncthreads();
-    for (int c = 0; c < GP_NB; ++c) {
-        if (failed >= 0) break;            // read after a barrier: uniform
-        // phase 1: column c of L (out), row c of W, V
-        if (threadIdx.x < GP_NB) {
-            const int p = threadIdx.x;
-            const dfl di = dinv[c];
-            if (p < c) {
-                const dfl w = df_neg(df_mul(di, P[prow(c) + p]));
-                P[prow(c) + p] = w;
-                V[p] = w;
-            } else if (p == c) {
-                df_store(T + (size_t)c * GP_NB + c, lcc[c]);
-                P[prow(c) + c] = di;
-                V[c] = di;
-            } else {
-                const dfl l = df_mul(P[prow(p) + c], di);
-                df_store(T + (size_t)c * GP_NB + p, l);
-                V[p] = df_neg(l);
-                P[prow(p) + c] = dfl{0.f, 0.f};   // restarts in phase 2 as acc_pc = L_pc V_c
+    for (int nb = 0;; ++nb) {
+        const int c0 = kDiagB * nb;
+        // the warps of one half own a row each of block nb + 1; the warp's
+        // rows below block nb reach from k0 on
+        const bool owner = (warp >> 3) == ((nb + 1) & 1);
+        const int k0 = (c0 + kDiagB - warp + kDiagWarps - 1) >> 4;
+        if (warp == kWarps) {
+            diag_block8(sh, c0, lane);
+        } else if (nb > 0) {               // the rest of block nb - 1's update
+            const int k1 = (c0 - warp + kDiagWarps - 1) >> 4;
+            const int kr = k1 + (owner ? 0 : 1);   // past the warp's row of block nb, exported with it
+            switch (nb >> 2) {
+                case 0: diag_dispatch_rest<0>(sh, R, kr, warp, lane); break;
+                case 1: diag_dispatch_rest<1>(sh, R, kr, warp, lane); break;
+                case 2: diag_dispatch_rest<2>(sh, R, kr, warp, lane); break;
+                default: diag_dispatch_rest<3>(sh, R, kr, warp, lane); break;
             }
         }
         __syncthreads();
-        if (c + 1 == GP_NB) break;
-        // phase 2: rows i > c, X_ip += L_ic V_p (p <= i), a warp per row; warp
-        // 0 takes only row c + 1 and its pivot, the others deal the rest two
-        // rows at a time (both rows' loads first: eight independent
-        // multiply-adds per lane).  A row i reaches only the 32-column blocks
-        // j <= i / 32, a test that is uniform across the warp.
-        dfl vl[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) vl[j] = V[lane + 32 * j];
-        if (warp == 0) {
-            const int i = c + 1;
-            const dfl m = df_neg(V[i]);    // L_ic
-            dfl* row = P + prow(i);
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const int p = lane + 32 * j;
-                if (32 * j <= i && p <= i) {
-                    const dfl x0 = row[p];
-                    const dfl x = df_fma(m, vl[j], x0);
-                    if (p == c + 1)
-                        take_pivot(c + 1, x);
-                    else
-                        row[p] = x;
-                }
-            }
-        } else {
-            constexpr int kRowStep = kWarps - 1;
-            for (int i = c + 1 + warp; i < GP_NB; i += 2 * kRowStep) {
-                const int i2 = i + kRowStep;
-                const bool two = i2 < GP_NB;
-                const dfl m1 = df_neg(V[i]);
-                const dfl m2 = two ? df_neg(V[i2]) : dfl{0.f, 0.f};
-                dfl* r1 = P + prow(i);
-                dfl* r2 = P + prow(two ? i2 : i);
-                dfl x1[4], x2[4];
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const int p = lane + 32 * j;
-                    if (32 * j <= i) x1[j] = (p <= i) ? r1[p] : dfl{0.f, 0.f};
-                    if (two && 32 * j <= i2) x2[j] = (p <= i2) ? r2[p] : dfl{0.f, 0.f};
-                }
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const int p = lane + 32 * j;
-                    if (32 * j <= i && p <= i) r1[p] = df_fma(m1, vl[j], x1[j]);
-                    if (two && 32 * j <= i2 && p <= i2) r2[p] = df_fma(m2, vl[j], x2[j]);
-                }
+        if (failed >= 0) break;            // uniform
+        diag_panels(sh, c0, warp, lane);
+        __syncthreads();
+        if (warp == kWarps) diag_write(sh, c0, T, P, lane);
+        if (warp < kWarps && nb + 1 < kDiagBlocks) {
+            switch ((nb + 1) >> 2) {
+                case 0: diag_dispatch_first<0>(sh, R, c0 + kDiagB, k0, owner, warp, lane); break;
+                case 1: diag_dispatch_first<1>(sh, R, c0 + kDiagB, k0, owner, warp, lane); break;
+                case 2: diag_dispatch_first<2>(sh, R, c0 + kDiagB, k0, owner, warp, lane); break;
+                default: diag_dispatch_first<3>(sh, R, c0 + kDiagB, k0, owner, warp, lane); break;
             }
         }
         __syncthreads();
+        if (nb + 1 == kDiagBlocks) break;
     }
     if (failed >= 0) {
         if (threadIdx.x == 0) {
@@ -204,9 +476,9 @@ __global__ void __launch_bounds__(kDiagThreads) k_diag_mixed(MixedBatch b, int J
         return;
     }
     // log-det: sum of log L_cc over the block in a fixed order (warp trees,
-    // then the four warp sums in turn); reciprocal diagonal out
-    // and the sum of 1 / L_cc^2 over the block's real rows (the refinement's
-    // estimate of the log-det's own error, k_refine_check)
+    // then, at the end of the kernel, the four warp sums in turn); reciprocal
+    // diagonal out and the sum of 1 / L_cc^2 over the block's real rows (the
+    // refinement's estimate of the log-det's own error, k_refine_check)
     if (threadIdx.x < GP_NB) {
         double v = log(df_to_double(lcc[threadIdx.x]));
         const double di = df_to_double(dinv[threadIdx.x]);
@@ -221,16 +493,6 @@ __global__ void __launch_bounds__(kDiagThreads) k_diag_mixed(MixedBatch b, int J
         }
         float2* rinv = b.Z + (size_t)t * b.z_stride + (size_t)4 * b.nt * GP_NB + J * GP_NB;
         df_store(rinv + threadIdx.x, dinv[threadIdx.x]);
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double ld = 0.0, pq = 0.0;
-        for (int w = 0; w < GP_NB / 32; ++w) {
-            ld += lsum[w];
-            pq += psum[w];
-        }
-        b.st[t].logdet += 2.0 * ld;
-        b.st[t].piv_inv += pq;
     }
     // W as a double-float tile (column-major, zeros above the diagonal) for
     // the diagonal-block products of the solves
@@ -247,38 +509,41 @@ __global__ void __launch_bounds__(kDiagThreads) k_diag_mixed(MixedBatch b, int J
     }
     // row c of W: exponent (of the largest high word, as the panel slicing
     // takes it) and slices; one warp per row, all on the FP32 pipes
-    __nv_bfloat16* WS = b.WS + (size_t)t * b.ws_stride;
+    uint8_t* WS = reinterpret_cast<uint8_t*>(b.WS + (size_t)t * b.ws_stride);
     int* WE = b.WE + (size_t)t * b.we_stride;
-    for (int c = warp; c < GP_NB; c += kWarps) {
+#pragma unroll 2
+    for (int c = warp; c < GP_NB; c += kDiagThreads / 32) {
         const dfl* w = P + prow(c);
-        float mx = 0.f;
-        for (int k = lane; k <= c; k += 32) mx = fmaxf(mx, fabsf(w[k].hi));
+        // lane handles columns 4*lane .. 4*lane+3 (half of one 16-byte piece)
+        const int k0 = 4 * lane;
+        float xh[4], xl[4], mx = 0.f;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const dfl v = (k0 + e <= c) ? w[k0 + e] : dfl{0.f, 0.f};
+            xh[e] = v.hi;
+            xl[e] = v.lo;
+            mx = fmaxf(mx, fabsf(v.hi));
+        }
         for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
         const int E = exponent_of(mx);
         if (lane == 0) WE[c] = E;
-        // x 2^(7 - E) exactly (two factors when 7 - E leaves the float range)
-        const int e2 = 7 - E;
-        const int ea = e2 > 127 ? 127 : (e2 < -126 ? -126 : e2);
-        const int eb = e2 - ea;
-        const float sa = __int_as_float((ea + 127) << 23);
-        const float sb = (eb == 0) ? 1.f : __int_as_float(((eb > 127 ? 127 : (eb < -126 ? -126 : eb)) + 127) << 23);
-        // lane handles columns 4*lane .. 4*lane+3 (half of one 16-byte piece)
-        const int k0 = 4 * lane;
-        float m[4][GP_MAX_SLICES];
+        float sa, sb;
+        slice_scale(E, sa, sb);
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-            const dfl x = (k0 + e <= c) ? w[k0 + e] : dfl{0.f, 0.f};
-            cut_slices(__fmul_rn(__fmul_rn(x.hi, sa), sb), __fmul_rn(__fmul_rn(x.lo, sa), sb), b.ps, m[e]);
+            xh[e] = __fmul_rn(__fmul_rn(xh[e], sa), sb);
+            xl[e] = __fmul_rn(__fmul_rn(xl[e], sa), sb);
         }
-        const uint32_t off = image_piece(c, k0 & ~7) + ((k0 & 4) ? 8u : 0u);
+        uint8_t* dst = WS + (size_t)(k0 >> 5) * kChunkBytes + image_piece(c, k0 & ~7) + ((k0 & 4) ? 8u : 0u);
+        float wt = 1.f;
 #pragma unroll
-        for (int a = 0; a < GP_MAX_SLICES; ++a) {
-            if (a >= b.ps) break;
-            uint2 v;
-            v.x = pack_bf16x2(m[0][a], m[1][a]);
-            v.y = pack_bf16x2(m[2][a], m[3][a]);
-            uint8_t* dst = reinterpret_cast<uint8_t*>(WS + (size_t)(a * kChunks + (k0 >> 5)) * kChunkElems);
-            *reinterpret_cast<uint2*>(dst + off) = v;
+        for (int a = 0; a < GP_PANEL_SLICES; ++a) {
+            float m[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) m[e] = cut_one(xh[e], xl[e], wt);
+            *reinterpret_cast<uint2*>(dst + (size_t)a * kChunks * kChunkBytes) =
+                make_uint2(pack_bf16x2(m[0], m[1]), pack_bf16x2(m[2], m[3]));
+            wt = __fmul_rn(wt, 0.00390625f);
         }
     }
     if (b.fwd) {
@@ -289,15 +554,28 @@ __global__ void __launch_bounds__(kDiagThreads) k_diag_mixed(MixedBatch b, int J
         // fixed order
         float2* zJ = b.Z + (size_t)t * b.z_stride + (size_t)J * GP_NB;
         const int k = (threadIdx.x >> 7) & 1, r = threadIdx.x & 127, h = threadIdx.x >> 8;
+        const bool active = h < 2;
         float2* zk = zJ + (size_t)k * b.nt * GP_NB;
-        if (threadIdx.x < 2 * GP_NB) bj[k][r] = df_load(zk + r);
+        if (h == 0) bj[k][r] = df_load(zk + r);
         __syncthreads();
         const dfl* w = P + prow(r);
         dfl sum = {0.f, 0.f};
-        for (int c = h; c <= r; c += 2) sum = df_fma(w[c], bj[k][c], sum);
+        if (active)
+            for (int c = h; c <= r; c += 2) sum = df_fma(w[c], bj[k][c], sum);
         if (h == 1) xpart[k][r] = sum;
         __syncthreads();
         if (h == 0) df_store(zk + r, df_add(sum, xpart[k][r]));
+    } else {
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) {
+        double ld = 0.0, pq = 0.0;
+        for (int w = 0; w < GP_NB / 32; ++w) {
+            ld += lsum[w];
+            pq += psum[w];
+        }
+        b.st[t].logdet += 2.0 * ld;
+        b.st[t].piv_inv += pq;
     }
 }
 

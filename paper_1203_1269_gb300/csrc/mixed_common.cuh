@@ -178,26 +178,19 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float a, float b) {
     return *reinterpret_cast<uint32_t*>(&v);
 }
 
-// Cut a double-float x (already scaled so |x| <= 2^7) into s slices: slice a
-// is the integer q_a (|q_a| <= 128) times 2^(-8a), so x = sum_a slice_a and
-// every product of slices carries its own weight 2^(-8(a+b)) into the
-// tensor-core accumulators.
-__device__ __forceinline__ void cut_slices(float xh, float xl, int s, float* m) {
-    float w = 1.f;
-#pragma unroll
-    for (int a = 0; a < GP_MAX_SLICES; ++a) {
-        if (a < s) {
-            const float q = rintf(xh);
-            m[a] = __fmul_rn(q, w);
-            w = __fmul_rn(w, 0.00390625f);
-            const float dh = __fsub_rn(xh, q);   // exact
-            two_sum(dh, xl, xh, xl);
-            xh = __fmul_rn(xh, 256.f);
-            xl = __fmul_rn(xl, 256.f);
-        } else {
-            m[a] = 0.f;
-        }
-    }
+// The next slice of a double-float x (scaled so |x| < 2^7 before the first
+// one): the integer q nearest x.hi, |q| <= 128, times the slice's weight w =
+// 2^(-8a), so that x = sum_a slice_a and every product of slices carries its
+// own weight 2^(-8(a+b)) into the tensor-core accumulators; x moves on to
+// 256 (x - q).  q comes from the float 1.5 2^23, whose unit is 1 (rintf's
+// instruction runs at a quarter of the rate of an addition).
+__device__ __forceinline__ float cut_one(float& xh, float& xl, float w) {
+    constexpr float kRound = 12582912.f;
+    const float q = __fsub_rn(__fadd_rn(xh, kRound), kRound);
+    two_sum(__fsub_rn(xh, q), xl, xh, xl);       // xh - q is exact
+    xh = __fmul_rn(xh, 256.f);
+    xl = __fmul_rn(xl, 256.f);
+    return __fmul_rn(q, w);
 }
 
 __device__ __forceinline__ void prefetch_l2(const void* p, uint32_t bytes) {
