@@ -190,6 +190,15 @@ cudaError_t launch_trsm_f64(const Batch& b, int J, cudaStream_t s);
 // the tiles of a trailing update: all, column J + 1 only, or the others
 enum : int { kUpdateAll = 0, kUpdateColumn = 1, kUpdateRest = 2 };
 cudaError_t launch_update_f64(const Batch& b, int J, cudaStream_t s, int which = kUpdateAll);
+cudaError_t launch_update_f64_tc(const Batch& b, int J, cudaStream_t s, int which);
+// Block columns from which the double path's trailing updates run on the
+// tensor cores (k_update_tc.cu), whatever the batch.  They are faster from
+// the first tile on (0.55 ms for a tile's 128^3 multiply-adds on one SM's FP64
+// pipe, about 11 us as digit products); up to 256 points the factor keeps
+// IEEE operations throughout, so the small designs that are fitted with p = 2
+// next to singularity (cond(R) 1e11, where any change of rounding shows in
+// the eighth digit of mu_hat) keep their bits.
+constexpr int kUpdateTcTiles = 3;
 cudaError_t launch_forward_solve(const Batch& b, double* Z, size_t z_stride, cudaStream_t s);
 cudaError_t launch_finalize(const Batch& b, const double* Z, size_t z_stride, double* nll,
                             double* mu, double* sigma2, double* logdet, int* status,

@@ -206,6 +206,7 @@ cudaError_t launch_update_f64(const Batch& b, int J, cudaStream_t s, int which) 
     const int m = b.nt - J - 1;
     const int tiles = which == kUpdateColumn ? m : (which == kUpdateRest ? m * (m - 1) / 2 : m * (m + 1) / 2);
     if (tiles <= 0) return cudaSuccess;
+    if (b.nt >= kUpdateTcTiles) return launch_update_f64_tc(b, J, s, which);
     k_update_f64<<<dim3(tiles, b.count), kThreads, 0, s>>>(b, J, which);
     return cudaGetLastError();
 }

@@ -1,0 +1,391 @@
+// k_update_tc.cu -- the trailing update of the double-precision Cholesky,
+// A_IK -= L_IJ L_KJ^T, as exact products of bf16 slices on the tensor cores
+// (after Ozaki, Ogita, Oishi & Rump, "Error-free transformations of matrix
+// multiplication by using fast routines of matrix multiplication", Numer.
+// Algorithms 59, 2012).
+//
+// An off-diagonal entry of L is at most 1 in magnitude, whatever the nugget:
+// sum_{k<i} l_ik^2 = 1 + delta - l_ii^2 and l_ii^2 >= delta for a positive
+// semidefinite R.  So every entry is cut at one fixed scale, with no row
+// exponents:
+//   X = rint(l 2^55) = sum_{a=0..6} q_a 256^(6-a),  |q_a| <= 128 (balanced digits),
+// each digit exact in bf16.  The product groups S_g = sum_{a+b=g} q_a q_b', g =
+// 0 .. 7, summed over the panel's 128 columns in fp32 are integers of at most 7
+// 2^21 < 2^24, hence exact; what is left out, a + b >= 8, is below 2^-64 of
+// 1 per term.  A row's dropped part of l is at most 2^-56, and the rows of L
+// have norm 1, so all panels together leave an error of about 2^-56 in an
+// entry of A, where each IEEE subtraction from A rounds to 2^-53 of it: the
+// factor is as accurate as with double multiply-adds.
+//
+// The digits are cut on the way into shared memory by eight converter
+// warps, from the double tiles themselves: no workspace, so the callers'
+// memory is the same on either path.
+//
+// Bound by the tensor pipe's shared-memory reads (34 digit products of K =
+// 128 columns, 12.7 k cycles a half tile) next to the converters' integer
+// work.  Measured, max |R - L L'| at n = 1500, d = 4, p = 1.5: 4.7e-16 (1.6e-15
+// with double multiply-adds on the FP64 pipe).  Twelve candidates at n = 4064:
+// the updates 16 ms instead of 256 ms (the FP64 pipe's 1.1 TF/s), the batch
+// 270 -> 55 ms; the double fit at n = 4064 54.6 -> 29.8 ms.
+#include "mixed_common.cuh"
+
+namespace gp {
+
+namespace {
+
+constexpr int kNS = 7;                        // digits per entry
+constexpr int kNG = 8;                        // accumulator groups a + b = g
+constexpr int kNT = 64;                       // columns of an output half tile
+static_assert(kNG * kNT <= 512, "accumulators exceed tensor memory");
+constexpr uint32_t kABytes = kNS * kChunkBytes;           // 128 rows x 32 columns, every digit
+constexpr uint32_t kBChunk = kChunkBytes / (GP_NB / kNT);
+constexpr uint32_t kStageBytes = kABytes + kNS * kBChunk;
+constexpr int kConvWarps = 8, kEpiWarps = 8;
+constexpr int kConvBase = 4, kEpiBase = kConvBase + kConvWarps;
+constexpr int kThreads = 32 * (kEpiBase + kEpiWarps);     // warpgroup 0: the MMA warp (and three idle ones)
+constexpr int kPieces = (GP_NB + kNT) / 32 * kChunks / kConvWarps;   // (32 rows x 8 columns) per warp and stage
+// registers after the split; their sum fits the launch's 96 a thread
+constexpr int kMmaRegs = 56, kConvRegs = 96, kEpiRegs = 112;
+static_assert(128 * kMmaRegs + 32 * kConvWarps * kConvRegs + 32 * kEpiWarps * kEpiRegs <= kThreads * 96,
+              "register split exceeds the launch's registers");
+static_assert((GP_NB + kNT) / 32 * 4 % kConvWarps == 0, "pieces per stage do not divide");
+
+// X + the digits' bias: byte 6 - a of the result is q_a + 128 (a >= 1), and
+// the bits from 48 up are q_0 as a signed number.  |l| >= 2 (possible only
+// on the way to a failed factorisation) is cut to 2.
+__device__ __forceinline__ unsigned long long biased_digits(double l) {
+    const unsigned hi = (unsigned)__double2hiint(l), lo = (unsigned)__double2loint(l);
+    const int e = (hi >> 20) & 0x7ff;
+    int r = 1023 - e;                                     // >= 0 for |l| < 2
+    unsigned long long m = ((unsigned long long)((hi & 0xfffffu) | 0x100000u) << 32) | lo;
+    if (r < 0) {
+        m = 0x1fffffffffffffull;
+        r = 0;
+    }
+    // 2 |X| before rounding: |l| 2^56 = m 2^(e - 1019) = (m << 4) >> r
+    const unsigned long long w = r < 64 ? (m << 4) >> r : 0ull;
+    const long long x = (long long)((w + 1) >> 1);
+    const long long s = (long long)(int)hi >> 63;
+    return (unsigned long long)((x ^ s) - s) + 0x0000808080808080ull;
+}
+
+// bf16 pair of two bytes' digits (y - 128 for byte k of u and of v)
+__device__ __forceinline__ uint32_t digit_pair(unsigned u, unsigned v, int k) {
+    const unsigned p = __byte_perm(u, v, k | (k << 4) | ((4 + k) << 8) | ((4 + k) << 12));
+    // 128 + (y & 127), and -128 or -256 by y's top bit: exact in bf16
+    const unsigned t = (p & 0x007f007fu) | 0x43004300u;
+    const unsigned c = (~p & 0x00800080u) | 0xc300c300u;
+    uint32_t r;
+    asm("add.rn.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(t), "r"(c));
+    return r;
+}
+
+__device__ __forceinline__ uint32_t top_pair(unsigned u, unsigned v) {
+    constexpr float kRound = 12582912.f;
+    const float a = __fsub_rn(__int_as_float(0x4b400000 + ((int)u >> 16)), kRound);
+    const float b = __fsub_rn(__int_as_float(0x4b400000 + ((int)v >> 16)), kRound);
+    return pack_bf16x2(a, b);
+}
+
+// Eight columns of one row into the digit images: piece at `dst`, digit a at
+// dst + a * stride.
+__device__ __forceinline__ void store_digits(const double (&l)[8], uint8_t* dst, uint32_t stride) {
+    unsigned yl[8], yh[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+        const unsigned long long y = biased_digits(l[e]);
+        yl[e] = (unsigned)y;
+        yh[e] = (unsigned)(y >> 32);
+    }
+#pragma unroll
+    for (int a = 0; a < kNS; ++a) {
+        uint4 v;
+        uint32_t* q = &v.x;
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+            q[e] = a == 0 ? top_pair(yh[2 * e], yh[2 * e + 1])
+                          : (a <= 2 ? digit_pair(yh[2 * e], yh[2 * e + 1], 2 - a)
+                                    : digit_pair(yl[2 * e], yl[2 * e + 1], 6 - a));
+        *reinterpret_cast<uint4*>(dst + a * stride) = v;
+    }
+}
+
+// The MMAs of one stage (two K = 16 steps): every digit product with a + b <
+// kNG into group a + b; the first stage of a tile overwrites the groups.
+template <bool FIRST>
+__device__ __forceinline__ void issue(uint32_t tacc, uint64_t ad0, uint64_t bd0) {
+    constexpr uint32_t idesc = idesc_bf16(kNT);
+#pragma unroll
+    for (int a = 0; a < kNS; ++a)
+#pragma unroll
+        for (int bb = 0; bb < kNS && a + bb < kNG; ++bb)
+#pragma unroll
+            for (int kk = 0; kk < 2; ++kk) {
+                const bool overwrite = FIRST && kk == 0 && (a == 0 || (a == 1 && bb == kNS - 1));
+                mma_bf16(tacc + (a + bb) * kNT, ad0 + (uint64_t)((a * kChunkBytes + kk * 32) >> 4),
+                         bd0 + (uint64_t)((bb * kBChunk + kk * 32) >> 4), idesc, overwrite ? 0u : 1u);
+            }
+}
+
+__device__ __forceinline__ void tmem_ld4(uint32_t taddr, float* v) {
+    uint32_t r[4];
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(taddr));
+#pragma unroll
+    for (int i = 0; i < 4; ++i) v[i] = __uint_as_float(r[i]);
+}
+
+// sum_g S_g 256^(5 - g), groups 6 and 7 rounded: the product of the two rows
+// in units of 2^-54
+__device__ __forceinline__ long long combine(const float (&s)[kNG]) {
+    const int t01 = __float2int_rn(s[0]) * 256 + __float2int_rn(s[1]);
+    long long v = (long long)t01 << 32;
+    v += (long long)__float2int_rn(s[2]) * (1 << 24);
+    v += (long long)__float2int_rn(s[3]) * (1 << 16);
+    v += (long long)__float2int_rn(s[4]) * (1 << 8);
+    v += __float2int_rn(s[5]);
+    const int t = __float2int_rn(s[6]) + ((__float2int_rn(s[7]) + 128) >> 8);
+    return v + ((t + 128) >> 8);
+}
+
+// Persistent: one CTA per SM walks the half tiles w = blockIdx.x + k gridDim.x
+// (instance-major).  The converter warps cut the operands of one 32-column
+// stage into a two-slot ring that runs on across tiles (each warp loads its
+// part of the next stage as it stores this one's), warp 0 issues the MMAs,
+// the epilogue warps sum the groups into 64-bit integers, release tensor
+// memory and then update C beside the next tile's MMAs.  Every wait is
+// bounded; a timeout marks the instances GP_ETIMEOUT and stops the CTA after
+// its MMAs have landed.
+__global__ void __launch_bounds__(kThreads, 1) k_update_f64_tc(Batch b, int J, int which, int per_inst) {
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    unsigned* live = reinterpret_cast<unsigned*>(smem + 2 * kStageBytes);   // a bit per instance
+    __shared__ __align__(8) uint64_t full_bar[2];
+    __shared__ __align__(8) uint64_t empty_bar[2];
+    __shared__ __align__(8) uint64_t tfull_bar, tempty_bar, drain_bar;
+    __shared__ uint32_t tmem_base;
+    __shared__ volatile int abort_flag;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int total = per_inst * b.count;
+    // the statuses are read once: a look-ahead's diagonal step may set one
+    // while this kernel runs, and the roles must agree on the tiles
+    for (int t0 = 32 * warp; t0 < b.count; t0 += kThreads) {
+        const bool ok = t0 + lane < b.count && *(volatile const int*)&b.st[t0 + lane].status == GP_OK;
+        const unsigned m = __ballot_sync(0xffffffffu, ok);
+        if (lane == 0) live[t0 >> 5] = m;
+    }
+    if (threadIdx.x == 0) {
+        for (int u = 0; u < 2; ++u) {
+            mbar_init(&full_bar[u], 32 * kConvWarps);
+            mbar_init(&empty_bar[u], 1);
+        }
+        mbar_init(&tfull_bar, 1);
+        mbar_init(&tempty_bar, 32 * kEpiWarps);
+        mbar_init(&drain_bar, 1);
+        abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(&tmem_base)));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tbase = tmem_base;
+
+    // first live work item from w on (total when there is none)
+    auto next_live = [&](int w) {
+        while (w < total) {
+            const int t = w / per_inst;
+            if (live[t >> 5] >> (t & 31) & 1) return w;
+            w += gridDim.x;
+        }
+        return total;
+    };
+    auto decode = [&](int w, int& t, int& I, int& K, int& col0) {
+        t = w / per_inst;
+        const int q = w - t * per_inst;
+        col0 = (q & 1) * kNT;
+        int ii, kk;
+        if (which == kUpdateColumn) {
+            ii = q >> 1;
+            kk = 0;
+        } else {
+            tri_decode(q >> 1, ii, kk);
+            if (which == kUpdateRest) {
+                ++ii;
+                ++kk;
+            }
+        }
+        I = J + 1 + ii;
+        K = J + 1 + kk;
+    };
+    auto tile = [&](int t, int I, int K) {
+        return b.A + (size_t)t * b.inst_stride + (size_t)tile_index(I, K, b.nt) * GP_TILE_ELEMS;
+    };
+
+    if (warp >= kEpiBase) {
+        regs_inc<kEpiRegs>();
+        const int q = warp & 3, half = (warp - kEpiBase) >> 2;
+        const int r = q * 32 + lane, c0 = 32 * half;
+        const uint32_t lane_addr = tbase + ((uint32_t)(q * 32) << 16) + c0;
+        int i = 0;
+        for (int w = next_live(blockIdx.x); w < total && !abort_flag; w = next_live(w + gridDim.x), ++i) {
+            int t, I, K, col0;
+            decode(w, t, I, K, col0);
+            double* C = tile(t, I, K) + (size_t)col0 * GP_NB;
+            if (threadIdx.x == 32 * kEpiBase) prefetch_l2(C, kNT * GP_NB * sizeof(double));
+            if (!mbar_wait(&tfull_bar, i & 1, &abort_flag)) {
+                abort_flag = 1;
+                break;
+            }
+            tc_fence_after();
+            long long v[32];
+#pragma unroll
+            for (int c = 0; c < 32; c += 4) {
+                float s[kNG][4];
+#pragma unroll
+                for (int g = 0; g < kNG; ++g) tmem_ld4(lane_addr + g * kNT + c, s[g]);
+                tmem_wait_ld();
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    float u[kNG];
+#pragma unroll
+                    for (int g = 0; g < kNG; ++g) u[g] = s[g][j];
+                    v[c + j] = combine(u);
+                }
+            }
+            tc_fence_before();
+            mbar_arrive(&tempty_bar);
+            double* p = C + (size_t)c0 * GP_NB + r;
+#pragma unroll
+            for (int c = 0; c < 32; c += 8) {
+                double cv[8];
+#pragma unroll
+                for (int j = 0; j < 8; ++j) cv[j] = p[(size_t)(c + j) * GP_NB];
+#pragma unroll
+                for (int j = 0; j < 8; ++j)
+                    p[(size_t)(c + j) * GP_NB] = fma(-__ll2double_rn(v[c + j]), 0x1p-54, cv[j]);
+            }
+        }
+    } else if (warp >= kConvBase) {
+        regs_inc<kConvRegs>();
+        const int cw = warp - kConvBase;
+        // this warp's pieces of a stage: 32 rows (of the 128 of A, then the 64
+        // of B) by 8 columns
+        auto source = [&](int w, int kc, int u) -> const double* {
+            int t, I, K, col0;
+            decode(w, t, I, K, col0);
+            const int piece = cw + kConvWarps * u, rg = piece >> 2, oct = piece & 3;
+            const double* base = rg < 4 ? tile(t, I, J) + 32 * rg : tile(t, K, J) + col0 + 32 * (rg - 4);
+            return base + (size_t)(32 * kc + 8 * oct) * GP_NB + lane;
+        };
+        double raw[kPieces][8];
+        int w = next_live(blockIdx.x), kc = 0;
+        if (w < total) {
+#pragma unroll
+            for (int u = 0; u < kPieces; ++u) {
+                const double* p = source(w, 0, u);
+#pragma unroll
+                for (int e = 0; e < 8; ++e) raw[u][e] = p[e * GP_NB];
+            }
+        }
+        for (int g = 0; w < total && !abort_flag; ++g) {
+            const int st = g & 1;
+            if (g >= 2 && !mbar_wait(&empty_bar[st], ((g >> 1) - 1) & 1, &abort_flag)) {
+                abort_flag = 1;
+                break;
+            }
+            const int kn = (kc + 1) & (kChunks - 1);
+            const int wn = kn == 0 ? next_live(w + gridDim.x) : w;
+            uint8_t* stage = smem + st * kStageBytes;
+#pragma unroll
+            for (int u = 0; u < kPieces; ++u) {
+                const int piece = cw + kConvWarps * u, rg = piece >> 2, oct = piece & 3;
+                const bool isA = rg < 4;
+                uint8_t* dst = stage + (isA ? 0u : kABytes) + image_piece((isA ? 32 * rg : 32 * (rg - 4)) + lane, 8 * oct);
+                store_digits(raw[u], dst, isA ? kChunkBytes : kBChunk);
+                if (wn < total) {
+                    const double* p = source(wn, kn, u);
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) raw[u][e] = p[e * GP_NB];
+                }
+            }
+            // the tensor core reads shared memory through the asynchronous proxy
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            mbar_arrive(&full_bar[st]);
+            w = wn;
+            kc = kn;
+        }
+    } else {
+        regs_dec<kMmaRegs>();
+        if (warp == 0 && lane == 0) {
+            int g = 0, i = 0;
+            for (int w = next_live(blockIdx.x); w < total && !abort_flag; w = next_live(w + gridDim.x), ++i) {
+                if (i >= 1 && !mbar_wait(&tempty_bar, (i - 1) & 1, &abort_flag)) {
+                    abort_flag = 1;
+                    break;
+                }
+                tc_fence_after();
+                for (int kc = 0; kc < kChunks; ++kc, ++g) {
+                    const int st = g & 1;
+                    if (!mbar_wait(&full_bar[st], (g >> 1) & 1, &abort_flag)) {
+                        abort_flag = 1;
+                        break;
+                    }
+                    tc_fence_after();
+                    const uint32_t sa = smem_u32(smem + st * kStageBytes);
+                    const uint64_t ad0 = smem_desc(sa, 16, 512, 4), bd0 = smem_desc(sa + kABytes, 16, 512, 4);
+                    if (kc == 0) issue<true>(tbase, ad0, bd0);
+                    else         issue<false>(tbase, ad0, bd0);
+                    mma_commit(&empty_bar[st]);
+                }
+                if (abort_flag) break;
+                mma_commit(&tfull_bar);
+            }
+            // every MMA issued has completed before tensor memory is released
+            mma_commit(&drain_bar);
+            mbar_wait(&drain_bar, 0);
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    if (abort_flag && threadIdx.x == 0)
+        for (int w = blockIdx.x; w < total; w += gridDim.x) b.st[w / per_inst].status = GP_ETIMEOUT;
+    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tbase));
+}
+
+int sm_count() {
+    static std::atomic<int> cache[kMaxDevices];
+    int dev = 0;
+    cudaGetDevice(&dev);
+    const bool cached = dev >= 0 && dev < kMaxDevices;
+    int n = cached ? cache[dev].load(std::memory_order_relaxed) : 0;
+    if (n == 0) {
+        if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) n = 1;
+        if (cached) cache[dev].store(n, std::memory_order_relaxed);
+    }
+    return n;
+}
+
+}  // namespace
+
+cudaError_t launch_update_f64_tc(const Batch& b, int J, cudaStream_t s, int which) {
+    const int m = b.nt - J - 1;
+    const int tiles = which == kUpdateColumn ? m : (which == kUpdateRest ? m * (m - 1) / 2 : m * (m + 1) / 2);
+    if (tiles <= 0) return cudaSuccess;
+    const size_t smem = 2 * (size_t)kStageBytes + 1024 + (size_t)(b.count + 31) / 32 * 4;
+    static std::atomic<size_t> attr[kMaxDevices];
+    cudaError_t e = raise_smem_limit(k_update_f64_tc, smem, attr);
+    if (e != cudaSuccess) return e;
+    const int per_inst = 2 * tiles;
+    const long long total = (long long)per_inst * b.count;
+    const int grid = (int)(total < sm_count() ? total : sm_count());
+    k_update_f64_tc<<<grid, kThreads, smem, s>>>(b, J, which, per_inst);
+    return cudaGetLastError();
+}
+
+}  // namespace gp
