@@ -205,63 +205,58 @@ int ensure_la(gp_ctx* ctx) {
 constexpr int kLookaheadMax = 16;
 
 // Factor `b.count` instances already assembled in b.A.  A small batch (a
-// fit's one instance) cannot fill the GPU with the serial diagonal step and
+// fit's one instance) cannot fill the GPU with the serial diagonal steps and
 // the panel of a block column, so it looks ahead by one: after the update
-// of column J + 1 (its tiles only), the diagonal step and panel of J + 1 run
-// on a high-priority stream beside the rest of update J (their CTAs fit on
-// an SM beside an update CTA).  Every tile still takes its updates in
-// block-column order on the main stream: the same bits as without.
+// of column J + 1 (its tiles only), block column J + 1 is factored and solved
+// on a high-priority stream beside the rest of update J.  Every tile still
+// takes its updates in block-column order on the main stream: the same bits
+// as without.
 int run_factor_f64(gp_ctx* ctx, const gp::Batch& b) {
     const int nt = b.nt;
-    if (b.count <= kLookaheadMax && nt > 1) {
-        int rc = ensure_la(ctx);
-        if (rc) return rc;
-        {
-            PhaseScope ps(ctx, GP_PHASE_POTRF, 1);
-            GP_CUDA(ctx, gp::launch_potrf_f64(b, 0, ctx->stream));
+    const bool tc = nt >= gp::kUpdateTcTiles;
+    // block column J finished: factored and solved
+    auto panel = [&](int J, cudaStream_t st) -> int {
+        if (tc) {
+            PhaseScope ps(ctx, GP_PHASE_POTRF, gp::panel_f64_launches(nt, J), st);
+            GP_CUDA(ctx, gp::launch_panel_f64(b, J, st));
+            return GP_OK;
         }
         {
-            PhaseScope ps(ctx, GP_PHASE_TRSM, 1);
-            GP_CUDA(ctx, gp::launch_trsm_f64(b, 0, ctx->stream));
+            PhaseScope ps(ctx, GP_PHASE_POTRF, 1, st);
+            GP_CUDA(ctx, gp::launch_potrf_f64(b, J, st));
         }
-        for (int J = 0; J + 1 < nt; ++J) {
-            {
-                PhaseScope ps(ctx, GP_PHASE_UPDATE, 1);
-                GP_CUDA(ctx, gp::launch_update_f64(b, J, ctx->stream, gp::kUpdateColumn));
-            }
-            GP_CUDA(ctx, cudaEventRecord(ctx->ev_la0, ctx->stream));
-            GP_CUDA(ctx, cudaStreamWaitEvent(ctx->la, ctx->ev_la0, 0));
-            {
-                PhaseScope ps(ctx, GP_PHASE_POTRF, 1, ctx->la);
-                GP_CUDA(ctx, gp::launch_potrf_f64(b, J + 1, ctx->la));
-            }
-            if (J + 2 < nt) {
-                PhaseScope ps(ctx, GP_PHASE_TRSM, 1, ctx->la);
-                GP_CUDA(ctx, gp::launch_trsm_f64(b, J + 1, ctx->la));
-            }
-            GP_CUDA(ctx, cudaEventRecord(ctx->ev_la1, ctx->la));
-            if (J + 2 < nt) {
-                PhaseScope ps(ctx, GP_PHASE_UPDATE, 1);
-                GP_CUDA(ctx, gp::launch_update_f64(b, J, ctx->stream, gp::kUpdateRest));
-            }
-            GP_CUDA(ctx, cudaStreamWaitEvent(ctx->stream, ctx->ev_la1, 0));
+        if (J + 1 < nt) {
+            PhaseScope ps(ctx, GP_PHASE_TRSM, 1, st);
+            GP_CUDA(ctx, gp::launch_trsm_f64(b, J, st));
         }
         return GP_OK;
+    };
+    auto update = [&](int J, int which) -> int {
+        PhaseScope ps(ctx, GP_PHASE_UPDATE, 1);
+        GP_CUDA(ctx, gp::launch_update_f64(b, J, ctx->stream, which));
+        return GP_OK;
+    };
+    const bool ahead = b.count <= kLookaheadMax && nt > 1;
+    int rc = ahead ? ensure_la(ctx) : GP_OK;
+    if (rc) return rc;
+    if ((rc = panel(0, ctx->stream))) return rc;
+    for (int J = 0; J + 1 < nt; ++J) {
+        if (!ahead) {
+            if ((rc = update(J, gp::kUpdateAll))) return rc;
+            if ((rc = panel(J + 1, ctx->stream))) return rc;
+            continue;
+        }
+        if ((rc = update(J, gp::kUpdateColumn))) return rc;
+        GP_CUDA(ctx, cudaEventRecord(ctx->ev_la0, ctx->stream));
+        GP_CUDA(ctx, cudaStreamWaitEvent(ctx->la, ctx->ev_la0, 0));
+        if ((rc = panel(J + 1, ctx->la))) return rc;
+        GP_CUDA(ctx, cudaEventRecord(ctx->ev_la1, ctx->la));
+        if (J + 2 < nt && (rc = update(J, gp::kUpdateRest))) return rc;
+        GP_CUDA(ctx, cudaStreamWaitEvent(ctx->stream, ctx->ev_la1, 0));
     }
-    for (int J = 0; J < b.nt; ++J) {
-        const int more = (J + 1 < b.nt) ? 1 : 0;
-        {
-            PhaseScope ps(ctx, GP_PHASE_POTRF, 1);
-            GP_CUDA(ctx, gp::launch_potrf_f64(b, J, ctx->stream));
-        }
-        if (more) {
-            PhaseScope ps(ctx, GP_PHASE_TRSM, 1);
-            GP_CUDA(ctx, gp::launch_trsm_f64(b, J, ctx->stream));
-        }
-        if (more) {
-            PhaseScope ps(ctx, GP_PHASE_UPDATE, 1);
-            GP_CUDA(ctx, gp::launch_update_f64(b, J, ctx->stream));
-        }
+    if (tc) {
+        PhaseScope ps(ctx, GP_PHASE_POTRF, 1);
+        GP_CUDA(ctx, gp::launch_logdet_f64(b, ctx->stream));
     }
     return GP_OK;
 }

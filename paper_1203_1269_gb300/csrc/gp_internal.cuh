@@ -172,6 +172,20 @@ inline cudaError_t raise_smem_limit(Kernel* kernel, size_t bytes, std::atomic<si
     return e;
 }
 
+// SMs of the current device (looked up once per device ordinal)
+inline int device_sms() {
+    static std::atomic<int> cache[kMaxDevices];
+    int dev = 0;
+    cudaGetDevice(&dev);
+    const bool cached = dev >= 0 && dev < kMaxDevices;
+    int n = cached ? cache[dev].load(std::memory_order_relaxed) : 0;
+    if (n == 0) {
+        if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) n = 1;
+        if (cached) cache[dev].store(n, std::memory_order_relaxed);
+    }
+    return n;
+}
+
 // ---- context accessors (gp_capi.cu) ----------------------------------------
 int ctx_fail(gp_ctx* ctx, int code, const char* fmt, ...);
 int ctx_device(const gp_ctx* ctx);
@@ -188,9 +202,17 @@ cudaError_t launch_assemble_dense(int n, int d, const double* x, const double* t
 cudaError_t launch_potrf_f64(const Batch& b, int J, cudaStream_t s);
 cudaError_t launch_trsm_f64(const Batch& b, int J, cudaStream_t s);
 // the tiles of a trailing update: all, column J + 1 only, or the others
-enum : int { kUpdateAll = 0, kUpdateColumn = 1, kUpdateRest = 2 };
+enum : int { kUpdateAll = 0, kUpdateColumn = 1, kUpdateRest = 2, kUpdateInner = 3 };
 cudaError_t launch_update_f64(const Batch& b, int J, cudaStream_t s, int which = kUpdateAll);
 cudaError_t launch_update_f64_tc(const Batch& b, int J, cudaStream_t s, int which);
+// columns 32 step .. 32 step + 31 of block column J, less the products of its columns before them
+cudaError_t launch_update_f64_inner(const Batch& b, int J, int step, cudaStream_t s);
+// block column J factored and solved (kUpdateTcTiles block columns and more), and the
+// log-determinant once they all are
+constexpr int kPanelStep = 32;
+int panel_f64_launches(int nt, int J);
+cudaError_t launch_panel_f64(const Batch& b, int J, cudaStream_t s);
+cudaError_t launch_logdet_f64(const Batch& b, cudaStream_t s);
 // Block columns from which the double path's trailing updates run on the
 // tensor cores (k_update_tc.cu), whatever the batch.  They are faster from
 // the first tile on (0.55 ms for a tile's 128^3 multiply-adds on one SM's FP64

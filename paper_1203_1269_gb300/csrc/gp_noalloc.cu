@@ -85,10 +85,15 @@ extern "C" int gp_nll_batch_noalloc(gp_ctx* ctx, int n, int d, const double* x, 
         e = gp::launch_validate_theta(b, stream);
         if (e == cudaSuccess) e = gp::launch_assemble_tiles(b, stream);
         for (int J = 0; J < nt && e == cudaSuccess; ++J) {
-            e = gp::launch_potrf_f64(b, J, stream);
-            if (e == cudaSuccess) e = gp::launch_trsm_f64(b, J, stream);
+            if (nt >= gp::kUpdateTcTiles) {
+                e = gp::launch_panel_f64(b, J, stream);
+            } else {
+                e = gp::launch_potrf_f64(b, J, stream);
+                if (e == cudaSuccess) e = gp::launch_trsm_f64(b, J, stream);
+            }
             if (e == cudaSuccess) e = gp::launch_update_f64(b, J, stream);
         }
+        if (nt >= gp::kUpdateTcTiles && e == cudaSuccess) e = gp::launch_logdet_f64(b, stream);
         const size_t zs = z_bytes / sizeof(double);
         if (e == cudaSuccess) e = gp::launch_forward_solve(b, Z, zs, stream);
         if (e == cudaSuccess)

@@ -1,5 +1,7 @@
 // k_chol_f64.cu -- blocked right-looking Cholesky R = L L' in IEEE double
-// over a batch of independent instances (one per theta candidate).
+// over a batch of independent instances (one per theta candidate), for
+// matrices of up to two block columns (launch_update_f64 sends larger ones to
+// k_update_tc.cu; their block columns are factored by k_panel_f64.cu).
 //
 // The paper factors R by Cholesky on the CPU and by LU on its GPU (Section
 // 3); here R is symmetric positive definite, so Cholesky is used throughout.

@@ -564,20 +564,6 @@ __global__ void __launch_bounds__(ER ? kGemmThreadsER : kGemmThreads, 1)
 
 }  // namespace
 
-// SMs of the current device (looked up once per device ordinal)
-static int sm_count() {
-    static std::atomic<int> cache[kMaxDevices];
-    int dev = 0;
-    cudaGetDevice(&dev);
-    const bool cached = dev >= 0 && dev < kMaxDevices;
-    int n = cached ? cache[dev].load(std::memory_order_relaxed) : 0;
-    if (n == 0) {
-        if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) n = 1;
-        if (cached) cache[dev].store(n, std::memory_order_relaxed);
-    }
-    return n;
-}
-
 template <int MODE, int NT, int NG, bool ER = false>
 static cudaError_t launch_gemm(const MixedBatch& b, int J, int per_inst, int ns, cudaStream_t s, int kind = 0) {
     const size_t smem = (size_t)2 * ns * (kChunkBytes + kChunkBytes / (GP_NB / NT)) + 1024;
@@ -585,7 +571,7 @@ static cudaError_t launch_gemm(const MixedBatch& b, int J, int per_inst, int ns,
     cudaError_t e = raise_smem_limit(k_split_gemm<MODE, NT, NG, ER>, smem, attr);
     if (e != cudaSuccess) return e;
     const long long total = (long long)per_inst * b.count;
-    const int grid = (int)(total < sm_count() ? total : sm_count());
+    const int grid = (int)(total < device_sms() ? total : device_sms());
     k_split_gemm<MODE, NT, NG, ER><<<grid, ER ? kGemmThreadsER : kGemmThreads, smem, s>>>(b, J, per_inst, kind);
     return cudaGetLastError();
 }

@@ -25,7 +25,7 @@
 // 128 columns, 12.7 k cycles a half tile) next to the converters' integer
 // work.  Measured, max |R - L L'| at n = 1500, d = 4, p = 1.5: 4.7e-16 (1.6e-15
 // with double multiply-adds on the FP64 pipe).  Twelve candidates at n = 4064:
-// the updates 16 ms instead of 256 ms (the FP64 pipe's 1.1 TF/s), the batch
+// the updates 17 ms instead of 256 ms (the FP64 pipe's 1.1 TF/s), the batch
 // 270 -> 55 ms; the double fit at n = 4064 54.6 -> 29.8 ms.
 #include "mixed_common.cuh"
 
@@ -35,20 +35,19 @@ namespace {
 
 constexpr int kNS = 7;                        // digits per entry
 constexpr int kNG = 8;                        // accumulator groups a + b = g
-constexpr int kNT = 64;                       // columns of an output half tile
-static_assert(kNG * kNT <= 512, "accumulators exceed tensor memory");
 constexpr uint32_t kABytes = kNS * kChunkBytes;           // 128 rows x 32 columns, every digit
-constexpr uint32_t kBChunk = kChunkBytes / (GP_NB / kNT);
-constexpr uint32_t kStageBytes = kABytes + kNS * kBChunk;
+// NT columns of an output tile (64: half tiles of the trailing update; 32: a
+// panel's inner update)
+constexpr uint32_t b_chunk(int nt) { return kChunkBytes / (GP_NB / nt); }
+constexpr uint32_t stage_bytes(int nt) { return kABytes + kNS * b_chunk(nt); }
 constexpr int kConvWarps = 8, kEpiWarps = 8;
 constexpr int kConvBase = 4, kEpiBase = kConvBase + kConvWarps;
 constexpr int kThreads = 32 * (kEpiBase + kEpiWarps);     // warpgroup 0: the MMA warp (and three idle ones)
-constexpr int kPieces = (GP_NB + kNT) / 32 * kChunks / kConvWarps;   // (32 rows x 8 columns) per warp and stage
+constexpr int kPieces = 3;                                // most (32 rows x 8 columns) pieces of a stage per warp
 // registers after the split; their sum fits the launch's 96 a thread
 constexpr int kMmaRegs = 56, kConvRegs = 96, kEpiRegs = 112;
 static_assert(128 * kMmaRegs + 32 * kConvWarps * kConvRegs + 32 * kEpiWarps * kEpiRegs <= kThreads * 96,
               "register split exceeds the launch's registers");
-static_assert((GP_NB + kNT) / 32 * 4 % kConvWarps == 0, "pieces per stage do not divide");
 
 // X + the digits' bias: byte 6 - a of the result is q_a + 128 (a >= 1), and
 // the bits from 48 up are q_0 as a signed number.  |l| >= 2 (possible only
@@ -112,9 +111,9 @@ __device__ __forceinline__ void store_digits(const double (&l)[8], uint8_t* dst,
 
 // The MMAs of one stage (two K = 16 steps): every digit product with a + b <
 // kNG into group a + b; the first stage of a tile overwrites the groups.
-template <bool FIRST>
+template <int kNT, bool FIRST>
 __device__ __forceinline__ void issue(uint32_t tacc, uint64_t ad0, uint64_t bd0) {
-    constexpr uint32_t idesc = idesc_bf16(kNT);
+    constexpr uint32_t idesc = idesc_bf16(kNT), kBChunk = b_chunk(kNT);
 #pragma unroll
     for (int a = 0; a < kNS; ++a)
 #pragma unroll
@@ -157,7 +156,19 @@ __device__ __forceinline__ long long combine(const float (&s)[kNG]) {
 // memory and then update C beside the next tile's MMAs.  Every wait is
 // bounded; a timeout marks the instances GP_ETIMEOUT and stops the CTA after
 // its MMAs have landed.
-__global__ void __launch_bounds__(kThreads, 1) k_update_f64_tc(Batch b, int J, int which, int per_inst) {
+//
+// NT = 32 (which = kUpdateInner, chunks = s): columns 32 s .. 32 s + 31 of block
+// column J itself take the products of its columns before them, for the rows
+// from 32 s of tile (J, J) down.
+template <int kNT>
+__global__ void __launch_bounds__(kThreads, 1)
+    k_update_f64_tc(Batch b, int J, int which, int per_inst, int chunks) {
+    constexpr bool kInner = kNT == 32;
+    constexpr uint32_t kBChunk = b_chunk(kNT), kStageBytes = stage_bytes(kNT);
+    constexpr int kStagePieces = (GP_NB + kNT) / 32 * 4;
+    constexpr int kEpiCols = kNT / 2;          // columns of an epilogue warp
+    static_assert(kNG * kNT <= 512, "accumulators exceed tensor memory");
+    static_assert(kStagePieces <= kPieces * kConvWarps, "pieces per stage");
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     unsigned* live = reinterpret_cast<unsigned*>(smem + 2 * kStageBytes);   // a bit per instance
@@ -207,6 +218,12 @@ __global__ void __launch_bounds__(kThreads, 1) k_update_f64_tc(Batch b, int J, i
     auto decode = [&](int w, int& t, int& I, int& K, int& col0) {
         t = w / per_inst;
         const int q = w - t * per_inst;
+        if (kInner) {
+            I = J + q;
+            K = J;
+            col0 = kNT * chunks;
+            return;
+        }
         col0 = (q & 1) * kNT;
         int ii, kk;
         if (which == kUpdateColumn) {
@@ -229,7 +246,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_update_f64_tc(Batch b, int J, i
     if (warp >= kEpiBase) {
         regs_inc<kEpiRegs>();
         const int q = warp & 3, half = (warp - kEpiBase) >> 2;
-        const int r = q * 32 + lane, c0 = 32 * half;
+        const int r = q * 32 + lane, c0 = kEpiCols * half;
         const uint32_t lane_addr = tbase + ((uint32_t)(q * 32) << 16) + c0;
         int i = 0;
         for (int w = next_live(blockIdx.x); w < total && !abort_flag; w = next_live(w + gridDim.x), ++i) {
@@ -242,9 +259,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_update_f64_tc(Batch b, int J, i
                 break;
             }
             tc_fence_after();
-            long long v[32];
+            long long v[kEpiCols];
 #pragma unroll
-            for (int c = 0; c < 32; c += 4) {
+            for (int c = 0; c < kEpiCols; c += 4) {
                 float s[kNG][4];
 #pragma unroll
                 for (int g = 0; g < kNG; ++g) tmem_ld4(lane_addr + g * kNT + c, s[g]);
@@ -259,9 +276,12 @@ __global__ void __launch_bounds__(kThreads, 1) k_update_f64_tc(Batch b, int J, i
             }
             tc_fence_before();
             mbar_arrive(&tempty_bar);
+            // the rows of the diagonal tile above the inner update's columns
+            // are finished
+            if (kInner && I == K && r < col0) continue;
             double* p = C + (size_t)c0 * GP_NB + r;
 #pragma unroll
-            for (int c = 0; c < 32; c += 8) {
+            for (int c = 0; c < kEpiCols; c += 8) {
                 double cv[8];
 #pragma unroll
                 for (int j = 0; j < 8; ++j) cv[j] = p[(size_t)(c + j) * GP_NB];
@@ -278,7 +298,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_update_f64_tc(Batch b, int J, i
         auto source = [&](int w, int kc, int u) -> const double* {
             int t, I, K, col0;
             decode(w, t, I, K, col0);
-            const int piece = cw + kConvWarps * u, rg = piece >> 2, oct = piece & 3;
+            const int piece = min(cw + kConvWarps * u, kStagePieces - 1), rg = piece >> 2, oct = piece & 3;
             const double* base = rg < 4 ? tile(t, I, J) + 32 * rg : tile(t, K, J) + col0 + 32 * (rg - 4);
             return base + (size_t)(32 * kc + 8 * oct) * GP_NB + lane;
         };
@@ -298,7 +318,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_update_f64_tc(Batch b, int J, i
                 abort_flag = 1;
                 break;
             }
-            const int kn = (kc + 1) & (kChunks - 1);
+            const int kn = kc + 1 == chunks ? 0 : kc + 1;
             const int wn = kn == 0 ? next_live(w + gridDim.x) : w;
             uint8_t* stage = smem + st * kStageBytes;
 #pragma unroll
@@ -306,7 +326,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_update_f64_tc(Batch b, int J, i
                 const int piece = cw + kConvWarps * u, rg = piece >> 2, oct = piece & 3;
                 const bool isA = rg < 4;
                 uint8_t* dst = stage + (isA ? 0u : kABytes) + image_piece((isA ? 32 * rg : 32 * (rg - 4)) + lane, 8 * oct);
-                store_digits(raw[u], dst, isA ? kChunkBytes : kBChunk);
+                if (piece < kStagePieces) store_digits(raw[u], dst, isA ? kChunkBytes : kBChunk);
                 if (wn < total) {
                     const double* p = source(wn, kn, u);
 #pragma unroll
@@ -329,7 +349,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_update_f64_tc(Batch b, int J, i
                     break;
                 }
                 tc_fence_after();
-                for (int kc = 0; kc < kChunks; ++kc, ++g) {
+                for (int kc = 0; kc < chunks; ++kc, ++g) {
                     const int st = g & 1;
                     if (!mbar_wait(&full_bar[st], (g >> 1) & 1, &abort_flag)) {
                         abort_flag = 1;
@@ -338,8 +358,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_update_f64_tc(Batch b, int J, i
                     tc_fence_after();
                     const uint32_t sa = smem_u32(smem + st * kStageBytes);
                     const uint64_t ad0 = smem_desc(sa, 16, 512, 4), bd0 = smem_desc(sa + kABytes, 16, 512, 4);
-                    if (kc == 0) issue<true>(tbase, ad0, bd0);
-                    else         issue<false>(tbase, ad0, bd0);
+                    if (kc == 0) issue<kNT, true>(tbase, ad0, bd0);
+                    else         issue<kNT, false>(tbase, ad0, bd0);
                     mma_commit(&empty_bar[st]);
                 }
                 if (abort_flag) break;
@@ -358,17 +378,22 @@ __global__ void __launch_bounds__(kThreads, 1) k_update_f64_tc(Batch b, int J, i
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tbase));
 }
 
-int sm_count() {
-    static std::atomic<int> cache[kMaxDevices];
-    int dev = 0;
-    cudaGetDevice(&dev);
-    const bool cached = dev >= 0 && dev < kMaxDevices;
-    int n = cached ? cache[dev].load(std::memory_order_relaxed) : 0;
-    if (n == 0) {
-        if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) n = 1;
-        if (cached) cache[dev].store(n, std::memory_order_relaxed);
-    }
-    return n;
+template <int NT>
+cudaError_t launch(const Batch& b, int J, cudaStream_t s, int which, int per_inst, int chunks) {
+    const size_t smem = 2 * (size_t)stage_bytes(NT) + 1024 + (size_t)(b.count + 31) / 32 * 4;
+    static std::atomic<size_t> attr[kMaxDevices];
+    cudaError_t e = raise_smem_limit(k_update_f64_tc<NT>, smem, attr);
+    if (e != cudaSuccess) return e;
+    const long long total = (long long)per_inst * b.count;
+    // the rest of an update runs beside the next block column's panel, whose
+    // kernels cannot share an SM with this one: a third of the SMs stay free
+    // for them (n = 4064, one candidate: 14.25 ms without the look-ahead, 14.4
+    // with every SM taken, 13.55 with a third or a half free; twelve: 38.6,
+    // 38.5, 37.3 and 44.2 ms)
+    const int cap = which == kUpdateRest ? device_sms() - device_sms() / 3 : device_sms();
+    const int grid = (int)(total < cap ? total : cap);
+    k_update_f64_tc<NT><<<grid, kThreads, smem, s>>>(b, J, which, per_inst, chunks);
+    return cudaGetLastError();
 }
 
 }  // namespace
@@ -377,15 +402,11 @@ cudaError_t launch_update_f64_tc(const Batch& b, int J, cudaStream_t s, int whic
     const int m = b.nt - J - 1;
     const int tiles = which == kUpdateColumn ? m : (which == kUpdateRest ? m * (m - 1) / 2 : m * (m + 1) / 2);
     if (tiles <= 0) return cudaSuccess;
-    const size_t smem = 2 * (size_t)kStageBytes + 1024 + (size_t)(b.count + 31) / 32 * 4;
-    static std::atomic<size_t> attr[kMaxDevices];
-    cudaError_t e = raise_smem_limit(k_update_f64_tc, smem, attr);
-    if (e != cudaSuccess) return e;
-    const int per_inst = 2 * tiles;
-    const long long total = (long long)per_inst * b.count;
-    const int grid = (int)(total < sm_count() ? total : sm_count());
-    k_update_f64_tc<<<grid, kThreads, smem, s>>>(b, J, which, per_inst);
-    return cudaGetLastError();
+    return launch<64>(b, J, s, which, 2 * tiles, kChunks);
+}
+
+cudaError_t launch_update_f64_inner(const Batch& b, int J, int step, cudaStream_t s) {
+    return launch<32>(b, J, s, kUpdateInner, b.nt - J, step);
 }
 
 }  // namespace gp
