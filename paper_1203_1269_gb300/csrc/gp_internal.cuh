@@ -202,13 +202,16 @@ cudaError_t launch_assemble_dense(int n, int d, const double* x, const double* t
 cudaError_t launch_potrf_f64(const Batch& b, int J, cudaStream_t s);
 cudaError_t launch_trsm_f64(const Batch& b, int J, cudaStream_t s);
 // the tiles of a trailing update: all, column J + 1 only, or the others
-enum : int { kUpdateAll = 0, kUpdateColumn = 1, kUpdateRest = 2, kUpdateInner = 3 };
+enum : int { kUpdateAll = 0, kUpdateColumn = 1, kUpdateRest = 2 };
 cudaError_t launch_update_f64(const Batch& b, int J, cudaStream_t s, int which = kUpdateAll);
 cudaError_t launch_update_f64_tc(const Batch& b, int J, cudaStream_t s, int which);
 // columns 32 step .. 32 step + 31 of block column J, less the products of its columns before them
 cudaError_t launch_update_f64_inner(const Batch& b, int J, int step, cudaStream_t s);
 // block column J factored and solved (kUpdateTcTiles block columns and more), and the
 // log-determinant once they all are
+// steps of X = L^-1 and R^-1 = X'X by rows of X (k_grad.cu, k_update_tc.cu)
+cudaError_t launch_inverse_apply(const Batch& b, int J, double* X, double* S, cudaStream_t s);
+cudaError_t launch_inverse_update(const Batch& b, int J, double* X, double* S, cudaStream_t s);
 constexpr int kPanelStep = 32;
 int panel_f64_launches(int nt, int J);
 cudaError_t launch_panel_f64(const Batch& b, int J, cudaStream_t s);

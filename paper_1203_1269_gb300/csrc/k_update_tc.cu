@@ -52,10 +52,11 @@ static_assert(128 * kMmaRegs + 32 * kConvWarps * kConvRegs + 32 * kEpiWarps * kE
 // X + the digits' bias: byte 6 - a of the result is q_a + 128 (a >= 1), and
 // the bits from 48 up are q_0 as a signed number.  |l| >= 2 (possible only
 // on the way to a failed factorisation) is cut to 2.
-__device__ __forceinline__ unsigned long long biased_digits(double l) {
+// E: the operand's exponent, X = rint(l 2^(55 - E)).
+__device__ __forceinline__ unsigned long long biased_digits(double l, int E) {
     const unsigned hi = (unsigned)__double2hiint(l), lo = (unsigned)__double2loint(l);
     const int e = (hi >> 20) & 0x7ff;
-    int r = 1023 - e;                                     // >= 0 for |l| < 2
+    int r = 1023 + E - e;                                 // >= 0 for |l| < 2^(E + 1)
     unsigned long long m = ((unsigned long long)((hi & 0xfffffu) | 0x100000u) << 32) | lo;
     if (r < 0) {
         m = 0x1fffffffffffffull;
@@ -88,11 +89,11 @@ __device__ __forceinline__ uint32_t top_pair(unsigned u, unsigned v) {
 
 // Eight columns of one row into the digit images: piece at `dst`, digit a at
 // dst + a * stride.
-__device__ __forceinline__ void store_digits(const double (&l)[8], uint8_t* dst, uint32_t stride) {
+__device__ __forceinline__ void store_digits(const double (&l)[8], int E, uint8_t* dst, uint32_t stride) {
     unsigned yl[8], yh[8];
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
-        const unsigned long long y = biased_digits(l[e]);
+        const unsigned long long y = biased_digits(l[e], E);
         yl[e] = (unsigned)y;
         yh[e] = (unsigned)(y >> 32);
     }
@@ -148,6 +149,8 @@ __device__ __forceinline__ long long combine(const float (&s)[kNG]) {
     return v + ((t + 128) >> 8);
 }
 
+enum : int { kFactorMode = 0, kInnerMode = 1, kInvApply = 2, kInvUpdate = 3 };
+
 // Persistent: one CTA per SM walks the half tiles w = blockIdx.x + k gridDim.x
 // (instance-major).  The converter warps cut the operands of one 32-column
 // stage into a two-slot ring that runs on across tiles (each warp loads its
@@ -157,13 +160,23 @@ __device__ __forceinline__ long long combine(const float (&s)[kNG]) {
 // bounded; a timeout marks the instances GP_ETIMEOUT and stops the CTA after
 // its MMAs have landed.
 //
-// NT = 32 (which = kUpdateInner, chunks = s): columns 32 s .. 32 s + 31 of block
-// column J itself take the products of its columns before them, for the rows
-// from 32 s of tile (J, J) down.
-template <int kNT>
+// MODE kInner (NT = 32, chunks = s): columns 32 s .. 32 s + 31 of block column J
+// itself take the products of its columns before them, for the rows from
+// 32 s of tile (J, J) down.
+//
+// MODE kInvApply, kInvUpdate: the same machine on the rows of X = L^-1
+// (k_grad.cu), whose columns are cut at their own exponents:
+//   apply   X_JK = -W_J S_JK                              K < J
+//   update  S_IK += L_IJ X_JK (I > J),  (R^-1)_IK += X_JI' X_JK (I <= J),  K <= J,
+// S and R^-1 sharing one set of tiles (row J of S is consumed by step J).
+// The exponents lie in the factor's own diagonal tiles, which the inverse no
+// longer needs: tile (K, K) holds those of X_JK's columns, of S_JK's columns
+// and of W_K's rows.
+template <int kNT, int MODE>
 __global__ void __launch_bounds__(kThreads, 1)
-    k_update_f64_tc(Batch b, int J, int which, int per_inst, int chunks) {
-    constexpr bool kInner = kNT == 32;
+    k_update_f64_tc(Batch b, int J, int which, int per_inst, int chunks, double* X, double* S) {
+    constexpr bool kInner = MODE == kInnerMode;
+    constexpr bool kInv = MODE == kInvApply || MODE == kInvUpdate;
     constexpr uint32_t kBChunk = b_chunk(kNT), kStageBytes = stage_bytes(kNT);
     constexpr int kStagePieces = (GP_NB + kNT) / 32 * 4;
     constexpr int kEpiCols = kNT / 2;          // columns of an epilogue warp
@@ -225,6 +238,21 @@ __global__ void __launch_bounds__(kThreads, 1)
             return;
         }
         col0 = (q & 1) * kNT;
+        if (MODE == kInvApply) {
+            I = J;
+            K = q >> 1;
+            return;
+        }
+        if (MODE == kInvUpdate) {
+            const int lower = (b.nt - 1 - J) * (J + 1), v = q >> 1;
+            if (v < lower) {
+                I = J + 1 + v / (J + 1);
+                K = v % (J + 1);
+            } else {
+                tri_decode(v - lower, I, K);
+            }
+            return;
+        }
         int ii, kk;
         if (which == kUpdateColumn) {
             ii = q >> 1;
@@ -239,9 +267,11 @@ __global__ void __launch_bounds__(kThreads, 1)
         I = J + 1 + ii;
         K = J + 1 + kk;
     };
-    auto tile = [&](int t, int I, int K) {
-        return b.A + (size_t)t * b.inst_stride + (size_t)tile_index(I, K, b.nt) * GP_TILE_ELEMS;
+    auto tile_of = [&](double* base, int t, int I, int K) {
+        return base + (size_t)t * b.inst_stride + (size_t)tile_index(I, K, b.nt) * GP_TILE_ELEMS;
     };
+    auto tile = [&](int t, int I, int K) { return tile_of(b.A, t, I, K); };
+    auto exps = [&](int t, int K, int slot) { return reinterpret_cast<const int*>(tile(t, K, K)) + slot * GP_NB; };
 
     if (warp >= kEpiBase) {
         regs_inc<kEpiRegs>();
@@ -252,8 +282,13 @@ __global__ void __launch_bounds__(kThreads, 1)
         for (int w = next_live(blockIdx.x); w < total && !abort_flag; w = next_live(w + gridDim.x), ++i) {
             int t, I, K, col0;
             decode(w, t, I, K, col0);
-            double* C = tile(t, I, K) + (size_t)col0 * GP_NB;
-            if (threadIdx.x == 32 * kEpiBase) prefetch_l2(C, kNT * GP_NB * sizeof(double));
+            double* C = (MODE == kInvApply    ? tile_of(X, t, I, K)
+                         : MODE == kInvUpdate ? tile_of(S, t, I, K)
+                                              : tile(t, I, K)) + (size_t)col0 * GP_NB;
+            // what the products are added to: nothing the first time a tile of S
+            // (K = J) or of R^-1 (I = J) is reached
+            const bool fresh = MODE == kInvApply || (MODE == kInvUpdate && (I > J ? K == J : I == J));
+            if (threadIdx.x == 32 * kEpiBase && !fresh) prefetch_l2(C, kNT * GP_NB * sizeof(double));
             if (!mbar_wait(&tfull_bar, i & 1, &abort_flag)) {
                 abort_flag = 1;
                 break;
@@ -280,37 +315,69 @@ __global__ void __launch_bounds__(kThreads, 1)
             // are finished
             if (kInner && I == K && r < col0) continue;
             double* p = C + (size_t)c0 * GP_NB + r;
+            // the rows' exponents (MODE kInvUpdate: of L_IJ none, of X_JI' its columns')
+            int ea = 0;
+            const int* eb = nullptr;
+            if (kInv) {
+                ea = MODE == kInvApply ? exps(t, J, 2)[r] : (I > J ? 0 : exps(t, I, 0)[r]);
+                eb = exps(t, K, MODE == kInvApply ? 1 : 0) + col0 + c0;
+            }
 #pragma unroll
             for (int c = 0; c < kEpiCols; c += 8) {
                 double cv[8];
 #pragma unroll
-                for (int j = 0; j < 8; ++j) cv[j] = p[(size_t)(c + j) * GP_NB];
+                for (int j = 0; j < 8; ++j) cv[j] = fresh ? 0.0 : p[(size_t)(c + j) * GP_NB];
 #pragma unroll
-                for (int j = 0; j < 8; ++j)
-                    p[(size_t)(c + j) * GP_NB] = fma(-__ll2double_rn(v[c + j]), 0x1p-54, cv[j]);
+                for (int j = 0; j < 8; ++j) {
+                    double scale = 0x1p-54;
+                    if (kInv) {
+                        const int e = 1023 - 54 + ea + eb[c + j];      // 0 below the normal range
+                        scale = __hiloint2double(e > 0 ? e << 20 : 0, 0);
+                    }
+                    const double d = __ll2double_rn(v[c + j]);
+                    p[(size_t)(c + j) * GP_NB] = fma(MODE == kInvUpdate ? d : -d, scale, cv[j]);
+                }
             }
         }
     } else if (warp >= kConvBase) {
         regs_inc<kConvRegs>();
         const int cw = warp - kConvBase;
-        // this warp's pieces of a stage: 32 rows (of the 128 of A, then the 64
-        // of B) by 8 columns
-        auto source = [&](int w, int kc, int u) -> const double* {
+        // this warp's pieces of a stage: 32 rows (of the 128 of A, then the NT
+        // of B) by 8 columns.  Operand rows run along a tile's columns for L and
+        // W, along its rows (eight consecutive doubles a lane) for X and S.
+        auto load = [&](int w, int kc, int u, double (&v)[8], int& E) {
             int t, I, K, col0;
             decode(w, t, I, K, col0);
             const int piece = min(cw + kConvWarps * u, kStagePieces - 1), rg = piece >> 2, oct = piece & 3;
-            const double* base = rg < 4 ? tile(t, I, J) + 32 * rg : tile(t, K, J) + col0 + 32 * (rg - 4);
-            return base + (size_t)(32 * kc + 8 * oct) * GP_NB + lane;
+            const bool isA = rg < 4;
+            const int row = (isA ? 32 * rg : col0 + 32 * (rg - 4)) + lane, k0 = 32 * kc + 8 * oct;
+            E = 0;
+            if (kInv) {
+                const bool byRow = isA && (MODE == kInvApply || I > J);
+                const double* src;
+                if (MODE == kInvApply) {
+                    src = isA ? tile_of(X, t, J, J) : tile_of(S, t, J, K);
+                    E = isA ? exps(t, J, 2)[row] : exps(t, K, 1)[row];
+                } else {
+                    src = byRow ? tile(t, I, J) : tile_of(X, t, J, isA ? I : K);
+                    if (!byRow) E = exps(t, isA ? I : K, 0)[row];
+                }
+                const double* p = byRow ? src + (size_t)k0 * GP_NB + row : src + (size_t)row * GP_NB + k0;
+                const int step = byRow ? GP_NB : 1;
+#pragma unroll
+                for (int e = 0; e < 8; ++e) v[e] = p[e * step];
+            } else {
+                const double* p = (isA ? tile(t, I, J) : tile(t, K, J)) + (size_t)k0 * GP_NB + row;
+#pragma unroll
+                for (int e = 0; e < 8; ++e) v[e] = p[e * GP_NB];
+            }
         };
         double raw[kPieces][8];
+        int exq[kPieces];
         int w = next_live(blockIdx.x), kc = 0;
         if (w < total) {
 #pragma unroll
-            for (int u = 0; u < kPieces; ++u) {
-                const double* p = source(w, 0, u);
-#pragma unroll
-                for (int e = 0; e < 8; ++e) raw[u][e] = p[e * GP_NB];
-            }
+            for (int u = 0; u < kPieces; ++u) load(w, 0, u, raw[u], exq[u]);
         }
         for (int g = 0; w < total && !abort_flag; ++g) {
             const int st = g & 1;
@@ -326,12 +393,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                 const int piece = cw + kConvWarps * u, rg = piece >> 2, oct = piece & 3;
                 const bool isA = rg < 4;
                 uint8_t* dst = stage + (isA ? 0u : kABytes) + image_piece((isA ? 32 * rg : 32 * (rg - 4)) + lane, 8 * oct);
-                if (piece < kStagePieces) store_digits(raw[u], dst, isA ? kChunkBytes : kBChunk);
-                if (wn < total) {
-                    const double* p = source(wn, kn, u);
-#pragma unroll
-                    for (int e = 0; e < 8; ++e) raw[u][e] = p[e * GP_NB];
-                }
+                if (piece < kStagePieces) store_digits(raw[u], exq[u], dst, isA ? kChunkBytes : kBChunk);
+                if (wn < total) load(wn, kn, u, raw[u], exq[u]);
             }
             // the tensor core reads shared memory through the asynchronous proxy
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -378,11 +441,12 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tbase));
 }
 
-template <int NT>
-cudaError_t launch(const Batch& b, int J, cudaStream_t s, int which, int per_inst, int chunks) {
+template <int NT, int MODE>
+cudaError_t launch(const Batch& b, int J, cudaStream_t s, int which, int per_inst, int chunks, double* X = nullptr,
+                   double* S = nullptr) {
     const size_t smem = 2 * (size_t)stage_bytes(NT) + 1024 + (size_t)(b.count + 31) / 32 * 4;
     static std::atomic<size_t> attr[kMaxDevices];
-    cudaError_t e = raise_smem_limit(k_update_f64_tc<NT>, smem, attr);
+    cudaError_t e = raise_smem_limit(k_update_f64_tc<NT, MODE>, smem, attr);
     if (e != cudaSuccess) return e;
     const long long total = (long long)per_inst * b.count;
     // the rest of an update runs beside the next block column's panel, whose
@@ -392,7 +456,7 @@ cudaError_t launch(const Batch& b, int J, cudaStream_t s, int which, int per_ins
     // 38.5, 37.3 and 44.2 ms)
     const int cap = which == kUpdateRest ? device_sms() - device_sms() / 3 : device_sms();
     const int grid = (int)(total < cap ? total : cap);
-    k_update_f64_tc<NT><<<grid, kThreads, smem, s>>>(b, J, which, per_inst, chunks);
+    k_update_f64_tc<NT, MODE><<<grid, kThreads, smem, s>>>(b, J, which, per_inst, chunks, X, S);
     return cudaGetLastError();
 }
 
@@ -402,11 +466,21 @@ cudaError_t launch_update_f64_tc(const Batch& b, int J, cudaStream_t s, int whic
     const int m = b.nt - J - 1;
     const int tiles = which == kUpdateColumn ? m : (which == kUpdateRest ? m * (m - 1) / 2 : m * (m + 1) / 2);
     if (tiles <= 0) return cudaSuccess;
-    return launch<64>(b, J, s, which, 2 * tiles, kChunks);
+    return launch<64, kFactorMode>(b, J, s, which, 2 * tiles, kChunks);
 }
 
 cudaError_t launch_update_f64_inner(const Batch& b, int J, int step, cudaStream_t s) {
-    return launch<32>(b, J, s, kUpdateInner, b.nt - J, step);
+    return launch<32, kInnerMode>(b, J, s, kUpdateAll, b.nt - J, step);
+}
+
+cudaError_t launch_inverse_apply(const Batch& b, int J, double* X, double* S, cudaStream_t s) {
+    if (J == 0) return cudaSuccess;
+    return launch<64, kInvApply>(b, J, s, kUpdateAll, 2 * J, kChunks, X, S);
+}
+
+cudaError_t launch_inverse_update(const Batch& b, int J, double* X, double* S, cudaStream_t s) {
+    const int tiles = (b.nt - 1 - J) * (J + 1) + (J + 1) * (J + 2) / 2;
+    return launch<64, kInvUpdate>(b, J, s, kUpdateAll, 2 * tiles, kChunks, X, S);
 }
 
 }  // namespace gp
