@@ -38,50 +38,76 @@ __device__ __forceinline__ double powabs(double diff, double p) {
     return (a == 0.0) ? 0.0 : pow(a, p);
 }
 
-// |dx|^p in double for a general p without a pow per term (the reduction
-// of P. T. P. Tang's table-driven logarithm, ACM TOMS 16 (1990), applied to
-// the power): a = 2^m F_j (1 + u) with F_j = 1 + j/64 the table point
-// nearest the mantissa (|u| <= 2^-7), so that
-//   a^p = [2^(m p) F_j^p] (1 + u)^p,
+// |dx|^p and exp(-S) in double without a pow or an exp per term (the reductions
+// of P. T. P. Tang's table-driven logarithm and exponential, ACM TOMS 16
+// (1990) and 15 (1989)): an FP64 instruction is worth 64 FP32 ones here, so
+// what counts is their number.
+//
+// a = 2^m x, x in [1, 2), c_j the double nearest 1 / (1 + j/64) for the table
+// point nearest x: u = x c_j - 1 by one fma (|u| <= 2^-7, one rounding), and
+//   a^p = [2^(m p) c_j^-p] (1 + u)^p,
 // the bracket as a double-double product of two tables computed on the host
 // in long double, (1 + u)^p - 1 = p u + c2 u^2 + ... + c7 u^7 (the u^8 term
 // is below 2^-62), and one rounding at the end: a^p = A_hi + (A_hi t +
-// A_lo).  m outside [-60, 4] takes pow.
+// A_lo): 15 double operations.  m outside [-60, 4] takes pow.
+//
+// exp(-S) = 2^(k/128) exp(r), k = round(-128 S / ln 2), r = -S - k ln2/128
+// (two fmas against ln2/128 as 32 + 53 bits), exp(r) - 1 = r + r^2 (1/2 + r/6 +
+// r^2/24 + r^3/120) (the next term is below 2^-60), times the table's 2^(j/128)
+// as a double-double, scaled by its exponent bits: 11 double operations.  S
+// above 700 takes exp.
 constexpr int kP64NBits = 6;
 constexpr int kP64N = 1 << kP64NBits;
 constexpr int kP64Mlo = -60, kP64Mhi = 4;
 constexpr int kP64Ms = kP64Mhi - kP64Mlo + 1;
+constexpr int kE64NBits = 7;
+constexpr int kE64N = 1 << kE64NBits;
 struct PowTab64 {
     int on;                       // general p on the power-exponential family
     double c[8];                  // c[k] = C(p, k), k = 1 .. 7
-    double inv[kP64N];            // 1 / F_j (rounded: the division's residual is formed exactly)
+    double inv[kP64N + 1];        // c_j (j = 64: 1/2, for x next to 2)
     double2 two[kP64Ms];          // 2^(m p), m = kP64Mlo .. kP64Mhi, as (hi, lo)
-    double2 f[kP64N];             // F_j^p as (hi, lo)
+    double2 f[kP64N + 1];         // c_j^-p as (hi, lo)
+    double2 e2[kE64N];            // 2^(j/128) as (hi, lo)
 };
-static_assert(sizeof(PowTab64) + 512 < 4096, "kernel parameters");
+static_assert(sizeof(PowTab64) + 512 < 32764, "kernel parameters");
 
 __device__ __forceinline__ double pow_tab64(double a, double p, const PowTab64& t) {
-    const long long rb = __double_as_longlong(a) + (1LL << (51 - kP64NBits));   // a > 0
-    const int e = (int)(rb >> 52);
-    if (e - 1023 < kP64Mlo || e - 1023 > kP64Mhi) return pow(a, p);
-    const int j = (int)(rb >> (52 - kP64NBits)) & (kP64N - 1);
-    const double Fm = __longlong_as_double(rb & ~((1LL << (52 - kP64NBits)) - 1));   // 2^m F_j
-    const double g = __longlong_as_double((long long)(2046 - e) << 52);              // 2^-m
-    const double fh = (a - Fm) * g;                                                   // exact
-    const double F = Fm * g;
-    const double iv = t.inv[j];
-    const double uh = fh * iv;
-    const double ul = fma(-uh, F, fh) * iv;
-    double q = fma(uh, t.c[7], t.c[6]);
-    q = fma(uh, q, t.c[5]);
-    q = fma(uh, q, t.c[4]);
-    q = fma(uh, q, t.c[3]);
-    q = fma(uh, q, t.c[2]);
-    const double tt = fma(t.c[1], uh, fma(t.c[1], ul, uh * uh * q));
-    const double2 T = t.two[e - 1023 - kP64Mlo], P = t.f[j];
+    const int hi = __double2hiint(a);                                      // a > 0
+    const int e = (hi >> 20) - 1023;
+    if (e < kP64Mlo || e > kP64Mhi) return pow(a, p);
+    const int j = ((hi & 0xfffff) + (1 << (19 - kP64NBits))) >> (20 - kP64NBits);
+    const double x = __hiloint2double((hi & 0xfffff) | 0x3ff00000, __double2loint(a));
+    const double u = fma(x, t.inv[j], -1.0);
+    double q = fma(u, t.c[7], t.c[6]);
+    q = fma(u, q, t.c[5]);
+    q = fma(u, q, t.c[4]);
+    q = fma(u, q, t.c[3]);
+    q = fma(u, q, t.c[2]);
+    const double tt = u * fma(u, q, t.c[1]);
+    const double2 T = t.two[e - kP64Mlo], P = t.f[j];
     const double ah = T.x * P.x;
     const double al = fma(T.x, P.x, -ah) + fma(T.x, P.y, T.y * P.x);
     return ah + fma(ah, tt, al);
+}
+
+__device__ __forceinline__ double exp_neg_tab64(double s, const PowTab64& t) {
+    if (!(s < 700.0)) return exp(-s);
+    constexpr double kInv = 128.0 / 0.693147180559945309417232121458176568;
+    constexpr double kHi = 0x1.62e42fefp-8;                                // ln2 / 128, 33 bits
+    constexpr double kLo = 0x1.473de6af278edp-41;                          // and the rest
+    constexpr double kRound = 6755399441055744.0;                          // 1.5 2^52
+    const double kr = fma(-s, kInv, kRound);
+    const int k = __double2loint(kr);
+    const double kd = kr - kRound;
+    const double r = fma(-kd, kLo, fma(-kd, kHi, -s));
+    double q = fma(r, 1.0 / 120.0, 1.0 / 24.0);
+    q = fma(r, q, 1.0 / 6.0);
+    q = fma(r, q, 0.5);
+    const double w = fma(r * r, q, r);
+    const double2 T = t.e2[k & (kE64N - 1)];
+    const double v = T.x + fma(T.x, w, T.y);
+    return __hiloint2double(__double2hiint(v) + ((k >> kE64NBits) << 20), __double2loint(v));
 }
 
 __device__ __forceinline__ double powabs_t(double diff, double p, const PowTab64& t) {
@@ -132,14 +158,22 @@ __global__ void k_validate_theta(Batch b) {
     b.st[t] = s;
 }
 
+constexpr int kThetaCache = 1024;
+
 // grid.x = packed tiles * kSplit, grid.y = candidate groups; DB = bound on d;
-// TAB: a general p on the power-exponential family, powers by pow_tab64
+// TAB: a general p on the power-exponential family, pow_tab64 and
+// exp_neg_tab64.  Bound by the FP64 pipe: 15 d double operations per entry and
+// d + 12 per entry and candidate (22 d and 2 d + 27 with the division's residual
+// formed apart and CUDA's exp).  n = 4064, d = 6: one candidate 2.97 -> 2.10 ms,
+// twelve 9.52 -> 5.78 ms, with R's largest relative error over 1 + S unchanged or
+// lower (1.50 and 2.43 -> 2.29 units of 2^-53 for p = 1.95 and 1.5).
 template <int DB, bool TAB>
 __global__ void __launch_bounds__(kThreads)
 k_assemble_tiles(Batch b, int group, PowTab64 ptab) {
     __shared__ double xs_r[GP_NB * DB];
     __shared__ double xs_c[kCols * DB];
     __shared__ PowTab64 pt;
+    __shared__ double th_s[kThetaCache];          // TAB: the group's theta, while it fits
     if (TAB)
         for (int q = threadIdx.x; q < (int)(sizeof(PowTab64) / sizeof(int)); q += kThreads)
             reinterpret_cast<int*>(&pt)[q] = reinterpret_cast<const int*>(&ptab)[q];
@@ -172,6 +206,12 @@ k_assemble_tiles(Batch b, int group, PowTab64 ptab) {
 
     const int t0 = blockIdx.y * group;
     const int t1 = min(b.count, t0 + group);
+    const bool cached = TAB && (t1 - t0) * DB <= kThetaCache;
+    if (cached) {
+        for (int q = threadIdx.x; q < (t1 - t0) * DB; q += kThreads)
+            th_s[q] = q % DB < d ? b.theta[(size_t)(t0 + q / DB) * d + q % DB] : 0.0;
+        __syncthreads();
+    }
     const size_t tile_off = (size_t)tile_lin * GP_TILE_ELEMS;
     const int r = threadIdx.x % GP_NB;           // row inside the tile
     const int cb = threadIdx.x / GP_NB;          // 0..1
@@ -199,6 +239,19 @@ k_assemble_tiles(Batch b, int group, PowTab64 ptab) {
             double v;
             if (pad) {
                 v = diag ? 1.0 : 0.0;
+            } else if (TAB) {
+                double s = 0.0;
+                if (cached) {
+#pragma unroll
+                    for (int k = 0; k < DB; ++k)
+                        if (k < d) s = fma(th_s[(t - t0) * DB + k], D[k], s);
+                } else {
+#pragma unroll
+                    for (int k = 0; k < DB; ++k)
+                        if (k < d) s = fma(__ldg(b.theta + (size_t)t * d + k), D[k], s);
+                }
+                v = exp_neg_tab64(s, pt);
+                if (diag) v += b.delta;
             } else {
                 const double* th = b.theta + (size_t)t * d;
                 double s = 0.0, q = 1.0;
@@ -448,11 +501,11 @@ static void pow_tab64_fill(double p, PowTab64& t) {
             const double h = (double)v;
             return make_double2(h, (double)(v - (long double)h));
         };
-        for (int j = 0; j < kP64N; ++j) {
-            const long double F = 1.0L + (long double)j / (long double)kP64N;
-            last.inv[j] = (double)(1.0L / F);
-            last.f[j] = split(powl(F, (long double)p));
+        for (int j = 0; j <= kP64N; ++j) {
+            last.inv[j] = (double)(1.0L / (1.0L + (long double)j / (long double)kP64N));
+            last.f[j] = split(powl((long double)last.inv[j], -(long double)p));
         }
+        for (int j = 0; j < kE64N; ++j) last.e2[j] = split(exp2l((long double)j / (long double)kE64N));
         for (int m = kP64Mlo; m <= kP64Mhi; ++m) last.two[m - kP64Mlo] = split(exp2l((long double)m * (long double)p));
         last_p = p;
     }
