@@ -7,12 +7,13 @@
 // On this GPU a double multiply-add takes a warp 64 cycles, issue and latency
 // alike, so what stays on the FP64 pipe is kept to the 32-wide triangles: a
 // quarter of the panel's multiply-adds, spread over all SMs by rows.  A block
-// column is bound by its chain: four 32-pivot sweeps of about 12 us, four
-// solves of 168 dependent double operations (6 us) and three inner updates.
-// Measured, one candidate at n = 4064: 190 us a block column (0.4 ms for the
-// 128-pivot sweep and 0.35 ms for the tile solve on the FP64 pipe alone); the
-// double fit 29.8 -> 13.6 ms, twelve candidates 55 -> 37.3 ms.
-#include "gp_internal.cuh"
+// column is bound by its chain: four 32-pivot sweeps of about 12 us (17 us
+// with a warp's terms all taken in the step of their column, 22 us as
+// unrolled code), four solves of about 8 us and three inner updates of 8 to
+// 13 us.  Measured, one candidate at n = 4064: 165 us a block column (0.4 ms
+// for a 128-pivot sweep in one CTA and 0.35 ms for the tile solve, on the FP64
+// pipe alone); the double fit 29.8 -> 10.5 ms with the solves after it.
+#include "mixed_common.cuh"
 
 namespace gp {
 
@@ -21,16 +22,16 @@ namespace {
 constexpr int kB = kPanelStep;                 // 32
 constexpr int kThreads = 128;
 constexpr int kWarps = kThreads / 32;
-constexpr int kUnit = 8;                       // rows a warp solves at a time
 
 __device__ __forceinline__ double* inst_tile(const Batch& b, int t, int I, int J) {
     return b.A + (size_t)t * b.inst_stride + (size_t)tile_index(I, J, b.nt) * GP_TILE_ELEMS;
 }
 
-// 1 / sqrt(a) for a normal a > 0: a float seed (2^-20), then y = y0 (1 + e/2 +
-// 3 e^2 / 8), e = 1 - a y0^2 (the next term, 5 e^3 / 16, is below 2^-58): five
-// double operations where sqrt and a division take 1360 cycles.
-__device__ __forceinline__ double rsqrt_f64(double a) {
+// v / sqrt(a) for a normal a > 0: a float seed y0 (2^-20), then v y0 (1 + e/2 +
+// 3 e^2 / 8), e = 1 - a y0^2 (the next term, 5 e^3 / 16, is below 2^-58): six
+// double operations, five of them in a chain, where sqrt and a division take
+// 1360 cycles.
+__device__ __forceinline__ double over_sqrt(double v, double a) {
     const int hi = __double2hiint(a), lo = __double2loint(a);
     const int e = (hi >> 20) - 1023;
     const int h = e >> 1;                               // a = m 2^(2h), m in [1, 4)
@@ -42,65 +43,117 @@ __device__ __forceinline__ double rsqrt_f64(double a) {
     const double y0 = __hiloint2double((ye << 20) | (int)((sb & 0x7fffff) >> 3), (int)(sb << 29));
     const double t = a * y0;
     const double err = fma(-t, y0, 1.0);
-    const double p = fma(err, 0.375, 0.5);
-    return fma(y0 * err, p, y0);
+    const double vy = v * y0;
+    const double q = err * fma(err, 0.375, 0.5);
+    return fma(vy, q, vy);
 }
 
-// L_ss of sub-block s.  Thread (lane, warp) holds row lane, columns warp + 4 j;
-// the warp that owns column c takes its pivot and publishes the finished
-// column, one barrier a column.
+// A pivot outside the normal range: v / sqrt(piv), or zeros (the sweep goes on
+// with them) and the column recorded when piv is not positive and finite.
+__device__ __noinline__ double odd_pivot(double v, double piv, int c, int lane, int* failed) {
+    if (piv > 0.0 && isfinite(piv)) return v * (1.0 / sqrt(piv));
+    if (lane == 0 && *failed < 0) *failed = c;
+    return 0.0;
+}
+
+// L_ss of sub-block s.  Thread (lane, warp) holds row lane, columns warp + 4 i;
+// one barrier a column.  The warp that owns column c + 1 takes its last term,
+// its pivot and the finished column in step c, 600 cycles of dependent double
+// operations and the sweep's critical path; the others' work fits beside
+// it.  Of the terms of four columns (a group), those for the next two groups
+// of columns are taken at once, the others in the next group, two columns by
+// four terms in each of a warp's three steps without a pivot.  Pivots are
+// tested by their bits (a comparison of doubles costs 64 cycles, too).  A group
+// is one iteration of a loop, in two forms (up to six and up to three columns
+// to come; the columns move down one register as they finish, and what moves
+// in past the last one is not used): unrolled over all columns the sweep
+// waits for its code.
+constexpr int kLsCols = 48;                    // rows of Ls, with room for the unused columns' reads
+
+template <int LEFT>
+__device__ __forceinline__ void diag32_columns(double (&a)[kB / kWarps], double (*Ls)[kLsCols], int j0, int warp,
+                                               int lane, int* failed) {
+    constexpr int kCols = kB / kWarps;
+    // pivot and finished column c, held in v by the warp that owns it
+    auto finish = [&](double& v, int c) {
+        const double piv = __shfl_sync(0xffffffffu, v, c);
+        const unsigned hi = (unsigned)__double2hiint(piv);
+        v = hi - 0x00100000u < 0x7fe00000u ? over_sqrt(v, piv)      // normal, positive and finite
+                                           : odd_pivot(v, piv, c, lane, failed);
+        Ls[c][lane] = v;
+    };
+    // the four terms of group j - 1 for columns i0, i0 + 1
+    auto pending = [&](int j, int i0) {
+        double l[4], lk[4][2];
+#pragma unroll
+        for (int u = 0; u < kWarps; ++u) {
+            const double* col = Ls[kWarps * (j - 1) + u];
+            l[u] = col[lane];
+#pragma unroll
+            for (int i = 0; i < 2; ++i) lk[u][i] = col[warp + kWarps * (j + i0 + i)];
+        }
+#pragma unroll
+        for (int u = 0; u < kWarps; ++u)
+#pragma unroll
+            for (int i = 0; i < 2; ++i)
+                if (i0 + i <= LEFT) a[i0 + i] = fma(-l[u], lk[u][i], a[i0 + i]);
+    };
+    if (j0 == 0) {
+        if (warp == 0) finish(a[0], 0);
+        __syncthreads();
+    }
+#pragma unroll 1
+    for (int j = j0; j < j0 + kCols / 2; ++j) {
+#pragma unroll
+        for (int q = 0; q < kWarps; ++q) {
+            const int c = kWarps * j + q;
+            const double lr = Ls[c][lane], l0 = Ls[c][warp + kWarps * j], l1 = Ls[c][warp + kWarps * (j + 1)];
+            if (warp == (q + 1) % kWarps) {
+                if (q < kWarps - 1) {
+                    a[0] = fma(-lr, l0, a[0]);
+                    finish(a[0], c + 1);
+                    a[1] = fma(-lr, l1, a[1]);
+                } else if (c + 1 < kB) {
+                    a[1] = fma(-lr, l1, a[1]);
+                    finish(a[1], c + 1);
+                }
+            } else {
+                if (warp > q) a[0] = fma(-lr, l0, a[0]);
+                a[1] = fma(-lr, l1, a[1]);
+                // this warp's step number among those without a pivot
+                const int step = q - (q > (warp + kWarps - 1) % kWarps ? 1 : 0);
+                if (j > 0) {
+                    if (step == 0) pending(j, 1);
+                    if (step == 1 && LEFT > 2) pending(j, 3);
+                    if (step == 2 && LEFT > 4) pending(j, 5);
+                }
+            }
+            __syncthreads();
+        }
+#pragma unroll
+        for (int i = 0; i + 1 < kCols; ++i) a[i] = a[i + 1];
+    }
+}
+
 __global__ void __launch_bounds__(kThreads) k_diag32_f64(Batch b, int J, int s) {
-    __shared__ double Ls[kB][kB + 1];              // Ls[c][r]
+    __shared__ double Ls[kB][kLsCols];             // Ls[c][r]
     __shared__ int failed;
     const int t = blockIdx.x;
     if (b.st[t].status != GP_OK) return;
     double* T = inst_tile(b, t, J, J) + (size_t)(kB * s) * GP_NB + kB * s;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    double a[kB / kWarps];
+    constexpr int kCols = kB / kWarps;
+    double a[kCols];
 #pragma unroll
-    for (int j = 0; j < kB / kWarps; ++j) {
-        const int k = warp + kWarps * j;
-        a[j] = lane >= k ? T[(size_t)k * GP_NB + lane] : 0.0;
+    for (int i = 0; i < kCols; ++i) {
+        const int k = warp + kWarps * i;
+        a[i] = lane >= k ? T[(size_t)k * GP_NB + lane] : 0.0;
     }
+    for (int q = threadIdx.x; q < kB * kLsCols; q += kThreads) (&Ls[0][0])[q] = 0.0;
     if (threadIdx.x == 0) failed = -1;
     __syncthreads();
-    // pivot and finished column c, held in a[c / 4] of warp c % 4
-    auto finish = [&](double& v, int c) {
-        const double piv = __shfl_sync(0xffffffffu, v, c);
-        double y = 0.0;
-        if (!(piv > 0.0) || !isfinite(piv)) {
-            if (lane == 0 && failed < 0) failed = c;   // the sweep goes on with zeros
-        } else if (piv < 0x1p-1000) {
-            y = 1.0 / sqrt(piv);
-        } else {
-            y = rsqrt_f64(piv);
-        }
-        v *= y;
-        Ls[c][lane] = v;
-    };
-    if (warp == 0) finish(a[0], 0);
-    __syncthreads();
-#pragma unroll
-    for (int j = 0; j < kB / kWarps; ++j)
-#pragma unroll
-        for (int q = 0; q < kWarps; ++q) {
-            const int c = kWarps * j + q;
-            const double lr = Ls[c][lane];
-            // column c + 1 first, and its pivot
-            constexpr int kLast = kB / kWarps - 1;
-            const int jn = q == kWarps - 1 ? j + 1 : j, qn = (q + 1) % kWarps;
-            if (warp == qn && jn <= kLast) {
-                const int jc = jn <= kLast ? jn : kLast;
-                a[jc] = fma(-lr, Ls[c][c + 1 < kB ? c + 1 : c], a[jc]);
-                finish(a[jc], c + 1);
-            }
-#pragma unroll
-            for (int i = j; i < kB / kWarps; ++i) {
-                const int k = warp + kWarps * i;
-                if (k > c && !(warp == qn && i == jn)) a[i] = fma(-lr, Ls[c][k], a[i]);
-            }
-            __syncthreads();
-        }
+    diag32_columns<kCols - 2>(a, Ls, 0, warp, lane, &failed);
+    diag32_columns<kCols / 2 - 1>(a, Ls, kCols / 2, warp, lane, &failed);
     if (failed >= 0) {
         if (threadIdx.x == 0) {
             b.st[t].status = GP_ENOTPD;
@@ -109,68 +162,81 @@ __global__ void __launch_bounds__(kThreads) k_diag32_f64(Batch b, int J, int s) 
         return;
     }
 #pragma unroll
-    for (int j = 0; j < kB / kWarps; ++j) {
-        const int k = warp + kWarps * j;
-        if (lane >= k) T[(size_t)k * GP_NB + lane] = a[j];
+    for (int i = 0; i < kCols; ++i) {
+        const int k = warp + kWarps * i;
+        if (lane >= k) T[(size_t)k * GP_NB + lane] = Ls[k][lane];
     }
 }
 
-// Rows below sub-block s, `per_warp` groups of eight rows a warp: lane (row
-// rr, kq) holds columns kq + 4 j of its row; x_c goes from its owner to the
+// Rows below sub-block s, `per_warp` groups of 32 / LANES rows a warp: lane (row
+// rr, kq) holds columns kq + LANES j of its row; x_c goes from its owner to the
 // row's other lanes by a shuffle, and column c leaves the columns after it in
-// the order of c.
+// the order of c.  Four lanes a row take 168 double operations for eight rows,
+// eight lanes 104 for four: less in all with four, sooner done with eight
+// where the rows do not fill the schedulers.
+template <int LANES>
 __global__ void __launch_bounds__(kThreads) k_solve32_f64(Batch b, int J, int s, int units, int per_warp) {
+    constexpr int kRows = 32 / LANES, kCols = kB / LANES;
     __shared__ double Ls[kB][kB + 1];
     __shared__ double inv[kB];
     const int t = blockIdx.y;
     if (b.st[t].status != GP_OK) return;
     const double* T = inst_tile(b, t, J, J) + (size_t)(kB * s) * GP_NB + kB * s;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int rr = lane & 7, kq = lane >> 3;
+    const int rr = lane % kRows, kq = lane / kRows;
     int u = (blockIdx.x * kWarps + warp) * per_warp;
     const int end = u + per_warp < units ? u + per_warp : units;
     auto rows = [&](int unit) {
-        const int row = kB * (s + 1) + kUnit * unit;
+        const int row = kB * (s + 1) + kRows * unit;
         return inst_tile(b, t, J + (row >> 7), J) + (size_t)(kB * s) * GP_NB + (row & 127) + rr;
     };
-    double a[kB / 4], nx[kB / 4];
+    double a[kCols], nx[kCols];
     if (u < end) {
         const double* p = rows(u);
 #pragma unroll
-        for (int j = 0; j < kB / 4; ++j) nx[j] = p[(size_t)(kq + 4 * j) * GP_NB];
+        for (int j = 0; j < kCols; ++j) nx[j] = p[(size_t)(kq + LANES * j) * GP_NB];
     }
     for (int q = threadIdx.x; q < kB * kB; q += kThreads) {
         const int r = q % kB, c = q / kB;
-        if (r >= c) Ls[c][r] = T[(size_t)c * GP_NB + r];
+        if (r >= c) cp_async8(&Ls[c][r], T + (size_t)c * GP_NB + r);
     }
-    __syncthreads();
-    if (threadIdx.x < kB) inv[threadIdx.x] = 1.0 / Ls[threadIdx.x][threadIdx.x];
+    if (threadIdx.x < kB) inv[threadIdx.x] = 1.0 / T[(size_t)threadIdx.x * (GP_NB + 1)];
+    cp_async_wait_all();
     __syncthreads();
     for (; u < end; ++u) {
         double* p = rows(u);
 #pragma unroll
-        for (int j = 0; j < kB / 4; ++j) a[j] = nx[j];
+        for (int j = 0; j < kCols; ++j) a[j] = nx[j];
         if (u + 1 < end) {
             const double* pn = rows(u + 1);
 #pragma unroll
-            for (int j = 0; j < kB / 4; ++j) nx[j] = pn[(size_t)(kq + 4 * j) * GP_NB];
+            for (int j = 0; j < kCols; ++j) nx[j] = pn[(size_t)(kq + LANES * j) * GP_NB];
         }
 #pragma unroll
         for (int c = 0; c < kB; ++c) {
-            const int jc = c / 4, qc = c % 4;
-            const double x = __shfl_sync(0xffffffffu, a[jc], 8 * qc + rr) * inv[c];
-            if (qc < 3) {
-                const double v = fma(-x, Ls[c][kq + 4 * jc], a[jc]);
+            const int jc = c / LANES, qc = c % LANES;
+            const double x = __shfl_sync(0xffffffffu, a[jc], kRows * qc + rr) * inv[c];
+            if (qc < LANES - 1) {
+                const double v = fma(-x, Ls[c][kq + LANES * jc], a[jc]);
                 a[jc] = kq > qc ? v : (kq == qc ? x : a[jc]);
-            } else if (kq == 3) {
+            } else if (kq == LANES - 1) {
                 a[jc] = x;
             }
 #pragma unroll
-            for (int j = jc + 1; j < kB / 4; ++j) a[j] = fma(-x, Ls[c][kq + 4 * j], a[j]);
+            for (int j = jc + 1; j < kCols; ++j) a[j] = fma(-x, Ls[c][kq + LANES * j], a[j]);
         }
 #pragma unroll
-        for (int j = 0; j < kB / 4; ++j) p[(size_t)(kq + 4 * j) * GP_NB] = a[j];
+        for (int j = 0; j < kCols; ++j) p[(size_t)(kq + LANES * j) * GP_NB] = a[j];
     }
+}
+
+template <int LANES>
+void launch_solve32(const Batch& b, int J, int s, int rows, int sms, cudaStream_t st) {
+    const int units = rows / (32 / LANES);
+    const long long warps = (long long)sms * 8;              // two CTAs an SM
+    const int per_warp = (int)(((long long)units * b.count + warps - 1) / warps);
+    const int grid = (units + kWarps * per_warp - 1) / (kWarps * per_warp);
+    k_solve32_f64<LANES><<<dim3(grid, b.count), kThreads, 0, st>>>(b, J, s, units, per_warp);
 }
 
 // log|R| = 2 sum log L_ii over the factor's diagonal (padded rows give 0),
@@ -207,12 +273,10 @@ cudaError_t launch_panel_f64(const Batch& b, int J, cudaStream_t st) {
             if (e != cudaSuccess) return e;
         }
         k_diag32_f64<<<b.count, kThreads, 0, st>>>(b, J, s);
-        const int units = ((b.nt - J) * GP_NB - kB * (s + 1)) / kUnit;
-        if (units > 0) {
-            const long long warps = (long long)sms * 8;      // two CTAs an SM
-            const int per_warp = (int)(((long long)units * b.count + warps - 1) / warps);
-            const int grid = (units + kWarps * per_warp - 1) / (kWarps * per_warp);
-            k_solve32_f64<<<dim3(grid, b.count), kThreads, 0, st>>>(b, J, s, units, per_warp);
+        const int rows = (b.nt - J) * GP_NB - kB * (s + 1);
+        if (rows > 0) {
+            if ((long long)rows * b.count <= 4 * 4LL * sms) launch_solve32<8>(b, J, s, rows, sms, st);
+            else                                            launch_solve32<4>(b, J, s, rows, sms, st);
         }
     }
     return cudaGetLastError();

@@ -8,25 +8,31 @@
 // sum_{k<i} l_ik^2 = 1 + delta - l_ii^2 and l_ii^2 >= delta for a positive
 // semidefinite R.  So every entry is cut at one fixed scale, with no row
 // exponents:
-//   X = rint(l 2^55) = sum_{a=0..6} q_a 256^(6-a),  |q_a| <= 128 (balanced digits),
-// each digit exact in bf16.  The product groups S_g = sum_{a+b=g} q_a q_b', g =
-// 0 .. 7, summed over the panel's 128 columns in fp32 are integers of at most 7
-// 2^21 < 2^24, hence exact; what is left out, a + b >= 8, is below 2^-64 of
-// 1 per term.  A row's dropped part of l is at most 2^-56, and the rows of L
-// have norm 1, so all panels together leave an error of about 2^-56 in an
-// entry of A, where each IEEE subtraction from A rounds to 2^-53 of it: the
-// factor is as accurate as with double multiply-adds.
+//   X = floor(l 2^56) = sum_{a=0..6} q_a 256^(6-a),  |q_a| <= 128 (a > 0), |q_0| <= 256
+// (balanced digits), each digit exact in fp16.  The product groups S_g =
+// sum_{a+b=g} q_a q_b', g = 0 .. 7, summed over the panel's 128 columns in fp32
+// are integers below 2^24, hence exact (at most 2^21 for a pair of lower
+// digits, of which a group has six at most, and less than 2^20 by
+// Cauchy-Schwarz for a pair with q_0, since the rows of L have norm 1); what
+// is left out, a + b >= 8, is below 2^-66 of 1 per term.  The dropped part of l
+// is at most 2^-56, so all panels together leave an error of about 2^-56 in
+// an entry of A, where each IEEE subtraction from A rounds to 2^-53 of it:
+// the factor is as accurate as with double multiply-adds.
 //
 // The digits are cut on the way into shared memory by eight converter
 // warps, from the double tiles themselves: no workspace, so the callers'
 // memory is the same on either path.
 //
-// Bound by the tensor pipe's shared-memory reads (34 digit products of K =
-// 128 columns, 12.7 k cycles a half tile) next to the converters' integer
-// work.  Measured, max |R - L L'| at n = 1500, d = 4, p = 1.5: 4.7e-16 (1.6e-15
-// with double multiply-adds on the FP64 pipe).  Twelve candidates at n = 4064:
-// the updates 17 ms instead of 256 ms (the FP64 pipe's 1.1 TF/s), the batch
-// 270 -> 55 ms; the double fit at n = 4064 54.6 -> 29.8 ms.
+// Bound by the tensor pipe: an M = 128, N = 64 product of K = 16 takes 80
+// cycles here (its operands' shared-memory reads), so a half tile's 272 take
+// 22 k cycles, then the groups' sum in front of the next tile 3 k (5 k with
+// every group through the conversion instruction).  The cutting runs beside
+// it since it costs 13 integer instructions an entry and 2 a digit (38 in
+// all, where it set the pace: 19.9 -> 15 us a half tile).
+// Measured, max |R - L L'| at n = 900, d = 2: 1.3e-16 (1.6e-15 with double
+// multiply-adds on the FP64 pipe).  Twelve candidates at n = 4064: 270 ms with
+// the updates on the FP64 pipe (256 of them), 28.8 ms now (updates 19); the
+// double fit at n = 4064 54.6 -> 10.5 ms.
 #include "mixed_common.cuh"
 
 namespace gp {
@@ -49,42 +55,37 @@ constexpr int kMmaRegs = 56, kConvRegs = 96, kEpiRegs = 112;
 static_assert(128 * kMmaRegs + 32 * kConvWarps * kConvRegs + 32 * kEpiWarps * kEpiRegs <= kThreads * 96,
               "register split exceeds the launch's registers");
 
-// X + the digits' bias: byte 6 - a of the result is q_a + 128 (a >= 1), and
-// the bits from 48 up are q_0 as a signed number.  |l| >= 2 (possible only
-// on the way to a failed factorisation) is cut to 2.
-// E: the operand's exponent, X = rint(l 2^(55 - E)).
-__device__ __forceinline__ unsigned long long biased_digits(double l, int E) {
+// X = floor(l 2^(56 - E)) plus the digits' bias: byte 6 - a of the result is q_a +
+// 128 (a >= 1), the 16 bits from 48 up q_0 + 512.  |l| >= 2^E (possible only on
+// the way to a failed factorisation) is cut to its significand, in [1, 2) 2^E.
+// 13 integer instructions, which this GPU issues at half the FP32 rate: the
+// converters' rate is what they cost.
+__device__ __forceinline__ uint2 biased_digits(double l, int E) {
     const unsigned hi = (unsigned)__double2hiint(l), lo = (unsigned)__double2loint(l);
-    const int e = (hi >> 20) & 0x7ff;
-    int r = 1023 + E - e;                                 // >= 0 for |l| < 2^(E + 1)
-    unsigned long long m = ((unsigned long long)((hi & 0xfffffu) | 0x100000u) << 32) | lo;
-    if (r < 0) {
-        m = 0x1fffffffffffffull;
-        r = 0;
-    }
-    // 2 |X| before rounding: |l| 2^56 = m 2^(e - 1019) = (m << 4) >> r
-    const unsigned long long w = r < 64 ? (m << 4) >> r : 0ull;
-    const long long x = (long long)((w + 1) >> 1);
-    const long long s = (long long)(int)hi >> 63;
-    return (unsigned long long)((x ^ s) - s) + 0x0000808080808080ull;
+    // r = 1023 + E - e in [0, 63]: l 2^(56 - E) = (m << 4) >> r for the 53-bit significand m
+    const int r = __viaddmin_s32_relu((int)((~hi & 0x7ff00000u) >> 20), 1023 + E - 2047, 63);
+    const unsigned long long m = (unsigned long long)((hi & 0xfffffu) | 0x100000u) << 32 | lo;
+    const unsigned long long w = (m << 4) >> r;
+    // -1 - w for a negative l: the floor
+    const unsigned s = (unsigned)((int)hi >> 31);
+    const unsigned long long x = (unsigned long long)((unsigned)(w >> 32) ^ s) << 32 | ((unsigned)w ^ s);
+    const unsigned long long y = x + 0x0200808080808080ull;
+    return make_uint2((unsigned)y, (unsigned)(y >> 32));
 }
 
-// bf16 pair of two bytes' digits (y - 128 for byte k of u and of v)
+// fp16 pair of two bytes' digits (y - 128 for byte k of u and of v): 0x6400 | y
+// is 1024 + y, and the subtraction is exact
 __device__ __forceinline__ uint32_t digit_pair(unsigned u, unsigned v, int k) {
     const unsigned p = __byte_perm(u, v, k | (k << 4) | ((4 + k) << 8) | ((4 + k) << 12));
-    // 128 + (y & 127), and -128 or -256 by y's top bit: exact in bf16
-    const unsigned t = (p & 0x007f007fu) | 0x43004300u;
-    const unsigned c = (~p & 0x00800080u) | 0xc300c300u;
     uint32_t r;
-    asm("add.rn.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(t), "r"(c));
+    asm("add.rn.f16x2 %0, %1, %2;" : "=r"(r) : "r"((p & 0x00ff00ffu) | 0x64006400u), "r"(0xe480e480u));   // - 1152
     return r;
 }
 
 __device__ __forceinline__ uint32_t top_pair(unsigned u, unsigned v) {
-    constexpr float kRound = 12582912.f;
-    const float a = __fsub_rn(__int_as_float(0x4b400000 + ((int)u >> 16)), kRound);
-    const float b = __fsub_rn(__int_as_float(0x4b400000 + ((int)v >> 16)), kRound);
-    return pack_bf16x2(a, b);
+    uint32_t r;
+    asm("add.rn.f16x2 %0, %1, %2;" : "=r"(r) : "r"(__byte_perm(u, v, 0x7632) | 0x64006400u), "r"(0xe600e600u));   // - 1536
+    return r;
 }
 
 // Eight columns of one row into the digit images: piece at `dst`, digit a at
@@ -93,9 +94,9 @@ __device__ __forceinline__ void store_digits(const double (&l)[8], int E, uint8_
     unsigned yl[8], yh[8];
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
-        const unsigned long long y = biased_digits(l[e], E);
-        yl[e] = (unsigned)y;
-        yh[e] = (unsigned)(y >> 32);
+        const uint2 y = biased_digits(l[e], E);
+        yl[e] = y.x;
+        yh[e] = y.y;
     }
 #pragma unroll
     for (int a = 0; a < kNS; ++a) {
@@ -110,11 +111,14 @@ __device__ __forceinline__ void store_digits(const double (&l)[8], int E, uint8_
     }
 }
 
+// Instruction descriptor: fp16 x fp16 -> f32, both K-major, M = 128, N = n.
+constexpr uint32_t idesc_f16(uint32_t n) { return (1u << 4) | ((n >> 3) << 17) | ((128u >> 4) << 24); }
+
 // The MMAs of one stage (two K = 16 steps): every digit product with a + b <
 // kNG into group a + b; the first stage of a tile overwrites the groups.
 template <int kNT, bool FIRST>
 __device__ __forceinline__ void issue(uint32_t tacc, uint64_t ad0, uint64_t bd0) {
-    constexpr uint32_t idesc = idesc_bf16(kNT), kBChunk = b_chunk(kNT);
+    constexpr uint32_t idesc = idesc_f16(kNT), kBChunk = b_chunk(kNT);
 #pragma unroll
     for (int a = 0; a < kNS; ++a)
 #pragma unroll
@@ -137,16 +141,22 @@ __device__ __forceinline__ void tmem_ld4(uint32_t taddr, float* v) {
 }
 
 // sum_g S_g 256^(5 - g), groups 6 and 7 rounded: the product of the two rows
-// in units of 2^-54
+// in units of 2^-56.  Groups 0 .. 2 (below 2^22) and 6, 7 (as one rounded
+// float) turn into integers by an addition; only 3 .. 5 need the conversion
+// instruction, an eighth of an addition's rate.
 __device__ __forceinline__ long long combine(const float (&s)[kNG]) {
-    const int t01 = __float2int_rn(s[0]) * 256 + __float2int_rn(s[1]);
-    long long v = (long long)t01 << 32;
-    v += (long long)__float2int_rn(s[2]) * (1 << 24);
+    constexpr float kRound = 12582912.f;                  // 1.5 2^23, unit 1
+    constexpr int kBits = 0x4b400000;
+    const int t0 = __float_as_int(__fadd_rn(s[0], kRound)) - kBits;
+    const int t1 = __float_as_int(__fadd_rn(s[1], kRound)) - kBits;
+    const int t2 = __float_as_int(__fadd_rn(s[2], kRound)) - kBits;
+    const float low = __fmaf_rn(s[7], 0x1p-8f, s[6]);
+    const int t6 = __float_as_int(__fmaf_rn(low, 0x1p-8f, kRound)) - kBits;
+    long long v = (long long)(t0 * 256 + t1) << 32;
+    v += (long long)t2 * (1 << 24);
     v += (long long)__float2int_rn(s[3]) * (1 << 16);
     v += (long long)__float2int_rn(s[4]) * (1 << 8);
-    v += __float2int_rn(s[5]);
-    const int t = __float2int_rn(s[6]) + ((__float2int_rn(s[7]) + 128) >> 8);
-    return v + ((t + 128) >> 8);
+    return v + (__float2int_rn(s[5]) + t6);
 }
 
 enum : int { kFactorMode = 0, kInnerMode = 1, kInvApply = 2, kInvUpdate = 3 };
@@ -237,14 +247,15 @@ __global__ void __launch_bounds__(kThreads, 1)
             col0 = kNT * chunks;
             return;
         }
-        col0 = (q & 1) * kNT;
+        constexpr int kParts = GP_NB / kNT;
+        col0 = (q % kParts) * kNT;
         if (MODE == kInvApply) {
             I = J;
-            K = q >> 1;
+            K = q / kParts;
             return;
         }
         if (MODE == kInvUpdate) {
-            const int lower = (b.nt - 1 - J) * (J + 1), v = q >> 1;
+            const int lower = (b.nt - 1 - J) * (J + 1), v = q / kParts;
             if (v < lower) {
                 I = J + 1 + v / (J + 1);
                 K = v % (J + 1);
@@ -255,10 +266,10 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         int ii, kk;
         if (which == kUpdateColumn) {
-            ii = q >> 1;
+            ii = q / kParts;
             kk = 0;
         } else {
-            tri_decode(q >> 1, ii, kk);
+            tri_decode(q / kParts, ii, kk);
             if (which == kUpdateRest) {
                 ++ii;
                 ++kk;
@@ -329,9 +340,9 @@ __global__ void __launch_bounds__(kThreads, 1)
                 for (int j = 0; j < 8; ++j) cv[j] = fresh ? 0.0 : p[(size_t)(c + j) * GP_NB];
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
-                    double scale = 0x1p-54;
+                    double scale = 0x1p-56;
                     if (kInv) {
-                        const int e = 1023 - 54 + ea + eb[c + j];      // 0 below the normal range
+                        const int e = 1023 - 56 + ea + eb[c + j];      // 0 below the normal range
                         scale = __hiloint2double(e > 0 ? e << 20 : 0, 0);
                     }
                     const double d = __ll2double_rn(v[c + j]);
@@ -345,39 +356,43 @@ __global__ void __launch_bounds__(kThreads, 1)
         // this warp's pieces of a stage: 32 rows (of the 128 of A, then the NT
         // of B) by 8 columns.  Operand rows run along a tile's columns for L and
         // W, along its rows (eight consecutive doubles a lane) for X and S.
-        auto load = [&](int w, int kc, int u, double (&v)[8], int& E) {
+        // A work item's pointers are formed once; a stage moves them on.
+        struct Piece {
+            const double* p;       // its first value
+            int step;              // to the next of the eight columns
+            int E;
+        };
+        auto source = [&](int w, int u) -> Piece {
             int t, I, K, col0;
             decode(w, t, I, K, col0);
             const int piece = min(cw + kConvWarps * u, kStagePieces - 1), rg = piece >> 2, oct = piece & 3;
             const bool isA = rg < 4;
-            const int row = (isA ? 32 * rg : col0 + 32 * (rg - 4)) + lane, k0 = 32 * kc + 8 * oct;
-            E = 0;
-            if (kInv) {
-                const bool byRow = isA && (MODE == kInvApply || I > J);
-                const double* src;
-                if (MODE == kInvApply) {
-                    src = isA ? tile_of(X, t, J, J) : tile_of(S, t, J, K);
-                    E = isA ? exps(t, J, 2)[row] : exps(t, K, 1)[row];
-                } else {
-                    src = byRow ? tile(t, I, J) : tile_of(X, t, J, isA ? I : K);
-                    if (!byRow) E = exps(t, isA ? I : K, 0)[row];
-                }
-                const double* p = byRow ? src + (size_t)k0 * GP_NB + row : src + (size_t)row * GP_NB + k0;
-                const int step = byRow ? GP_NB : 1;
-#pragma unroll
-                for (int e = 0; e < 8; ++e) v[e] = p[e * step];
+            const int row = (isA ? 32 * rg : col0 + 32 * (rg - 4)) + lane;
+            if (!kInv)
+                return {(isA ? tile(t, I, J) : tile(t, K, J)) + (size_t)(8 * oct) * GP_NB + row, GP_NB, 0};
+            const bool byRow = isA && (MODE == kInvApply || I > J);
+            const double* src;
+            int E = 0;
+            if (MODE == kInvApply) {
+                src = isA ? tile_of(X, t, J, J) : tile_of(S, t, J, K);
+                E = isA ? exps(t, J, 2)[row] : exps(t, K, 1)[row];
             } else {
-                const double* p = (isA ? tile(t, I, J) : tile(t, K, J)) + (size_t)k0 * GP_NB + row;
-#pragma unroll
-                for (int e = 0; e < 8; ++e) v[e] = p[e * GP_NB];
+                src = byRow ? tile(t, I, J) : tile_of(X, t, J, isA ? I : K);
+                if (!byRow) E = exps(t, isA ? I : K, 0)[row];
             }
+            return byRow ? Piece{src + (size_t)(8 * oct) * GP_NB + row, GP_NB, E}
+                         : Piece{src + (size_t)row * GP_NB + 8 * oct, 1, E};
         };
         double raw[kPieces][8];
-        int exq[kPieces];
+        Piece at[kPieces];
         int w = next_live(blockIdx.x), kc = 0;
         if (w < total) {
 #pragma unroll
-            for (int u = 0; u < kPieces; ++u) load(w, 0, u, raw[u], exq[u]);
+            for (int u = 0; u < kPieces; ++u) {
+                at[u] = source(w, u);
+#pragma unroll
+                for (int e = 0; e < 8; ++e) raw[u][e] = at[u].p[e * (kInv ? at[u].step : GP_NB)];
+            }
         }
         for (int g = 0; w < total && !abort_flag; ++g) {
             const int st = g & 1;
@@ -393,8 +408,13 @@ __global__ void __launch_bounds__(kThreads, 1)
                 const int piece = cw + kConvWarps * u, rg = piece >> 2, oct = piece & 3;
                 const bool isA = rg < 4;
                 uint8_t* dst = stage + (isA ? 0u : kABytes) + image_piece((isA ? 32 * rg : 32 * (rg - 4)) + lane, 8 * oct);
-                if (piece < kStagePieces) store_digits(raw[u], exq[u], dst, isA ? kChunkBytes : kBChunk);
-                if (wn < total) load(wn, kn, u, raw[u], exq[u]);
+                if (piece < kStagePieces) store_digits(raw[u], kInv ? at[u].E : 0, dst, isA ? kChunkBytes : kBChunk);
+                if (wn < total) {
+                    if (kn == 0) at[u] = source(wn, u);
+                    else         at[u].p += 32 * (kInv ? at[u].step : GP_NB);
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) raw[u][e] = at[u].p[e * (kInv ? at[u].step : GP_NB)];
+                }
             }
             // the tensor core reads shared memory through the asynchronous proxy
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -466,6 +486,9 @@ cudaError_t launch_update_f64_tc(const Batch& b, int J, cudaStream_t s, int whic
     const int m = b.nt - J - 1;
     const int tiles = which == kUpdateColumn ? m : (which == kUpdateRest ? m * (m - 1) / 2 : m * (m + 1) / 2);
     if (tiles <= 0) return cudaSuccess;
+    // quarter tiles where the half tiles would leave half of the SMs idle (the
+    // same bits; a tile's chain is 22 us in halves, about 15 in quarters)
+    if ((long long)4 * tiles * b.count <= device_sms()) return launch<32, kFactorMode>(b, J, s, which, 4 * tiles, kChunks);
     return launch<64, kFactorMode>(b, J, s, which, 2 * tiles, kChunks);
 }
 
