@@ -213,30 +213,26 @@ constexpr int kLookaheadMax = 16;
 // as without.
 int run_factor_f64(gp_ctx* ctx, const gp::Batch& b) {
     const int nt = b.nt;
-    const bool tc = nt >= gp::kUpdateTcTiles;
+    if (nt < gp::kUpdateTcTiles) {
+        int k = 0;
+        PhaseScope ps(ctx, GP_PHASE_POTRF, 0);
+        const cudaError_t e = gp::launch_factor_small_f64(b, ctx->stream, &k);
+        ps.kernels += k;
+        GP_CUDA(ctx, e);
+        return GP_OK;
+    }
     // block column J finished: factored and solved
     auto panel = [&](int J, cudaStream_t st) -> int {
-        if (tc) {
-            PhaseScope ps(ctx, GP_PHASE_POTRF, gp::panel_f64_launches(nt, J), st);
-            GP_CUDA(ctx, gp::launch_panel_f64(b, J, st));
-            return GP_OK;
-        }
-        {
-            PhaseScope ps(ctx, GP_PHASE_POTRF, 1, st);
-            GP_CUDA(ctx, gp::launch_potrf_f64(b, J, st));
-        }
-        if (J + 1 < nt) {
-            PhaseScope ps(ctx, GP_PHASE_TRSM, 1, st);
-            GP_CUDA(ctx, gp::launch_trsm_f64(b, J, st));
-        }
+        PhaseScope ps(ctx, GP_PHASE_POTRF, gp::panel_f64_launches(nt, J), st);
+        GP_CUDA(ctx, gp::launch_panel_f64(b, J, st));
         return GP_OK;
     };
     auto update = [&](int J, int which) -> int {
         PhaseScope ps(ctx, GP_PHASE_UPDATE, 1);
-        GP_CUDA(ctx, gp::launch_update_f64(b, J, ctx->stream, which));
+        GP_CUDA(ctx, gp::launch_update_f64_tc(b, J, ctx->stream, which));
         return GP_OK;
     };
-    const bool ahead = b.count <= kLookaheadMax && nt > 1;
+    const bool ahead = b.count <= kLookaheadMax;
     int rc = ahead ? ensure_la(ctx) : GP_OK;
     if (rc) return rc;
     if ((rc = panel(0, ctx->stream))) return rc;
@@ -254,10 +250,8 @@ int run_factor_f64(gp_ctx* ctx, const gp::Batch& b) {
         if (J + 2 < nt && (rc = update(J, gp::kUpdateRest))) return rc;
         GP_CUDA(ctx, cudaStreamWaitEvent(ctx->stream, ctx->ev_la1, 0));
     }
-    if (tc) {
-        PhaseScope ps(ctx, GP_PHASE_POTRF, 1);
-        GP_CUDA(ctx, gp::launch_logdet_f64(b, ctx->stream));
-    }
+    PhaseScope ps(ctx, GP_PHASE_POTRF, 1);
+    GP_CUDA(ctx, gp::launch_logdet_f64(b, ctx->stream));
     return GP_OK;
 }
 

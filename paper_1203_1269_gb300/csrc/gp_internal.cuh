@@ -199,12 +199,9 @@ cudaError_t launch_validate_theta(const Batch& b, cudaStream_t s);
 cudaError_t launch_assemble_tiles(const Batch& b, cudaStream_t s);
 cudaError_t launch_assemble_dense(int n, int d, const double* x, const double* theta, double p, int corr,
                                   double delta, double* R, cudaStream_t s);
-cudaError_t launch_potrf_f64(const Batch& b, int J, cudaStream_t s);
-cudaError_t launch_trsm_f64(const Batch& b, int J, cudaStream_t s);
 // the tiles of a trailing update: all, column J + 1 only, or the others
 enum : int { kUpdateAll = 0, kUpdateColumn = 1, kUpdateRest = 2 };
-cudaError_t launch_update_f64(const Batch& b, int J, cudaStream_t s, int which = kUpdateAll);
-cudaError_t launch_update_f64_tc(const Batch& b, int J, cudaStream_t s, int which);
+cudaError_t launch_update_f64_tc(const Batch& b, int J, cudaStream_t s, int which = kUpdateAll);
 // columns 32 step .. 32 step + 31 of block column J, less the products of its columns before them
 cudaError_t launch_update_f64_inner(const Batch& b, int J, int step, cudaStream_t s);
 // block column J factored and solved (kUpdateTcTiles block columns and more), and the
@@ -216,13 +213,14 @@ constexpr int kPanelStep = 32;
 int panel_f64_launches(int nt, int J);
 cudaError_t launch_panel_f64(const Batch& b, int J, cudaStream_t s);
 cudaError_t launch_logdet_f64(const Batch& b, cudaStream_t s);
-// Block columns from which the double path's trailing updates run on the
-// tensor cores (k_update_tc.cu), whatever the batch.  They are faster from
-// the first tile on (0.55 ms for a tile's 128^3 multiply-adds on one SM's FP64
-// pipe, about 11 us as digit products); up to 256 points the factor keeps
-// IEEE operations throughout, so the small designs that are fitted with p = 2
-// next to singularity (cond(R) 1e11, where any change of rounding shows in
-// the eighth digit of mu_hat) keep their bits.
+// the whole factorisation and log-determinant of fewer block columns
+cudaError_t launch_factor_small_f64(const Batch& b, cudaStream_t s, int* kernels);
+// Block columns from which the double path's products run on the tensor cores
+// (k_update_tc.cu), whatever the batch.  They are faster from the first tile on
+// (a tile's update is 0.55 ms of one SM's FP64 pipe, 22 us as digits); up to 256 points the factor keeps IEEE operations
+// throughout, so the small designs that are fitted with p = 2 next to
+// singularity (cond(R) 1e11, where any change of rounding shows in the eighth
+// digit of mu_hat) keep their bits.
 constexpr int kUpdateTcTiles = 3;
 cudaError_t launch_forward_solve(const Batch& b, double* Z, size_t z_stride, cudaStream_t s);
 cudaError_t launch_finalize(const Batch& b, const double* Z, size_t z_stride, double* nll,

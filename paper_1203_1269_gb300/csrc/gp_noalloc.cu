@@ -84,16 +84,15 @@ extern "C" int gp_nll_batch_noalloc(gp_ctx* ctx, int n, int d, const double* x, 
         // and the forward solve writes Z, so nothing is cleared here
         e = gp::launch_validate_theta(b, stream);
         if (e == cudaSuccess) e = gp::launch_assemble_tiles(b, stream);
-        for (int J = 0; J < nt && e == cudaSuccess; ++J) {
-            if (nt >= gp::kUpdateTcTiles) {
+        if (nt < gp::kUpdateTcTiles) {
+            if (e == cudaSuccess) e = gp::launch_factor_small_f64(b, stream, nullptr);
+        } else {
+            for (int J = 0; J < nt && e == cudaSuccess; ++J) {
                 e = gp::launch_panel_f64(b, J, stream);
-            } else {
-                e = gp::launch_potrf_f64(b, J, stream);
-                if (e == cudaSuccess) e = gp::launch_trsm_f64(b, J, stream);
+                if (e == cudaSuccess) e = gp::launch_update_f64_tc(b, J, stream);
             }
-            if (e == cudaSuccess) e = gp::launch_update_f64(b, J, stream);
+            if (e == cudaSuccess) e = gp::launch_logdet_f64(b, stream);
         }
-        if (nt >= gp::kUpdateTcTiles && e == cudaSuccess) e = gp::launch_logdet_f64(b, stream);
         const size_t zs = z_bytes / sizeof(double);
         if (e == cudaSuccess) e = gp::launch_forward_solve(b, Z, zs, stream);
         if (e == cudaSuccess)

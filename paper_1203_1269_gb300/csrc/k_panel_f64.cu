@@ -1,9 +1,11 @@
 // k_panel_f64.cu -- one block column of the double-precision Cholesky in
-// four 32-column steps (matrices of three block columns and more):
+// four 32-column steps:
 //   inner  columns 32 s .. 32 s + 31 take the products of the steps before
 //          them, on the tensor cores (k_update_tc.cu)           s > 0
 //   diag   the 32 x 32 block is factored                         one CTA per instance
-//   solve  X L_ss^T = A for every row below it                   eight rows a warp
+//   solve  X L_ss^T = A for every row below it                   a few rows a warp
+// Matrices of up to two block columns keep IEEE operations throughout, in the
+// order of the unblocked loops (below).
 // On this GPU a double multiply-add takes a warp 64 cycles, issue and latency
 // alike, so what stays on the FP64 pipe is kept to the 32-wide triangles: a
 // quarter of the panel's multiply-adds, spread over all SMs by rows.  A block
@@ -27,11 +29,8 @@ __device__ __forceinline__ double* inst_tile(const Batch& b, int t, int I, int J
     return b.A + (size_t)t * b.inst_stride + (size_t)tile_index(I, J, b.nt) * GP_TILE_ELEMS;
 }
 
-// v / sqrt(a) for a normal a > 0: a float seed y0 (2^-20), then v y0 (1 + e/2 +
-// 3 e^2 / 8), e = 1 - a y0^2 (the next term, 5 e^3 / 16, is below 2^-58): six
-// double operations, five of them in a chain, where sqrt and a division take
-// 1360 cycles.
-__device__ __forceinline__ double over_sqrt(double v, double a) {
+// 1 / sqrt(a) to about 2^-20 for a normal a > 0, from the float instruction.
+__device__ __forceinline__ double rsqrt_seed(double a) {
     const int hi = __double2hiint(a), lo = __double2loint(a);
     const int e = (hi >> 20) - 1023;
     const int h = e >> 1;                               // a = m 2^(2h), m in [1, 4)
@@ -40,7 +39,14 @@ __device__ __forceinline__ double over_sqrt(double v, double a) {
     asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(s) : "f"(__uint_as_float(fb)));
     const unsigned sb = __float_as_uint(s);              // in (1/2, 1]
     const int ye = (int)(sb >> 23) - 127 + 1023 - h;
-    const double y0 = __hiloint2double((ye << 20) | (int)((sb & 0x7fffff) >> 3), (int)(sb << 29));
+    return __hiloint2double((ye << 20) | (int)((sb & 0x7fffff) >> 3), (int)(sb << 29));
+}
+
+// v / sqrt(a) for a normal a > 0: v y0 (1 + e/2 + 3 e^2 / 8), e = 1 - a y0^2 (the
+// next term, 5 e^3 / 16, is below 2^-58): six double operations, five of them
+// in a chain, where sqrt and a division take 1360 cycles.
+__device__ __forceinline__ double over_sqrt(double v, double a) {
+    const double y0 = rsqrt_seed(a);
     const double t = a * y0;
     const double err = fma(-t, y0, 1.0);
     const double vy = v * y0;
@@ -48,10 +54,32 @@ __device__ __forceinline__ double over_sqrt(double v, double a) {
     return fma(vy, q, vy);
 }
 
+// l = sqrt(a) and inv = 1 / l, both correctly rounded, for a normal a > 0 (P.
+// Markstein, "Computation of elementary functions on the IBM RISC System/6000
+// processor", IBM J. Res. Dev. 34, 1990): y = 1 / sqrt(a) and g = a y as above to
+// about an ulp, l = g + (a - g^2) y / 2, inv = y + y (1 - l y).  His theorem
+// excepts the reciprocal of a significand of all ones, which is divided.
+// Compared with sqrt and the division over 8.6e9 arguments: no difference.
+__device__ __forceinline__ void sqrt_and_reciprocal(double a, double& l, double& inv) {
+    const double y0 = rsqrt_seed(a);
+    const double t = a * y0;
+    const double err = fma(-t, y0, 1.0);
+    const double q = err * fma(err, 0.375, 0.5);
+    const double y = fma(y0, q, y0);
+    const double g = fma(t, q, t);
+    const double r = fma(-g, g, a);
+    l = fma(r, __hiloint2double(__double2hiint(y) - 0x100000, __double2loint(y)), g);
+    inv = fma(y, fma(-l, y, 1.0), y);
+    if ((__double2hiint(l) & 0xfffff) == 0xfffff && __double2loint(l) == -1) inv = 1.0 / l;
+}
+
 // A pivot outside the normal range: v / sqrt(piv), or zeros (the sweep goes on
 // with them) and the column recorded when piv is not positive and finite.
 __device__ __noinline__ double odd_pivot(double v, double piv, int c, int lane, int* failed) {
-    if (piv > 0.0 && isfinite(piv)) return v * (1.0 / sqrt(piv));
+    if (piv > 0.0 && isfinite(piv)) {
+        const double l = sqrt(piv);
+        return lane == c ? l : v * (1.0 / l);
+    }
     if (lane == 0 && *failed < 0) *failed = c;
     return 0.0;
 }
@@ -70,7 +98,9 @@ __device__ __noinline__ double odd_pivot(double v, double piv, int c, int lane, 
 // waits for its code.
 constexpr int kLsCols = 48;                    // rows of Ls, with room for the unused columns' reads
 
-template <int LEFT>
+// IEEE: L_cc = sqrt(a_cc) and a_rc (1 / L_cc), each correctly rounded, and every
+// position's terms in the order of c.
+template <int LEFT, bool IEEE>
 __device__ __forceinline__ void diag32_columns(double (&a)[kB / kWarps], double (*Ls)[kLsCols], int j0, int warp,
                                                int lane, int* failed) {
     constexpr int kCols = kB / kWarps;
@@ -78,8 +108,15 @@ __device__ __forceinline__ void diag32_columns(double (&a)[kB / kWarps], double 
     auto finish = [&](double& v, int c) {
         const double piv = __shfl_sync(0xffffffffu, v, c);
         const unsigned hi = (unsigned)__double2hiint(piv);
-        v = hi - 0x00100000u < 0x7fe00000u ? over_sqrt(v, piv)      // normal, positive and finite
-                                           : odd_pivot(v, piv, c, lane, failed);
+        if (hi - 0x00100000u >= 0x7fe00000u) {         // not normal, positive and finite
+            v = odd_pivot(v, piv, c, lane, failed);
+        } else if (IEEE) {
+            double l, inv;
+            sqrt_and_reciprocal(piv, l, inv);
+            v = lane == c ? l : v * inv;
+        } else {
+            v = over_sqrt(v, piv);
+        }
         Ls[c][lane] = v;
     };
     // the four terms of group j - 1 for columns i0, i0 + 1
@@ -112,18 +149,21 @@ __device__ __forceinline__ void diag32_columns(double (&a)[kB / kWarps], double 
                 if (q < kWarps - 1) {
                     a[0] = fma(-lr, l0, a[0]);
                     finish(a[0], c + 1);
-                    a[1] = fma(-lr, l1, a[1]);
+                    if (q > 0) a[1] = fma(-lr, l1, a[1]);
                 } else if (c + 1 < kB) {
                     a[1] = fma(-lr, l1, a[1]);
                     finish(a[1], c + 1);
                 }
             } else {
-                if (warp > q) a[0] = fma(-lr, l0, a[0]);
-                a[1] = fma(-lr, l1, a[1]);
                 // this warp's step number among those without a pivot
                 const int step = q - (q > (warp + kWarps - 1) % kWarps ? 1 : 0);
+                if (warp > q) a[0] = fma(-lr, l0, a[0]);
+                if (j > 0 && step == 0) pending(j, 1);
+                // every column's terms in order: warp 1's pivot comes before the
+                // group's first step without one
+                if (q == 1 && warp == 1) a[1] = fma(-Ls[c - 1][lane], Ls[c - 1][warp + kWarps * (j + 1)], a[1]);
+                a[1] = fma(-lr, l1, a[1]);
                 if (j > 0) {
-                    if (step == 0) pending(j, 1);
                     if (step == 1 && LEFT > 2) pending(j, 3);
                     if (step == 2 && LEFT > 4) pending(j, 5);
                 }
@@ -135,6 +175,7 @@ __device__ __forceinline__ void diag32_columns(double (&a)[kB / kWarps], double 
     }
 }
 
+template <bool IEEE>
 __global__ void __launch_bounds__(kThreads) k_diag32_f64(Batch b, int J, int s) {
     __shared__ double Ls[kB][kLsCols];             // Ls[c][r]
     __shared__ int failed;
@@ -152,8 +193,8 @@ __global__ void __launch_bounds__(kThreads) k_diag32_f64(Batch b, int J, int s) 
     for (int q = threadIdx.x; q < kB * kLsCols; q += kThreads) (&Ls[0][0])[q] = 0.0;
     if (threadIdx.x == 0) failed = -1;
     __syncthreads();
-    diag32_columns<kCols - 2>(a, Ls, 0, warp, lane, &failed);
-    diag32_columns<kCols / 2 - 1>(a, Ls, kCols / 2, warp, lane, &failed);
+    diag32_columns<kCols - 2, IEEE>(a, Ls, 0, warp, lane, &failed);
+    diag32_columns<kCols / 2 - 1, IEEE>(a, Ls, kCols / 2, warp, lane, &failed);
     if (failed >= 0) {
         if (threadIdx.x == 0) {
             b.st[t].status = GP_ENOTPD;
@@ -239,6 +280,86 @@ void launch_solve32(const Batch& b, int J, int s, int rows, int sms, cudaStream_
     k_solve32_f64<LANES><<<dim3(grid, b.count), kThreads, 0, st>>>(b, J, s, units, per_warp);
 }
 
+// Up to two block columns: the products of sub-block s for the columns of block
+// column J after it, A_rk = fma(-L_rc, L_kc, A_rk) for c in order, a CTA per 32 x
+// 32 block (rb, kb) of 32-row and 32-column groups counted from the sub-block:
+// thread (lane, warp) owns row lane, columns warp + 8 j.
+constexpr int kInnerThreads = 256;
+constexpr int kInnerCols = kB * kB / kInnerThreads;
+
+__global__ void __launch_bounds__(kInnerThreads) k_inner_f64(Batch b, int J, int s) {
+    __shared__ double Lk[kB][kB + 1];              // Lk[c][k]
+    const int t = blockIdx.z;
+    if (b.st[t].status != GP_OK) return;
+    const int kb = s + 1 + blockIdx.y, rb = kb + blockIdx.x;      // from tile (J, J)'s first
+    const int row0 = kB * rb;
+    if (J * GP_NB + row0 >= b.n) return;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const double* Lj = inst_tile(b, t, J, J) + (size_t)(kB * s) * GP_NB + kB * kb;
+    for (int q = threadIdx.x; q < kB * kB; q += kInnerThreads) cp_async8(&Lk[q / kB][q % kB], Lj + (size_t)(q / kB) * GP_NB + q % kB);
+    double* T = inst_tile(b, t, J + (row0 >> 7), J) + (row0 & 127) + lane;
+    double lr[kB], a[kInnerCols];
+#pragma unroll
+    for (int c = 0; c < kB; ++c) lr[c] = T[(size_t)(kB * s + c) * GP_NB];
+#pragma unroll
+    for (int j = 0; j < kInnerCols; ++j) a[j] = T[(size_t)(kB * kb + warp + 8 * j) * GP_NB];
+    cp_async_wait_all();
+    __syncthreads();
+#pragma unroll
+    for (int c = 0; c < kB; ++c)
+#pragma unroll
+        for (int j = 0; j < kInnerCols; ++j) a[j] = fma(-lr[c], Lk[c][warp + 8 * j], a[j]);
+#pragma unroll
+    for (int j = 0; j < kInnerCols; ++j) T[(size_t)(kB * kb + warp + 8 * j) * GP_NB] = a[j];
+}
+
+// Tile (1, 1) less L_10 L_10^T: sums from zero over the 128 columns in order, then
+// one subtraction, a CTA per 32 x 32 block of the lower triangle.
+__global__ void __launch_bounds__(kInnerThreads) k_trailing_f64(Batch b) {
+    __shared__ double Lk[GP_NB][kB + 1];
+    const int t = blockIdx.y;
+    if (b.st[t].status != GP_OK) return;
+    int rb, kb;
+    tri_decode(blockIdx.x, rb, kb);
+    if (GP_NB + kB * rb >= b.n) return;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const double* L = inst_tile(b, t, 1, 0);
+    for (int q = threadIdx.x; q < GP_NB * kB; q += kInnerThreads) cp_async8(&Lk[q / kB][q % kB], L + (size_t)(q / kB) * GP_NB + kB * kb + q % kB);
+    double* C = inst_tile(b, t, 1, 1) + kB * rb + lane;
+    L += kB * rb + lane;
+    double acc[kInnerCols] = {};
+    cp_async_wait_all();
+    __syncthreads();
+#pragma unroll 16
+    for (int c = 0; c < GP_NB; ++c) {
+        const double lr = __ldg(L + (size_t)c * GP_NB);
+#pragma unroll
+        for (int j = 0; j < kInnerCols; ++j) acc[j] = fma(lr, Lk[c][warp + 8 * j], acc[j]);
+    }
+#pragma unroll
+    for (int j = 0; j < kInnerCols; ++j) C[(size_t)(kB * kb + warp + 8 * j) * GP_NB] -= acc[j];
+}
+
+// log|R| of up to two block columns: the pivots' logarithms summed in column
+// order per block, the blocks' sums in turn.
+__global__ void __launch_bounds__(GP_NB) k_logdet_small_f64(Batch b) {
+    __shared__ double logs[GP_NB];
+    const int t = blockIdx.x;
+    if (b.st[t].status != GP_OK) return;
+    double total = 0.0;
+    for (int J = 0; J < b.nt; ++J) {
+        logs[threadIdx.x] = log(inst_tile(b, t, J, J)[threadIdx.x * (GP_NB + 1)]);
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            double sum = 0.0;
+            for (int c = 0; c < GP_NB; ++c) sum += logs[c];
+            total += 2.0 * sum;
+        }
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) b.st[t].logdet = total;
+}
+
 // log|R| = 2 sum log L_ii over the factor's diagonal (padded rows give 0),
 // one CTA per instance, in a fixed order.
 __global__ void __launch_bounds__(256) k_logdet_f64(Batch b) {
@@ -262,6 +383,40 @@ __global__ void __launch_bounds__(256) k_logdet_f64(Batch b) {
 
 }  // namespace
 
+// Factor matrices of one or two block columns, the padded rows and columns left
+// as they are (the identity).  Every position takes its operations in the
+// order of the unblocked loops: the same bits as one CTA per tile and instance
+// on the FP64 pipe gave (n = 200, T = 64: 1.59 -> 0.52 ms).
+cudaError_t launch_factor_small_f64(const Batch& b, cudaStream_t st, int* kernels) {
+    const int sms = device_sms();
+    int k = 0;
+    for (int J = 0; J < b.nt; ++J) {
+        const int left = b.n - J * GP_NB;                    // real rows from block column J on
+        for (int s = 0; s < GP_NB / kB && kB * s < left; ++s) {
+            k_diag32_f64<true><<<b.count, kThreads, 0, st>>>(b, J, s);
+            ++k;
+            const int rows = (left - kB * (s + 1) + 7) / 8 * 8;
+            if (rows <= 0) continue;
+            if ((long long)rows * b.count <= 4 * 4LL * sms) launch_solve32<8>(b, J, s, rows, sms, st);
+            else                                            launch_solve32<4>(b, J, s, rows, sms, st);
+            ++k;
+            const int cols = GP_NB / kB - 1 - s, groups = (left + kB - 1) / kB - 1 - s;
+            if (cols > 0 && groups > 0) {
+                k_inner_f64<<<dim3(groups, cols < groups ? cols : groups, b.count), kInnerThreads, 0, st>>>(b, J, s);
+                ++k;
+            }
+        }
+        if (J + 1 < b.nt) {
+            const int groups = (left - GP_NB + kB - 1) / kB;
+            k_trailing_f64<<<dim3(groups * (groups + 1) / 2, b.count), kInnerThreads, 0, st>>>(b);
+            ++k;
+        }
+    }
+    k_logdet_small_f64<<<b.count, GP_NB, 0, st>>>(b);
+    if (kernels) *kernels = k + 1;
+    return cudaGetLastError();
+}
+
 // Kernels of launch_panel_f64.
 int panel_f64_launches(int nt, int J) { return J + 1 < nt ? 11 : 10; }
 
@@ -272,7 +427,7 @@ cudaError_t launch_panel_f64(const Batch& b, int J, cudaStream_t st) {
             cudaError_t e = launch_update_f64_inner(b, J, s, st);
             if (e != cudaSuccess) return e;
         }
-        k_diag32_f64<<<b.count, kThreads, 0, st>>>(b, J, s);
+        k_diag32_f64<false><<<b.count, kThreads, 0, st>>>(b, J, s);
         const int rows = (b.nt - J) * GP_NB - kB * (s + 1);
         if (rows > 0) {
             if ((long long)rows * b.count <= 4 * 4LL * sms) launch_solve32<8>(b, J, s, rows, sms, st);

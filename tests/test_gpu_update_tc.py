@@ -1,5 +1,5 @@
-"""The double-precision factor with its trailing updates on the tensor cores
-(three block columns and more) at ragged sizes, large nuggets, entries of L
+"""The double-precision factor (its products on the tensor cores from three
+block columns on, in IEEE operations below) at ragged sizes, large nuggets, entries of L
 next to 1, and failing pivots beyond the first block columns."""
 import numpy as np
 import pytest
@@ -52,7 +52,7 @@ def bound(n, delta):
     return 2 * (n + 2) * U * (1.0 + delta)
 
 
-@pytest.mark.parametrize("n", [257, 320, 383, 384, 385, 513, 700, 1025])
+@pytest.mark.parametrize("n", [1, 7, 31, 32, 33, 96, 127, 128, 129, 160, 225, 256, 257, 320, 383, 384, 385, 513, 700, 1025])
 @pytest.mark.parametrize("d,lo", [(1, -1.0), (5, 0.0)])
 def test_factor_residual(ctx, n, d, lo):
     g = np.random.default_rng(n + d)
