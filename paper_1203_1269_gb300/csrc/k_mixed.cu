@@ -33,6 +33,23 @@ namespace {
 
 // ----------------------------------------------------------- kernels -------
 
+// The next slice of a double-float x (scaled so |x| < 2^7 before the first
+// one): the integer q nearest x.hi, |q| <= 128, times the slice's weight w =
+// 2^(-8a), so that x = sum_a slice_a and every product of slices carries its
+// own weight 2^(-8(a+b)) into the tensor-core accumulators; x moves on to
+// 256 (x - q).  q comes from the float 1.5 2^23, whose unit is 1: rintf's
+// instruction has a longer latency, which shows here, where eight warps' rows
+// are all there is to run (the panels' slicing, next_slice8, has warps enough
+// and too many additions: the kriging pass lost 0.8% to this form).
+__device__ __forceinline__ float cut_one(float& xh, float& xl, float w) {
+    constexpr float kRound = 12582912.f;
+    const float q = __fsub_rn(__fadd_rn(xh, kRound), kRound);
+    two_sum(__fsub_rn(xh, q), xl, xh, xl);       // xh - q is exact
+    xh = __fmul_rn(xh, 256.f);
+    xl = __fmul_rn(xl, 256.f);
+    return __fmul_rn(q, w);
+}
+
 // Diagonal block of column J in double-float on the FP32 pipes (an FP64
 // instruction costs about 64 FP32 ones here): L_JJ = chol(A_JJ), log-det,
 // the reciprocal diagonal, and W = L_JJ^-1 with the slices of W's rows.

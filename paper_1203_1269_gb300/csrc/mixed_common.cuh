@@ -178,21 +178,6 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float a, float b) {
     return *reinterpret_cast<uint32_t*>(&v);
 }
 
-// The next slice of a double-float x (scaled so |x| < 2^7 before the first
-// one): the integer q nearest x.hi, |q| <= 128, times the slice's weight w =
-// 2^(-8a), so that x = sum_a slice_a and every product of slices carries its
-// own weight 2^(-8(a+b)) into the tensor-core accumulators; x moves on to
-// 256 (x - q).  q comes from the float 1.5 2^23, whose unit is 1 (rintf's
-// instruction runs at a quarter of the rate of an addition).
-__device__ __forceinline__ float cut_one(float& xh, float& xl, float w) {
-    constexpr float kRound = 12582912.f;
-    const float q = __fsub_rn(__fadd_rn(xh, kRound), kRound);
-    two_sum(__fsub_rn(xh, q), xl, xh, xl);       // xh - q is exact
-    xh = __fmul_rn(xh, 256.f);
-    xl = __fmul_rn(xl, 256.f);
-    return __fmul_rn(q, w);
-}
-
 __device__ __forceinline__ void prefetch_l2(const void* p, uint32_t bytes) {
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
 }

@@ -45,7 +45,13 @@ __device__ __forceinline__ void st_global_v8(void* p, uint4 a, uint4 b) {
 __device__ __forceinline__ uint4 next_slice8(float (&xh)[8], float (&xl)[8], float w) {
     float m[8];
 #pragma unroll
-    for (int e = 0; e < 8; ++e) m[e] = cut_one(xh[e], xl[e], w);
+    for (int e = 0; e < 8; ++e) {
+        const float qv = rintf(xh[e]);
+        m[e] = __fmul_rn(qv, w);
+        two_sum(__fsub_rn(xh[e], qv), xl[e], xh[e], xl[e]);
+        xh[e] = __fmul_rn(xh[e], 256.f);
+        xl[e] = __fmul_rn(xl[e], 256.f);
+    }
     uint4 pk;
     pk.x = pack_bf16x2(m[0], m[1]);
     pk.y = pack_bf16x2(m[2], m[3]);
