@@ -54,7 +54,12 @@ typedef struct gp_model gp_model;
 typedef struct gp_plan gp_plan;
 
 /* Arithmetic of the factorisation.
- * GP_FP64:  assembly, Cholesky and solves in IEEE double.
+ * GP_FP64:  double precision throughout: assembly, pivots, row solves and
+ *           substitutions in IEEE double; from three block columns (n > 256)
+ *           on, the products of the Cholesky factorisation as exact digit
+ *           products on the tensor cores (7 digits of 8 bits per entry),
+ *           subtracted in double: the factor's backward error is that of
+ *           IEEE multiply-adds or smaller.
  * GP_MIXED: the panel solves and trailing updates of the blocked Cholesky
  *           on the tensor cores: operands split into bf16 slices, exact fp32
  *           accumulation of the product groups (Ozaki-style), recombined in
@@ -256,10 +261,11 @@ int gp_nll_batch(gp_ctx* ctx, int n, int d, const double* x, const double* y, in
  * depend on theta); for every gp_correlation.  Section 2 names a multi-start
  * gradient-based search as a possibly faster alternative to its GA; this is
  * the gradient such a search needs.  -2logL, mu_hat and w come from the
- * IEEE-double factor (nll equals gp_nll_batch's GP_FP64 result); R^-1 is
- * formed from that factor in double-float, about 48 bits (L^-1 by tile
- * diagonals, then L^-T L^-1: twice the factorisation's n^3/6 multiply-adds),
- * so the gradient's relative error is about cond(R) 2^-47 at worst.  nll,
+ * double-precision factor (nll equals gp_nll_batch's GP_FP64 result); R^-1 is
+ * formed from that factor by rows of L^-1 (twice the factorisation's n^3/6
+ * multiply-adds), as digit products on the tensor cores added in double, so
+ * the gradient's relative error is about cond(R) 2^-53 times a modest factor;
+ * the powers |dx|^p of a general p carry double-float precision there.  nll,
  * status as gp_nll_batch; grad rows are NaN where the status is not GP_OK.
  * d <= 16 (GP_ENOTSUP above).
  * Asynchronous. */

@@ -10,6 +10,8 @@
 // the powers with p = 1 for the Matern families.
 #pragma once
 
+#include <cmath>
+
 #include "df.cuh"
 #include "gp_internal.cuh"
 
@@ -34,6 +36,48 @@ __device__ __forceinline__ dfl matern_q_df(dfl h, int corr, dfl third) {
     if (corr == GP_CORR_MATERN32) return df_add(dfl{1.f, 0.f}, h);
     if (corr == GP_CORR_MATERN52) return df_add(dfl{1.f, 0.f}, df_fma(df_mul(h, h), third, h));
     return dfl{1.f, 0.f};
+}
+
+// exp(-S) in double without CUDA's exp (the reduction of P. T. P. Tang, ACM TOMS
+// 15 (1989)): an FP64 instruction is worth 64 FP32 ones here, so what counts is
+// their number, 11 against about 20.
+// exp(-S) = 2^(k/128) exp(r), k = round(-128 S / ln 2), r = -S - k ln2/128
+// (two fmas against ln2/128 as 32 + 53 bits), exp(r) - 1 = r + r^2 (1/2 + r/6 +
+// r^2/24 + r^3/120) (the next term is below 2^-60), times the table's 2^(j/128)
+// as a double-double, scaled by its exponent bits: 11 double operations.  S
+// above 700 takes exp.
+constexpr int kE64NBits = 7;
+constexpr int kE64N = 1 << kE64NBits;
+struct ExpTab64 {
+    double2 e2[kE64N];            // 2^(j/128) as (hi, lo)
+};
+
+__device__ __forceinline__ double exp_neg_tab64(double s, const ExpTab64& t) {
+    if (!(s < 700.0)) return exp(-s);
+    constexpr double kInv = 128.0 / 0.693147180559945309417232121458176568;
+    constexpr double kHi = 0x1.62e42fefp-8;                                // ln2 / 128, 33 bits
+    constexpr double kLo = 0x1.473de6af278edp-41;                          // and the rest
+    constexpr double kRound = 6755399441055744.0;                          // 1.5 2^52
+    const double kr = fma(-s, kInv, kRound);
+    const int k = __double2loint(kr);
+    const double kd = kr - kRound;
+    const double r = fma(-kd, kLo, fma(-kd, kHi, -s));
+    double q = fma(r, 1.0 / 120.0, 1.0 / 24.0);
+    q = fma(r, q, 1.0 / 6.0);
+    q = fma(r, q, 0.5);
+    const double w = fma(r * r, q, r);
+    const double2 T = t.e2[k & (kE64N - 1)];
+    const double v = T.x + fma(T.x, w, T.y);
+    return __hiloint2double(__double2hiint(v) + ((k >> kE64NBits) << 20), __double2loint(v));
+}
+
+// The table, in long double (64 significant bits or more).
+inline void exp_tab64_fill(ExpTab64& t) {
+    for (int j = 0; j < kE64N; ++j) {
+        const long double v = exp2l((long double)j / (long double)kE64N);
+        t.e2[j].x = (double)v;
+        t.e2[j].y = (double)(v - (long double)t.e2[j].x);
+    }
 }
 
 }  // namespace gp

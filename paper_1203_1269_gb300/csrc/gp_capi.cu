@@ -681,21 +681,20 @@ int auto_nll_batch(gp_ctx* ctx, int n, int d, const double* x, const double* y, 
 }
 
 // Workspace per candidate of gp_nll_grad_batch: the factor, L^-1, R^-1,
-// [a | w], its record, tile partial sums, and mu / sigma2 / log|R| (which
-// the caller does not ask for).
+// [a | w], its record, and mu / sigma2 / log|R| (which the caller does not ask
+// for).
 struct GradSizes {
-    size_t a, z, st, part, sc, per;
+    size_t a, z, st, sc, per;
 };
 
-GradSizes grad_sizes(int n, int d) {
+GradSizes grad_sizes(int n) {
     const int nt = gp::num_tiles(n);
     GradSizes g;
     g.a = align256(gp::packed_elems(n) * sizeof(double));
     g.z = align256((size_t)2 * nt * GP_NB * sizeof(double));
     g.st = align256(sizeof(gp::InstState));
-    g.part = align256((size_t)gp::packed_tiles(nt) * d * sizeof(double));
     g.sc = align256(3 * sizeof(double));
-    g.per = 3 * g.a + g.z + g.st + g.part + g.sc;
+    g.per = 3 * g.a + g.z + g.st + g.sc;
     return g;
 }
 
@@ -1324,8 +1323,8 @@ int gp_nll_grad_batch(gp_ctx* ctx, int n, int d, const double* x, const double* 
     if (!x || !y || !theta || !nll || !grad || !status) return fail(ctx, GP_EINVAL, "null pointer argument");
     GP_CUDA(ctx, cudaSetDevice(ctx->device));
     const int nt = gp::num_tiles(n);
-    const GradSizes g = grad_sizes(n, d);
-    const size_t a_bytes = g.a, z_bytes = g.z, st_bytes = g.st, part_bytes = g.part;
+    const GradSizes g = grad_sizes(n);
+    const size_t a_bytes = g.a, z_bytes = g.z, st_bytes = g.st;
     Chunking ch;
     if (!chunk_batch(ctx->opt, ctx->budget, ctx->models_bytes, g.per, 0, T, &ch))
         return fail(ctx, GP_ENOMEM, "one instance (%zu bytes) exceeds the HBM budget", g.per);
@@ -1338,7 +1337,6 @@ int gp_nll_grad_batch(gp_ctx* ctx, int n, int d, const double* x, const double* 
     double* Ri = (double*)c; c += a_bytes * Tc;
     double* Z = (double*)c; c += z_bytes * Tc;
     gp::InstState* st = (gp::InstState*)c; c += st_bytes * Tc;
-    double* partial = (double*)c; c += part_bytes * Tc;
     double* sc = (double*)c;
     for (int c0 = 0; c0 < T; c0 += Tc) {
         const int cnt = (T - c0 < Tc) ? (T - c0) : Tc;
@@ -1361,7 +1359,7 @@ int gp_nll_grad_batch(gp_ctx* ctx, int n, int d, const double* x, const double* 
                                              ctx->stream));
         }
         int kernels = 0;
-        cudaError_t e = gp::launch_grad(b, Z, zs, X, Ri, partial, status + c0, grad + (size_t)c0 * d,
+        cudaError_t e = gp::launch_grad(b, Z, zs, X, Ri, status + c0, grad + (size_t)c0 * d,
                                         ctx->stream, &kernels);
         ctx->launches += kernels;
         ctx->phase_launches[GP_PHASE_SOLVE] += kernels;
@@ -1834,7 +1832,7 @@ int gp_call_bytes(gp_ctx* ctx, int call, int n, int d, int count, int prec, size
         if (count < 1 || count > gp::kMaxCandidates)
             return fail(ctx, GP_EINVAL, "T = %d outside [1, 2^30]", count);
         if (d > 16) return fail(ctx, GP_ENOTSUP, "the gradient is built for d <= 16 (d = %d)", d);
-        return batch(grad_sizes(n, d).per, 0, bytes);
+        return batch(grad_sizes(n).per, 0, bytes);
     }
     case GP_CALL_FIT: {
         const size_t total = model_sizes(n, d).total;

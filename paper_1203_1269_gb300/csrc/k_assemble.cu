@@ -38,10 +38,10 @@ __device__ __forceinline__ double powabs(double diff, double p) {
     return (a == 0.0) ? 0.0 : pow(a, p);
 }
 
-// |dx|^p and exp(-S) in double without a pow or an exp per term (the reductions
-// of P. T. P. Tang's table-driven logarithm and exponential, ACM TOMS 16
-// (1990) and 15 (1989)): an FP64 instruction is worth 64 FP32 ones here, so
-// what counts is their number.
+// |dx|^p in double for a general p without a pow per term (the reduction of P. T.
+// P. Tang's table-driven logarithm, ACM TOMS 16 (1990), applied to the power):
+// an FP64 instruction is worth 64 FP32 ones here, so what counts is their
+// number.
 //
 // a = 2^m x, x in [1, 2), c_j the double nearest 1 / (1 + j/64) for the table
 // point nearest x: u = x c_j - 1 by one fma (|u| <= 2^-7, one rounding), and
@@ -50,25 +50,17 @@ __device__ __forceinline__ double powabs(double diff, double p) {
 // in long double, (1 + u)^p - 1 = p u + c2 u^2 + ... + c7 u^7 (the u^8 term
 // is below 2^-62), and one rounding at the end: a^p = A_hi + (A_hi t +
 // A_lo): 15 double operations.  m outside [-60, 4] takes pow.
-//
-// exp(-S) = 2^(k/128) exp(r), k = round(-128 S / ln 2), r = -S - k ln2/128
-// (two fmas against ln2/128 as 32 + 53 bits), exp(r) - 1 = r + r^2 (1/2 + r/6 +
-// r^2/24 + r^3/120) (the next term is below 2^-60), times the table's 2^(j/128)
-// as a double-double, scaled by its exponent bits: 11 double operations.  S
-// above 700 takes exp.
 constexpr int kP64NBits = 6;
 constexpr int kP64N = 1 << kP64NBits;
 constexpr int kP64Mlo = -60, kP64Mhi = 4;
 constexpr int kP64Ms = kP64Mhi - kP64Mlo + 1;
-constexpr int kE64NBits = 7;
-constexpr int kE64N = 1 << kE64NBits;
 struct PowTab64 {
     int on;                       // general p on the power-exponential family
     double c[8];                  // c[k] = C(p, k), k = 1 .. 7
     double inv[kP64N + 1];        // c_j (j = 64: 1/2, for x next to 2)
     double2 two[kP64Ms];          // 2^(m p), m = kP64Mlo .. kP64Mhi, as (hi, lo)
     double2 f[kP64N + 1];         // c_j^-p as (hi, lo)
-    double2 e2[kE64N];            // 2^(j/128) as (hi, lo)
+    ExpTab64 e;                   // exp_neg_tab64's table
 };
 static_assert(sizeof(PowTab64) + 512 < 32764, "kernel parameters");
 
@@ -89,25 +81,6 @@ __device__ __forceinline__ double pow_tab64(double a, double p, const PowTab64& 
     const double ah = T.x * P.x;
     const double al = fma(T.x, P.x, -ah) + fma(T.x, P.y, T.y * P.x);
     return ah + fma(ah, tt, al);
-}
-
-__device__ __forceinline__ double exp_neg_tab64(double s, const PowTab64& t) {
-    if (!(s < 700.0)) return exp(-s);
-    constexpr double kInv = 128.0 / 0.693147180559945309417232121458176568;
-    constexpr double kHi = 0x1.62e42fefp-8;                                // ln2 / 128, 33 bits
-    constexpr double kLo = 0x1.473de6af278edp-41;                          // and the rest
-    constexpr double kRound = 6755399441055744.0;                          // 1.5 2^52
-    const double kr = fma(-s, kInv, kRound);
-    const int k = __double2loint(kr);
-    const double kd = kr - kRound;
-    const double r = fma(-kd, kLo, fma(-kd, kHi, -s));
-    double q = fma(r, 1.0 / 120.0, 1.0 / 24.0);
-    q = fma(r, q, 1.0 / 6.0);
-    q = fma(r, q, 0.5);
-    const double w = fma(r * r, q, r);
-    const double2 T = t.e2[k & (kE64N - 1)];
-    const double v = T.x + fma(T.x, w, T.y);
-    return __hiloint2double(__double2hiint(v) + ((k >> kE64NBits) << 20), __double2loint(v));
 }
 
 __device__ __forceinline__ double powabs_t(double diff, double p, const PowTab64& t) {
@@ -250,7 +223,7 @@ k_assemble_tiles(Batch b, int group, PowTab64 ptab) {
                     for (int k = 0; k < DB; ++k)
                         if (k < d) s = fma(__ldg(b.theta + (size_t)t * d + k), D[k], s);
                 }
-                v = exp_neg_tab64(s, pt);
+                v = exp_neg_tab64(s, pt.e);
                 if (diag) v += b.delta;
             } else {
                 const double* th = b.theta + (size_t)t * d;
@@ -505,7 +478,7 @@ static void pow_tab64_fill(double p, PowTab64& t) {
             last.inv[j] = (double)(1.0L / (1.0L + (long double)j / (long double)kP64N));
             last.f[j] = split(powl((long double)last.inv[j], -(long double)p));
         }
-        for (int j = 0; j < kE64N; ++j) last.e2[j] = split(exp2l((long double)j / (long double)kE64N));
+        exp_tab64_fill(last.e);
         for (int m = kP64Mlo; m <= kP64Mhi; ++m) last.two[m - kP64Mlo] = split(exp2l((long double)m * (long double)p));
         last_p = p;
     }

@@ -24,7 +24,7 @@
 // The inverse in double-float multiply-adds on the FP32 pipes, along the tile
 // diagonals of X, took 36.6 ms of the gradient's 49 at n = 4064, T = 1.
 #include "corr.cuh"
-#include "gp_internal.cuh"
+#include "mixed_common.cuh"
 
 namespace gp {
 
@@ -37,72 +37,111 @@ __device__ __forceinline__ T* tile_at(T* base, size_t stride, int t, int I, int 
     return base + (size_t)t * stride + (size_t)tile_index(I, J, nt) * GP_TILE_ELEMS;
 }
 
-// X_JJ = L_JJ^-1 (lower; zeros above the diagonal), one CTA per (J, instance),
-// in double: row i of W from rows j < i, W_ij = -(1/L_ii) sum_{k=j}^{i-1} L_ik W_kj.
-// Dynamic smem: L and W as packed lower triangles (row r at r (r + 1) / 2).
+// X_JJ = W_J = L_JJ^-1 (lower; zeros above the diagonal) in double, a CTA per 32
+// columns of it (their rows above are zero): lane = column, warp w holds rows
+// c0 + w + 4 i of acc_ij = sum_{m<k} L_im W_mj in registers.  Step k finishes row
+// k (W_kj = -acc_kj / L_kk, W_kk = 1 / L_kk), one barrier, and adds its term to the
+// rows after it.  Four rows are one iteration of a loop (the rows move down
+// one register as they finish), in forms for up to 31, 23, 15 and 7 rows left.
+// 0.13 ms for every block of n = 4064 at once (0.45 ms with one CTA a block
+// and a dependent sum per entry).
 constexpr int kPackedTri = GP_NB * (GP_NB + 1) / 2;
+constexpr int kInvThreads = 128;
+constexpr int kInvWarps = kInvThreads / 32;
+constexpr int kInvCols = 32;
+constexpr int kInvRows = GP_NB / kInvWarps;            // rows of a warp
 __device__ __forceinline__ int prow(int r) { return r * (r + 1) / 2; }
 
-__global__ void __launch_bounds__(kThreads) k_inv_diag(Batch b, double* X) {
-    extern __shared__ double sm[];
-    double* Lp = sm;
-    double* Wp = sm + kPackedTri;
-    __shared__ double dinv[GP_NB];
-    const int J = blockIdx.x, t = blockIdx.y;
-    if (b.st[t].status != GP_OK) return;
-    const double* L = tile_at(b.A, b.inst_stride, t, J, J, b.nt);
-    for (int q = threadIdx.x; q < GP_TILE_ELEMS; q += kThreads) {
-        const int r = q % GP_NB, c = q / GP_NB;
-        if (r >= c) {
-            const double l = L[q];
-            Lp[prow(r) + c] = l;
-            Wp[prow(r) + c] = 0.0;
-            if (r == c) dinv[r] = 1.0 / l;    // one division per pivot
+// Rows k = k0 .. k0 + 31, or up to row 127 where LEFT rows of a warp are left.
+template <int LEFT>
+__device__ __forceinline__ void inv_rows(double (&acc)[kInvRows], const double* Lp, const double* dinv,
+                                         double (*Wk)[kInvCols], double* Xt, int k0, int c0, int warp, int lane) {
+#pragma unroll 1
+    for (int g = 0; g < 8; ++g) {
+#pragma unroll
+        for (int q = 0; q < kInvWarps; ++q) {
+            const int k = k0 + kInvWarps * g + q;
+            if (warp == q) {
+                const double w = c0 + lane == k ? dinv[k] : -dinv[k] * acc[0];
+                Wk[k & 1][lane] = w;
+                Xt[(size_t)(c0 + lane) * GP_NB + k] = w;
+            }
+            __syncthreads();
+            const double w = Wk[k & 1][lane];
+            if (warp > q) acc[0] = fma(Lp[prow(k - q + warp) + k], w, acc[0]);
+#pragma unroll
+            for (int i = 1; i <= LEFT; ++i) {
+                const int r = k - q + warp + kInvWarps * i;
+                if (i <= LEFT - 7 || r < GP_NB) acc[i] = fma(Lp[prow(r) + k], w, acc[i]);
+            }
         }
-    }
-    __syncthreads();
-    for (int i = 0; i < GP_NB; ++i) {
-        const double inv = dinv[i];
-        for (int j = threadIdx.x; j < i; j += kThreads) {
-            double s = 0.0;
-            for (int k = j; k < i; ++k) s = fma(Lp[prow(i) + k], Wp[prow(k) + j], s);
-            Wp[prow(i) + j] = -inv * s;
-        }
-        if (threadIdx.x == 0) Wp[prow(i) + i] = inv;
-        __syncthreads();
-    }
-    double* Xt = tile_at(X, b.inst_stride, t, J, J, b.nt);
-    for (int q = threadIdx.x; q < GP_TILE_ELEMS; q += kThreads) {
-        const int r = q % GP_NB, c = q / GP_NB;
-        Xt[q] = (r >= c) ? Wp[prow(r) + c] : 0.0;
-    }
-    // the exponents of W's rows, |W_rc| < 2^E, into the factor's diagonal tile
-    // (its slot 2; the factor's own diagonal block is not needed any more)
-    if (threadIdx.x < GP_NB) {
-        const int r = threadIdx.x;
-        unsigned m = 0;
-        for (int c = 0; c <= r; ++c) m = max(m, (unsigned)__double2hiint(Wp[prow(r) + c]) & 0x7fffffffu);
-        reinterpret_cast<int*>(tile_at(b.A, b.inst_stride, t, J, J, b.nt))[2 * GP_NB + r] = (int)(m >> 20) - 1022;
+#pragma unroll
+        for (int i = 0; i < LEFT; ++i) acc[i] = acc[i + 1];
     }
 }
 
+__global__ void __launch_bounds__(kInvThreads) k_inv_diag(Batch b, double* X) {
+    extern __shared__ double Lp[];                     // packed lower triangle, row r at r (r + 1) / 2
+    __shared__ double dinv[GP_NB];
+    __shared__ double Wk[2][kInvCols];
+    const int J = blockIdx.x, t = blockIdx.y, c0 = kInvCols * blockIdx.z;
+    if (b.st[t].status != GP_OK) return;
+    const double* L = tile_at(b.A, b.inst_stride, t, J, J, b.nt);
+    double* Xt = tile_at(X, b.inst_stride, t, J, J, b.nt);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int q = threadIdx.x; q < GP_TILE_ELEMS; q += kInvThreads) {
+        const int r = q % GP_NB, c = q / GP_NB;
+        if (r >= c && c >= c0) cp_async8(Lp + prow(r) + c, L + q);
+        if (r < c0 && c >= c0 && c < c0 + kInvCols) Xt[q] = 0.0;
+    }
+    if ((int)threadIdx.x >= c0) dinv[threadIdx.x] = 1.0 / L[threadIdx.x * (GP_NB + 1)];
+    cp_async_wait_all();
+    __syncthreads();
+    double acc[kInvRows];
+#pragma unroll
+    for (int i = 0; i < kInvRows; ++i) acc[i] = 0.0;
+    if (c0 <= 0) inv_rows<31>(acc, Lp, dinv, Wk, Xt, 0, c0, warp, lane);
+    if (c0 <= 32) inv_rows<23>(acc, Lp, dinv, Wk, Xt, 32, c0, warp, lane);
+    if (c0 <= 64) inv_rows<15>(acc, Lp, dinv, Wk, Xt, 64, c0, warp, lane);
+    inv_rows<7>(acc, Lp, dinv, Wk, Xt, 96, c0, warp, lane);
+}
+
+// Exponents of W_J's rows, |W_rc| < 2^E, into slot 2 of the factor's diagonal
+// tile (the factor's own diagonal block is not needed any more).
+__global__ void __launch_bounds__(GP_NB) k_row_exponents(Batch b, const double* X) {
+    const int J = blockIdx.x, t = blockIdx.y, r = threadIdx.x;
+    if (b.st[t].status != GP_OK) return;
+    const double* T = tile_at(X, b.inst_stride, t, J, J, b.nt) + r;
+    unsigned m = 0;
+#pragma unroll 16
+    for (int c = 0; c < GP_NB; ++c) m = max(m, (unsigned)__double2hiint(T[(size_t)c * GP_NB]) & 0x7fffffffu);
+    reinterpret_cast<int*>(tile_at(b.A, b.inst_stride, t, J, J, b.nt))[2 * GP_NB + r] = (int)(m >> 20) - 1022;
+}
+
 // Exponents of the columns of tiles (J, K), K = blockIdx.x, of `src`: |entry| <
-// 2^E, into slot `slot` of the factor's diagonal tile (K, K).  A warp per
-// column, its 128 entries in one coalesced kilobyte.
+// 2^E, into slot `slot` of the factor's diagonal tile (K, K).  A warp per four
+// columns, 128 entries in a coalesced kilobyte each.
+constexpr int kExpSplit = 4;
 __global__ void __launch_bounds__(kThreads) k_col_exponents(Batch b, const double* src, int J, int slot) {
     const int K = blockIdx.x, t = blockIdx.y;
     if (b.st[t].status != GP_OK) return;
     const double* T = tile_at(src, b.inst_stride, t, J, K, b.nt);
     int* out = reinterpret_cast<int*>(tile_at(b.A, b.inst_stride, t, K, K, b.nt)) + slot * GP_NB;
     const int lane = threadIdx.x & 31;
-#pragma unroll 4
-    for (int c = threadIdx.x >> 5; c < GP_NB; c += kThreads / 32) {
-        unsigned m = 0;
+    constexpr int kCols = GP_NB / kExpSplit / (kThreads / 32);
+    const int c0 = (GP_NB / kExpSplit) * blockIdx.z + kCols * (threadIdx.x >> 5);
+    unsigned m[kCols];
+#pragma unroll
+    for (int c = 0; c < kCols; ++c) {
+        m[c] = 0;
 #pragma unroll
         for (int u = 0; u < 4; ++u)
-            m = max(m, (unsigned)__double2hiint(T[(size_t)c * GP_NB + 32 * u + lane]) & 0x7fffffffu);
-        m = __reduce_max_sync(0xffffffffu, m);
-        if (lane == 0) out[c] = (int)(m >> 20) - 1022;
+            m[c] = max(m[c], (unsigned)__double2hiint(T[(size_t)(c0 + c) * GP_NB + 32 * u + lane]) & 0x7fffffffu);
+    }
+#pragma unroll
+    for (int c = 0; c < kCols; ++c) {
+        m[c] = __reduce_max_sync(0xffffffffu, m[c]);
+        if (lane == 0) out[c0 + c] = (int)(m[c] >> 20) - 1022;
     }
 }
 
@@ -124,102 +163,148 @@ __global__ void k_residual_vec(Batch b, double* Z, size_t zs) {
 //   dlog rho_k / dtheta_k = -D_k                       (eq. 2, Matern 1/2)
 //                         = -h / (1 + h) c D_k          (3/2, h = c theta_k D_k)
 //                         = -h (1 + h) / (3 + 3h + h^2) c D_k   (5/2)
-template <int DB>
+//
+// A CTA takes a quarter of a tile (whole tiles left a last wave of 72 CTAs to
+// themselves at n = 4064: FP64 pipes 85% busy on average, 54% of the time), and
+// its sums go to the factor's memory, which nothing needs any more.
+// G candidates share an element's powers, whose double-float logarithms and
+// conversions are half of its cost; theta comes scaled from shared memory and
+// exp(-S) from the assembly's table (11 double operations): FP64-bound, about
+// d + 25 + (7 d + 14) / G double operations per element and candidate (16 d + 2 d
+// + 30 each with CUDA's exp and a candidate at a time).  n = 1024, d = 6, T = 16:
+// 2.12 -> 0.94 ms; n = 4064, T = 1: 2.11 -> 1.72 ms.
+constexpr int kGradSplit = 4;
+
+template <int DB, int G>
 __global__ void __launch_bounds__(kThreads) k_grad_tiles(Batch b, const double* Ri, const double* Z, size_t zs,
-                                                         double* partial, int ntiles) {
+                                                         ExpTab64 etab) {
     __shared__ double red[kThreads / 32][DB];
     __shared__ dfl tab[kExpTab];
-    fill_exp2_table(tab);
-    __syncthreads();
-    const int t = blockIdx.y, nt = b.nt, n = b.n, d = b.d;
-    const InstState st = b.st[t];
-    if (st.status != GP_OK) return;
-    int J = 0;
-    {
-        long long rem = blockIdx.x;
-        while (rem >= nt - J) { rem -= nt - J; ++J; }
-    }
-    const int I = J + (int)(blockIdx.x - tile_index(J, J, nt));
-    const double* R1 = tile_at(Ri, b.inst_stride, t, I, J, nt);
-    const int pmode = pow_mode(b.p);
-    const dfl pd = df_from_double(b.p);
-    const double* w = Z + (size_t)t * zs + (size_t)nt * GP_NB;
-    const double* th = b.theta + (size_t)t * d;
-    const double nq = n / st.Q;
+    __shared__ ExpTab64 et;
+    __shared__ double th[G][DB], nq[G];
+    __shared__ int live[G];
+    const int t0 = blockIdx.y * G, nt = b.nt, n = b.n, d = b.d;
     const int corr = b.corr;
     const bool matern = corr_is_matern(corr);
     const double cm = corr_theta_scale(corr);
-    double acc[DB];
+    fill_exp2_table(tab);
+    for (int q = threadIdx.x; q < (int)(sizeof(ExpTab64) / sizeof(double)); q += kThreads)
+        reinterpret_cast<double*>(&et)[q] = reinterpret_cast<const double*>(&etab)[q];
+    for (int q = threadIdx.x; q < G * DB; q += kThreads) {
+        const int g = q / DB, k = q % DB;
+        th[g][k] = (t0 + g < b.count && k < d) ? cm * b.theta[(size_t)(t0 + g) * d + k] : 0.0;
+    }
+    if (threadIdx.x < G) {
+        live[threadIdx.x] = t0 + (int)threadIdx.x < b.count && b.st[t0 + threadIdx.x].status == GP_OK;
+        if (live[threadIdx.x]) nq[threadIdx.x] = n / b.st[t0 + threadIdx.x].Q;
+    }
+    __syncthreads();
+    int J = 0;
+    {
+        long long rem = blockIdx.x / kGradSplit;
+        while (rem >= nt - J) { rem -= nt - J; ++J; }
+    }
+    const int I = J + (int)(blockIdx.x / kGradSplit - tile_index(J, J, nt));
+    const int pmode = pow_mode(b.p);
+    const dfl pd = df_from_double(b.p);
+    // a thread's elements all lie in one row
+    static_assert(kThreads % GP_NB == 0, "rows per thread");
+    const int r = threadIdx.x % GP_NB, gi = I * GP_NB + r;
+    double acc[G][DB], wi[G];
 #pragma unroll
-    for (int k = 0; k < DB; ++k) acc[k] = 0.0;
-    for (int q = threadIdx.x; q < GP_TILE_ELEMS; q += kThreads) {
-        const int r = q % GP_NB, c = q / GP_NB;
-        const int gi = I * GP_NB + r, gj = J * GP_NB + c;
+    for (int g = 0; g < G; ++g) {
+        wi[g] = (live[g] && gi < n) ? nq[g] * Z[(size_t)(t0 + g) * zs + (size_t)nt * GP_NB + gi] : 0.0;
+#pragma unroll
+        for (int k = 0; k < DB; ++k) acc[g][k] = 0.0;
+    }
+    constexpr int kCols = GP_NB / kGradSplit;
+    const int c0 = kCols * (blockIdx.x % kGradSplit);
+    for (int c = c0 + threadIdx.x / GP_NB; c < c0 + kCols; c += kThreads / GP_NB) {
+        const int gj = J * GP_NB + c;
         if (gi >= n || gj >= n || gi <= gj) continue;
-        const double m = R1[q] - nq * w[gi] * w[gj];
-        double D[DB], h[DB];
-        double s = 0.0, qp = 1.0;
+        double D[DB];
 #pragma unroll
         for (int k = 0; k < DB; ++k) {
             D[k] = 0.0;
-            h[k] = 0.0;
             if (k < d) {
                 const double a = fabs(b.x[(size_t)gi * d + k] - b.x[(size_t)gj * d + k]);
                 // |dx|^p for general p in double-float (FP64 pow is scarce here)
                 D[k] = (matern || pmode == kPowOne) ? a
                                                     : (pmode == kPowTwo ? a * a
-                                                                        : df_to_double(df_powabs(df_from_double(a), pmode, b.p, pd, tab)));
-                h[k] = cm * th[k] * D[k];
-                s += h[k];
-                if (matern) qp *= matern_q(h[k], corr);
+                                                                        : df_to_double_positive(df_powabs(df_from_positive(a), pmode, b.p, pd, tab)));
             }
         }
-        const double mr = 2.0 * m * qp * exp(-s);
 #pragma unroll
-        for (int k = 0; k < DB; ++k) {
-            if (k < d) {
-                double dl = -D[k];
-                if (corr == GP_CORR_MATERN32) dl = -h[k] / (1.0 + h[k]) * cm * D[k];
-                if (corr == GP_CORR_MATERN52) dl = -h[k] * (1.0 + h[k]) / (3.0 + 3.0 * h[k] + h[k] * h[k]) * cm * D[k];
-                acc[k] = fma(mr, dl, acc[k]);
-            }
+        for (int g = 0; g < G; ++g) {
+            if (!live[g]) continue;
+            const int t = t0 + g;
+            const double m = tile_at(Ri, b.inst_stride, t, I, J, nt)[c * GP_NB + r] -
+                             wi[g] * Z[(size_t)t * zs + (size_t)nt * GP_NB + gj];
+            double s = 0.0, qp = m;
+#pragma unroll
+            for (int k = 0; k < DB; ++k)
+                if (k < d) {
+                    s = fma(th[g][k], D[k], s);
+                    if (matern) qp *= matern_q(th[g][k] * D[k], corr);
+                }
+            const double mr = qp * exp_neg_tab64(s, et);
+#pragma unroll
+            for (int k = 0; k < DB; ++k)
+                if (k < d) {
+                    double dl = D[k];
+                    if (corr == GP_CORR_MATERN32 || corr == GP_CORR_MATERN52) {
+                        const double h = th[g][k] * D[k];
+                        dl *= corr == GP_CORR_MATERN32 ? h / (1.0 + h) * cm
+                                                       : h * (1.0 + h) / (3.0 + 3.0 * h + h * h) * cm;
+                    }
+                    acc[g][k] = fma(mr, dl, acc[g][k]);
+                }
         }
     }
-    // fixed-order block reduction of the d sums
+    // fixed-order block reduction of each candidate's d sums; both (i, j) and
+    // (j, i), and the derivative's sign
     const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
 #pragma unroll
-    for (int k = 0; k < DB; ++k) {
-        double v = acc[k];
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-        if (lane == 0) red[wp][k] = v;
-    }
-    __syncthreads();
-    if (threadIdx.x < d) {
-        double v = 0.0;
-        for (int i = 0; i < kThreads / 32; ++i) v += red[i][threadIdx.x];
-        partial[((size_t)t * ntiles + blockIdx.x) * d + threadIdx.x] = v;
+    for (int g = 0; g < G; ++g) {
+        if (!live[g]) continue;
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < DB; ++k) {
+            double v = acc[g][k];
+            for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+            if (lane == 0) red[wp][k] = v;
+        }
+        __syncthreads();
+        if (threadIdx.x < d) {
+            double v = 0.0;
+            for (int i = 0; i < kThreads / 32; ++i) v += red[i][threadIdx.x];
+            b.A[(size_t)(t0 + g) * b.inst_stride + (size_t)blockIdx.x * d + threadIdx.x] = -2.0 * v;
+        }
     }
 }
 
-// grad[t][k] = sum over tiles, in tile order; NaN where the likelihood
-// itself failed (status: the finalize kernel's, which also flags Q = 0)
-__global__ void k_grad_reduce(Batch b, const double* partial, int ntiles, const int* status, double* grad) {
+// grad[t][k] = the sum of the tile parts' sums, in a fixed order (a warp per k);
+// NaN where the likelihood itself failed (status: the finalize kernel's, which
+// also flags Q = 0)
+__global__ void k_grad_reduce(Batch b, int parts, const int* status, double* grad) {
     const int t = blockIdx.x, d = b.d;
-    const int k = threadIdx.x;
+    const int k = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (k >= d) return;
     if (b.st[t].status != GP_OK || status[t] != GP_OK) {
-        grad[(size_t)t * d + k] = __longlong_as_double(0x7ff8000000000000LL);
+        if (lane == 0) grad[(size_t)t * d + k] = __longlong_as_double(0x7ff8000000000000LL);
         return;
     }
+    const double* partial = b.A + (size_t)t * b.inst_stride;
     double v = 0.0;
-    for (int q = 0; q < ntiles; ++q) v += partial[((size_t)t * ntiles + q) * d + k];
-    grad[(size_t)t * d + k] = v;
+    for (int q = lane; q < parts; q += 32) v += partial[(size_t)q * d + k];
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    if (lane == 0) grad[(size_t)t * d + k] = v;
 }
 
 }  // namespace
 
-cudaError_t launch_grad(const Batch& b, double* Z, size_t zs, double* X, double* Ri, double* partial,
-                        const int* status, double* grad, cudaStream_t s, int* kernels) {
+cudaError_t launch_grad(const Batch& b, double* Z, size_t zs, double* X, double* Ri, const int* status,
+                        double* grad, cudaStream_t s, int* kernels) {
     const int nt = b.nt;
     int k = 0;
     k_residual_vec<<<b.count, kThreads, 0, s>>>(b, Z, zs);
@@ -228,34 +313,42 @@ cudaError_t launch_grad(const Batch& b, double* Z, size_t zs, double* X, double*
     if (e != cudaSuccess) return e;
     k += solve_f64_launches(nt, true);
     {
-        const size_t smem = (size_t)2 * kPackedTri * sizeof(double);
+        const size_t smem = (size_t)kPackedTri * sizeof(double);
         static std::atomic<size_t> attr[kMaxDevices];
         e = raise_smem_limit(k_inv_diag, smem, attr);
         if (e != cudaSuccess) return e;
-        k_inv_diag<<<dim3(nt, b.count), kThreads, smem, s>>>(b, X);
-        ++k;
+        k_inv_diag<<<dim3(nt, b.count, GP_NB / kInvCols), kInvThreads, smem, s>>>(b, X);
+        k_row_exponents<<<dim3(nt, b.count), GP_NB, 0, s>>>(b, X);
+        k += 2;
     }
     for (int J = 0; J < nt; ++J) {
         if (J > 0) {
-            k_col_exponents<<<dim3(J, b.count), kThreads, 0, s>>>(b, Ri, J, 1);
+            k_col_exponents<<<dim3(J, b.count, kExpSplit), kThreads, 0, s>>>(b, Ri, J, 1);
             e = launch_inverse_apply(b, J, X, Ri, s);
             if (e != cudaSuccess) return e;
             k += 2;
         }
-        k_col_exponents<<<dim3(J + 1, b.count), kThreads, 0, s>>>(b, X, J, 0);
+        k_col_exponents<<<dim3(J + 1, b.count, kExpSplit), kThreads, 0, s>>>(b, X, J, 0);
         e = launch_inverse_update(b, J, X, Ri, s);
         if (e != cudaSuccess) return e;
         k += 2;
     }
     const int ntiles = (int)packed_tiles(nt);
-    if (b.d <= 4)
-        k_grad_tiles<4><<<dim3(ntiles, b.count), kThreads, 0, s>>>(b, Ri, Z, zs, partial, ntiles);
-    else if (b.d <= 8)
-        k_grad_tiles<8><<<dim3(ntiles, b.count), kThreads, 0, s>>>(b, Ri, Z, zs, partial, ntiles);
-    else
-        k_grad_tiles<16><<<dim3(ntiles, b.count), kThreads, 0, s>>>(b, Ri, Z, zs, partial, ntiles);
+    ExpTab64 et;
+    exp_tab64_fill(et);
+    // four candidates an element where their CTAs fill most of the SMs
+    const int parts = kGradSplit * ntiles;
+    const int G = (long long)ntiles * ((b.count + 3) / 4) * 4 >= 3LL * device_sms() && b.count > 1 ? 4 : 1;
+    const dim3 grid(parts, (b.count + G - 1) / G);
+#define GP_GRAD_TILES(DB)                                                                                   \
+    (G == 4 ? k_grad_tiles<DB, 4><<<grid, kThreads, 0, s>>>(b, Ri, Z, zs, et)              \
+            : k_grad_tiles<DB, 1><<<grid, kThreads, 0, s>>>(b, Ri, Z, zs, et))
+    if (b.d <= 4)      GP_GRAD_TILES(4);
+    else if (b.d <= 8) GP_GRAD_TILES(8);
+    else               GP_GRAD_TILES(16);
+#undef GP_GRAD_TILES
     ++k;
-    k_grad_reduce<<<b.count, 64, 0, s>>>(b, partial, ntiles, status, grad);
+    k_grad_reduce<<<b.count, 32 * 16, 0, s>>>(b, parts, status, grad);
     ++k;
     if (kernels) *kernels = k;
     return cudaGetLastError();

@@ -64,7 +64,7 @@ def test_columns_of_very_different_sizes(ctx):
     assert np.max(np.abs(gg - ref)) <= tol(len(x), cond) * np.max(np.abs(ref))
 
 
-@pytest.mark.parametrize("n", [200, 300, 700])
+@pytest.mark.parametrize("n", [200, 300, 700, 2000])
 def test_alone_and_in_a_batch(ctx, n):
     g = np.random.default_rng(n)
     x = inputs.random_lhd(g, n, 5)
