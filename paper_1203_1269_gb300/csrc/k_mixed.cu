@@ -80,20 +80,24 @@ __device__ __forceinline__ float cut_one(float& xh, float& xl, float w) {
 // little else (per term and warp four loads of V shared by its rows, one
 // load per pair of rows).  It first reaches the next block's columns and
 // rows, which go to shared memory; a 17th warp then factors the next 8 x 8
-// block while the others finish the update, and writes the finished rows and
-// columns out while they begin the next.  Three barriers per eight columns.
+// block while the others finish the update.  Three more warps write the
+// finished rows and columns out and take what follows from a finished row of
+// W -- its slices, the tiles the solves read, the forward solve's x_J, the
+// pivots' logarithms -- beside the sweep.  Three barriers per eight columns.
 //
 // Bound by FP32 issue: the 128^3 / 3 multiply-adds of 15 instructions are
 // 0.10 M cycles on an SM's four schedulers at the measured 1.04 cycles each;
-// the sweep takes 0.21 M, the rest being the panels and the 8 x 8 blocks of
-// the last columns, and the kernel 131 us for up to 152 candidates (254 us
-// with the triangle in shared memory and two barriers a column, where the
-// loads, stores and index arithmetic took three of four issue slots; 160 us
-// with registers but a barrier pair per column, 850 of whose 2000 cycles were
-// the pivot's dependent chain).  n = 1024, T = 100: 4.46 -> 3.50 ms a batch;
-// n = 64, T = 100: 0.363 -> 0.260 ms; n = 4000, T = 256: 130.0 -> 128.2 ms.
-constexpr int kDiagWarps = 16;                         // warps that hold the triangle, plus one
-constexpr int kDiagThreads = 32 * (kDiagWarps + 1);
+// the sweep takes about twice that, the rest being the panels and the 8 x 8
+// blocks of the last columns.  Measured, a block column at up to 152
+// candidates: 254 us with the triangle in shared memory and two barriers a
+// column (loads, stores and index arithmetic took three of four issue slots),
+// 160 us with registers but a barrier pair per column, 131 us with the rows'
+// slices and copies after the sweep, 126 us now.  n = 1024, T = 100: 4.46 -> 3.46
+// ms a batch; n = 64, T = 100: 0.363 -> 0.247 ms; n = 4000, T = 256: 130.0 -> 127.2
+// ms.
+constexpr int kDiagWarps = 16;                         // warps that hold the triangle
+constexpr int kDiagHelpers = 4;                        // one for the 8 x 8 blocks, three for finished rows
+constexpr int kDiagThreads = 32 * (kDiagWarps + kDiagHelpers);
 constexpr int kDiagRows = GP_NB / kDiagWarps;          // rows per warp
 constexpr int kDiagB = 8;
 constexpr int kDiagBlocks = GP_NB / kDiagB;
@@ -113,6 +117,8 @@ struct DiagShared {
     float4 ld[kDiagB][kDiagB / 2];   // the block's L: column c, rows 2 u and 2 u + 1 in pairs
     dfl dinv[GP_NB];            // 1 / L_cc
     dfl lcc[GP_NB];             // L_cc
+    dfl bj[2][GP_NB];           // the forward solve's right-hand sides
+    double lsum[GP_NB / 32], psum[GP_NB / 32];
     int failed;
 };
 
@@ -195,42 +201,40 @@ __device__ __noinline__ void diag_block8_slow(DiagShared& sh, int c0, int lane) 
     }
 }
 
-// The 8 x 8 block at c0 (one warp): lane r < 8 holds its row r.  Every lane
-// takes each pivot and the results go out at the end, so the eight columns
-// are one straight-line chain: a pivot, the column, a shuffle and the next
-// pivot's last term, the other terms beside it.
+// The 8 x 8 block at c0 (one warp): lane r + 8 u holds columns 2 u and 2 u + 1 of
+// row r.  Every lane takes each pivot and the results go out at the end, so
+// the eight columns are one straight-line chain: a pivot, the column, a
+// shuffle and the next pivot's last term, the other terms beside it.
 __device__ __forceinline__ void diag_block8(DiagShared& sh, int c0, int lane) {
-    const int r = lane & 7;
-    df2 a[kDiagB / 2];
-    dfl l[kDiagB], y[kDiagB];
-#pragma unroll
-    for (int u = 0; u < kDiagB / 2; ++u) a[u] = df2_pack(sh.col[2 * u][c0 + r], sh.col[2 * u + 1][c0 + r]);
+    const int r = lane & 7, u = lane >> 3;
+    df2 a = df2_pack(sh.col[2 * u][c0 + r], sh.col[2 * u + 1][c0 + r]);
+    dfl l0 = {0.f, 0.f}, l1 = {0.f, 0.f}, yr = {0.f, 0.f};     // L_{r, 2u}, L_{r, 2u+1}, 1 / L_rr
     bool ok = true;
 #pragma unroll
     for (int cc = 0; cc < kDiagB; ++cc) {
-        const dfl acc = (cc & 1) ? df2_second(a[cc / 2]) : df2_first(a[cc / 2]);
-        const dfl piv = df_shfl(acc, cc);
+        const int from = 8 * (cc / 2);                          // lanes from + r hold column cc
+        const dfl acc = (cc & 1) ? df2_second(a) : df2_first(a);
+        const dfl piv = df_shfl(acc, from + cc);
         ok = ok && pivot_in_range(piv);
-        y[cc] = pivot_rsqrt(piv);
-        l[cc] = df_mul(acc, y[cc]);        // on lane cc: a y, the pivot's square root
-        const df2 la = df2_dup(l[cc]);
-        const f32x2 nl = f2_neg(la.hi);
-#pragma unroll
-        for (int u = (cc + 1) / 2; u < kDiagB / 2; ++u) {
-            const df2 lq = df2_pack(df_shfl(l[cc], 2 * u), df_shfl(l[cc], 2 * u + 1));
-            a[u] = df2_fnma(f2_mul(nl, lq.hi), la, lq, a[u]);
+        const dfl y = pivot_rsqrt(piv);
+        const dfl l = df_mul(acc, y);                           // at row cc: a y, the pivot's square root
+        if (r == cc) yr = y;
+        if (u == cc / 2) {
+            if (cc & 1) l1 = l;
+            else        l0 = l;
+        }
+        if (cc + 1 < kDiagB) {
+            const df2 la = df2_dup(df_shfl(l, from + r));
+            const df2 lq = df2_pack(df_shfl(l, from + 2 * u), df_shfl(l, from + 2 * u + 1));
+            a = df2_fnma(f2_mul(f2_neg(la.hi), lq.hi), la, lq, a);
         }
     }
     if (ok) {
-        if (lane < kDiagB) {
-#pragma unroll
-            for (int cc = 0; cc < kDiagB; ++cc) {
-                ld_store(sh, lane, cc, l[cc]);
-                if (lane == cc) {
-                    sh.dinv[c0 + cc] = y[cc];
-                    sh.lcc[c0 + cc] = l[cc];
-                }
-            }
+        ld_store(sh, r, 2 * u, l0);
+        ld_store(sh, r, 2 * u + 1, l1);
+        if (r / 2 == u) {
+            sh.dinv[c0 + r] = yr;
+            sh.lcc[c0 + r] = (r & 1) ? l1 : l0;
         }
     } else {
         diag_block8_slow(sh, c0, lane);
@@ -287,17 +291,19 @@ __device__ __forceinline__ void diag_panels(DiagShared& sh, int c0, int warp, in
 }
 
 // Block c0's columns of L into the tile T and its rows of W into the packed
-// triangle P, from the vectors V (one warp).
-__device__ __forceinline__ void diag_write(const DiagShared& sh, int c0, float2* T, dfl* P, int lane) {
-    if (lane < kDiagB) {
+// triangle P, from the vectors V (the helper warps h = 0 .. 3, two columns and
+// rows each).
+__device__ __forceinline__ void diag_write(const DiagShared& sh, int c0, float2* T, dfl* P, int h, int lane) {
+    if (h == 0 && lane < kDiagB) {
 #pragma unroll
         for (int cc = 0; cc < kDiagB; ++cc) {
             const float* p = reinterpret_cast<const float*>(&sh.ld[cc][lane >> 1]) + (lane & 1);
             if (lane >= cc) T[(size_t)(c0 + cc) * GP_NB + c0 + lane] = make_float2(p[0], p[2]);
         }
     }
-#pragma unroll 2
-    for (int cc = 0; cc < kDiagB; ++cc)
+#pragma unroll
+    for (int q = 0; q < kDiagB / kDiagHelpers; ++q) {
+        const int cc = h + kDiagHelpers * q;
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             const int p = lane + 32 * j;
@@ -307,6 +313,99 @@ __device__ __forceinline__ void diag_write(const DiagShared& sh, int c0, float2*
             else if (p >= c0 + kDiagB)
                 T[(size_t)(c0 + cc) * GP_NB + p] = make_float2(-v.x, -v.z);
         }
+    }
+}
+
+// Row c of W: exponent (of the largest high word, as the panel slicing takes
+// it) and slices; one warp, lane l columns 4 l .. 4 l + 3 (half of one 16-byte
+// piece).
+__device__ __forceinline__ void diag_slices(const dfl* P, uint8_t* WS, int* WE, int c, int lane) {
+    const dfl* w = P + prow(c);
+    const int k0 = 4 * lane;
+    float xh[4], xl[4], mx = 0.f;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        const dfl v = (k0 + e <= c) ? w[k0 + e] : dfl{0.f, 0.f};
+        xh[e] = v.hi;
+        xl[e] = v.lo;
+        mx = fmaxf(mx, fabsf(v.hi));
+    }
+    for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    const int E = exponent_of(mx);
+    if (lane == 0) WE[c] = E;
+    float sa, sb;
+    slice_scale(E, sa, sb);
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        xh[e] = __fmul_rn(__fmul_rn(xh[e], sa), sb);
+        xl[e] = __fmul_rn(__fmul_rn(xl[e], sa), sb);
+    }
+    uint8_t* dst = WS + (size_t)(k0 >> 5) * kChunkBytes + image_piece(c, k0 & ~7) + ((k0 & 4) ? 8u : 0u);
+    float wt = 1.f;
+#pragma unroll
+    for (int a = 0; a < GP_PANEL_SLICES; ++a) {
+        float m[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) m[e] = cut_one(xh[e], xl[e], wt);
+        *reinterpret_cast<uint2*>(dst + (size_t)a * kChunks * kChunkBytes) =
+            make_uint2(pack_bf16x2(m[0], m[1]), pack_bf16x2(m[2], m[3]));
+        wt = __fmul_rn(wt, 0.00390625f);
+    }
+}
+
+// Rows c0 .. c0 + 7 of W as parts of the double-float tiles that the solves read:
+// column-major (forward) and row-major (backward), zeros above the diagonal;
+// `parts` warps.
+__device__ __forceinline__ void diag_tiles(const dfl* P, float2* Wt, float2* Wr, int c0, int part, int parts,
+                                           int lane) {
+    for (int c = part; c < kDiagB; c += parts)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int r = c0 + c, p = lane + 32 * j;
+            const dfl v = p <= r ? P[prow(r) + p] : dfl{0.f, 0.f};
+            Wr[(size_t)r * GP_NB + p] = make_float2(v.hi, v.lo);
+        }
+    const int r = c0 + (lane & 7);
+#pragma unroll 4
+    for (int p = (lane >> 3) + 4 * part; p < GP_NB; p += 4 * parts) {
+        const dfl v = p <= r ? P[prow(r) + p] : dfl{0.f, 0.f};
+        Wt[(size_t)p * GP_NB + r] = make_float2(v.hi, v.lo);
+    }
+}
+
+// Rows c0 .. c0 + 7 of the forward solve x_J = W (b_J - sum_{K<J} L_JK x_K), the sum
+// already subtracted by the slicing of panels K < J, in double-float (one
+// warp): lane (row, right-hand side k, half h) sums the columns h, h + 2, ...
+// of its row, then the two halves add.
+__device__ __forceinline__ void diag_forward(const DiagShared& sh, const dfl* P, float2* zJ, size_t npad, int c0,
+                                             int lane) {
+    const int r = c0 + (lane & 7), k = (lane >> 3) & 1, h = lane >> 4;
+    const dfl* w = P + prow(r);
+    dfl sum = {0.f, 0.f};
+#pragma unroll 4
+    for (int c = h; c <= r; c += 2) sum = df_fma(w[c], sh.bj[k][c], sum);
+    const dfl other = df_shfl(sum, (lane & 15) + 16);
+    if (h == 0) df_store(zJ + (size_t)k * npad + r, df_add(sum, other));
+}
+
+// log L_cc and 1 / L_cc^2 over columns 32 q .. 32 q + 31 (one warp), and the
+// reciprocal diagonal out: sums by a warp tree, the four quarters' in turn at
+// the end of the kernel.  The squares (over real rows only) are the
+// refinement's estimate of the log-det's own error (k_refine_check).
+__device__ __forceinline__ void diag_logs(DiagShared& sh, float2* rinv, int q, int real_rows, int lane) {
+    const int c = 32 * q + lane;
+    double v = log(df_to_double(sh.lcc[c]));
+    const double di = df_to_double(sh.dinv[c]);
+    double s = c < real_rows ? di * di : 0.0;
+    for (int o = 16; o > 0; o >>= 1) {
+        v += __shfl_down_sync(0xffffffffu, v, o);
+        s += __shfl_down_sync(0xffffffffu, s, o);
+    }
+    if (lane == 0) {
+        sh.lsum[q] = v;
+        sh.psum[q] = s;
+    }
+    df_store(rinv + c, sh.dinv[c]);
 }
 
 // A thread's part of the triangle: rows 2 m and 2 m + 1 of its warp in column
@@ -413,13 +512,6 @@ __device__ __forceinline__ void diag_dispatch_rest(const DiagShared& sh, DiagReg
 __global__ void __launch_bounds__(kDiagThreads, 1) k_diag_mixed(MixedBatch b, int J) {
     extern __shared__ dfl P[];             // kPacked double-float values: A_JJ in, W out
     __shared__ DiagShared sh;
-    __shared__ dfl bj[2][GP_NB];
-    __shared__ dfl xpart[2][GP_NB];
-    __shared__ double lsum[GP_NB / 32];
-    __shared__ double psum[GP_NB / 32];
-    dfl (&dinv)[GP_NB] = sh.dinv;
-    dfl (&lcc)[GP_NB] = sh.lcc;
-    int& failed = sh.failed;
     const int t = blockIdx.x;
     if (b.st[t].status != GP_OK) return;
     float2* T = df_tile(b, b.A, t, J, J);
@@ -427,11 +519,20 @@ __global__ void __launch_bounds__(kDiagThreads, 1) k_diag_mixed(MixedBatch b, in
         const int rr = q & 127, cc = q >> 7;
         if (rr >= cc) cp_async8(P + prow(rr) + cc, T + q);
     }
-    if (threadIdx.x == 0) failed = -1;
-    cp_async_wait_all();
-    __syncthreads();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     constexpr int kWarps = kDiagWarps;
+    const int helper = warp - kWarps;      // 0: the 8 x 8 blocks, 1 .. 3: finished rows
+    const size_t npad = (size_t)b.nt * GP_NB;
+    float2* zJ = b.Z + (size_t)t * b.z_stride + (size_t)J * GP_NB;
+    uint8_t* WS = reinterpret_cast<uint8_t*>(b.WS + (size_t)t * b.ws_stride);
+    int* WE = b.WE + (size_t)t * b.we_stride;
+    float2* Wt = b.WT + (size_t)t * b.wt_stride + (size_t)J * GP_TILE_ELEMS;
+    float2* Wr = b.WR + (size_t)t * b.wt_stride + (size_t)J * GP_TILE_ELEMS;
+    if (b.fwd && threadIdx.x < 2 * GP_NB)
+        sh.bj[threadIdx.x >> 7][threadIdx.x & 127] = df_load(zJ + (threadIdx.x >> 7) * npad + (threadIdx.x & 127));
+    if (threadIdx.x == 0) sh.failed = -1;
+    cp_async_wait_all();
+    __syncthreads();
     DiagRegs R;
 #pragma unroll
     for (int m = 0; m < kDiagRows / 2; ++m)
@@ -451,14 +552,28 @@ __global__ void __launch_bounds__(kDiagThreads, 1) k_diag_mixed(MixedBatch b, in
             R.x[m][0] = df2{0, 0};
         }
     __syncthreads();
+    // what follows from the finished rows of block nb, by helpers 1 .. 3
+    auto finished = [&](int nb) {
+        const int c0 = kDiagB * nb;
+        if (helper == 3) {                 // a chain of up to 64 dependent multiply-adds
+            if (b.fwd) diag_forward(sh, P, zJ, npad, c0, lane);
+        } else {
+#pragma unroll 2
+            for (int q = 0; q < kDiagB / 2; ++q) diag_slices(P, WS, WE, c0 + 2 * q + helper - 1, lane);
+            diag_tiles(P, Wt, Wr, c0, helper - 1, 2, lane);
+            if (helper == 1 && (nb & 3) == 3) diag_logs(sh, zJ + 4 * npad, nb >> 2, b.n - J * GP_NB, lane);
+        }
+    };
     for (int nb = 0;; ++nb) {
         const int c0 = kDiagB * nb;
         // the warps of one half own a row each of block nb + 1; the warp's
         // rows below block nb reach from k0 on
         const bool owner = (warp >> 3) == ((nb + 1) & 1);
         const int k0 = (c0 + kDiagB - warp + kDiagWarps - 1) >> 4;
-        if (warp == kWarps) {
+        if (helper == 0) {
             diag_block8(sh, c0, lane);
+        } else if (nb > 0 && helper > 0) {
+            finished(nb - 1);
         } else if (nb > 0) {               // the rest of block nb - 1's update
             const int k1 = (c0 - warp + kDiagWarps - 1) >> 4;
             const int kr = k1 + (owner ? 0 : 1);   // past the warp's row of block nb, exported with it
@@ -470,11 +585,11 @@ __global__ void __launch_bounds__(kDiagThreads, 1) k_diag_mixed(MixedBatch b, in
             }
         }
         __syncthreads();
-        if (failed >= 0) break;            // uniform
+        if (sh.failed >= 0) break;         // uniform
         diag_panels(sh, c0, warp, lane);
         __syncthreads();
-        if (warp == kWarps) diag_write(sh, c0, T, P, lane);
-        if (warp < kWarps && nb + 1 < kDiagBlocks) {
+        if (helper >= 0) diag_write(sh, c0, T, P, helper, lane);
+        if (helper < 0 && nb + 1 < kDiagBlocks) {
             switch ((nb + 1) >> 2) {
                 case 0: diag_dispatch_first<0>(sh, R, c0 + kDiagB, k0, owner, warp, lane); break;
                 case 1: diag_dispatch_first<1>(sh, R, c0 + kDiagB, k0, owner, warp, lane); break;
@@ -485,111 +600,25 @@ __global__ void __launch_bounds__(kDiagThreads, 1) k_diag_mixed(MixedBatch b, in
         __syncthreads();
         if (nb + 1 == kDiagBlocks) break;
     }
-    if (failed >= 0) {
+    if (sh.failed >= 0) {
         if (threadIdx.x == 0) {
             b.st[t].status = GP_ENOTPD;
-            b.st[t].fail_col = J * GP_NB + failed;
+            b.st[t].fail_col = J * GP_NB + sh.failed;
         }
         return;
     }
-    // log-det: sum of log L_cc over the block in a fixed order (warp trees,
-    // then, at the end of the kernel, the four warp sums in turn); reciprocal
-    // diagonal out and the sum of 1 / L_cc^2 over the block's real rows (the
-    // refinement's estimate of the log-det's own error, k_refine_check)
-    if (threadIdx.x < GP_NB) {
-        double v = log(df_to_double(lcc[threadIdx.x]));
-        const double di = df_to_double(dinv[threadIdx.x]);
-        double q = (J * GP_NB + (int)threadIdx.x < b.n) ? di * di : 0.0;
-        for (int o = 16; o > 0; o >>= 1) {
-            v += __shfl_down_sync(0xffffffffu, v, o);
-            q += __shfl_down_sync(0xffffffffu, q, o);
-        }
-        if (lane == 0) {
-            lsum[warp] = v;
-            psum[warp] = q;
-        }
-        float2* rinv = b.Z + (size_t)t * b.z_stride + (size_t)4 * b.nt * GP_NB + J * GP_NB;
-        df_store(rinv + threadIdx.x, dinv[threadIdx.x]);
-    }
-    // W as a double-float tile (column-major, zeros above the diagonal) for
-    // the diagonal-block products of the solves
-    // and row-major (W^T column-major) for the backward substitution
-    {
-        float2* Wt = b.WT + (size_t)t * b.wt_stride + (size_t)J * GP_TILE_ELEMS;
-        float2* Wr = b.WR + (size_t)t * b.wt_stride + (size_t)J * GP_TILE_ELEMS;
-        for (int q = threadIdx.x; q < GP_TILE_ELEMS; q += kDiagThreads) {
-            const int rr = q & 127, cc = q >> 7;
-            Wt[q] = (rr >= cc) ? make_float2(P[prow(rr) + cc].hi, P[prow(rr) + cc].lo) : make_float2(0.f, 0.f);
-            // row cc, column rr of W
-            Wr[q] = (cc >= rr) ? make_float2(P[prow(cc) + rr].hi, P[prow(cc) + rr].lo) : make_float2(0.f, 0.f);
-        }
-    }
-    // row c of W: exponent (of the largest high word, as the panel slicing
-    // takes it) and slices; one warp per row, all on the FP32 pipes
-    uint8_t* WS = reinterpret_cast<uint8_t*>(b.WS + (size_t)t * b.ws_stride);
-    int* WE = b.WE + (size_t)t * b.we_stride;
-#pragma unroll 2
-    for (int c = warp; c < GP_NB; c += kDiagThreads / 32) {
-        const dfl* w = P + prow(c);
-        // lane handles columns 4*lane .. 4*lane+3 (half of one 16-byte piece)
-        const int k0 = 4 * lane;
-        float xh[4], xl[4], mx = 0.f;
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const dfl v = (k0 + e <= c) ? w[k0 + e] : dfl{0.f, 0.f};
-            xh[e] = v.hi;
-            xl[e] = v.lo;
-            mx = fmaxf(mx, fabsf(v.hi));
-        }
-        for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-        const int E = exponent_of(mx);
-        if (lane == 0) WE[c] = E;
-        float sa, sb;
-        slice_scale(E, sa, sb);
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            xh[e] = __fmul_rn(__fmul_rn(xh[e], sa), sb);
-            xl[e] = __fmul_rn(__fmul_rn(xl[e], sa), sb);
-        }
-        uint8_t* dst = WS + (size_t)(k0 >> 5) * kChunkBytes + image_piece(c, k0 & ~7) + ((k0 & 4) ? 8u : 0u);
-        float wt = 1.f;
-#pragma unroll
-        for (int a = 0; a < GP_PANEL_SLICES; ++a) {
-            float m[4];
-#pragma unroll
-            for (int e = 0; e < 4; ++e) m[e] = cut_one(xh[e], xl[e], wt);
-            *reinterpret_cast<uint2*>(dst + (size_t)a * kChunks * kChunkBytes) =
-                make_uint2(pack_bf16x2(m[0], m[1]), pack_bf16x2(m[2], m[3]));
-            wt = __fmul_rn(wt, 0.00390625f);
-        }
-    }
-    if (b.fwd) {
-        // forward solve, block J: x_J = W (b_J - sum_{K<J} L_JK x_K), the sum
-        // already subtracted by the slicing of panels K < J; b_J in, x_J out
-        // (Z columns 0, 1), in double-float: thread (k, r, h) sums the
-        // columns c = h, h + 2, ... of row r, then the two halves add in a
-        // fixed order
-        float2* zJ = b.Z + (size_t)t * b.z_stride + (size_t)J * GP_NB;
-        const int k = (threadIdx.x >> 7) & 1, r = threadIdx.x & 127, h = threadIdx.x >> 8;
-        const bool active = h < 2;
-        float2* zk = zJ + (size_t)k * b.nt * GP_NB;
-        if (h == 0) bj[k][r] = df_load(zk + r);
-        __syncthreads();
-        const dfl* w = P + prow(r);
-        dfl sum = {0.f, 0.f};
-        if (active)
-            for (int c = h; c <= r; c += 2) sum = df_fma(w[c], bj[k][c], sum);
-        if (h == 1) xpart[k][r] = sum;
-        __syncthreads();
-        if (h == 0) df_store(zk + r, df_add(sum, xpart[k][r]));
-    } else {
-        __syncthreads();
-    }
+    // the last block's rows, by every warp
+    constexpr int kLast = GP_NB - kDiagB;
+    if (warp < kDiagB)           diag_slices(P, WS, WE, kLast + warp, lane);
+    else if (warp == 8)        { if (b.fwd) diag_forward(sh, P, zJ, npad, kLast, lane); }
+    else if (warp == 9)          diag_logs(sh, zJ + 4 * npad, 3, b.n - J * GP_NB, lane);
+    else                         diag_tiles(P, Wt, Wr, kLast, warp - 10, kDiagThreads / 32 - 10, lane);
+    __syncthreads();
     if (threadIdx.x == 0) {
         double ld = 0.0, pq = 0.0;
         for (int w = 0; w < GP_NB / 32; ++w) {
-            ld += lsum[w];
-            pq += psum[w];
+            ld += sh.lsum[w];
+            pq += sh.psum[w];
         }
         b.st[t].logdet += 2.0 * ld;
         b.st[t].piv_inv += pq;
