@@ -272,10 +272,13 @@ __device__ __forceinline__ dfl df_powabs(dfl d, int mode, double p, dfl pd, cons
 }
 
 // tab[j] = 2^(-j/N), j = 0 .. N - 1, as double-float (the block's threads in
-// turn; the caller synchronises before the table is read).
-__device__ __forceinline__ void fill_exp2_table(dfl* tab) {
-    for (int j = threadIdx.x; j < kExpTab; j += blockDim.x)
-        tab[j] = df_from_double(exp2(-(double)j / (double)kExpTab));
+// turn; the caller synchronises before the table is read).  `src` is the
+// device's copy (exp2_table): a CTA of its own 1024 exp2 is 7 us of an SM's FP64
+// pipe, which small problems spent half of their assembly on (n = 64, T = 100:
+// 41 -> 24 us).
+__device__ __forceinline__ void load_exp2_table(dfl* tab, const float2* src) {
+    for (int j = threadIdx.x; j < kExpTab; j += blockDim.x) tab[j] = df_load(src + j);
 }
+__device__ __forceinline__ dfl exp2_entry(int j) { return df_from_double(exp2(-(double)j / (double)kExpTab)); }
 
 }  // namespace gp

@@ -1100,6 +1100,11 @@ int gp_create(gp_ctx** out, int device, size_t hbm_budget_bytes, void* cuda_stre
         delete ctx;
         return GP_ECUDA;
     }
+    if (gp::init_exp2_table() != cudaSuccess) {
+        cudaGetLastError();
+        delete ctx;
+        return GP_ECUDA;
+    }
     ctx->budget = hbm_budget_bytes ? hbm_budget_bytes : (free_b / 4) * 3;
     int sms = 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) == cudaSuccess && sms > 0)

@@ -186,6 +186,11 @@ inline int device_sms() {
     return n;
 }
 
+// The current device's table of 2^(-j/1024) as double-float (k_assemble.cu),
+// filled once per device by init_exp2_table (gp_create; it synchronises).
+cudaError_t init_exp2_table();
+const float2* exp2_table();
+
 // ---- context accessors (gp_capi.cu) ----------------------------------------
 int ctx_fail(gp_ctx* ctx, int code, const char* fmt, ...);
 int ctx_device(const gp_ctx* ctx);

@@ -112,6 +112,13 @@ __device__ __forceinline__ void store_entry(const Batch& b, int t, size_t off, d
     }
 }
 
+__device__ float2 g_exp2_table[kExpTab];
+
+__global__ void k_exp2_table() {
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j < kExpTab) df_store(g_exp2_table + j, exp2_entry(j));
+}
+
 // Validate theta and reset each instance's record.
 __global__ void k_validate_theta(Batch b) {
     int t = blockIdx.x * blockDim.x + threadIdx.x;
@@ -257,7 +264,7 @@ k_assemble_tiles(Batch b, int group, PowTab64 ptab) {
 // bound (the benchmark's d = 6: 10.84 -> 9.92 ms, the same bits).
 template <int DB, int COLS, bool MATERN, bool EXACT = false>
 __global__ void __launch_bounds__(kThreads)
-k_assemble_tiles_df(Batch b, int group) {
+k_assemble_tiles_df(Batch b, int group, const float2* etab) {
     constexpr int kSplitDf = GP_NB / COLS;
     constexpr int kColsDf = COLS;
     constexpr int kEntriesDf = GP_NB * COLS / kThreads;
@@ -293,7 +300,7 @@ k_assemble_tiles_df(Batch b, int group) {
                         : dfl{0.f, 0.f};
     }
     for (int q = threadIdx.x; q < t1 - t0; q += kThreads) live[q] = (b.st[t0 + q].status == GP_OK);
-    fill_exp2_table(tab);
+    load_exp2_table(tab, etab);
     __syncthreads();
     const dfl delta = df_from_double(b.delta);
     constexpr bool matern = MATERN;                          // the family is a template argument
@@ -444,6 +451,46 @@ __global__ void k_assemble_dense(int n, int d, const double* __restrict__ x,
 
 }  // namespace
 
+namespace {
+std::mutex g_exp2_mutex;
+std::atomic<const float2*> g_exp2_addr[kMaxDevices];
+}  // namespace
+
+// The table is a constant: filled when the first context on a device is
+// created, before any call that reads it, and kept.
+// On a stream of its own, so that the caller's may be capturing.
+cudaError_t init_exp2_table() {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
+    std::lock_guard<std::mutex> lock(g_exp2_mutex);
+    if (g_exp2_addr[dev].load(std::memory_order_acquire)) return cudaSuccess;
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    void* p = nullptr;
+    cudaStream_t s = nullptr;
+    e = cudaGetSymbolAddress(&p, g_exp2_table);
+    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
+    if (e == cudaSuccess) {
+        k_exp2_table<<<kExpTab / 128, 128, 0, s>>>();
+        e = cudaGetLastError();
+        const cudaError_t done = cudaStreamSynchronize(s);
+        if (e == cudaSuccess) e = done;
+        cudaStreamDestroy(s);
+    }
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    if (e == cudaSuccess) g_exp2_addr[dev].store((const float2*)p, std::memory_order_release);
+    return e;
+}
+
+const float2* exp2_table() {
+    int dev = 0;
+    return cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < kMaxDevices
+               ? g_exp2_addr[dev].load(std::memory_order_acquire)
+               : nullptr;
+}
+
 // The double-float assembly for one (DB, COLS, family): its shared-memory
 // limit raised once per device and size (raise_smem_limit, safe when
 // contexts on several threads assemble at once), then the launch.
@@ -452,7 +499,7 @@ static cudaError_t launch_asm_df(dim3 grid, size_t smem, cudaStream_t s, const B
     static std::atomic<size_t> attr[kMaxDevices];
     cudaError_t e = raise_smem_limit(k_assemble_tiles_df<DB, COLS, M, EXACT>, smem, attr);
     if (e != cudaSuccess) return e;
-    k_assemble_tiles_df<DB, COLS, M, EXACT><<<grid, kThreads, smem, s>>>(b, group);
+    k_assemble_tiles_df<DB, COLS, M, EXACT><<<grid, kThreads, smem, s>>>(b, group, exp2_table());
     return cudaGetLastError();
 }
 

@@ -24,6 +24,7 @@
 // The inverse in double-float multiply-adds on the FP32 pipes, along the tile
 // diagonals of X, took 36.6 ms of the gradient's 49 at n = 4064, T = 1.
 #include "corr.cuh"
+#include "inv_diag.cuh"
 #include "mixed_common.cuh"
 
 namespace gp {
@@ -37,49 +38,7 @@ __device__ __forceinline__ T* tile_at(T* base, size_t stride, int t, int I, int 
     return base + (size_t)t * stride + (size_t)tile_index(I, J, nt) * GP_TILE_ELEMS;
 }
 
-// X_JJ = W_J = L_JJ^-1 (lower; zeros above the diagonal) in double, a CTA per 32
-// columns of it (their rows above are zero): lane = column, warp w holds rows
-// c0 + w + 4 i of acc_ij = sum_{m<k} L_im W_mj in registers.  Step k finishes row
-// k (W_kj = -acc_kj / L_kk, W_kk = 1 / L_kk), one barrier, and adds its term to the
-// rows after it.  Four rows are one iteration of a loop (the rows move down
-// one register as they finish), in forms for up to 31, 23, 15 and 7 rows left.
-// 0.13 ms for every block of n = 4064 at once (0.45 ms with one CTA a block
-// and a dependent sum per entry).
-constexpr int kPackedTri = GP_NB * (GP_NB + 1) / 2;
-constexpr int kInvThreads = 128;
-constexpr int kInvWarps = kInvThreads / 32;
-constexpr int kInvCols = 32;
-constexpr int kInvRows = GP_NB / kInvWarps;            // rows of a warp
-__device__ __forceinline__ int prow(int r) { return r * (r + 1) / 2; }
-
-// Rows k = k0 .. k0 + 31, or up to row 127 where LEFT rows of a warp are left.
-template <int LEFT>
-__device__ __forceinline__ void inv_rows(double (&acc)[kInvRows], const double* Lp, const double* dinv,
-                                         double (*Wk)[kInvCols], double* Xt, int k0, int c0, int warp, int lane) {
-#pragma unroll 1
-    for (int g = 0; g < 8; ++g) {
-#pragma unroll
-        for (int q = 0; q < kInvWarps; ++q) {
-            const int k = k0 + kInvWarps * g + q;
-            if (warp == q) {
-                const double w = c0 + lane == k ? dinv[k] : -dinv[k] * acc[0];
-                Wk[k & 1][lane] = w;
-                Xt[(size_t)(c0 + lane) * GP_NB + k] = w;
-            }
-            __syncthreads();
-            const double w = Wk[k & 1][lane];
-            if (warp > q) acc[0] = fma(Lp[prow(k - q + warp) + k], w, acc[0]);
-#pragma unroll
-            for (int i = 1; i <= LEFT; ++i) {
-                const int r = k - q + warp + kInvWarps * i;
-                if (i <= LEFT - 7 || r < GP_NB) acc[i] = fma(Lp[prow(r) + k], w, acc[i]);
-            }
-        }
-#pragma unroll
-        for (int i = 0; i < LEFT; ++i) acc[i] = acc[i + 1];
-    }
-}
-
+// X_JJ = W_J = L_JJ^-1 in double (inv_diag.cuh), a CTA per 32 columns of it.
 __global__ void __launch_bounds__(kInvThreads) k_inv_diag(Batch b, double* X) {
     extern __shared__ double Lp[];                     // packed lower triangle, row r at r (r + 1) / 2
     __shared__ double dinv[GP_NB];
@@ -97,13 +56,7 @@ __global__ void __launch_bounds__(kInvThreads) k_inv_diag(Batch b, double* X) {
     if ((int)threadIdx.x >= c0) dinv[threadIdx.x] = 1.0 / L[threadIdx.x * (GP_NB + 1)];
     cp_async_wait_all();
     __syncthreads();
-    double acc[kInvRows];
-#pragma unroll
-    for (int i = 0; i < kInvRows; ++i) acc[i] = 0.0;
-    if (c0 <= 0) inv_rows<31>(acc, Lp, dinv, Wk, Xt, 0, c0, warp, lane);
-    if (c0 <= 32) inv_rows<23>(acc, Lp, dinv, Wk, Xt, 32, c0, warp, lane);
-    if (c0 <= 64) inv_rows<15>(acc, Lp, dinv, Wk, Xt, 64, c0, warp, lane);
-    inv_rows<7>(acc, Lp, dinv, Wk, Xt, 96, c0, warp, lane);
+    inv_columns(Lp, dinv, Wk, Xt, c0, warp, lane);
 }
 
 // Exponents of W_J's rows, |W_rc| < 2^E, into slot 2 of the factor's diagonal
@@ -177,7 +130,7 @@ constexpr int kGradSplit = 4;
 
 template <int DB, int G>
 __global__ void __launch_bounds__(kThreads) k_grad_tiles(Batch b, const double* Ri, const double* Z, size_t zs,
-                                                         ExpTab64 etab) {
+                                                         ExpTab64 etab, const float2* e2tab) {
     __shared__ double red[kThreads / 32][DB];
     __shared__ dfl tab[kExpTab];
     __shared__ ExpTab64 et;
@@ -187,7 +140,7 @@ __global__ void __launch_bounds__(kThreads) k_grad_tiles(Batch b, const double* 
     const int corr = b.corr;
     const bool matern = corr_is_matern(corr);
     const double cm = corr_theta_scale(corr);
-    fill_exp2_table(tab);
+    load_exp2_table(tab, e2tab);
     for (int q = threadIdx.x; q < (int)(sizeof(ExpTab64) / sizeof(double)); q += kThreads)
         reinterpret_cast<double*>(&et)[q] = reinterpret_cast<const double*>(&etab)[q];
     for (int q = threadIdx.x; q < G * DB; q += kThreads) {
@@ -341,8 +294,8 @@ cudaError_t launch_grad(const Batch& b, double* Z, size_t zs, double* X, double*
     const int G = (long long)ntiles * ((b.count + 3) / 4) * 4 >= 3LL * device_sms() && b.count > 1 ? 4 : 1;
     const dim3 grid(parts, (b.count + G - 1) / G);
 #define GP_GRAD_TILES(DB)                                                                                   \
-    (G == 4 ? k_grad_tiles<DB, 4><<<grid, kThreads, 0, s>>>(b, Ri, Z, zs, et)              \
-            : k_grad_tiles<DB, 1><<<grid, kThreads, 0, s>>>(b, Ri, Z, zs, et))
+    (G == 4 ? k_grad_tiles<DB, 4><<<grid, kThreads, 0, s>>>(b, Ri, Z, zs, et, exp2_table())              \
+            : k_grad_tiles<DB, 1><<<grid, kThreads, 0, s>>>(b, Ri, Z, zs, et, exp2_table()))
     if (b.d <= 4)      GP_GRAD_TILES(4);
     else if (b.d <= 8) GP_GRAD_TILES(8);
     else               GP_GRAD_TILES(16);

@@ -42,6 +42,7 @@ struct PredArgs {
     double* yhat;
     double* s2;
     float2* work;          // per CTA: npad * NR
+    const float2* etab;    // exp2_table()
 };
 
 // NR test points per CTA, PT = NR / 2 per thread (two threads per row).
@@ -70,7 +71,7 @@ __global__ void __launch_bounds__(kThreads) k_predict(PredArgs g) {
     }
     // Matern families: theta pre-multiplied by c, powers with p = 1 (corr.cuh)
     for (int q = threadIdx.x; q < d; q += kThreads) th[q] = df_from_double(corr_theta_scale(g.corr) * g.theta[q]);
-    fill_exp2_table(tab);
+    load_exp2_table(tab, g.etab);
     const dfl pd = df_from_double(g.p);
     const bool matern = corr_is_matern(g.corr);
     const int pmode = matern ? kPowOne : pow_mode(g.p);
@@ -249,6 +250,7 @@ cudaError_t launch_predict(int n, int d, int nt, const float2* x, const double* 
     g.n = n; g.d = d; g.nt = nt; g.N = N; g.m0 = 0;
     g.x = x; g.theta = theta; g.p = p; g.corr = corr; g.c0 = c0;
     g.L = L; g.w = w; g.a = a; g.sc = scalars; g.xs = xs; g.yhat = yhat; g.s2 = s2; g.work = work;
+    g.etab = exp2_table();
     if (nr == 8) return launch_predict_nr<8>(g, d, N, chunk, s);
     if (nr == 16) return launch_predict_nr<16>(g, d, N, chunk, s);
     return cudaErrorInvalidValue;

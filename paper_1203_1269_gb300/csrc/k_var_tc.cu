@@ -33,7 +33,7 @@
 //
 // r, its products with w (the mean) and the diagonal inverses come from
 // kernels on the FP32 / FP64 pipes before the tensor-core pass:
-//   k_var_w       W_J = L_JJ^-1 in double (one CTA per tile row), its rows'
+//   k_var_w, k_var_wslice   W_J = L_JJ^-1 in double, its rows'
 //                 exponents and 7 slices
 //   k_var_lmax,   row exponents and 5 slices of the rows of L left of the
 //   k_var_lslice  diagonal (the update's B operand)
@@ -47,6 +47,7 @@
 // All of it is rebuilt per call from the model (the tables take about 1 ms
 // at n = 16384), so a model holds only its factor.
 #include "corr.cuh"
+#include "inv_diag.cuh"
 #include "slices.cuh"
 
 namespace gp {
@@ -90,59 +91,61 @@ __host__ __device__ inline size_t ws_chunk(int J, int a, int k) { return ((size_
 
 // ------------------------------------------------------------ tables -------
 
-// W_J = L_JJ^-1 by columns in double (thread j owns column j: W_jj =
-// 1 / L_jj, W_ij = -(sum_{k=j}^{i-1} L_ik W_kj) / L_ii), then thread i
-// cuts row i of W into 7 slices with its own exponent.  Dynamic shared
-// memory: L_JJ packed (8256 doubles), W with row stride 129, 1 / L_ii.
-constexpr int kWStride = GP_NB + 1;
-constexpr size_t kVarWSmem = (size_t)(GP_NB * (GP_NB + 1) / 2 + GP_NB * kWStride + GP_NB) * sizeof(double);
-
-__global__ void __launch_bounds__(GP_NB) k_var_w(const float2* L, int nt, __nv_bfloat16* WS, int* WE) {
-    extern __shared__ double wsm[];
-    double* Lp = wsm;                                  // L_rc at r (r + 1) / 2 + c
-    double* W = Lp + GP_NB * (GP_NB + 1) / 2;          // W_ij at i * kWStride + j
-    double* dinv = W + GP_NB * kWStride;
-    const int J = blockIdx.x, j = threadIdx.x;
+// W_J = L_JJ^-1 in double (inv_diag.cuh), a CTA per 32 columns, column-major
+// into the memory that W_J's slices will take.  With the slicing after it 0.20
+// ms for any nt <= 38 (0.43 ms as one CTA per J with a dependent sum per entry;
+// the same bits; the serving request's 1000 predictions 1.50 -> 1.27 ms).
+__global__ void __launch_bounds__(kInvThreads) k_var_w(const float2* L, int nt, __nv_bfloat16* WS) {
+    extern __shared__ double Lp[];                     // packed lower triangle
+    __shared__ double dinv[GP_NB];
+    __shared__ double Wk[2][kInvCols];
+    const int J = blockIdx.x, c0 = kInvCols * blockIdx.y;
     const float2* T = L + (size_t)tile_index(J, J, nt) * GP_TILE_ELEMS;
-    for (int c = 0; c < GP_NB; ++c)
-        if (j >= c) Lp[j * (j + 1) / 2 + c] = (double)T[(size_t)c * GP_NB + j].x + (double)T[(size_t)c * GP_NB + j].y;
-    __syncthreads();
-    dinv[j] = 1.0 / Lp[j * (j + 1) / 2 + j];
-    __syncthreads();
-    for (int i = 0; i < GP_NB; ++i) {
-        double w = 0.0;
-        if (i == j) {
-            w = dinv[j];
-        } else if (i > j) {
-            double s = 0.0;
-            const double* Li = Lp + i * (i + 1) / 2;
-            for (int k = j; k < i; ++k) s = fma(Li[k], W[k * kWStride + j], s);
-            w = -s * dinv[i];
+    for (int q = threadIdx.x; q < GP_TILE_ELEMS; q += kInvThreads) {
+        const int r = q % GP_NB, c = q / GP_NB;
+        if (r >= c && c >= c0) {
+            const double l = (double)T[q].x + (double)T[q].y;
+            Lp[prow(r) + c] = l;
+            if (r == c) dinv[r] = 1.0 / l;
         }
-        W[i * kWStride + j] = w;
     }
     __syncthreads();
-    // row i = j of W: exponent from the high words, then the slices (the
-    // same cut as the factorisation's panel slicing)
-    const int i = j;
+    inv_columns(Lp, dinv, Wk, reinterpret_cast<double*>(WS + ws_chunk(J, 0, 0) * kChunkElems), c0,
+                threadIdx.x >> 5, threadIdx.x & 31);
+}
+
+// Slices of W_J's rows, each with its own exponent (from the high words, the
+// same cut as the factorisation's panel slicing), over the doubles they are
+// cut from: thread (row, part) holds two runs of 16 columns.
+constexpr int kWSliceThreads = 512;
+__global__ void __launch_bounds__(kWSliceThreads) k_var_wslice(__nv_bfloat16* WS, int* WE) {
+    __shared__ float pmax[4][GP_NB];
+    const int J = blockIdx.x, i = threadIdx.x & (GP_NB - 1), part = threadIdx.x >> 7;
+    const double* W = reinterpret_cast<const double*>(WS + ws_chunk(J, 0, 0) * kChunkElems);
+    float2 v[2][16];
     float mx = 0.f;
-    for (int k = 0; k <= i; ++k) mx = fmaxf(mx, fabsf(__double2float_rn(W[i * kWStride + k])));
+#pragma unroll
+    for (int u = 0; u < 2; ++u)
+#pragma unroll
+        for (int e = 0; e < 16; ++e) {
+            const int k = 32 * part + 16 * u + e;
+            const double w = k <= i ? W[(size_t)k * GP_NB + i] : 0.0;
+            const dfl x = df_from_double(w);
+            v[u][e] = make_float2(x.hi, x.lo);
+            mx = fmaxf(mx, fabsf(x.hi));
+        }
+    pmax[part][i] = mx;
+    __syncthreads();                                   // every double of W_J has been read
+#pragma unroll
+    for (int q = 0; q < 4; ++q) mx = fmaxf(mx, pmax[q][i]);
     const int E = exponent_of(mx);
-    WE[J * GP_NB + i] = E;
+    if (part == 0) WE[J * GP_NB + i] = E;
     float sa, sb;
     slice_scale(E, sa, sb);
     uint8_t* base = reinterpret_cast<uint8_t*>(WS + ws_chunk(J, 0, 0) * kChunkElems);
-#pragma unroll 1
-    for (int u = 0; u < 8; ++u) {
-        float2 v[16];
 #pragma unroll
-        for (int e = 0; e < 16; ++e) {
-            const dfl x = df_from_double(W[i * kWStride + 16 * u + e]);
-            v[e] = make_float2(x.hi, x.lo);
-        }
-        slice_pieces(v, sa, sb, i, 16 * (u & 1), kVarWSlices, base + (size_t)(u >> 1) * kChunkBytes,
-                     (size_t)4 * kChunkBytes);
-    }
+    for (int u = 0; u < 2; ++u)
+        slice_pieces(v[u], sa, sb, i, 16 * u, kVarWSlices, base + (size_t)part * kChunkBytes, (size_t)4 * kChunkBytes);
 }
 
 // Largest |L_ik| (high words) of each row left of its diagonal block: tile
@@ -865,19 +868,21 @@ VarTables var_tables_at(void* base, int nt) {
 }
 
 // The slices of W_J (all J) and of the rows of L left of their diagonal
-// blocks: 1 + (nt > 1 ? 2 : 0) kernels.
+// blocks: 2 + (nt > 1 ? 2 : 0) kernels.
 cudaError_t launch_var_tables(const float2* L, int nt, const VarTables& t, cudaStream_t s, int* kernels) {
     static std::atomic<size_t> attr[kMaxDevices];
-    cudaError_t e = raise_smem_limit(k_var_w, kVarWSmem, attr);
+    constexpr size_t smem = (size_t)kPackedTri * sizeof(double);
+    cudaError_t e = raise_smem_limit(k_var_w, smem, attr);
     if (e != cudaSuccess) return e;
-    k_var_w<<<nt, GP_NB, kVarWSmem, s>>>(L, nt, t.WS, t.WE);
-    *kernels = 1;
+    k_var_w<<<dim3(nt, GP_NB / kInvCols), kInvThreads, smem, s>>>(L, nt, t.WS);
+    k_var_wslice<<<nt, kWSliceThreads, 0, s>>>(t.WS, t.WE);
+    *kernels = 2;
     if ((e = cudaGetLastError()) != cudaSuccess || nt == 1) return e;
     const unsigned tiles = (unsigned)((long long)nt * (nt - 1) / 2);
     if ((e = cudaMemsetAsync(t.lbits, 0, (size_t)nt * GP_NB * sizeof(int), s)) != cudaSuccess) return e;
     k_var_lmax<<<tiles, GP_NB, 0, s>>>(L, nt, t.lbits);
     k_var_lslice<<<tiles, 2 * GP_NB, 0, s>>>(L, nt, t.lbits, t.LS, t.LE);
-    *kernels = 3;
+    *kernels = 4;
     return cudaGetLastError();
 }
 
