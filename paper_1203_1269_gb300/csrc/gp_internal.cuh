@@ -227,6 +227,67 @@ cudaError_t launch_factor_small_f64(const Batch& b, cudaStream_t s, int* kernels
 // singularity (cond(R) 1e11, where any change of rounding shows in the eighth
 // digit of mu_hat) keep their bits.
 constexpr int kUpdateTcTiles = 3;
+
+// Launches of a chain of kernels in one stream.  With `ahead`, the kernel is set
+// up on the GPU while the one before it still runs (programmatic stream
+// serialization); its first statement, grid_dependency(), waits until that one
+// has completed with its writes visible, so no result depends on the flag.  Only
+// for kernels that begin with grid_dependency().
+//
+// Where few blocks run it saves 1 to 1.5 us a launch, and a block column of the
+// factor is a dozen launches (ms, without -> with; candidates x n):
+//   double factor: 1x200 .577 -> .518, 16x300 1.11 -> 1.03, 16x1024 3.06 -> 2.88,
+//     8x2048 6.43 -> 6.13, 1x4064 9.06 -> 8.28, 1x8192 27.9 -> 27.1;
+//   split factor: 100x64 .286 -> .263, 32x256 .501 -> .467, 8x1024 1.86 -> 1.80,
+//     1x4000 7.43 -> 7.19.
+// Where many do it costs: a block that waits takes its place beside one that
+// runs, so that several blocks of the next kernel share an SM (and its FP64 or
+// shared-memory rate) while others idle, and the second stream's slicing finds
+// no room: 16x200 .750 -> .760, 64x200 1.11 -> 1.22, 128x300 2.17 -> 2.55, 32x1024 4.28 -> 4.83 (all
+// double), 8x4064 the same either way, split 8x16384 188 -> 190 to 193.
+// kAhead* are the lines between the two.  The first launch after a wait for the
+// other stream is a plain one.
+constexpr int kAheadSmallF64 = 8;      // candidates, double, up to two block columns
+constexpr int kAheadCountF64 = 16;     // the same, more block columns
+constexpr int kAheadColumnsF64 = 128;  // candidates x block columns, double
+constexpr int kAheadColumnsMixed = 256;
+
+inline bool ahead_f64(const Batch& b) {
+    return b.count <= (b.nt < kUpdateTcTiles ? kAheadSmallF64 : kAheadCountF64) &&
+           (long long)b.count * b.nt <= kAheadColumnsF64;
+}
+
+inline bool ahead_mixed(const MixedBatch& b) { return (long long)b.count * b.nt <= kAheadColumnsMixed; }
+
+inline bool ahead_assemble(const Batch& b) {
+    return b.Adf ? (long long)b.count * b.nt <= kAheadColumnsMixed : ahead_f64(b);
+}
+
+template <typename T>
+struct NotDeduced {
+    using type = T;
+};
+template <typename... P>
+inline cudaError_t launch_chained(bool ahead, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
+                                  cudaStream_t s, typename NotDeduced<P>::type... args) {
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &attr;
+    cfg.numAttrs = ahead ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
+__device__ __forceinline__ void grid_dependency() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 cudaError_t launch_forward_solve(const Batch& b, double* Z, size_t z_stride, cudaStream_t s);
 cudaError_t launch_finalize(const Batch& b, const double* Z, size_t z_stride, double* nll,
                             double* mu, double* sigma2, double* logdet, int* status,

@@ -150,6 +150,7 @@ constexpr int kThetaCache = 1024;
 template <int DB, bool TAB>
 __global__ void __launch_bounds__(kThreads)
 k_assemble_tiles(Batch b, int group, PowTab64 ptab) {
+    grid_dependency();
     __shared__ double xs_r[GP_NB * DB];
     __shared__ double xs_c[kCols * DB];
     __shared__ PowTab64 pt;
@@ -265,6 +266,7 @@ k_assemble_tiles(Batch b, int group, PowTab64 ptab) {
 template <int DB, int COLS, bool MATERN, bool EXACT = false>
 __global__ void __launch_bounds__(kThreads)
 k_assemble_tiles_df(Batch b, int group, const float2* etab) {
+    grid_dependency();
     constexpr int kSplitDf = GP_NB / COLS;
     constexpr int kColsDf = COLS;
     constexpr int kEntriesDf = GP_NB * COLS / kThreads;
@@ -499,7 +501,8 @@ static cudaError_t launch_asm_df(dim3 grid, size_t smem, cudaStream_t s, const B
     static std::atomic<size_t> attr[kMaxDevices];
     cudaError_t e = raise_smem_limit(k_assemble_tiles_df<DB, COLS, M, EXACT>, smem, attr);
     if (e != cudaSuccess) return e;
-    k_assemble_tiles_df<DB, COLS, M, EXACT><<<grid, kThreads, smem, s>>>(b, group, exp2_table());
+    launch_chained(ahead_assemble(b), k_assemble_tiles_df<DB, COLS, M, EXACT>, grid, kThreads, smem, s, b,
+                   group, exp2_table());
     return cudaGetLastError();
 }
 
@@ -588,14 +591,14 @@ cudaError_t launch_assemble_tiles(const Batch& b, cudaStream_t s) {
     if (b.d <= 16 && !corr_is_matern(b.corr) && pow_mode(b.p) == kPowGeneral) pow_tab64_fill(b.p, pt);
     const bool tab = pt.on != 0;
     if (b.d <= 4)
-        tab ? k_assemble_tiles<4, true><<<grid, kThreads, 0, s>>>(b, group, pt)
-            : k_assemble_tiles<4, false><<<grid, kThreads, 0, s>>>(b, group, pt);
+        tab ? launch_chained(ahead_assemble(b), k_assemble_tiles<4, true>, grid, kThreads, 0, s, b, group, pt)
+            : launch_chained(ahead_assemble(b), k_assemble_tiles<4, false>, grid, kThreads, 0, s, b, group, pt);
     else if (b.d <= 8)
-        tab ? k_assemble_tiles<8, true><<<grid, kThreads, 0, s>>>(b, group, pt)
-            : k_assemble_tiles<8, false><<<grid, kThreads, 0, s>>>(b, group, pt);
+        tab ? launch_chained(ahead_assemble(b), k_assemble_tiles<8, true>, grid, kThreads, 0, s, b, group, pt)
+            : launch_chained(ahead_assemble(b), k_assemble_tiles<8, false>, grid, kThreads, 0, s, b, group, pt);
     else if (b.d <= 16)
-        tab ? k_assemble_tiles<16, true><<<grid, kThreads, 0, s>>>(b, group, pt)
-            : k_assemble_tiles<16, false><<<grid, kThreads, 0, s>>>(b, group, pt);
+        tab ? launch_chained(ahead_assemble(b), k_assemble_tiles<16, true>, grid, kThreads, 0, s, b, group, pt)
+            : launch_chained(ahead_assemble(b), k_assemble_tiles<16, false>, grid, kThreads, 0, s, b, group, pt);
     else
         k_assemble_tiles_generic<<<grid, kThreads, 0, s>>>(b, group);
     return cudaGetLastError();

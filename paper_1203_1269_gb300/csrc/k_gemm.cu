@@ -155,6 +155,7 @@ __device__ __forceinline__ void sum_panel_groups(const float (&d)[NG][CB], int j
 template <int MODE, int NT, int NG, bool ER = false>
 __global__ void __launch_bounds__(ER ? kGemmThreadsER : kGemmThreads, 1)
     k_split_gemm(MixedBatch b, int J, int per_inst, int kind) {
+    grid_dependency();
     static_assert(NG * NT <= 512, "accumulators exceed tensor memory");
     static_assert(!ER || (MODE == 1 && NT == 128 && NG == 4) || (MODE == 0 && NT == 64),
                   "early release is built for the 128-column update and the panel solve");
@@ -572,7 +573,8 @@ static cudaError_t launch_gemm(const MixedBatch& b, int J, int per_inst, int ns,
     if (e != cudaSuccess) return e;
     const long long total = (long long)per_inst * b.count;
     const int grid = (int)(total < device_sms() ? total : device_sms());
-    k_split_gemm<MODE, NT, NG, ER><<<grid, ER ? kGemmThreadsER : kGemmThreads, smem, s>>>(b, J, per_inst, kind);
+    launch_chained(MODE != 0 && ahead_mixed(b), k_split_gemm<MODE, NT, NG, ER>, grid,
+                   ER ? kGemmThreadsER : kGemmThreads, smem, s, b, J, per_inst, kind);
     return cudaGetLastError();
 }
 

@@ -40,6 +40,7 @@ __device__ __forceinline__ T* tile_at(T* base, size_t stride, int t, int I, int 
 
 // X_JJ = W_J = L_JJ^-1 in double (inv_diag.cuh), a CTA per 32 columns of it.
 __global__ void __launch_bounds__(kInvThreads) k_inv_diag(Batch b, double* X) {
+    grid_dependency();
     extern __shared__ double Lp[];                     // packed lower triangle, row r at r (r + 1) / 2
     __shared__ double dinv[GP_NB];
     __shared__ double Wk[2][kInvCols];
@@ -62,6 +63,7 @@ __global__ void __launch_bounds__(kInvThreads) k_inv_diag(Batch b, double* X) {
 // Exponents of W_J's rows, |W_rc| < 2^E, into slot 2 of the factor's diagonal
 // tile (the factor's own diagonal block is not needed any more).
 __global__ void __launch_bounds__(GP_NB) k_row_exponents(Batch b, const double* X) {
+    grid_dependency();
     const int J = blockIdx.x, t = blockIdx.y, r = threadIdx.x;
     if (b.st[t].status != GP_OK) return;
     const double* T = tile_at(X, b.inst_stride, t, J, J, b.nt) + r;
@@ -76,6 +78,7 @@ __global__ void __launch_bounds__(GP_NB) k_row_exponents(Batch b, const double* 
 // columns, 128 entries in a coalesced kilobyte each.
 constexpr int kExpSplit = 4;
 __global__ void __launch_bounds__(kThreads) k_col_exponents(Batch b, const double* src, int J, int slot) {
+    grid_dependency();
     const int K = blockIdx.x, t = blockIdx.y;
     if (b.st[t].status != GP_OK) return;
     const double* T = tile_at(src, b.inst_stride, t, J, K, b.nt);
@@ -100,6 +103,7 @@ __global__ void __launch_bounds__(kThreads) k_col_exponents(Batch b, const doubl
 
 // e = b - mu_hat a in column 1 of Z (w = L^-T e follows by the backward solve)
 __global__ void k_residual_vec(Batch b, double* Z, size_t zs) {
+    grid_dependency();
     const int t = blockIdx.x;
     const InstState st = b.st[t];
     if (st.status != GP_OK) return;
@@ -131,6 +135,7 @@ constexpr int kGradSplit = 4;
 template <int DB, int G>
 __global__ void __launch_bounds__(kThreads) k_grad_tiles(Batch b, const double* Ri, const double* Z, size_t zs,
                                                          ExpTab64 etab, const float2* e2tab) {
+    grid_dependency();
     __shared__ double red[kThreads / 32][DB];
     __shared__ dfl tab[kExpTab];
     __shared__ ExpTab64 et;
@@ -240,6 +245,7 @@ __global__ void __launch_bounds__(kThreads) k_grad_tiles(Batch b, const double* 
 // NaN where the likelihood itself failed (status: the finalize kernel's, which
 // also flags Q = 0)
 __global__ void k_grad_reduce(Batch b, int parts, const int* status, double* grad) {
+    grid_dependency();
     const int t = blockIdx.x, d = b.d;
     const int k = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (k >= d) return;
@@ -260,7 +266,7 @@ cudaError_t launch_grad(const Batch& b, double* Z, size_t zs, double* X, double*
                         double* grad, cudaStream_t s, int* kernels) {
     const int nt = b.nt;
     int k = 0;
-    k_residual_vec<<<b.count, kThreads, 0, s>>>(b, Z, zs);
+    launch_chained(ahead_f64(b), k_residual_vec, b.count, kThreads, 0, s, b, Z, zs);
     ++k;
     cudaError_t e = launch_backward_solve(b, Z, zs, 1, s);   // w = L^-T (b - mu a), double factor
     if (e != cudaSuccess) return e;
@@ -270,18 +276,18 @@ cudaError_t launch_grad(const Batch& b, double* Z, size_t zs, double* X, double*
         static std::atomic<size_t> attr[kMaxDevices];
         e = raise_smem_limit(k_inv_diag, smem, attr);
         if (e != cudaSuccess) return e;
-        k_inv_diag<<<dim3(nt, b.count, GP_NB / kInvCols), kInvThreads, smem, s>>>(b, X);
-        k_row_exponents<<<dim3(nt, b.count), GP_NB, 0, s>>>(b, X);
+        launch_chained(ahead_f64(b), k_inv_diag, dim3(nt, b.count, GP_NB / kInvCols), kInvThreads, smem, s, b, X);
+        launch_chained(ahead_f64(b), k_row_exponents, dim3(nt, b.count), GP_NB, 0, s, b, X);
         k += 2;
     }
     for (int J = 0; J < nt; ++J) {
         if (J > 0) {
-            k_col_exponents<<<dim3(J, b.count, kExpSplit), kThreads, 0, s>>>(b, Ri, J, 1);
+            launch_chained(ahead_f64(b), k_col_exponents, dim3(J, b.count, kExpSplit), kThreads, 0, s, b, Ri, J, 1);
             e = launch_inverse_apply(b, J, X, Ri, s);
             if (e != cudaSuccess) return e;
             k += 2;
         }
-        k_col_exponents<<<dim3(J + 1, b.count, kExpSplit), kThreads, 0, s>>>(b, X, J, 0);
+        launch_chained(ahead_f64(b), k_col_exponents, dim3(J + 1, b.count, kExpSplit), kThreads, 0, s, b, X, J, 0);
         e = launch_inverse_update(b, J, X, Ri, s);
         if (e != cudaSuccess) return e;
         k += 2;
@@ -294,14 +300,14 @@ cudaError_t launch_grad(const Batch& b, double* Z, size_t zs, double* X, double*
     const int G = (long long)ntiles * ((b.count + 3) / 4) * 4 >= 3LL * device_sms() && b.count > 1 ? 4 : 1;
     const dim3 grid(parts, (b.count + G - 1) / G);
 #define GP_GRAD_TILES(DB)                                                                                   \
-    (G == 4 ? k_grad_tiles<DB, 4><<<grid, kThreads, 0, s>>>(b, Ri, Z, zs, et, exp2_table())              \
-            : k_grad_tiles<DB, 1><<<grid, kThreads, 0, s>>>(b, Ri, Z, zs, et, exp2_table()))
+    (G == 4 ? launch_chained(ahead_f64(b), k_grad_tiles<DB, 4>, grid, kThreads, 0, s, b, Ri, Z, zs, et, exp2_table()) \
+            : launch_chained(ahead_f64(b), k_grad_tiles<DB, 1>, grid, kThreads, 0, s, b, Ri, Z, zs, et, exp2_table()))
     if (b.d <= 4)      GP_GRAD_TILES(4);
     else if (b.d <= 8) GP_GRAD_TILES(8);
     else               GP_GRAD_TILES(16);
 #undef GP_GRAD_TILES
     ++k;
-    k_grad_reduce<<<b.count, 32 * 16, 0, s>>>(b, parts, status, grad);
+    launch_chained(ahead_f64(b), k_grad_reduce, b.count, 32 * 16, 0, s, b, parts, status, grad);
     ++k;
     if (kernels) *kernels = k;
     return cudaGetLastError();

@@ -510,6 +510,7 @@ __device__ __forceinline__ void diag_dispatch_rest(const DiagShared& sh, DiagReg
 }
 
 __global__ void __launch_bounds__(kDiagThreads, 1) k_diag_mixed(MixedBatch b, int J) {
+    grid_dependency();
     extern __shared__ dfl P[];             // kPacked double-float values: A_JJ in, W out
     __shared__ DiagShared sh;
     const int t = blockIdx.x;
@@ -680,6 +681,7 @@ __device__ __forceinline__ void fwd_apply(const MixedBatch& b, int t, int I, int
 }
 
 __global__ void __launch_bounds__(kSplitThreads) k_split_panel(MixedBatch b, int J, int ns, int gemv) {
+    grid_dependency();
     __shared__ float pmax[kSplitParts][kSplitRows];
     __shared__ dfl xs[2][GP_NB];
     __shared__ dfl red[kSplitParts][2][kSplitRows];
@@ -728,6 +730,7 @@ __global__ void __launch_bounds__(kSplitThreads) k_split_panel(MixedBatch b, int
 // chunk as in k_split_panel), so every tile is read once and every slice
 // written in 32-byte stores; the row maximum spans all 16 parts.
 __global__ void __launch_bounds__(kSplitThreads) k_split_fused(MixedBatch b, int J) {
+    grid_dependency();
     __shared__ float pmax[kFusedParts][kFusedRows];
     __shared__ dfl xs[2][GP_NB];
     __shared__ dfl red[kFusedParts / 2][2][kFusedRows];
@@ -810,6 +813,7 @@ __device__ dfl block_sum_df(dfl v, dfl* red) {
 // [1 Y] (zero on padded rows) into Z columns 0, 1: the right-hand sides of
 // the forward solve that the factorisation carries out block by block
 __global__ void k_rhs_init(MixedBatch b) {
+    grid_dependency();
     const int t = blockIdx.y;
     const int gi = blockIdx.x * blockDim.x + threadIdx.x;
     if (gi >= b.nt * GP_NB) return;
@@ -908,6 +912,7 @@ __device__ __forceinline__ void fwd_diag_step(const MixedBatch& b, int t, int c0
 }
 
 __global__ void __launch_bounds__(kSubThreads) k_fwd_diag(MixedBatch b, int c0, int J) {
+    grid_dependency();
     __shared__ dfl rhs[2][GP_NB];
     __shared__ dfl part[2][2][GP_NB];
     const int t = blockIdx.x;
@@ -919,6 +924,7 @@ __global__ void __launch_bounds__(kSubThreads) k_fwd_diag(MixedBatch b, int c0, 
 // the CTA finishing tile (J + 1, J) second then takes block J + 1's
 // diagonal step
 __global__ void __launch_bounds__(kSubThreads) k_fwd_tiles(MixedBatch b, int c0, int J) {
+    grid_dependency();
     __shared__ dfl xs[2][GP_NB / 2];
     __shared__ dfl part[2][2][GP_NB];
     __shared__ dfl rhs[2][GP_NB];
@@ -1004,6 +1010,7 @@ __device__ __forceinline__ void bwd_diag_step(const MixedBatch& b, int t, int c0
 }
 
 __global__ void __launch_bounds__(kSubThreads) k_bwd_diag(MixedBatch b, int c0, int K, int add_to) {
+    grid_dependency();
     __shared__ dfl rhs[2][GP_NB];
     __shared__ dfl part[2][2][GP_NB];
     const int t = blockIdx.x;
@@ -1017,6 +1024,7 @@ __global__ void __launch_bounds__(kSubThreads) k_bwd_diag(MixedBatch b, int c0, 
 // second then takes block K - 1's diagonal step
 constexpr int kBwdTs = GP_NB / 2 + 1;
 __global__ void __launch_bounds__(kSubThreads) k_bwd_tiles(MixedBatch b, int c0, int K, int add_to) {
+    grid_dependency();
     extern __shared__ dfl T[];                  // GP_NB x kBwdTs
     __shared__ dfl xs[2][GP_NB / 2];
     __shared__ dfl part[2][2][GP_NB];
@@ -1068,6 +1076,7 @@ constexpr int kResCols = GP_NB / 2;
 static_assert(kRpTile == 2 * 2 * GP_NB + 2 * 2 * kResCols, "residual partial layout");
 
 __global__ void __launch_bounds__(kResThreads) k_resid_tiles(MixedBatch b) {
+    grid_dependency();
     extern __shared__ dfl T[];                  // kResCols x kTs
     __shared__ dfl xa[2][kResCols];             // x_J on this half's columns
     __shared__ dfl xb[2][GP_NB];                // x_I
@@ -1137,6 +1146,7 @@ __global__ void __launch_bounds__(kResThreads) k_resid_tiles(MixedBatch b) {
 // into Z columns 2, 3; padded rows: R is the identity there and x is zero,
 // so r = 0.  One CTA per (row block I, instance).
 __global__ void __launch_bounds__(kResThreads) k_resid_reduce(MixedBatch b) {
+    grid_dependency();
     const int t = blockIdx.y, I = blockIdx.x;
     if (b.st[t].status != GP_OK || b.st[t].refine_done) return;
     const int nt = b.nt, n = b.n;
@@ -1161,6 +1171,7 @@ __global__ void __launch_bounds__(kResThreads) k_resid_reduce(MixedBatch b) {
 // a = L^-1 1 and b = L^-1 Y (Z columns 0, 1 after the forward solve) into
 // columns 8, 9, where the refinement's sums read them
 __global__ void k_keep_forward(MixedBatch b) {
+    grid_dependency();
     const int t = blockIdx.y;
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const int npad = b.nt * GP_NB;
@@ -1197,6 +1208,7 @@ __device__ __forceinline__ double split_unit(int s) {
 }
 
 __global__ void __launch_bounds__(kSolveThreads) k_refine_check(MixedBatch b, int step) {
+    grid_dependency();
     __shared__ dfl red[kSolveThreads / 32];
     const int t = blockIdx.x;
     InstState* st = b.st + t;
@@ -1263,6 +1275,7 @@ __global__ void __launch_bounds__(kSolveThreads) k_refine_check(MixedBatch b, in
 // unit of the split factorisation (2^-40 at 5 slices).
 __global__ void k_df_finalize(MixedBatch b, double* nll, double* mu, double* sigma2, double* logdet,
                               int* status) {
+    grid_dependency();
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= b.count) return;
     const InstState st = b.st[t];
@@ -1334,27 +1347,27 @@ cudaError_t launch_diag_mixed(const MixedBatch& b, int J, cudaStream_t s) {
     static std::atomic<size_t> attr[kMaxDevices];
     cudaError_t e = raise_smem_limit(k_diag_mixed, smem, attr);
     if (e != cudaSuccess) return e;
-    k_diag_mixed<<<b.count, kDiagThreads, smem, s>>>(b, J);
+    launch_chained(ahead_mixed(b), k_diag_mixed, b.count, kDiagThreads, smem, s, b, J);
     return cudaGetLastError();
 }
 
 cudaError_t launch_split_panel(const MixedBatch& b, int J, int ns, int gemv, cudaStream_t s) {
     const int m = b.nt - J - 1;
     if (m <= 0) return cudaSuccess;
-    k_split_panel<<<dim3(2 * m, b.count), kSplitThreads, 0, s>>>(b, J, ns, gemv);
+    launch_chained(gemv && ahead_mixed(b), k_split_panel, dim3(2 * m, b.count), kSplitThreads, 0, s, b, J, ns, gemv);
     return cudaGetLastError();
 }
 
 cudaError_t launch_split_fused(const MixedBatch& b, int J, cudaStream_t s) {
     const int m = b.nt - J - 2;
     if (m <= 0) return cudaSuccess;
-    k_split_fused<<<dim3(4 * m, b.count), kSplitThreads, 0, s>>>(b, J);
+    launch_chained(ahead_mixed(b), k_split_fused, dim3(4 * m, b.count), kSplitThreads, 0, s, b, J);
     return cudaGetLastError();
 }
 
 cudaError_t launch_rhs_init(const MixedBatch& b, cudaStream_t s) {
     const int npad = b.nt * GP_NB;
-    k_rhs_init<<<dim3((npad + 255) / 256, b.count), 256, 0, s>>>(b);
+    launch_chained(ahead_mixed(b), k_rhs_init, dim3((npad + 255) / 256, b.count), 256, 0, s, b);
     return cudaGetLastError();
 }
 
@@ -1366,9 +1379,9 @@ cudaError_t launch_df_forward(const MixedBatch& b, int c0, int init, cudaStream_
     }
     cudaError_t e = cudaMemsetAsync(b.SC, 0, (size_t)b.count * b.sc_stride * sizeof(int), s);
     if (e != cudaSuccess) return e;
-    k_fwd_diag<<<b.count, kSubThreads, 0, s>>>(b, c0, 0);
+    launch_chained(ahead_mixed(b), k_fwd_diag, b.count, kSubThreads, 0, s, b, c0, 0);
     for (int J = 0; J + 1 < b.nt; ++J)
-        k_fwd_tiles<<<dim3(2 * (b.nt - 1 - J), b.count), kSubThreads, 0, s>>>(b, c0, J);
+        launch_chained(ahead_mixed(b), k_fwd_tiles, dim3(2 * (b.nt - 1 - J), b.count), kSubThreads, 0, s, b, c0, J);
     return cudaGetLastError();
 }
 
@@ -1379,9 +1392,9 @@ cudaError_t launch_df_backward(const MixedBatch& b, int c0, int add_to, cudaStre
     if (e != cudaSuccess) return e;
     e = cudaMemsetAsync(b.SC, 0, (size_t)b.count * b.sc_stride * sizeof(int), s);
     if (e != cudaSuccess) return e;
-    k_bwd_diag<<<b.count, kSubThreads, 0, s>>>(b, c0, b.nt - 1, add_to);
+    launch_chained(ahead_mixed(b), k_bwd_diag, b.count, kSubThreads, 0, s, b, c0, b.nt - 1, add_to);
     for (int K = b.nt - 1; K > 0; --K)
-        k_bwd_tiles<<<dim3(2 * K, b.count), kSubThreads, smem, s>>>(b, c0, K, add_to);
+        launch_chained(ahead_mixed(b), k_bwd_tiles, dim3(2 * K, b.count), kSubThreads, smem, s, b, c0, K, add_to);
     return cudaGetLastError();
 }
 
@@ -1390,14 +1403,16 @@ cudaError_t launch_df_residual(const MixedBatch& b, cudaStream_t s) {
     static std::atomic<size_t> attr[kMaxDevices];
     cudaError_t e = raise_smem_limit(k_resid_tiles, smem, attr);
     if (e != cudaSuccess) return e;
-    k_resid_tiles<<<dim3(2 * (unsigned)packed_tiles(b.nt), b.count), kResThreads, smem, s>>>(b);
-    k_resid_reduce<<<dim3(b.nt, b.count), kResThreads, 0, s>>>(b);
+    launch_chained(ahead_mixed(b), k_resid_tiles, dim3(2 * (unsigned)packed_tiles(b.nt), b.count), kResThreads,
+                   smem, s, b);
+    launch_chained(ahead_mixed(b), k_resid_reduce, dim3(b.nt, b.count), kResThreads, 0, s, b);
     return cudaGetLastError();
 }
 
 cudaError_t launch_df_finalize(const MixedBatch& b, double* nll, double* mu, double* sigma2, double* logdet,
                                int* status, cudaStream_t s) {
-    k_df_finalize<<<(b.count + 127) / 128, 128, 0, s>>>(b, nll, mu, sigma2, logdet, status);
+    launch_chained(ahead_mixed(b), k_df_finalize, (b.count + 127) / 128, 128, 0, s, b, nll, mu, sigma2, logdet,
+                   status);
     return cudaGetLastError();
 }
 
@@ -1409,12 +1424,12 @@ cudaError_t launch_split_model(const MixedBatch& v, float2* Zm, double* scalars,
 
 cudaError_t launch_keep_forward(const MixedBatch& b, cudaStream_t s) {
     const int npad = b.nt * GP_NB;
-    k_keep_forward<<<dim3((2 * npad + 255) / 256, b.count), 256, 0, s>>>(b);
+    launch_chained(ahead_mixed(b), k_keep_forward, dim3((2 * npad + 255) / 256, b.count), 256, 0, s, b);
     return cudaGetLastError();
 }
 
 cudaError_t launch_refine_check(const MixedBatch& b, int step, cudaStream_t s) {
-    k_refine_check<<<b.count, kSolveThreads, 0, s>>>(b, step);
+    launch_chained(ahead_mixed(b), k_refine_check, b.count, kSolveThreads, 0, s, b, step);
     return cudaGetLastError();
 }
 

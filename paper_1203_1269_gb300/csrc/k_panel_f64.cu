@@ -177,6 +177,7 @@ __device__ __forceinline__ void diag32_columns(double (&a)[kB / kWarps], double 
 
 template <bool IEEE>
 __global__ void __launch_bounds__(kThreads) k_diag32_f64(Batch b, int J, int s) {
+    grid_dependency();
     __shared__ double Ls[kB][kLsCols];             // Ls[c][r]
     __shared__ int failed;
     const int t = blockIdx.x;
@@ -217,6 +218,7 @@ __global__ void __launch_bounds__(kThreads) k_diag32_f64(Batch b, int J, int s) 
 // where the rows do not fill the schedulers.
 template <int LANES>
 __global__ void __launch_bounds__(kThreads) k_solve32_f64(Batch b, int J, int s, int units, int per_warp) {
+    grid_dependency();
     constexpr int kRows = 32 / LANES, kCols = kB / LANES;
     __shared__ double Ls[kB][kB + 1];
     __shared__ double inv[kB];
@@ -277,7 +279,8 @@ void launch_solve32(const Batch& b, int J, int s, int rows, int sms, cudaStream_
     const long long warps = (long long)sms * 8;              // two CTAs an SM
     const int per_warp = (int)(((long long)units * b.count + warps - 1) / warps);
     const int grid = (units + kWarps * per_warp - 1) / (kWarps * per_warp);
-    k_solve32_f64<LANES><<<dim3(grid, b.count), kThreads, 0, st>>>(b, J, s, units, per_warp);
+    launch_chained(ahead_f64(b), k_solve32_f64<LANES>, dim3(grid, b.count), kThreads, 0, st, b, J, s, units,
+                   per_warp);
 }
 
 // Up to two block columns: the products of sub-block s for the columns of block
@@ -288,6 +291,7 @@ constexpr int kInnerThreads = 256;
 constexpr int kInnerCols = kB * kB / kInnerThreads;
 
 __global__ void __launch_bounds__(kInnerThreads) k_inner_f64(Batch b, int J, int s) {
+    grid_dependency();
     __shared__ double Lk[kB][kB + 1];              // Lk[c][k]
     const int t = blockIdx.z;
     if (b.st[t].status != GP_OK) return;
@@ -316,6 +320,7 @@ __global__ void __launch_bounds__(kInnerThreads) k_inner_f64(Batch b, int J, int
 // Tile (1, 1) less L_10 L_10^T: sums from zero over the 128 columns in order, then
 // one subtraction, a CTA per 32 x 32 block of the lower triangle.
 __global__ void __launch_bounds__(kInnerThreads) k_trailing_f64(Batch b) {
+    grid_dependency();
     __shared__ double Lk[GP_NB][kB + 1];
     const int t = blockIdx.y;
     if (b.st[t].status != GP_OK) return;
@@ -343,6 +348,7 @@ __global__ void __launch_bounds__(kInnerThreads) k_trailing_f64(Batch b) {
 // log|R| of up to two block columns: the pivots' logarithms summed in column
 // order per block, the blocks' sums in turn.
 __global__ void __launch_bounds__(GP_NB) k_logdet_small_f64(Batch b) {
+    grid_dependency();
     __shared__ double logs[GP_NB];
     const int t = blockIdx.x;
     if (b.st[t].status != GP_OK) return;
@@ -393,7 +399,7 @@ cudaError_t launch_factor_small_f64(const Batch& b, cudaStream_t st, int* kernel
     for (int J = 0; J < b.nt; ++J) {
         const int left = b.n - J * GP_NB;                    // real rows from block column J on
         for (int s = 0; s < GP_NB / kB && kB * s < left; ++s) {
-            k_diag32_f64<true><<<b.count, kThreads, 0, st>>>(b, J, s);
+            launch_chained(ahead_f64(b), k_diag32_f64<true>, b.count, kThreads, 0, st, b, J, s);
             ++k;
             const int rows = (left - kB * (s + 1) + 7) / 8 * 8;
             if (rows <= 0) continue;
@@ -402,17 +408,19 @@ cudaError_t launch_factor_small_f64(const Batch& b, cudaStream_t st, int* kernel
             ++k;
             const int cols = GP_NB / kB - 1 - s, groups = (left + kB - 1) / kB - 1 - s;
             if (cols > 0 && groups > 0) {
-                k_inner_f64<<<dim3(groups, cols < groups ? cols : groups, b.count), kInnerThreads, 0, st>>>(b, J, s);
+                launch_chained(ahead_f64(b), k_inner_f64, dim3(groups, cols < groups ? cols : groups, b.count),
+                               kInnerThreads, 0, st, b, J, s);
                 ++k;
             }
         }
         if (J + 1 < b.nt) {
             const int groups = (left - GP_NB + kB - 1) / kB;
-            k_trailing_f64<<<dim3(groups * (groups + 1) / 2, b.count), kInnerThreads, 0, st>>>(b);
+            launch_chained(ahead_f64(b), k_trailing_f64, dim3(groups * (groups + 1) / 2, b.count),
+                           kInnerThreads, 0, st, b);
             ++k;
         }
     }
-    k_logdet_small_f64<<<b.count, GP_NB, 0, st>>>(b);
+    launch_chained(ahead_f64(b), k_logdet_small_f64, b.count, GP_NB, 0, st, b);
     if (kernels) *kernels = k + 1;
     return cudaGetLastError();
 }
@@ -427,7 +435,7 @@ cudaError_t launch_panel_f64(const Batch& b, int J, cudaStream_t st) {
             cudaError_t e = launch_update_f64_inner(b, J, s, st);
             if (e != cudaSuccess) return e;
         }
-        k_diag32_f64<false><<<b.count, kThreads, 0, st>>>(b, J, s);
+        launch_chained(s > 0 && ahead_f64(b), k_diag32_f64<false>, b.count, kThreads, 0, st, b, J, s);
         const int rows = (b.nt - J) * GP_NB - kB * (s + 1);
         if (rows > 0) {
             if ((long long)rows * b.count <= 4 * 4LL * sms) launch_solve32<8>(b, J, s, rows, sms, st);

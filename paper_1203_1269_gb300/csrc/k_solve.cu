@@ -75,6 +75,7 @@ __device__ __forceinline__ void stage_diag(const double* L, double* D) {
 
 // Z <- [1 Y] (padded rows zero), the forward solve's right-hand sides
 __global__ void k_rhs_f64(Batch b, double* Z, size_t zs) {
+    grid_dependency();
     const int npad = b.nt * GP_NB;
     double* z0 = Z + (size_t)blockIdx.y * zs;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < npad; i += gridDim.x * blockDim.x) {
@@ -89,6 +90,7 @@ __global__ void k_rhs_f64(Batch b, double* Z, size_t zs) {
 // tiles left of it; L_JJ z = Z_J by columns, x_c = v_c (1 / L_cc), then
 // v_r -= L_rc x_c for r > c, in the order of c.
 __global__ void __launch_bounds__(2 * GP_NB) k_fwd_diag_f64(Batch b, double* Z, size_t zs, int J) {
+    grid_dependency();
     extern __shared__ double D[];
     __shared__ double xc[2][GP_NB];
     __shared__ double inv[GP_NB];
@@ -129,6 +131,7 @@ __global__ void __launch_bounds__(2 * GP_NB) k_fwd_diag_f64(Batch b, double* Z, 
 // columns 16 g .. 16 g + 15 of row r): Z_I -= L_IJ z_J, the 8 column parts
 // added in order.
 __global__ void __launch_bounds__(kFwdTileThreads) k_fwd_tiles_f64(Batch b, double* Z, size_t zs, int J) {
+    grid_dependency();
     constexpr int kRows = GP_NB / kTileSplit;
     __shared__ double xs[2][GP_NB];
     __shared__ double part[8][2][kRows];
@@ -167,6 +170,7 @@ __global__ void __launch_bounds__(kFwdTileThreads) k_fwd_tiles_f64(Batch b, doub
 // Z_I from the last column back, x_c = v_c (1 / L_cc), then v_r -= L_cr x_c for
 // r < c.
 __global__ void __launch_bounds__(GP_NB) k_bwd_diag_f64(Batch b, double* Z, size_t zs, int col, int I) {
+    grid_dependency();
     extern __shared__ double D[];
     __shared__ double xc[GP_NB];
     __shared__ double inv[GP_NB];
@@ -207,6 +211,7 @@ __global__ void __launch_bounds__(GP_NB) k_bwd_diag_f64(Batch b, double* Z, size
 // Backward, tiles (I, K), K < I, a CTA for 32 columns each (one per warp, lane
 // l rows l, l + 32, l + 64, l + 96, then a shuffle sum): Z_K -= L_IK^T w_I.
 __global__ void __launch_bounds__(kBwdTileThreads) k_bwd_tiles_f64(Batch b, double* Z, size_t zs, int col, int I) {
+    grid_dependency();
     __shared__ double ws[GP_NB];
     const int t = blockIdx.y;
     if (b.st[t].status != GP_OK) return;
@@ -229,6 +234,7 @@ __global__ void __launch_bounds__(kBwdTileThreads) k_bwd_tiles_f64(Batch b, doub
 __global__ void __launch_bounds__(kThreads) k_finalize(Batch b, const double* Z, size_t zs,
                                                        double* nll, double* mu, double* sigma2,
                                                        double* logdet, int* status) {
+    grid_dependency();
     __shared__ double red[kThreads / 32];
     const int t = blockIdx.x;
     InstState st = b.st[t];
@@ -282,6 +288,7 @@ __global__ void __launch_bounds__(kThreads) k_finalize(Batch b, const double* Z,
 // becomes e = b - mu_hat a = L^-1 (Y - 1 mu_hat), ready for the backward
 // solve that gives the kriging weights w = R^-1 (Y - 1 mu_hat).
 __global__ void k_fit_finish(Batch b, double* Z, size_t zs, double* scalars) {
+    grid_dependency();
     const int t = blockIdx.x;
     const InstState st = b.st[t];
     if (st.status != GP_OK) return;
@@ -298,7 +305,7 @@ __global__ void k_fit_finish(Batch b, double* Z, size_t zs, double* scalars) {
 }  // namespace
 
 cudaError_t launch_fit_finish(const Batch& b, double* Z, size_t zs, double* scalars, cudaStream_t s) {
-    k_fit_finish<<<b.count, kThreads, 0, s>>>(b, Z, zs, scalars);
+    launch_chained(ahead_f64(b), k_fit_finish, b.count, kThreads, 0, s, b, Z, zs, scalars);
     return cudaGetLastError();
 }
 
@@ -309,10 +316,13 @@ cudaError_t launch_forward_solve(const Batch& b, double* Z, size_t zs, cudaStrea
     cudaError_t e = raise_smem_limit(k_fwd_diag_f64, kDiagSmem, attr);
     if (e != cudaSuccess) return e;
     const int nt = b.nt;
-    k_rhs_f64<<<dim3((nt * GP_NB + kThreads - 1) / kThreads, b.count), kThreads, 0, s>>>(b, Z, zs);
+    launch_chained(ahead_f64(b), k_rhs_f64, dim3((nt * GP_NB + kThreads - 1) / kThreads, b.count), kThreads, 0,
+                   s, b, Z, zs);
     for (int J = 0; J < nt; ++J) {
-        k_fwd_diag_f64<<<b.count, 2 * GP_NB, kDiagSmem, s>>>(b, Z, zs, J);
-        if (J + 1 < nt) k_fwd_tiles_f64<<<dim3(kTileSplit * (nt - 1 - J), b.count), kFwdTileThreads, 0, s>>>(b, Z, zs, J);
+        launch_chained(ahead_f64(b), k_fwd_diag_f64, b.count, 2 * GP_NB, kDiagSmem, s, b, Z, zs, J);
+        if (J + 1 < nt)
+            launch_chained(ahead_f64(b), k_fwd_tiles_f64, dim3(kTileSplit * (nt - 1 - J), b.count),
+                           kFwdTileThreads, 0, s, b, Z, zs, J);
     }
     return cudaGetLastError();
 }
@@ -322,15 +332,17 @@ cudaError_t launch_backward_solve(const Batch& b, double* Z, size_t zs, int col,
     cudaError_t e = raise_smem_limit(k_bwd_diag_f64, kDiagSmem, attr);
     if (e != cudaSuccess) return e;
     for (int I = b.nt - 1; I >= 0; --I) {
-        k_bwd_diag_f64<<<b.count, GP_NB, kDiagSmem, s>>>(b, Z, zs, col, I);
-        if (I > 0) k_bwd_tiles_f64<<<dim3(kTileSplit * I, b.count), kBwdTileThreads, 0, s>>>(b, Z, zs, col, I);
+        launch_chained(ahead_f64(b), k_bwd_diag_f64, b.count, GP_NB, kDiagSmem, s, b, Z, zs, col, I);
+        if (I > 0)
+            launch_chained(ahead_f64(b), k_bwd_tiles_f64, dim3(kTileSplit * I, b.count), kBwdTileThreads, 0, s,
+                           b, Z, zs, col, I);
     }
     return cudaGetLastError();
 }
 
 cudaError_t launch_finalize(const Batch& b, const double* Z, size_t zs, double* nll, double* mu,
                             double* sigma2, double* logdet, int* status, cudaStream_t s) {
-    k_finalize<<<b.count, kThreads, 0, s>>>(b, Z, zs, nll, mu, sigma2, logdet, status);
+    launch_chained(ahead_f64(b), k_finalize, b.count, kThreads, 0, s, b, Z, zs, nll, mu, sigma2, logdet, status);
     return cudaGetLastError();
 }
 

@@ -185,6 +185,7 @@ enum : int { kFactorMode = 0, kInnerMode = 1, kInvApply = 2, kInvUpdate = 3 };
 template <int kNT, int MODE>
 __global__ void __launch_bounds__(kThreads, 1)
     k_update_f64_tc(Batch b, int J, int which, int per_inst, int chunks, double* X, double* S) {
+    grid_dependency();
     constexpr bool kInner = MODE == kInnerMode;
     constexpr bool kInv = MODE == kInvApply || MODE == kInvUpdate;
     constexpr uint32_t kBChunk = b_chunk(kNT), kStageBytes = stage_bytes(kNT);
@@ -476,7 +477,8 @@ cudaError_t launch(const Batch& b, int J, cudaStream_t s, int which, int per_ins
     // 38.5, 37.3 and 44.2 ms)
     const int cap = which == kUpdateRest ? device_sms() - device_sms() / 3 : device_sms();
     const int grid = (int)(total < cap ? total : cap);
-    k_update_f64_tc<NT, MODE><<<grid, kThreads, smem, s>>>(b, J, which, per_inst, chunks, X, S);
+    launch_chained(which != kUpdateColumn && ahead_f64(b), k_update_f64_tc<NT, MODE>, grid, kThreads, smem, s, b, J,
+                   which, per_inst, chunks, X, S);
     return cudaGetLastError();
 }
 
