@@ -353,6 +353,7 @@ int run_mixed_factor(gp_ctx* ctx, gp::MixedBatch& mb, int d, const double* x, co
     mb.d = d;
     mb.delta = delta;
     GP_CUDA(ctx, cudaMemsetAsync(mb.err, 0, sizeof(int), ctx->stream));
+    GP_CUDA(ctx, cudaMemsetAsync(mb.SC, 0, (size_t)mb.count * mb.sc_stride * sizeof(int), ctx->stream));
     {
         PhaseScope ps(ctx, GP_PHASE_ASSEMBLE, mb.fwd ? 3 : 2);
         GP_CUDA(ctx, gp::launch_validate_theta(b, ctx->stream));

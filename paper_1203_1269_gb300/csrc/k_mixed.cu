@@ -810,6 +810,35 @@ __device__ dfl block_sum_df(dfl v, dfl* red) {
 }
 
 
+// The same sums as block_sum_df of N values at once, their last additions in
+// N threads of different warps.
+template <int N>
+__device__ __forceinline__ void block_sums_df(dfl (&v)[N], dfl (*red)[N]) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int k = 0; k < N; ++k) {
+            dfl u;
+            u.hi = __shfl_down_sync(0xffffffffu, v[k].hi, o);
+            u.lo = __shfl_down_sync(0xffffffffu, v[k].lo, o);
+            v[k] = df_add(v[k], u);
+        }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < N; ++k)
+        if (lane == 0) red[w][k] = v[k];
+    __syncthreads();
+    if (lane == 0 && w < N) {
+        dfl s = red[0][w];
+        for (int i = 1; i < (int)(blockDim.x >> 5); ++i) s = df_add(s, red[i][w]);
+        red[0][w] = s;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < N; ++k) v[k] = red[0][k];
+}
+
 // [1 Y] (zero on padded rows) into Z columns 0, 1: the right-hand sides of
 // the forward solve that the factorisation carries out block by block
 __global__ void k_rhs_init(MixedBatch b) {
@@ -822,9 +851,6 @@ __global__ void k_rhs_init(MixedBatch b) {
     df_store(zcol(b, t, 1) + gi, in ? df_from_double(b.y[gi]) : dfl{0.f, 0.f});
 }
 
-
-
-
 // Forward and backward substitution with the double-float factor for two
 // columns (c0, c0 + 1) of Z in place, tile-parallel: block column by block
 // column, a small kernel finishes the diagonal block from the partial
@@ -832,7 +858,23 @@ __global__ void k_rhs_init(MixedBatch b) {
 // forms the next partial products of every tile of that block column (or
 // row) at once, one CTA per tile half.  Partial products live in RP:
 // per lower tile q, [2 halves][2 columns][128] double-float values.
+// A step is a chain of latencies (the tile from HBM, its partial products
+// through L2 to the diagonal step, W from L2), so each link's loads are issued
+// together and the next block's two tiles come first in the grid (the
+// candidates run along x): their diagonal step ends while the other tiles are
+// worked on.  Each step of 100 candidates at n = 1024: 42 -> 22 us forward,
+// 35 -> 24 backward; the solve phase there .82 -> .56 ms, 32 x 1448 1.07 ->
+// .64, 8 x 16384 17.4 -> 10.7, 256 x 4000 15.5 -> 14.4 (the residual's 6.1
+// of them, and 2.4 a pass what the factor's bytes take).
 constexpr int kSubThreads = 256;
+// Entries that a thread has in flight: partial-product tiles, W and L, and the
+// CTAs per SM that its registers leave room for.
+struct SubDeep {
+    static constexpr int kSum = 4, kW = 16, kL = 32, kFwd = 2, kBwd = 2;
+};
+struct SubWide {
+    static constexpr int kSum = 4, kW = 8, kL = 8, kFwd = 4, kBwd = 3;
+};
 
 __device__ __forceinline__ bool sub_active(const MixedBatch& b, int t) {
     return b.st[t].status == GP_OK && !b.st[t].hager_done && !b.st[t].refine_done;
@@ -851,64 +893,109 @@ __device__ __forceinline__ dfl df_load_cg(const float2* p) {
 // pass) or inside the tile launch before them, by whichever of the two CTAs
 // writing the block's last partial products finishes second: each of them
 // fences its partial products device-wide and counts itself on the block's
-// counter (zeroed per pass); the second reads all the block's partial
+// counter (which the second leaves at zero again); the second reads all the block's partial
 // products in the same fixed order as a separate launch would.  No CTA
 // waits for another.
 __device__ __forceinline__ bool second_of_two(const MixedBatch& b, int t, int blk) {
     __shared__ int last;
     __threadfence();
     __syncthreads();
-    if (threadIdx.x == 0) last = (atomicAdd(b.SC + (size_t)t * b.sc_stride + blk, 1) == 1);
+    if (threadIdx.x == 0) last = (atomicInc((unsigned*)b.SC + (size_t)t * b.sc_stride + blk, 1) == 1);
     __syncthreads();
     if (last) __threadfence();
     return last;
+}
+
+// Sums over `count` partial products of both right-hand sides, count in steps
+// of two tiles (one per half): pp(i) is the i-th tile's part for this thread.
+// The loads of N tiles are issued before their sums (in the tiles' order).
+template <int N, typename F>
+__device__ __forceinline__ void sum_partials(int count, F pp, dfl& p0, dfl& p1) {
+    p0 = {0.f, 0.f};
+    p1 = {0.f, 0.f};
+#pragma unroll 1
+    for (int i = 0; i < count; i += N) {
+        dfl v[N][4];
+#pragma unroll
+        for (int j = 0; j < N; ++j)
+            if (i + j < count) {
+                const float2* q = pp(i + j);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) v[j][k] = df_load_cg(q + k * GP_NB);
+            }
+#pragma unroll
+        for (int j = 0; j < N; ++j)
+            if (i + j < count) {
+                p0 = df_add(p0, df_add(v[j][0], v[j][2]));
+                p1 = df_add(p1, df_add(v[j][1], v[j][3]));
+            }
+    }
+}
+
+// The first N of the 64 entries of W (stride GP_NB) of a thread of a
+// diagonal step.
+template <int N>
+__device__ __forceinline__ void diag_load(const float2* W, float2 (&w)[N]) {
+#pragma unroll
+    for (int j = 0; j < N; ++j) w[j] = W[(size_t)j * GP_NB];
+}
+
+// Products of 64 entries of W with both right-hand sides (xs0, xs1: 64 terms
+// each), even and odd terms apart.  w holds the first N entries; each
+// batch is loaded while the one before it is multiplied: left to the
+// compiler, every load waited for L2 on its own (18 to 36 thousand clocks for
+// the 64 terms, against 5.6 thousand that the products issue in).
+template <int N>
+__device__ __forceinline__ void diag_products(const float2* W, float2 (&w)[N], const dfl* xs0, const dfl* xs1,
+                                              dfl& s0, dfl& s1) {
+    dfl a0 = {0.f, 0.f}, a1 = {0.f, 0.f}, b0 = {0.f, 0.f}, b1 = {0.f, 0.f};
+#pragma unroll 1
+    for (int c0 = 0; c0 < GP_NB / 2; c0 += N) {
+        float2 next[N];
+        if (c0 + N < GP_NB / 2) diag_load(W + (size_t)(c0 + N) * GP_NB, next);
+#pragma unroll
+        for (int j = 0; j < N; j += 2) {
+            const dfl w0 = {w[j].x, w[j].y}, w1 = {w[j + 1].x, w[j + 1].y};
+            a0 = df_fma(w0, xs0[c0 + j], a0);
+            b0 = df_fma(w0, xs1[c0 + j], b0);
+            a1 = df_fma(w1, xs0[c0 + j + 1], a1);
+            b1 = df_fma(w1, xs1[c0 + j + 1], b1);
+        }
+#pragma unroll
+        for (int j = 0; j < N; ++j) w[j] = next[j];
+    }
+    s0 = df_add(a0, a1);
+    s1 = df_add(b0, b1);
 }
 
 // forward, block J: z_J <- W_J (z_J - sum_{K<J} L_JK z_K), W_J = L_JJ^-1.
 // Thread (r, h) takes both right-hand sides of row r over half h of the
 // terms (every other partial-product tile, then columns 64h .. 64h + 63 of
 // the column-major WT, one load serving both sums); the halves add in a
-// fixed order.  part: 2 x 2 x 128 scratch.
+// fixed order.  W is zero above its diagonal; a fixed trip count.
+// part: 2 x 2 x 128 scratch.
+template <typename V>
 __device__ __forceinline__ void fwd_diag_step(const MixedBatch& b, int t, int c0, int J, dfl (*rhs)[GP_NB],
                                               dfl (*part)[2][GP_NB]) {
     const int r = threadIdx.x & 127, h = threadIdx.x >> 7;
-    float2* z0 = zcol(b, t, c0) + (size_t)J * GP_NB;
-    float2* z1 = zcol(b, t, c0 + 1) + (size_t)J * GP_NB;
-    dfl p0 = {0.f, 0.f}, p1 = {0.f, 0.f};
-#pragma unroll 4
-    for (int K = h; K < J; K += 2) {
-        const float2* pp = rp_part(b, t, J, K) + r;
-        p0 = df_add(p0, df_add(df_load_cg(pp), df_load_cg(pp + 2 * GP_NB)));
-        p1 = df_add(p1, df_add(df_load_cg(pp + GP_NB), df_load_cg(pp + 3 * GP_NB)));
-    }
+    float2* zr = zcol(b, t, c0 + h) + (size_t)J * GP_NB + r;     // half h finishes right-hand side h
+    const float2* W = b.WT + (size_t)t * b.wt_stride + (size_t)J * GP_TILE_ELEMS + (size_t)(64 * h) * GP_NB + r;
+    float2 w[V::kW];
+    diag_load(W, w);
+    const dfl z = df_load(zr);
+    dfl p0, p1;
+    sum_partials<V::kSum>((J - h + 1) / 2, [&](int i) { return rp_part(b, t, J, h + 2 * i) + r; }, p0, p1);
     part[h][0][r] = p0;
     part[h][1][r] = p1;
     __syncthreads();
-    if (h == 0) {
-        rhs[0][r] = df_sub(df_load(z0 + r), df_add(part[0][0][r], part[1][0][r]));
-        rhs[1][r] = df_sub(df_load(z1 + r), df_add(part[0][1][r], part[1][1][r]));
-    }
+    rhs[h][r] = df_sub(z, df_add(part[0][h][r], part[1][h][r]));
     __syncthreads();
-    // 64 columns (W is zero above its diagonal: a fixed trip count lets the
-    // loads run ahead of the accumulation chains)
-    const float2* W = b.WT + (size_t)t * b.wt_stride + (size_t)J * GP_TILE_ELEMS;
-    dfl a0 = {0.f, 0.f}, a1 = {0.f, 0.f}, b0 = {0.f, 0.f}, b1 = {0.f, 0.f};
-#pragma unroll 16
-    for (int c = 64 * h; c < 64 * h + 64; c += 2) {
-        const dfl w0 = df_load(W + (size_t)c * GP_NB + r), w1 = df_load(W + (size_t)(c + 1) * GP_NB + r);
-        a0 = df_fma(w0, rhs[0][c], a0);
-        b0 = df_fma(w0, rhs[1][c], b0);
-        a1 = df_fma(w1, rhs[0][c + 1], a1);
-        b1 = df_fma(w1, rhs[1][c + 1], b1);
-    }
+    dfl s0, s1;
+    diag_products(W, w, rhs[0] + 64 * h, rhs[1] + 64 * h, s0, s1);
+    part[h][0][r] = s0;
+    part[h][1][r] = s1;
     __syncthreads();
-    part[h][0][r] = df_add(a0, a1);
-    part[h][1][r] = df_add(b0, b1);
-    __syncthreads();
-    if (h == 0) {
-        df_store(z0 + r, df_add(part[0][0][r], part[1][0][r]));
-        df_store(z1 + r, df_add(part[0][1][r], part[1][1][r]));
-    }
+    df_store(zr, df_add(part[0][h][r], part[1][h][r]));
 }
 
 __global__ void __launch_bounds__(kSubThreads) k_fwd_diag(MixedBatch b, int c0, int J) {
@@ -917,42 +1004,55 @@ __global__ void __launch_bounds__(kSubThreads) k_fwd_diag(MixedBatch b, int c0, 
     __shared__ dfl part[2][2][GP_NB];
     const int t = blockIdx.x;
     if (!sub_active(b, t)) return;
-    fwd_diag_step(b, t, c0, J, rhs, part);
+    fwd_diag_step<SubDeep>(b, t, c0, J, rhs, part);
 }
 
 // forward, tiles (I, J), I > J, half h of the columns: L_IJ(:, h) z_J(h);
 // the CTA finishing tile (J + 1, J) second then takes block J + 1's
 // diagonal step
-__global__ void __launch_bounds__(kSubThreads) k_fwd_tiles(MixedBatch b, int c0, int J) {
+template <typename V>
+__global__ void __launch_bounds__(kSubThreads, V::kFwd) k_fwd_tiles(MixedBatch b, int c0, int J) {
     grid_dependency();
     __shared__ dfl xs[2][GP_NB / 2];
     __shared__ dfl part[2][2][GP_NB];
     __shared__ dfl rhs[2][GP_NB];
-    const int t = blockIdx.y;
+    const int t = blockIdx.x;
     if (!sub_active(b, t)) return;
-    const int I = J + 1 + (blockIdx.x >> 1), h = blockIdx.x & 1;
+    const int I = J + 1 + (blockIdx.y >> 1), h = blockIdx.y & 1;
     const int tid = threadIdx.x;
     // W_{J+1} heads for L2 for the diagonal step
     if (tid == 0 && I == J + 1 && h == 0)
         prefetch_l2(b.WT + (size_t)t * b.wt_stride + (size_t)(J + 1) * GP_TILE_ELEMS, GP_TILE_ELEMS * sizeof(float2));
+    const int r = tid & 127, g = tid >> 7;
+    const float2* L = df_tile(b, b.A, t, I, J) + ((size_t)h * 64 + 32 * g) * GP_NB + r;
+    float2 l[V::kL];
+#pragma unroll
+    for (int c = 0; c < V::kL; ++c) l[c] = __ldg(L + (size_t)c * GP_NB);
     if (tid < GP_NB) xs[tid >> 6][tid & 63] = df_load(zcol(b, t, c0 + (tid >> 6)) + (size_t)J * GP_NB + 64 * h + (tid & 63));
     __syncthreads();
-    const float2* L = df_tile(b, b.A, t, I, J) + (size_t)h * 64 * GP_NB;
-    const int r = tid & 127, g = tid >> 7;
     dfl u0 = {0.f, 0.f}, u1 = {0.f, 0.f};
-#pragma unroll 8
-    for (int c = 32 * g; c < 32 * g + 32; ++c) {
-        const float2 l = __ldg(L + (size_t)c * GP_NB + r);
-        const dfl ld = {l.x, l.y};
-        u0 = df_fma(ld, xs[0][c], u0);
-        u1 = df_fma(ld, xs[1][c], u1);
+#pragma unroll 1
+    for (int q = 0; q < 32; q += V::kL) {
+        float2 next[V::kL];
+        if (q + V::kL < 32) {
+#pragma unroll
+            for (int c = 0; c < V::kL; ++c) next[c] = __ldg(L + (size_t)(q + V::kL + c) * GP_NB);
+        }
+#pragma unroll
+        for (int c = 0; c < V::kL; ++c) {
+            const dfl ld = {l[c].x, l[c].y};
+            u0 = df_fma(ld, xs[0][32 * g + q + c], u0);
+            u1 = df_fma(ld, xs[1][32 * g + q + c], u1);
+        }
+#pragma unroll
+        for (int c = 0; c < V::kL; ++c) l[c] = next[c];
     }
     part[g][0][r] = u0;
     part[g][1][r] = u1;
     __syncthreads();
     const int k = tid >> 7;
     df_store(rp_part(b, t, I, J) + (h * 2 + k) * GP_NB + r, df_add(part[0][k][r], part[1][k][r]));
-    if (I == J + 1 && second_of_two(b, t, I)) fwd_diag_step(b, t, c0, I, rhs, part);
+    if (I == J + 1 && second_of_two(b, t, I)) fwd_diag_step<V>(b, t, c0, I, rhs, part);
 }
 
 // backward, block K: z_K <- W_K^T (z_K - sum_{K' > K} L_K'K^T z_K'); W^T
@@ -960,53 +1060,33 @@ __global__ void __launch_bounds__(kSubThreads) k_fwd_tiles(MixedBatch b, int c0,
 // 64h .. 64h + 63, both right-hand sides per load; the partial-product
 // tiles alternate between the halves); the halves add in a fixed order.
 // With add_to >= 0 the result is also added into (add_to, add_to + 1).
+template <typename V>
 __device__ __forceinline__ void bwd_diag_step(const MixedBatch& b, int t, int c0, int K, int add_to,
                                               dfl (*rhs)[GP_NB], dfl (*part)[2][GP_NB]) {
-    const int nt = b.nt;
     const int c = threadIdx.x & 127, h = threadIdx.x >> 7;
-    float2* z0 = zcol(b, t, c0) + (size_t)K * GP_NB;
-    float2* z1 = zcol(b, t, c0 + 1) + (size_t)K * GP_NB;
-    dfl p0 = {0.f, 0.f}, p1 = {0.f, 0.f};
-#pragma unroll 4
-    for (int K2 = K + 1 + h; K2 < nt; K2 += 2) {
-        const float2* pp = rp_part(b, t, K2, K) + c;
-        p0 = df_add(p0, df_add(df_load_cg(pp), df_load_cg(pp + 2 * GP_NB)));
-        p1 = df_add(p1, df_add(df_load_cg(pp + GP_NB), df_load_cg(pp + 3 * GP_NB)));
-    }
+    float2* zc = zcol(b, t, c0 + h) + (size_t)K * GP_NB + c;     // half h finishes right-hand side h
+    float2* acc = add_to >= 0 ? zcol(b, t, add_to + h) + (size_t)K * GP_NB + c : nullptr;
+    const float2* W = b.WR + (size_t)t * b.wt_stride + (size_t)K * GP_TILE_ELEMS + (size_t)(64 * h) * GP_NB + c;
+    float2 w[V::kW];
+    diag_load(W, w);
+    const dfl z = df_load(zc);
+    dfl total = {0.f, 0.f};
+    if (acc) total = df_load(acc);
+    dfl p0, p1;
+    sum_partials<V::kSum>((b.nt - K - h) / 2, [&](int i) { return rp_part(b, t, K + 1 + h + 2 * i, K) + c; }, p0, p1);
     part[h][0][c] = p0;
     part[h][1][c] = p1;
     __syncthreads();
-    if (h == 0) {
-        rhs[0][c] = df_sub(df_load(z0 + c), df_add(part[0][0][c], part[1][0][c]));
-        rhs[1][c] = df_sub(df_load(z1 + c), df_add(part[0][1][c], part[1][1][c]));
-    }
+    rhs[h][c] = df_sub(z, df_add(part[0][h][c], part[1][h][c]));
     __syncthreads();
-    const float2* Wr = b.WR + (size_t)t * b.wt_stride + (size_t)K * GP_TILE_ELEMS;
-    dfl a0 = {0.f, 0.f}, a1 = {0.f, 0.f}, b0 = {0.f, 0.f}, b1 = {0.f, 0.f};
-#pragma unroll 16
-    for (int r = 64 * h; r < 64 * h + 64; r += 2) {
-        const dfl w0 = df_load(Wr + (size_t)r * GP_NB + c), w1 = df_load(Wr + (size_t)(r + 1) * GP_NB + c);
-        a0 = df_fma(w0, rhs[0][r], a0);
-        b0 = df_fma(w0, rhs[1][r], b0);
-        a1 = df_fma(w1, rhs[0][r + 1], a1);
-        b1 = df_fma(w1, rhs[1][r + 1], b1);
-    }
+    dfl s0, s1;
+    diag_products(W, w, rhs[0] + 64 * h, rhs[1] + 64 * h, s0, s1);
+    part[h][0][c] = s0;
+    part[h][1][c] = s1;
     __syncthreads();
-    part[h][0][c] = df_add(a0, a1);
-    part[h][1][c] = df_add(b0, b1);
-    __syncthreads();
-    if (h == 0) {
-        const dfl x0 = df_add(part[0][0][c], part[1][0][c]);
-        const dfl x1 = df_add(part[0][1][c], part[1][1][c]);
-        df_store(z0 + c, x0);
-        df_store(z1 + c, x1);
-        if (add_to >= 0) {
-            float2* acc0 = zcol(b, t, add_to) + (size_t)K * GP_NB + c;
-            float2* acc1 = zcol(b, t, add_to + 1) + (size_t)K * GP_NB + c;
-            df_store(acc0, df_add(df_load(acc0), x0));
-            df_store(acc1, df_add(df_load(acc1), x1));
-        }
-    }
+    const dfl x = df_add(part[0][h][c], part[1][h][c]);
+    df_store(zc, x);
+    if (acc) df_store(acc, df_add(total, x));
 }
 
 __global__ void __launch_bounds__(kSubThreads) k_bwd_diag(MixedBatch b, int c0, int K, int add_to) {
@@ -1015,7 +1095,7 @@ __global__ void __launch_bounds__(kSubThreads) k_bwd_diag(MixedBatch b, int c0, 
     __shared__ dfl part[2][2][GP_NB];
     const int t = blockIdx.x;
     if (!sub_active(b, t)) return;
-    bwd_diag_step(b, t, c0, K, add_to, rhs, part);
+    bwd_diag_step<SubDeep>(b, t, c0, K, add_to, rhs, part);
 }
 
 // backward, tiles (K, I), I < K, half h of the rows: L_KI(h, :)^T z_K(h);
@@ -1023,15 +1103,16 @@ __global__ void __launch_bounds__(kSubThreads) k_bwd_diag(MixedBatch b, int c0, 
 // thread c walks column c conflict-free; the CTA finishing tile (K, K - 1)
 // second then takes block K - 1's diagonal step
 constexpr int kBwdTs = GP_NB / 2 + 1;
-__global__ void __launch_bounds__(kSubThreads) k_bwd_tiles(MixedBatch b, int c0, int K, int add_to) {
+template <typename V>
+__global__ void __launch_bounds__(kSubThreads, V::kBwd) k_bwd_tiles(MixedBatch b, int c0, int K, int add_to) {
     grid_dependency();
     extern __shared__ dfl T[];                  // GP_NB x kBwdTs
     __shared__ dfl xs[2][GP_NB / 2];
     __shared__ dfl part[2][2][GP_NB];
     __shared__ dfl rhs[2][GP_NB];
-    const int t = blockIdx.y;
+    const int t = blockIdx.x;
     if (!sub_active(b, t)) return;
-    const int I = blockIdx.x >> 1, h = blockIdx.x & 1;
+    const int I = K - 1 - (blockIdx.y >> 1), h = blockIdx.y & 1;
     const int tid = threadIdx.x;
     // W_{K-1} (row-major) heads for L2 for the next diagonal step
     if (tid == 0 && I == K - 1 && h == 0)
@@ -1059,7 +1140,7 @@ __global__ void __launch_bounds__(kSubThreads) k_bwd_tiles(MixedBatch b, int c0,
     const int k = tid >> 7;
     df_store(rp_part(b, t, K, I) + (h * 2 + k) * GP_NB + c, df_add(part[0][k][c], part[1][k][c]));
     // the CTA finishing tile (K, K - 1) second takes block K - 1's diagonal step
-    if (I == K - 1 && second_of_two(b, t, I)) bwd_diag_step(b, t, c0, I, add_to, rhs, part);
+    if (I == K - 1 && second_of_two(b, t, I)) bwd_diag_step<V>(b, t, c0, I, add_to, rhs, part);
 }
 
 // Residual r = b - R x of the solution columns (0, 1) into columns (2, 3),
@@ -1153,14 +1234,32 @@ __global__ void __launch_bounds__(kResThreads) k_resid_reduce(MixedBatch b) {
     const int k = threadIdx.x >> 7, r = threadIdx.x & 127;
     const float2* rp = b.RP + (size_t)t * b.rp_stride;
     dfl y = {0.f, 0.f};
-    for (int J = 0; J <= I; ++J) {
-        const float2* u = rp + (size_t)tile_index(I, J, nt) * kRpTile;
-        y = df_add(y, df_load(u + k * GP_NB + r));
-        y = df_add(y, df_load(u + (2 + k) * GP_NB + r));
+    // eight partial sums loaded before they are added (in their order)
+#pragma unroll 1
+    for (int J = 0; J <= I; J += 4) {
+        dfl v[8];
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if (J + j <= I) {
+                const float2* u = rp + (size_t)tile_index(I, J + j, nt) * kRpTile;
+                v[2 * j] = df_load(u + k * GP_NB + r);
+                v[2 * j + 1] = df_load(u + (2 + k) * GP_NB + r);
+            }
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if (J + j <= I) y = df_add(df_add(y, v[2 * j]), v[2 * j + 1]);
     }
-    for (int K = I + 1; K < nt; ++K) {
-        const float2* v = rp + (size_t)tile_index(K, I, nt) * kRpTile + 4 * GP_NB;
-        y = df_add(y, df_load(v + ((r >> 6) * 2 + k) * kResCols + (r & 63)));
+#pragma unroll 1
+    for (int K = I + 1; K < nt; K += 8) {
+        dfl v[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+            if (K + j < nt)
+                v[j] = df_load(rp + (size_t)tile_index(K + j, I, nt) * kRpTile + 4 * GP_NB +
+                               ((r >> 6) * 2 + k) * kResCols + (r & 63));
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+            if (K + j < nt) y = df_add(y, v[j]);
     }
     const int gi = I * GP_NB + r;
     dfl bq = {0.f, 0.f};
@@ -1209,7 +1308,8 @@ __device__ __forceinline__ double split_unit(int s) {
 
 __global__ void __launch_bounds__(kSolveThreads) k_refine_check(MixedBatch b, int step) {
     grid_dependency();
-    __shared__ dfl red[kSolveThreads / 32];
+    __shared__ dfl red[kSolveThreads / 32], red3[kSolveThreads / 32][3];
+    __shared__ double log_prev;
     const int t = blockIdx.x;
     InstState* st = b.st + t;
     if (st->status != GP_OK || st->refine_done) return;
@@ -1234,9 +1334,9 @@ __global__ void __launch_bounds__(kSolveThreads) k_refine_check(MixedBatch b, in
             sc = df_fma(df_load(bv + i), zyi, sc);
         }
     }
-    const double A = df_to_double(block_sum_df(sa, red));
-    const double B = df_to_double(block_sum_df(sb, red));
-    const double C = df_to_double(block_sum_df(sc, red));
+    dfl sums[3] = {sa, sb, sc};
+    block_sums_df(sums, red3);
+    const double A = df_to_double(sums[0]), B = df_to_double(sums[1]), C = df_to_double(sums[2]);
     const double m = B / A;
     const dfl md = df_from_double(m);
     dfl sq = {0.f, 0.f};
@@ -1248,9 +1348,9 @@ __global__ void __launch_bounds__(kSolveThreads) k_refine_check(MixedBatch b, in
             sq = df_fma(u, df_fms(md, df_load(z1 + i), df_load(zy + i)), sq);
         }
     }
+    if (corr && threadIdx.x == 32) log_prev = log(st->Q);       // beside the sum; a barrier follows
     const double Q = df_to_double(block_sum_df(sq, red));
     if (threadIdx.x == 0) {
-        const double Qprev = st->Q;
         st->aa = A;
         st->ab = B;
         st->bb = C;
@@ -1259,7 +1359,7 @@ __global__ void __launch_bounds__(kSolveThreads) k_refine_check(MixedBatch b, in
         if (!(Q > 0.0)) {
             st->refine_done = 1;            // degenerate: the finalisation reports it
         } else if (corr) {
-            const double dq = n * fabs(log(Q) - log(Qprev));
+            const double dq = n * fabs(log(Q) - log_prev);
             double rho = 0.0625;
             if (step > 1 && st->dq_prev > 0.0) rho = fmin(0.5, fmax(dq / st->dq_prev, 1.52587890625e-05));
             const double rest = dq * rho / (1.0 - rho);
@@ -1371,30 +1471,40 @@ cudaError_t launch_rhs_init(const MixedBatch& b, cudaStream_t s) {
     return cudaGetLastError();
 }
 
+// The tile launches of a substitution: many CTAs are bound by what an SM
+// issues and run more of them with fewer loads in flight; few are bound by
+// latency.  The line is at eight CTAs per SM (solve phase, ms, wide / deep:
+// 256 x 4000 14.5 / 15.7, 128 x 2047 2.19 / 2.27, 100 x 1024 .60 / .59,
+// 8 x 16384 12.2 / 11.1, 32 x 1448 .77 / .70).
+static bool sub_wide(dim3 grid) { return (long long)grid.x * grid.y > 8 * device_sms(); }
+
 cudaError_t launch_df_forward(const MixedBatch& b, int c0, int init, cudaStream_t s) {
     if (init) {
         if (c0 != 0) return cudaErrorInvalidValue;
         cudaError_t e = launch_rhs_init(b, s);
         if (e != cudaSuccess) return e;
     }
-    cudaError_t e = cudaMemsetAsync(b.SC, 0, (size_t)b.count * b.sc_stride * sizeof(int), s);
-    if (e != cudaSuccess) return e;
-    launch_chained(ahead_mixed(b), k_fwd_diag, b.count, kSubThreads, 0, s, b, c0, 0);
-    for (int J = 0; J + 1 < b.nt; ++J)
-        launch_chained(ahead_mixed(b), k_fwd_tiles, dim3(2 * (b.nt - 1 - J), b.count), kSubThreads, 0, s, b, c0, J);
+    launch_chained(true, k_fwd_diag, b.count, kSubThreads, 0, s, b, c0, 0);
+    for (int J = 0; J + 1 < b.nt; ++J) {
+        const dim3 grid(b.count, 2 * (b.nt - 1 - J));
+        launch_chained(true, sub_wide(grid) ? k_fwd_tiles<SubWide> : k_fwd_tiles<SubDeep>, grid, kSubThreads, 0,
+                       s, b, c0, J);
+    }
     return cudaGetLastError();
 }
 
 cudaError_t launch_df_backward(const MixedBatch& b, int c0, int add_to, cudaStream_t s) {
     const size_t smem = (size_t)GP_NB * kBwdTs * sizeof(dfl);
-    static std::atomic<size_t> attr[kMaxDevices];
-    cudaError_t e = raise_smem_limit(k_bwd_tiles, smem, attr);
+    static std::atomic<size_t> attr[2][kMaxDevices];
+    cudaError_t e = raise_smem_limit(k_bwd_tiles<SubDeep>, smem, attr[0]);
+    if (e == cudaSuccess) e = raise_smem_limit(k_bwd_tiles<SubWide>, smem, attr[1]);
     if (e != cudaSuccess) return e;
-    e = cudaMemsetAsync(b.SC, 0, (size_t)b.count * b.sc_stride * sizeof(int), s);
-    if (e != cudaSuccess) return e;
-    launch_chained(ahead_mixed(b), k_bwd_diag, b.count, kSubThreads, 0, s, b, c0, b.nt - 1, add_to);
-    for (int K = b.nt - 1; K > 0; --K)
-        launch_chained(ahead_mixed(b), k_bwd_tiles, dim3(2 * K, b.count), kSubThreads, smem, s, b, c0, K, add_to);
+    launch_chained(true, k_bwd_diag, b.count, kSubThreads, 0, s, b, c0, b.nt - 1, add_to);
+    for (int K = b.nt - 1; K > 0; --K) {
+        const dim3 grid(b.count, 2 * K);
+        launch_chained(true, sub_wide(grid) ? k_bwd_tiles<SubWide> : k_bwd_tiles<SubDeep>, grid, kSubThreads,
+                       smem, s, b, c0, K, add_to);
+    }
     return cudaGetLastError();
 }
 
@@ -1403,7 +1513,7 @@ cudaError_t launch_df_residual(const MixedBatch& b, cudaStream_t s) {
     static std::atomic<size_t> attr[kMaxDevices];
     cudaError_t e = raise_smem_limit(k_resid_tiles, smem, attr);
     if (e != cudaSuccess) return e;
-    launch_chained(ahead_mixed(b), k_resid_tiles, dim3(2 * (unsigned)packed_tiles(b.nt), b.count), kResThreads,
+    launch_chained(true, k_resid_tiles, dim3(2 * (unsigned)packed_tiles(b.nt), b.count), kResThreads,
                    smem, s, b);
     launch_chained(ahead_mixed(b), k_resid_reduce, dim3(b.nt, b.count), kResThreads, 0, s, b);
     return cudaGetLastError();
@@ -1411,7 +1521,7 @@ cudaError_t launch_df_residual(const MixedBatch& b, cudaStream_t s) {
 
 cudaError_t launch_df_finalize(const MixedBatch& b, double* nll, double* mu, double* sigma2, double* logdet,
                                int* status, cudaStream_t s) {
-    launch_chained(ahead_mixed(b), k_df_finalize, (b.count + 127) / 128, 128, 0, s, b, nll, mu, sigma2, logdet,
+    launch_chained(true, k_df_finalize, (b.count + 127) / 128, 128, 0, s, b, nll, mu, sigma2, logdet,
                    status);
     return cudaGetLastError();
 }

@@ -26,10 +26,11 @@ def dev(a):
 
 
 # (n, candidates of the plain batch): past 8 or 16 candidates or 128 (double)
-# and 256 (split) candidates x block columns
+# and 256 (split) candidates x block columns; at 1300 x 70 the substitutions
+# have more than eight CTAs per SM and take their other variant
 @pytest.mark.parametrize("prec,n,T", [("fp64", 40, 9), ("fp64", 256, 9), ("fp64", 257, 17), ("fp64", 700, 24),
                                       ("fp64", 1300, 12), ("mixed", 64, 257), ("mixed", 200, 130),
-                                      ("mixed", 390, 65), ("mixed", 1300, 24)])
+                                      ("mixed", 390, 65), ("mixed", 1300, 24), ("mixed", 1300, 70)])
 def test_few_candidates_give_the_batch_bits(ctx, prec, n, T):
     g = np.random.default_rng(n + T)
     d, p, delta, few = 3, 1.95, 1e-6, 2
