@@ -341,7 +341,39 @@ int ensure_aux(gp_ctx* ctx) {
     return GP_OK;
 }
 
-// Assemble and factor (split precision) the instances of `mb`.
+// Look-ahead of the split path: the SMs that the rest of a fused update leaves
+// to the factoring of the next pair of block columns (m block columns remain
+// with that pair), or 0 where the whole update first is as fast.  The update's
+// kernel holds its SMs to its end, so the split is made beforehand, from the
+// measured costs: a tile of the rest kTile us of one SM; a block column of the
+// pair kLatency us in which only the candidates' diagonal steps run, then
+// kFront us of one SM per tile (slices, panel solve, column update), on the SMs
+// left and, once the rest has ended, on all.
+int lookahead_sms(int m, int count) {
+    constexpr double kTile = 13.4, kFront = 90.0, kLatency = 140.0;
+    const int sms = gp::device_sms();
+    const double rest = kTile * (m - 1) * (m - 2) / 2 * count, work = kFront * m * count / 2;
+    int best = 0;
+    double least = 0.97 * (rest / sms + 2 * (kLatency + work / sms));      // two launches more
+    for (int r = count; r < sms; ++r) {
+        const double end = rest / (sms - r);
+        double t = 0.0;
+        for (int k = 0; k < 2; ++k) {
+            t += kLatency;
+            const double beside = t < end ? std::min(work, (end - t) * r) : 0.0;
+            t += beside / r + (work - beside) / sms;
+        }
+        if (std::max(t, end) < least) {
+            least = std::max(t, end);
+            best = r;
+        }
+    }
+    return best;
+}
+
+// Assemble and factor (split precision) the instances of `mb`.  A small batch
+// looks ahead by a pair of block columns: every tile still takes its updates
+// in block-column order, the same bits as without.
 int run_mixed_factor(gp_ctx* ctx, gp::MixedBatch& mb, int d, const double* x, const double* theta, double p,
                      double delta) {
     gp::Batch b{};
@@ -361,18 +393,21 @@ int run_mixed_factor(gp_ctx* ctx, gp::MixedBatch& mb, int d, const double* x, co
         if (mb.fwd) GP_CUDA(ctx, gp::launch_rhs_init(mb, ctx->stream));
     }
     const int nt = mb.nt;
+    const bool ahead = mb.fuse && nt >= gp::kLookaheadMixedTiles && mb.count <= gp::kLookaheadMixedMax;
+    mb.lookahead = ahead;
     int rc = ensure_aux(ctx);
+    if (!rc && ahead) rc = ensure_la(ctx);
     if (rc) return rc;
     // Diagonal block J and the slices of panel J's tiles for the panel solve
     // touch disjoint buffers: the slicing runs on the second stream while
     // the diagonal kernel (latency-bound, about one CTA per SM) runs on the
     // main one, and the panel solve waits for both.
-    auto diag_and_slices = [&](int J) -> int {
+    auto diag_and_slices = [&](int J, cudaStream_t st) -> int {
         const bool slices = J + 1 < nt;
-        if (slices) GP_CUDA(ctx, cudaEventRecord(ctx->ev_fork, ctx->stream));
+        if (slices) GP_CUDA(ctx, cudaEventRecord(ctx->ev_fork, st));
         {
-            PhaseScope ps(ctx, GP_PHASE_POTRF, 1);
-            GP_CUDA(ctx, gp::launch_diag_mixed(mb, J, ctx->stream));
+            PhaseScope ps(ctx, GP_PHASE_POTRF, 1, st);
+            GP_CUDA(ctx, gp::launch_diag_mixed(mb, J, st));
         }
         if (slices) {
             GP_CUDA(ctx, cudaStreamWaitEvent(ctx->aux, ctx->ev_fork, 0));
@@ -380,55 +415,73 @@ int run_mixed_factor(gp_ctx* ctx, gp::MixedBatch& mb, int d, const double* x, co
             ctx->phase_launches[GP_PHASE_SPLIT] += 1;
             GP_CUDA(ctx, gp::launch_split_panel(mb, J, mb.ps, 0, ctx->aux));
             GP_CUDA(ctx, cudaEventRecord(ctx->ev_join, ctx->aux));
-            // the time the main stream waits here is the slicing left exposed
-            PhaseScope ps(ctx, GP_PHASE_SPLIT, 0);
-            GP_CUDA(ctx, cudaStreamWaitEvent(ctx->stream, ctx->ev_join, 0));
+            // the time the stream waits here is the slicing left exposed
+            PhaseScope ps(ctx, GP_PHASE_SPLIT, 0, st);
+            GP_CUDA(ctx, cudaStreamWaitEvent(st, ctx->ev_join, 0));
         }
         return GP_OK;
     };
-    auto panel = [&](int J) -> int {
-        PhaseScope ps(ctx, GP_PHASE_TRSM, 1);
-        GP_CUDA(ctx, gp::launch_gemm_panel(mb, J, ctx->stream));
+    auto panel = [&](int J, cudaStream_t st) -> int {
+        PhaseScope ps(ctx, GP_PHASE_TRSM, 1, st);
+        GP_CUDA(ctx, gp::launch_gemm_panel(mb, J, st));
         return GP_OK;
     };
-    int J = 0;
-    while (J < nt) {
-        rc = diag_and_slices(J);
-        if (rc) return rc;
-        if (J + 1 == nt) break;
-        rc = panel(J);
-        if (rc) return rc;
+    // Block column J factored, solved and sliced; with panel pairs (J, J + 1)
+    // also column J + 1, updated from panel J, factored and solved: the
+    // trailing tiles then take both panels in one K = 256 pass.
+    auto pair_at = [&](int J) { return mb.fuse && J + 2 < nt; };
+    auto front = [&](int J, cudaStream_t st) -> int {
+        int e = diag_and_slices(J, st);
+        if (e || J + 1 == nt) return e;
+        if ((e = panel(J, st))) return e;
+        {
+            PhaseScope ps(ctx, GP_PHASE_SPLIT, 1, st);
+            GP_CUDA(ctx, gp::launch_split_panel(mb, J, mb.s, 1, st));
+        }
+        if (!pair_at(J)) return GP_OK;
+        {
+            PhaseScope ps(ctx, GP_PHASE_UPDATE, 1, st);
+            GP_CUDA(ctx, gp::launch_gemm_update_column(mb, J, st));
+        }
+        if ((e = diag_and_slices(J + 1, st))) return e;
+        return panel(J + 1, st);
+    };
+    auto fused = [&](int J, int which) -> int {
+        PhaseScope ps(ctx, GP_PHASE_UPDATE, 1);
+        GP_CUDA(ctx, gp::launch_gemm_update_fused(mb, J, which, ctx->stream));
+        return GP_OK;
+    };
+    if ((rc = front(0, ctx->stream))) return rc;
+    for (int J = 0; J + 1 < nt;) {
+        if (!pair_at(J)) {
+            {
+                PhaseScope ps(ctx, GP_PHASE_UPDATE, 1);
+                GP_CUDA(ctx, gp::launch_gemm_update(mb, J, ctx->stream));
+            }
+            if ((rc = front(++J, ctx->stream))) return rc;
+            continue;
+        }
         {
             PhaseScope ps(ctx, GP_PHASE_SPLIT, 1);
-            GP_CUDA(ctx, gp::launch_split_panel(mb, J, mb.s, 1, ctx->stream));
+            GP_CUDA(ctx, gp::launch_split_fused(mb, J, ctx->stream));
         }
-        if (mb.fuse && J + 2 < nt) {
-            // panel pair (J, J + 1): update column J + 1 from panel J, factor and
-            // solve panel J + 1, then apply both panels to the trailing tiles in
-            // one K = 256 pass
-            {
-                PhaseScope ps(ctx, GP_PHASE_UPDATE, 1);
-                GP_CUDA(ctx, gp::launch_gemm_update_column(mb, J, ctx->stream));
-            }
-            rc = diag_and_slices(J + 1);
-            if (rc) return rc;
-            rc = panel(J + 1);
-            if (rc) return rc;
-            {
-                PhaseScope ps(ctx, GP_PHASE_SPLIT, 1);
-                GP_CUDA(ctx, gp::launch_split_fused(mb, J, ctx->stream));
-            }
-            {
-                PhaseScope ps(ctx, GP_PHASE_UPDATE, 1);
-                GP_CUDA(ctx, gp::launch_gemm_update_fused(mb, J, ctx->stream));
-            }
-            J += 2;
+        J += 2;
+        if (ahead && J + 2 < nt && (mb.lookahead = lookahead_sms(nt - J, mb.count)) > 0) {
+            // the next pair's columns first; the pair is then factored on a
+            // high-priority stream beside the rest of the update
+            if ((rc = fused(J - 2, gp::kUpdateColumn))) return rc;
+            GP_CUDA(ctx, cudaEventRecord(ctx->ev_la0, ctx->stream));
+            GP_CUDA(ctx, cudaStreamWaitEvent(ctx->la, ctx->ev_la0, 0));
+            if ((rc = front(J, ctx->la))) return rc;
+            GP_CUDA(ctx, cudaEventRecord(ctx->ev_la1, ctx->la));
+            if ((rc = fused(J - 2, gp::kUpdateRest))) return rc;
+            GP_CUDA(ctx, cudaStreamWaitEvent(ctx->stream, ctx->ev_la1, 0));
         } else {
-            PhaseScope ps(ctx, GP_PHASE_UPDATE, 1);
-            GP_CUDA(ctx, gp::launch_gemm_update(mb, J, ctx->stream));
-            J += 1;
+            if ((rc = fused(J - 2, gp::kUpdateAll))) return rc;
+            if ((rc = front(J, ctx->stream))) return rc;
         }
     }
+    mb.lookahead = 0;
     return GP_OK;
 }
 

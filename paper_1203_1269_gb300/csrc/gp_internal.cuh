@@ -130,6 +130,7 @@ struct MixedBatch {
     size_t z_stride;
     float2* RP;                   // per-tile partial sums of the tile-parallel solves and residual
     size_t rp_stride;
+    int lookahead;                // SMs that the rest of an update leaves to the next block columns (0: none)
     int* SC;                      // per-block counters of the tile-parallel substitutions
     size_t sc_stride;
     const double* y;
@@ -227,6 +228,15 @@ cudaError_t launch_factor_small_f64(const Batch& b, cudaStream_t s, int* kernels
 // singularity (cond(R) 1e11, where any change of rounding shows in the eighth
 // digit of mu_hat) keep their bits.
 constexpr int kUpdateTcTiles = 3;
+// The split path looks ahead with at most so many candidates and at least so
+// many block columns (ms, without -> with; candidates x n): 32x1448 3.63 ->
+// 3.52, 16x2048 4.36 -> 4.10, 8x4000 9.76 -> 8.90, 32x4000 20.2 -> 19.1, 4x8192
+// 24.4 -> 21.3, 1x12000 29.4 -> 26.6, 8x16384 175.4 -> 170.9.  With fewer block
+// columns the launches set up ahead give more (1x512 .76 against .78), and with
+// more candidates the diagonal steps themselves fill the SMs (64x2048 8.30 ->
+// 8.15 but 64x4000 34.2 -> 34.5, 100x1024 3.24 -> 3.28, 128x2047 14.04 -> 14.11).
+constexpr int kLookaheadMixedMax = 48;
+constexpr int kLookaheadMixedTiles = 12;
 
 // Launches of a chain of kernels in one stream.  With `ahead`, the kernel is set
 // up on the GPU while the one before it still runs (programmatic stream
@@ -257,7 +267,9 @@ inline bool ahead_f64(const Batch& b) {
            (long long)b.count * b.nt <= kAheadColumnsF64;
 }
 
-inline bool ahead_mixed(const MixedBatch& b) { return (long long)b.count * b.nt <= kAheadColumnsMixed; }
+inline bool ahead_mixed(const MixedBatch& b) {
+    return !b.lookahead && (long long)b.count * b.nt <= kAheadColumnsMixed;
+}
 
 inline bool ahead_assemble(const Batch& b) {
     return b.Adf ? (long long)b.count * b.nt <= kAheadColumnsMixed : ahead_f64(b);
@@ -350,7 +362,7 @@ cudaError_t launch_split_panel(const MixedBatch& b, int J, int ns, int gemv, cud
 cudaError_t launch_gemm_panel(const MixedBatch& b, int J, cudaStream_t s);
 cudaError_t launch_gemm_update(const MixedBatch& b, int J, cudaStream_t s);
 cudaError_t launch_gemm_update_column(const MixedBatch& b, int J, cudaStream_t s);
-cudaError_t launch_gemm_update_fused(const MixedBatch& b, int J, cudaStream_t s);
+cudaError_t launch_gemm_update_fused(const MixedBatch& b, int J, int which, cudaStream_t s);
 cudaError_t launch_split_fused(const MixedBatch& b, int J, cudaStream_t s);
 cudaError_t launch_df_forward(const MixedBatch& b, int c0, int init, cudaStream_t s);
 cudaError_t launch_rhs_init(const MixedBatch& b, cudaStream_t s);

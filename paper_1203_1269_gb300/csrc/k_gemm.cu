@@ -178,9 +178,10 @@ __global__ void __launch_bounds__(ER ? kGemmThreadsER : kGemmThreads, 1)
 
     // kind (MODE 1): 0 trailing tiles from J + 1 (K = 128), 1 the single
     // column J + 1 (look-ahead, K = 128), 2 trailing tiles from J + 2 with
-    // the two panels J, J + 1 fused (K = 256)
+    // the two panels J, J + 1 fused (K = 256), 3 the first two columns of 2,
+    // 4 the rest of 2
     const int ns = (MODE == 0) ? b.ps : b.s;
-    const bool fused = (MODE == 1 && kind == 2);
+    const bool fused = (MODE == 1 && kind >= 2);
     const int nch = fused ? 2 * kChunks : kChunks;
     constexpr uint32_t kBBytes = kChunkBytes / (GP_NB / NT);      // B rows col0..col0+NT of a chunk
     const uint32_t a_bytes = (uint32_t)ns * kChunkBytes;
@@ -200,14 +201,26 @@ __global__ void __launch_bounds__(ER ? kGemmThreadsER : kGemmThreads, 1)
         } else if (kind == 1) {
             I = J + 1 + tile;
             K = J + 1;
+        } else if (kind == 3) {
+            const int m = b.nt - J - 2;
+            K = tile < m ? J + 2 : J + 3;
+            I = tile < m ? J + 2 + tile : J + 3 + tile - m;
         } else {
             int ii, kk;
             tri_decode(tile, ii, kk);
-            const int base = (kind == 2) ? J + 2 : J + 1;
+            const int base = (kind == 4) ? J + 4 : (kind == 2) ? J + 2 : J + 1;
             I = base + ii;
             K = base + kk;
         }
     };
+
+    // The diagonal step of a later block column may run beside kind 4 and fail a
+    // candidate: its warps must agree on the tiles they skip, so they go by
+    // what the CTA read at its start.
+    __shared__ uint8_t live[kLookaheadMixedMax];
+    if (MODE == 1 && kind == 4)
+        for (int i = threadIdx.x; i < b.count; i += blockDim.x) live[i] = b.st[i].status == GP_OK;
+    auto alive = [&](int t) { return (MODE == 1 && kind == 4) ? live[t] != 0 : b.st[t].status == GP_OK; };
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
@@ -252,7 +265,7 @@ __global__ void __launch_bounds__(ER ? kGemmThreadsER : kGemmThreads, 1)
         for (int w = blockIdx.x; w < total && !abort_flag; w += gridDim.x) {
             int t, I, K, col0;
             decode(w, t, I, K, col0);
-            if (b.st[t].status != GP_OK) continue;
+            if (!alive(t)) continue;
             float2* C = df_tile(b, b.A, t, I, K) + (size_t)col0 * GP_NB;
             if (MODE == 1 && threadIdx.x == 32 * kEpiBase) prefetch_l2(C, (uint32_t)(NT * GP_NB * sizeof(float2)));
             if (!mbar_wait(&tfull_bar[0], i & 1, &abort_flag)) {
@@ -376,7 +389,7 @@ __global__ void __launch_bounds__(ER ? kGemmThreadsER : kGemmThreads, 1)
             for (int w = blockIdx.x; w < total && !abort_flag; w += gridDim.x) {
                 int t, I, K, col0;
                 decode(w, t, I, K, col0);
-                if (b.st[t].status != GP_OK) continue;
+                if (!alive(t)) continue;
                 const __nv_bfloat16* gA = fused ? pf_block(b, t, I) : ps_block(b, t, I);
                 const __nv_bfloat16* gBb = (MODE == 0) ? (b.WS + (size_t)t * b.ws_stride)
                                                        : (fused ? pf_block(b, t, K) : ps_block(b, t, K));
@@ -407,7 +420,7 @@ __global__ void __launch_bounds__(ER ? kGemmThreadsER : kGemmThreads, 1)
             for (int w = blockIdx.x; w < total && !abort_flag; w += gridDim.x) {
                 int t, I, K, col0;
                 decode(w, t, I, K, col0);
-                if (b.st[t].status != GP_OK) continue;
+                if (!alive(t)) continue;
                 // accumulator set i % NBUF is free once the epilogue has drained
                 // tile i - NBUF (the group-wise release: group by group, in the first stage)
                 const int buf = i % NBUF;
@@ -468,7 +481,7 @@ __global__ void __launch_bounds__(ER ? kGemmThreadsER : kGemmThreads, 1)
         for (int w = blockIdx.x; w < total && !abort_flag; w += gridDim.x) {
             int t, I, K, col0;
             decode(w, t, I, K, col0);
-            if (b.st[t].status != GP_OK) continue;
+            if (!alive(t)) continue;
             float2* C = df_tile(b, b.A, t, I, K) + (size_t)col0 * GP_NB;
             // the C tile (contiguous) heads for L2 while this tile's MMAs run
             if (MODE == 1 && threadIdx.x == 64) prefetch_l2(C, (uint32_t)(NT * GP_NB * sizeof(float2)));
@@ -572,7 +585,8 @@ static cudaError_t launch_gemm(const MixedBatch& b, int J, int per_inst, int ns,
     cudaError_t e = raise_smem_limit(k_split_gemm<MODE, NT, NG, ER>, smem, attr);
     if (e != cudaSuccess) return e;
     const long long total = (long long)per_inst * b.count;
-    const int grid = (int)(total < device_sms() ? total : device_sms());
+    const int cap = kind == 4 ? device_sms() - b.lookahead : device_sms();
+    const int grid = (int)(total < cap ? total : cap);
     launch_chained(MODE != 0 && ahead_mixed(b), k_split_gemm<MODE, NT, NG, ER>, grid,
                    ER ? kGemmThreadsER : kGemmThreads, smem, s, b, J, per_inst, kind);
     return cudaGetLastError();
@@ -626,13 +640,14 @@ cudaError_t launch_gemm_update_column(const MixedBatch& b, int J, cudaStream_t s
     return launch_update128(b, J, m, b.s, s, 1);
 }
 
-cudaError_t launch_gemm_update_fused(const MixedBatch& b, int J, cudaStream_t s) {
+cudaError_t launch_gemm_update_fused(const MixedBatch& b, int J, int which, cudaStream_t s) {
     const int m = b.nt - J - 2;
-    if (m <= 0) return cudaSuccess;
-    if (b.update_tile == 64) return launch_gemm<1, 64, 4>(b, J, m * (m + 1), b.s, s, 2);
-    return launch_update128(b, J, m * (m + 1) / 2, b.s, s, 2);
+    const int tiles = which == kUpdateAll ? m * (m + 1) / 2 : which == kUpdateColumn ? 2 * m - 1 : (m - 2) * (m - 1) / 2;
+    const int kind = which == kUpdateAll ? 2 : which == kUpdateColumn ? 3 : 4;
+    if (m <= 0 || tiles <= 0) return cudaSuccess;
+    if (b.update_tile == 64) return launch_gemm<1, 64, 4>(b, J, 2 * tiles, b.s, s, kind);
+    return launch_update128(b, J, tiles, b.s, s, kind);
 }
-
 
 cudaError_t launch_gemm_update(const MixedBatch& b, int J, cudaStream_t s) {
     const int m = b.nt - J - 1;
