@@ -33,9 +33,31 @@ __device__ __forceinline__ double matern_q(double h, int corr) {
 
 // q(h) in double-float (h >= 0); third = 1/3 as double-float
 __device__ __forceinline__ dfl matern_q_df(dfl h, int corr, dfl third) {
-    if (corr == GP_CORR_MATERN32) return df_add(dfl{1.f, 0.f}, h);
-    if (corr == GP_CORR_MATERN52) return df_add(dfl{1.f, 0.f}, df_fma(df_mul(h, h), third, h));
+    if (corr == GP_CORR_MATERN32) return df_add_float(1.f, h);
+    if (corr == GP_CORR_MATERN52) return df_add_float(1.f, df_fma(df_mul(h, h), third, h));
     return dfl{1.f, 0.f};
+}
+
+// the same for two values at once, bit for bit (nthird: the negated high word)
+__device__ __forceinline__ df2 matern_q_df2(df2 h, int corr, df2 third, f32x2 nthird) {
+    const f32x2 one = f2_pack(1.f, 1.f), zero = f2_pack(0.f, 0.f);
+    if (corr != GP_CORR_MATERN32 && corr != GP_CORR_MATERN52) return {one, zero};
+    df2 w = h;
+    if (corr == GP_CORR_MATERN52) {
+        const df2 m = df2_mul(f2_neg(h.hi), h, h);
+        const f32x2 pn = f2_mul(m.hi, nthird);
+        f32x2 e = f2_fma(m.hi, third.hi, pn);
+        e = f2_fma(m.hi, third.lo, e);
+        e = f2_fma(m.lo, third.hi, e);
+        f32x2 s, t;
+        f2_two_diff(h.hi, pn, s, t);
+        f2_fast_two_sum(s, f2_add(t, f2_add(h.lo, e)), w.hi, w.lo);
+    }
+    const f32x2 s = f2_add(one, w.hi), bb = f2_sub(s, one);
+    const f32x2 e = f2_add(f2_sub(one, f2_sub(s, bb)), f2_sub(w.hi, bb));
+    df2 r;
+    f2_fast_two_sum(s, f2_add(e, w.lo), r.hi, r.lo);
+    return r;
 }
 
 // exp(-S) in double without CUDA's exp (the reduction of P. T. P. Tang, ACM TOMS

@@ -49,6 +49,16 @@ __device__ __forceinline__ dfl df_add(dfl a, dfl b) {
     return {s, e};
 }
 
+// a + b for a float a: the bits of df_add({a, 0}, b), whose second TwoSum and
+// last FastTwoSum change nothing then
+__device__ __forceinline__ dfl df_add_float(float a, dfl b) {
+    float s, e;
+    two_sum(a, b.hi, s, e);
+    e = __fadd_rn(e, b.lo);
+    fast_two_sum(s, e, s, e);
+    return {s, e};
+}
+
 __device__ __forceinline__ dfl df_neg(dfl a) { return {-a.hi, -a.lo}; }
 
 __device__ __forceinline__ dfl df_sub(dfl a, dfl b) { return df_add(a, df_neg(b)); }
@@ -126,6 +136,11 @@ __device__ __forceinline__ f32x2 f2_fma(f32x2 a, f32x2 b, f32x2 c) {
     return r;
 }
 __device__ __forceinline__ f32x2 f2_neg(f32x2 a) { return a ^ 0x8000000080000000ull; }
+// a b where its only use is an addition, rounded by itself: a pair's mul.rn and
+// add.rn were seen contracted into one fma there, the scalar ones are not
+__device__ __forceinline__ f32x2 f2_mul_alone(f32x2 a, f32x2 b) {
+    return f2_pack(__fmul_rn(f2_first(a), f2_first(b)), __fmul_rn(f2_second(a), f2_second(b)));
+}
 
 // c - a b, half by half the bits of df_fma(df_neg(a), b, c) and of
 // df_fma(a, df_neg(b), c): p = -(a.hi b.hi), which the caller forms with
@@ -142,6 +157,30 @@ __device__ __forceinline__ df2 df2_fnma(f32x2 p, df2 a, df2 b, df2 c) {
     df2 r;
     r.hi = f2_add(s, t);
     r.lo = f2_sub(t, f2_sub(r.hi, s));
+    return r;
+}
+
+// Sum of a and -bn, half by half the bits of two_sum(a, -bn)
+__device__ __forceinline__ void f2_two_diff(f32x2 a, f32x2 bn, f32x2& s, f32x2& e) {
+    const f32x2 s0 = f2_sub(a, bn), bb = f2_sub(s0, a);
+    e = f2_sub(f2_sub(a, f2_sub(s0, bb)), f2_add(bn, bb));
+    s = s0;
+}
+// fast_two_sum(a, b), half by half
+__device__ __forceinline__ void f2_fast_two_sum(f32x2 a, f32x2 b, f32x2& s, f32x2& e) {
+    const f32x2 s0 = f2_add(a, b);
+    e = f2_sub(b, f2_sub(s0, a));
+    s = s0;
+}
+// a b from an = -a.hi: the bits of df_mul
+__device__ __forceinline__ df2 df2_mul(f32x2 an, df2 a, df2 b) {
+    const f32x2 pn = f2_mul(an, b.hi);
+    f32x2 e = f2_fma(a.hi, b.hi, pn);
+    e = f2_fma(a.hi, b.lo, e);
+    e = f2_fma(a.lo, b.hi, e);
+    df2 r;
+    r.hi = f2_sub(e, pn);
+    r.lo = f2_sub(e, f2_add(r.hi, pn));
     return r;
 }
 
@@ -234,6 +273,47 @@ __device__ __forceinline__ dfl df_exp_neg(dfl S, const dfl* tab) {
     const float sc = __int_as_float((127 - (k >> kExpTabBits)) << 23);   // 2^-m, -120 <= m <= 125
     e.hi = __fmul_rn(e.hi, sc);
     e.lo = __fmul_rn(e.lo, sc);
+    return e;
+}
+
+// The same for two values at once, their operations in pairs where both halves
+// take them: bit for bit df_exp_neg of each half (S >= 0 here).  The rounding to
+// an integer goes through an added 1.5 2^23, which also leaves k in the
+// low bits of the sum.
+__device__ __forceinline__ df2 df2_exp_neg(df2 S, const dfl* tab) {
+    constexpr double kLn2OverN = 0.693147180559945309417232121458176568 / kExpTab;
+    constexpr float kCHi = (float)kLn2OverN;
+    constexpr float kCLo = (float)(kLn2OverN - (double)kCHi);
+    constexpr float kNOverLn2 = (float)(kExpTab / 0.693147180559945309417232121458176568);
+    const f32x2 round = f2_pack(12582912.f, 12582912.f);
+    const f32x2 kr = f2_add(f2_mul_alone(S.hi, f2_pack(kNOverLn2, kNOverLn2)), round);
+    const f32x2 kf = f2_sub(kr, round);
+    const int k0 = __float_as_int(f2_first(kr)) - 0x4b400000, k1 = __float_as_int(f2_second(kr)) - 0x4b400000;
+    const f32x2 p1n = f2_mul(kf, f2_pack(-kCHi, -kCHi));
+    const f32x2 e1 = f2_fma(kf, f2_pack(kCHi, kCHi), p1n);
+    const f32x2 p2 = f2_mul_alone(kf, f2_pack(kCLo, kCLo));
+    const f32x2 r0 = f2_add(S.hi, p1n);
+    const f32x2 l0 = f2_sub(f2_sub(S.lo, e1), p2);
+    const f32x2 rh = f2_add(r0, l0), bb = f2_sub(rh, r0);
+    const f32x2 rl = f2_add(f2_sub(r0, f2_sub(rh, bb)), f2_sub(l0, bb));
+    f32x2 q = f2_fma(rh, f2_pack(-1.f / 6.f, -1.f / 6.f), f2_pack(0.5f, 0.5f));
+    q = f2_fma(rh, q, rl);
+    q = f2_mul_alone(rh, q);
+    const f32x2 one = f2_pack(1.f, 1.f);
+    const f32x2 s0 = f2_sub(one, rh);
+    const f32x2 t0 = f2_sub(q, f2_add(f2_add(rh, f2_sub(s0, one)), rl));
+    df2 w;
+    f2_fast_two_sum(s0, t0, w.hi, w.lo);
+    const df2 T = df2_pack(tab[k0 & (kExpTab - 1)], tab[k1 & (kExpTab - 1)]);
+    df2 e = df2_mul(f2_neg(w.hi), w, T);
+    // 2^-m by the exponent bits
+    const f32x2 sc = f2_pack(__int_as_float((127 - (k0 >> kExpTabBits)) << 23),
+                             __int_as_float((127 - (k1 >> kExpTabBits)) << 23));
+    e.hi = f2_mul(e.hi, sc);
+    e.lo = f2_mul(e.lo, sc);
+    const bool in0 = f2_first(S.hi) < 86.6f, in1 = f2_second(S.hi) < 86.6f;
+    e.hi = f2_pack(in0 ? f2_first(e.hi) : 0.f, in1 ? f2_second(e.hi) : 0.f);
+    e.lo = f2_pack(in0 ? f2_first(e.lo) : 0.f, in1 ? f2_second(e.lo) : 0.f);
     return e;
 }
 

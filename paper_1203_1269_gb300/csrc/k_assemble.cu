@@ -263,8 +263,19 @@ k_assemble_tiles(Batch b, int group, PowTab64 ptab) {
 // (double-float), the group's status flags.
 // EXACT: DB is d itself, so the loops over the dimensions have a constant
 // bound (the benchmark's d = 6: 10.84 -> 9.92 ms, the same bits).
-template <int DB, int COLS, bool MATERN, bool EXACT = false>
-__global__ void __launch_bounds__(kThreads)
+// PAIR: two candidates at once in paired FP32 instructions, half the issue
+// slots of what both take (a scalar warp issues in 82 to 87 % of the cycles
+// with the FP32 pipe at 56 % (power-exponential, d = 6) and 78 % (Matern 5/2, d
+// = 8); the same bits).  Matern: always, 5.59 -> 4.60 ms at 128 x 2047, d = 8.
+// Power-exponential: where a CTA has at least kPairMinGroup candidates and d <=
+// kPairMaxD: 9.91 -> 8.93 ms at 256 x 4000, d = 6, .391 -> .356 at 100 x 1024;
+// with few the powers are what counts and a half pair is lost (3 x 2000 .163 ->
+// .188), above d = 10 the doubled powers leave too few warps (64 x 1024, d = 14
+// .509 -> .524).
+constexpr int kPairMinGroup = 16;
+constexpr int kPairMaxD = 10;
+template <int DB, int COLS, bool MATERN, bool PAIR, bool EXACT = false>
+__global__ void __launch_bounds__(kThreads, PAIR && !MATERN && DB > 8 ? 4 : 0)
 k_assemble_tiles_df(Batch b, int group, const float2* etab) {
     grid_dependency();
     constexpr int kSplitDf = GP_NB / COLS;
@@ -273,9 +284,13 @@ k_assemble_tiles_df(Batch b, int group, const float2* etab) {
     extern __shared__ double dsm[];
     double* xs_r = dsm;                                  // GP_NB * DB
     double* xs_c = xs_r + GP_NB * DB;                    // kColsDf * DB
-    dfl* th = reinterpret_cast<dfl*>(xs_c + kColsDf * DB); // group * DB
-    dfl* tab = th + (size_t)group * DB;                  // kExpTab
-    int* live = reinterpret_cast<int*>(tab + kExpTab);   // group
+    // theta of a pair of candidates: high words, their negatives and low words
+    // (without PAIR the two words of each candidate)
+    static_assert(PAIR || !MATERN, "the Matern families take candidates in pairs");
+    constexpr int kTh = PAIR ? 3 : 2;
+    f32x2* th = reinterpret_cast<f32x2*>(xs_c + kColsDf * DB);   // (group + 1) / 2 * DB * kTh
+    dfl* tab = reinterpret_cast<dfl*>(th + (size_t)(group + 1) / 2 * DB * kTh);   // kExpTab
+    int* live = reinterpret_cast<int*>(tab + kExpTab);   // group, rounded up to a pair
     const int nt = b.nt, n = b.n, d = b.d;
     const int tile_lin = blockIdx.x / kSplitDf;
     const int part = blockIdx.x % kSplitDf;
@@ -296,19 +311,31 @@ k_assemble_tiles_df(Batch b, int group, const float2* etab) {
         const int c = q / DB, k = q % DB, gj = col0 + c;
         xs_c[q] = (gj < n && k < d) ? b.x[(size_t)gj * d + k] : 0.0;
     }
-    for (int q = threadIdx.x; q < (t1 - t0) * DB; q += kThreads) {
-        const int tt = q / DB, k = q % DB;
-        th[q] = (k < d) ? df_from_double(corr_theta_scale(b.corr) * b.theta[(size_t)(t0 + tt) * d + k])
-                        : dfl{0.f, 0.f};
+    const int pairs = (t1 - t0 + 1) / 2;
+    for (int q = threadIdx.x; q < pairs * DB; q += kThreads) {
+        const int k = q % DB, i0 = t0 + 2 * (q / DB), i1 = min(i0 + 1, t1 - 1);
+        const double scale = corr_theta_scale(b.corr);
+        const dfl v0 = k < d ? df_from_double(scale * b.theta[(size_t)i0 * d + k]) : dfl{0.f, 0.f};
+        const dfl v1 = k < d ? df_from_double(scale * b.theta[(size_t)i1 * d + k]) : dfl{0.f, 0.f};
+        if (PAIR) {
+            th[3 * q] = f2_pack(v0.hi, v1.hi);
+            th[3 * q + 1] = f2_pack(-v0.hi, -v1.hi);
+            th[3 * q + 2] = f2_pack(v0.lo, v1.lo);
+        } else {
+            dfl* one = reinterpret_cast<dfl*>(th) + 2 * (q / DB) * DB + k;
+            one[0] = v0;
+            one[DB] = v1;
+        }
     }
-    for (int q = threadIdx.x; q < t1 - t0; q += kThreads) live[q] = (b.st[t0 + q].status == GP_OK);
+    for (int q = threadIdx.x; q < 2 * pairs; q += kThreads) live[q] = t0 + q < t1 && b.st[t0 + q].status == GP_OK;
     load_exp2_table(tab, etab);
     __syncthreads();
     const dfl delta = df_from_double(b.delta);
     constexpr bool matern = MATERN;                          // the family is a template argument
     const int pmode = matern ? kPowOne : pow_mode(b.p);      // Matern: h = c theta |dx|
     const dfl pd = df_from_double(b.p);
-    const dfl third = df_from_double(1.0 / 3.0);
+    const df2 third = df2_dup(df_from_double(1.0 / 3.0));
+    const f32x2 nthird = f2_neg(third.hi);
     const size_t tile_off = (size_t)tile_lin * GP_TILE_ELEMS;
     const int r = threadIdx.x % GP_NB;
     const int cb = threadIdx.x / GP_NB;
@@ -320,63 +347,118 @@ k_assemble_tiles_df(Batch b, int group, const float2* etab) {
         const size_t off = tile_off + (size_t)(part * kColsDf + c) * GP_NB + r;
         const bool pad = (gi >= n) || (gj >= n);
         const bool diag = (gi == gj);
-        dfl D[DB];
+        auto power = [&](int k) {
+            return (k < (EXACT ? DB : d) && !pad) ? power_term(xs_r[r * DB + k] - xs_c[c * DB + k], pmode, b.p, pd, tab)
+                                                  : dfl{0.f, 0.f};
+        };
+        if constexpr (!PAIR) {
+            dfl D[DB];
 #pragma unroll
-        for (int k = 0; k < DB; ++k)
-            D[k] = (k < (EXACT ? DB : d) && !pad) ? power_term(xs_r[r * DB + k] - xs_c[c * DB + k], pmode, b.p, pd, tab)
-                                   : dfl{0.f, 0.f};
+            for (int k = 0; k < DB; ++k) D[k] = power(k);
 #pragma unroll 1
-        for (int t = t0; t < t1; ++t) {
-            if (!live[t - t0]) continue;
-            dfl v;
-            if (pad) {
-                v = {diag ? 1.f : 0.f, 0.f};
-            } else {
-                const dfl* tt = th + (size_t)(t - t0) * DB;
-                float sh = 0.f, sl = 0.f;
-                dfl qp = {1.f, 0.f};                // Matern: prod_k q(h_k)
-                // k >= d is uniform across the warp: leave the unrolled loop
-                // there rather than issue its predicated-off iterations; the
-                // first term enters S exactly (the TwoSum of 0 and it is exact)
+            for (int t = t0; t < t1; ++t) {
+                if (!live[t - t0]) continue;
+                dfl v;
+                if (pad) {
+                    v = {diag ? 1.f : 0.f, 0.f};
+                } else {
+                    const dfl* tt = reinterpret_cast<const dfl*>(th) + (size_t)(t - t0) * DB;
+                    float sh = 0.f, sl = 0.f;
+                    // k >= d is uniform across the warp: leave the unrolled loop
+                    // there rather than issue its predicated-off iterations; the
+                    // first term enters S exactly (the TwoSum of 0 and it is exact)
 #pragma unroll
-                for (int k = 0; k < DB; ++k) {
-                    if (k >= (EXACT ? DB : d)) break;
-                    const dfl a = tt[k];
-                    float ph = __fmul_rn(a.hi, D[k].hi);
-                    if (matern) {
-                        // h_k = a D_k itself is needed for q(h_k): its high
-                        // word enters the TwoSum, its low word sl
-                        const float pe = __fmaf_rn(a.hi, D[k].hi, -ph);
-                        const float pl = __fmaf_rn(a.hi, D[k].lo, __fmul_rn(a.lo, D[k].hi));
-                        dfl h;
-                        fast_two_sum(ph, __fadd_rn(pe, pl), h.hi, h.lo);
-                        qp = df_mul(qp, matern_q_df(h, b.corr, third));
-                        ph = h.hi;
-                        sl = __fadd_rn(sl, h.lo);
-                    } else {
+                    for (int k = 0; k < DB; ++k) {
+                        if (k >= (EXACT ? DB : d)) break;
+                        const dfl a = tt[k];
+                        const float ph = __fmul_rn(a.hi, D[k].hi);
                         sl = __fadd_rn(sl, __fmaf_rn(a.hi, D[k].hi, -ph));
                         sl = __fmaf_rn(a.hi, D[k].lo, sl);
                         sl = __fmaf_rn(a.lo, D[k].hi, sl);
+                        if (k == 0) {
+                            sh = ph;
+                        } else {
+                            float s2, e2;
+                            two_sum(sh, ph, s2, e2);
+                            sh = s2;
+                            sl = __fadd_rn(sl, e2);
+                        }
+                    }
+                    dfl S;
+                    fast_two_sum(sh, sl, S.hi, S.lo);   // |sl| << sh: every term is >= 0
+                    v = df_exp_neg(S, tab);
+                    if (diag) v = df_add(v, delta);
+                }
+                const size_t i = (size_t)t * b.inst_stride + off;
+                const float2 hl = make_float2(v.hi, v.lo);
+                b.Adf[i] = hl;
+                b.Rdf[i] = hl;
+            }
+            continue;
+        }
+        // the same for two candidates at once in paired FP32 instructions
+        df2 D[DB];
+#pragma unroll
+        for (int k = 0; k < DB; ++k) D[k] = df2_dup(power(k));
+#pragma unroll 1
+        for (int pr = 0; pr < pairs; ++pr) {
+            const int2 alive = reinterpret_cast<const int2*>(live)[pr];
+            if (!(alive.x | alive.y)) continue;
+            df2 v;
+            if (pad) {
+                v = df2_dup(dfl{diag ? 1.f : 0.f, 0.f});
+            } else {
+                const f32x2* tt = th + (size_t)pr * DB * kTh;
+                f32x2 sh = f2_pack(0.f, 0.f), sl = sh;
+                df2 qp = {f2_pack(1.f, 1.f), sh};            // Matern: prod_k q(h_k)
+                // products are formed negated (pn): a pair has no negated operand
+#pragma unroll
+                for (int k = 0; k < DB; ++k) {
+                    if (k >= (EXACT ? DB : d)) break;
+                    const df2 a = {tt[kTh * k], tt[kTh * k + 2]};
+                    f32x2 pn = f2_mul(tt[kTh * k + 1], D[k].hi);
+                    if (matern) {
+                        // h_k = a D_k itself is needed for q(h_k): its high
+                        // word enters the TwoSum, its low word sl
+                        const f32x2 pe = f2_fma(a.hi, D[k].hi, pn);
+                        const f32x2 pl = f2_fma(a.hi, D[k].lo, f2_mul(a.lo, D[k].hi));
+                        const f32x2 w = f2_add(pe, pl);
+                        df2 h;
+                        h.hi = f2_sub(w, pn);
+                        h.lo = f2_sub(w, f2_add(h.hi, pn));
+                        qp = df2_mul(f2_neg(qp.hi), qp, matern_q_df2(h, b.corr, third, nthird));
+                        pn = f2_neg(h.hi);
+                        sl = f2_add(sl, h.lo);
+                    } else {
+                        sl = f2_add(sl, f2_fma(a.hi, D[k].hi, pn));
+                        sl = f2_fma(a.hi, D[k].lo, sl);
+                        sl = f2_fma(a.lo, D[k].hi, sl);
                     }
                     if (k == 0) {
-                        sh = ph;
+                        sh = f2_neg(pn);
                     } else {
-                        float s2, e2;
-                        two_sum(sh, ph, s2, e2);
-                        sh = s2;
-                        sl = __fadd_rn(sl, e2);
+                        f32x2 e2;
+                        f2_two_diff(sh, pn, sh, e2);
+                        sl = f2_add(sl, e2);
                     }
                 }
-                dfl S;
-                fast_two_sum(sh, sl, S.hi, S.lo);   // |sl| << sh: every term is >= 0
-                v = df_exp_neg(S, tab);
-                if (matern) v = df_mul(v, qp);
-                if (diag) v = df_add(v, delta);
+                df2 S;
+                f2_fast_two_sum(sh, sl, S.hi, S.lo);   // |sl| << sh: every term is >= 0
+                v = df2_exp_neg(S, tab);
+                if (matern) v = df2_mul(f2_neg(v.hi), v, qp);
+                if (diag) v = df2_pack(df_add(df2_first(v), delta), df_add(df2_second(v), delta));
             }
-            const size_t i = (size_t)t * b.inst_stride + off;
-            const float2 hl = make_float2(v.hi, v.lo);
-            b.Adf[i] = hl;
-            b.Rdf[i] = hl;
+            const size_t i = (size_t)(t0 + 2 * pr) * b.inst_stride + off;
+            if (alive.x) {
+                const float2 hl = make_float2(f2_first(v.hi), f2_first(v.lo));
+                b.Adf[i] = hl;
+                b.Rdf[i] = hl;
+            }
+            if (alive.y) {
+                const float2 hl = make_float2(f2_second(v.hi), f2_second(v.lo));
+                b.Adf[i + b.inst_stride] = hl;
+                b.Rdf[i + b.inst_stride] = hl;
+            }
         }
     }
 }
@@ -496,12 +578,12 @@ const float2* exp2_table() {
 // The double-float assembly for one (DB, COLS, family): its shared-memory
 // limit raised once per device and size (raise_smem_limit, safe when
 // contexts on several threads assemble at once), then the launch.
-template <int DB, int COLS, bool M, bool EXACT = false>
+template <int DB, int COLS, bool M, bool PAIR, bool EXACT = false>
 static cudaError_t launch_asm_df(dim3 grid, size_t smem, cudaStream_t s, const Batch& b, int group) {
     static std::atomic<size_t> attr[kMaxDevices];
-    cudaError_t e = raise_smem_limit(k_assemble_tiles_df<DB, COLS, M, EXACT>, smem, attr);
+    cudaError_t e = raise_smem_limit(k_assemble_tiles_df<DB, COLS, M, PAIR, EXACT>, smem, attr);
     if (e != cudaSuccess) return e;
-    launch_chained(ahead_assemble(b), k_assemble_tiles_df<DB, COLS, M, EXACT>, grid, kThreads, smem, s, b,
+    launch_chained(ahead_assemble(b), k_assemble_tiles_df<DB, COLS, M, PAIR, EXACT>, grid, kThreads, smem, s, b,
                    group, exp2_table());
     return cudaGetLastError();
 }
@@ -562,15 +644,17 @@ cudaError_t launch_assemble_tiles(const Batch& b, cudaStream_t s) {
         grid = dim3((unsigned)(tiles * split), (unsigned)g_df);
         // 16 columns (the default): DB = d exactly; 32: d rounded up to 4, 8 or 16
         const int DB = (cols == 16) ? b.d : (b.d <= 4 ? 4 : (b.d <= 8 ? 8 : 16));
+        const bool m = corr_is_matern(b.corr), pair = cols == 16 && b.d <= kPairMaxD && group >= kPairMinGroup;
+        const size_t duos = (size_t)(group + 1) / 2;
         const size_t smem = (size_t)(GP_NB + cols) * DB * sizeof(double) +
-                            ((size_t)group * DB + kExpTab) * sizeof(dfl) + (size_t)group * sizeof(int);
-        const bool m = corr_is_matern(b.corr);
+                            (duos * DB * (m || pair ? 3 : 2) + kExpTab) * sizeof(dfl) + duos * sizeof(int2);
         cudaError_t e;
         if (cols == 16) {
 #define GP_ASM_EXACT(D)                                                                                  \
     case D:                                                                                              \
-        e = m ? launch_asm_df<D, 16, true, true>(grid, smem, s, b, group)                                \
-              : launch_asm_df<D, 16, false, true>(grid, smem, s, b, group);                             \
+        e = m ? launch_asm_df<D, 16, true, true, true>(grid, smem, s, b, group)                          \
+          : pair ? launch_asm_df<D, 16, false, D <= kPairMaxD, true>(grid, smem, s, b, group)            \
+                 : launch_asm_df<D, 16, false, false, true>(grid, smem, s, b, group);                    \
         break
             switch (b.d) {
                 GP_ASM_EXACT(1); GP_ASM_EXACT(2); GP_ASM_EXACT(3); GP_ASM_EXACT(4);
@@ -581,9 +665,9 @@ cudaError_t launch_assemble_tiles(const Batch& b, cudaStream_t s) {
             }
 #undef GP_ASM_EXACT
         } else {
-            if (DB == 4) e = m ? launch_asm_df<4, 32, true>(grid, smem, s, b, group) : launch_asm_df<4, 32, false>(grid, smem, s, b, group);
-            else if (DB == 8) e = m ? launch_asm_df<8, 32, true>(grid, smem, s, b, group) : launch_asm_df<8, 32, false>(grid, smem, s, b, group);
-            else e = m ? launch_asm_df<16, 32, true>(grid, smem, s, b, group) : launch_asm_df<16, 32, false>(grid, smem, s, b, group);
+            if (DB == 4) e = m ? launch_asm_df<4, 32, true, true>(grid, smem, s, b, group) : launch_asm_df<4, 32, false, false>(grid, smem, s, b, group);
+            else if (DB == 8) e = m ? launch_asm_df<8, 32, true, true>(grid, smem, s, b, group) : launch_asm_df<8, 32, false, false>(grid, smem, s, b, group);
+            else e = m ? launch_asm_df<16, 32, true, true>(grid, smem, s, b, group) : launch_asm_df<16, 32, false, false>(grid, smem, s, b, group);
         }
         return e;
     }
