@@ -640,14 +640,22 @@ cudaError_t launch_assemble_tiles(const Batch& b, cudaStream_t s) {
         if (g_df < 1) g_df = 1;
         if (g_df > b.count) g_df = b.count;
         group = (int)((b.count + g_df - 1) / g_df);
-        g_df = (b.count + group - 1) / group;
-        grid = dim3((unsigned)(tiles * split), (unsigned)g_df);
         // 16 columns (the default): DB = d exactly; 32: d rounded up to 4, 8 or 16
         const int DB = (cols == 16) ? b.d : (b.d <= 4 ? 4 : (b.d <= 8 ? 8 : 16));
         const bool m = corr_is_matern(b.corr), pair = cols == 16 && b.d <= kPairMaxD && group >= kPairMinGroup;
+        const size_t duo = (size_t)DB * (m || pair ? 3 : 2) * sizeof(dfl);       // theta of two candidates
+        // a group's theta takes at most half of the shared memory where pairs
+        // enlarge it, as much as fits otherwise
+        const int most = 2 * (int)((m || pair ? 96 * 1024 : 192 * 1024) / (duo + sizeof(int2)));
+        if (group > most) {
+            g_df = (b.count + most - 1) / most;
+            group = (int)((b.count + g_df - 1) / g_df);
+        }
+        g_df = (b.count + group - 1) / group;
+        grid = dim3((unsigned)(tiles * split), (unsigned)g_df);
         const size_t duos = (size_t)(group + 1) / 2;
-        const size_t smem = (size_t)(GP_NB + cols) * DB * sizeof(double) +
-                            (duos * DB * (m || pair ? 3 : 2) + kExpTab) * sizeof(dfl) + duos * sizeof(int2);
+        const size_t smem = (size_t)(GP_NB + cols) * DB * sizeof(double) + duos * duo + kExpTab * sizeof(dfl) +
+                            duos * sizeof(int2);
         cudaError_t e;
         if (cols == 16) {
 #define GP_ASM_EXACT(D)                                                                                  \

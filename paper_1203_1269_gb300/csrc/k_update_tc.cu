@@ -1,5 +1,5 @@
 // k_update_tc.cu -- the trailing update of the double-precision Cholesky,
-// A_IK -= L_IJ L_KJ^T, as exact products of bf16 slices on the tensor cores
+// A_IK -= L_IJ L_KJ^T, as exact products of 8-bit digits on the tensor cores
 // (after Ozaki, Ogita, Oishi & Rump, "Error-free transformations of matrix
 // multiplication by using fast routines of matrix multiplication", Numer.
 // Algorithms 59, 2012).
@@ -32,7 +32,7 @@
 // Measured, max |R - L L'| at n = 900, d = 2: 1.3e-16 (1.6e-15 with double
 // multiply-adds on the FP64 pipe).  Twelve candidates at n = 4064: 270 ms with
 // the updates on the FP64 pipe (256 of them), 28.8 ms now (updates 19); the
-// double fit at n = 4064 54.6 -> 10.5 ms.
+// double fit at n = 4064 54.6 -> 10.5 ms (9.6 with its launches set up ahead).
 #include "mixed_common.cuh"
 
 namespace gp {

@@ -1,7 +1,7 @@
 """The split path's assembly with two candidates in a pair of FP32 lanes
 against single candidates: the same bits, whatever the partner (none, refused,
 or with entries that underflow), for every family, dimension and exponent
-mode."""
+mode, and with more candidates than the theta of one group holds."""
 import numpy as np
 import pytest
 
@@ -27,6 +27,7 @@ def gp():
 
 @pytest.mark.parametrize("corr,n,d,p,T", [("powexp", 1100, 1, 1.95, 33), ("powexp", 1100, 6, 1.0, 32),
                                           ("powexp", 1153, 10, 2.0, 35), ("powexp", 1100, 11, 1.5, 33),
+                                          ("powexp", 1030, 10, 1.95, 1701), ("matern32", 1030, 16, 1.0, 1031),
                                           ("matern12", 130, 3, 1.0, 5), ("matern32", 129, 8, 1.0, 4),
                                           ("matern52", 300, 16, 1.0, 7)])
 def test_pairs_give_the_single_candidate_bits(gp, corr, n, d, p, T):
