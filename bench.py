@@ -349,12 +349,16 @@ def run_gp(args):
         upd_ms, upd_n = phases["update"]
         flops = update_flops(w.n) * w.T * args.steps
         achieved = flops / (upd_ms / 1e3) / 1e12 if upd_ms > 0 else None
-        fp64_peak = fp64_dgemm_tflops(dev)
-        roof = {"kernel": "k_update_f64", "bound": "alu", "achieved": achieved, "peak": fp64_peak,
-                "unit": "TFLOP/s", "frac": (achieved / fp64_peak) if achieved else None,
-                "traffic": stored_traffic("k_update_f64", ["k_chol_f64.cu"]),
-                "peak_source": "FP64 dense, measured in this run: cuBLAS DGEMM (torch.matmul, "
-                               "4096^3, best of 5, CUDA events)",
+        # from three block columns on, each update runs as 34 products of
+        # 8-bit digits on the tensor cores
+        digits = 34
+        peak = pk["bf16_tflops_sustained"]
+        roof = {"kernel": "k_update_f64_tc", "bound": "tensor", "achieved": achieved * digits if achieved else None,
+                "peak": peak, "unit": "TFLOP/s", "frac": (achieved * digits / peak) if achieved else None,
+                "traffic": stored_traffic("k_update_f64_tc", ["k_update_tc.cu", "mixed_common.cuh"]),
+                "peak_source": ("bf16 dense sustained, measured (MEASURED_PEAKS.json)" if pk_src == "measured"
+                                else "bf16 dense sustained, fallback (1.7 PFLOP/s; MEASURED_PEAKS.json absent)"),
+                "update_fp64_tflops": achieved, "fp64_dgemm_tflops_measured": fp64_dgemm_tflops(dev),
                 "launches_timed": upd_n, "avg_launch_ms": upd_ms / max(upd_n, 1),
                 "algorithmic_flops_per_launch": flops / max(upd_n, 1)}
     else:
