@@ -184,6 +184,21 @@ __device__ __forceinline__ df2 df2_mul(f32x2 an, df2 a, df2 b) {
     return r;
 }
 
+// c + l x for one l and two x: bit for bit df_fma(l, x, c) of each half
+// (xn = -x.hi)
+__device__ __forceinline__ df2 df2_fma_shared(dfl l, df2 x, f32x2 xn, df2 c) {
+    const f32x2 lh = f2_pack(l.hi, l.hi), ll = f2_pack(l.lo, l.lo);
+    const f32x2 pn = f2_mul(lh, xn);
+    f32x2 e = f2_fma(lh, x.hi, pn);
+    e = f2_fma(lh, x.lo, e);
+    e = f2_fma(ll, x.hi, e);
+    f32x2 s, t;
+    f2_two_diff(c.hi, pn, s, t);
+    df2 r;
+    f2_fast_two_sum(s, f2_add(t, f2_add(c.lo, e)), r.hi, r.lo);
+    return r;
+}
+
 __device__ __forceinline__ dfl df2_first(df2 v) { return {f2_first(v.hi), f2_first(v.lo)}; }
 __device__ __forceinline__ dfl df2_second(df2 v) { return {f2_second(v.hi), f2_second(v.lo)}; }
 __device__ __forceinline__ df2 df2_pack(dfl a, dfl b) { return {f2_pack(a.hi, b.hi), f2_pack(a.lo, b.lo)}; }

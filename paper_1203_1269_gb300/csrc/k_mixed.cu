@@ -864,8 +864,31 @@ __global__ void k_rhs_init(MixedBatch b) {
 // candidates run along x): their diagonal step ends while the other tiles are
 // worked on.  Each step of 100 candidates at n = 1024: 42 -> 22 us forward,
 // 35 -> 24 backward; the solve phase there .82 -> .56 ms, 32 x 1448 1.07 ->
-// .64, 8 x 16384 17.4 -> 10.7, 256 x 4000 15.5 -> 14.4 (the residual's 6.1
-// of them, and 2.4 a pass what the factor's bytes take).
+// .64, 8 x 16384 17.4 -> 10.7, 256 x 4000 15.5 -> 14.4 (2.4 a pass is what the
+// factor's bytes take).
+// N entries of both right-hand sides side by side, for the paired FP32
+// instructions: hl = {hi of both, lo of both}, and the negated high words.  A
+// product with L then takes half the issue slots of two scalar ones (the
+// residual issued in 67 % of the cycles, the forward tiles in 70): the solve
+// phase of 256 x 4000 14.4 -> 13.3 ms, 128 x 2047 2.11 -> 1.95, 8 x 16384 10.7 ->
+// 10.1, 100 x 1024 .565 -> .525; the same bits.
+template <int N>
+struct SubX {
+    float4 hl[N];
+    float2 n[N];
+    __device__ __forceinline__ void set(int i, int k, dfl v) {
+        float* p = reinterpret_cast<float*>(hl + i);
+        p[k] = v.hi;
+        p[2 + k] = v.lo;
+        reinterpret_cast<float*>(n + i)[k] = -v.hi;
+    }
+    __device__ __forceinline__ df2 fma(dfl l, int i, df2 c) const {
+        const float4 x = hl[i];
+        const float2 m = n[i];
+        return df2_fma_shared(l, df2{f2_pack(x.x, x.y), f2_pack(x.z, x.w)}, f2_pack(m.x, m.y), c);
+    }
+};
+
 constexpr int kSubThreads = 256;
 // Entries that a thread has in flight: partial-product tiles, W and L, and the
 // CTAs per SM that its registers leave room for.
@@ -940,32 +963,29 @@ __device__ __forceinline__ void diag_load(const float2* W, float2 (&w)[N]) {
     for (int j = 0; j < N; ++j) w[j] = W[(size_t)j * GP_NB];
 }
 
-// Products of 64 entries of W with both right-hand sides (xs0, xs1: 64 terms
-// each), even and odd terms apart.  w holds the first N entries; each
+// Products of 64 entries of W with both right-hand sides (from entry
+// `first` of xs), even and odd terms apart.  w holds the first N entries; each
 // batch is loaded while the one before it is multiplied: left to the
 // compiler, every load waited for L2 on its own (18 to 36 thousand clocks for
 // the 64 terms, against 5.6 thousand that the products issue in).
 template <int N>
-__device__ __forceinline__ void diag_products(const float2* W, float2 (&w)[N], const dfl* xs0, const dfl* xs1,
+__device__ __forceinline__ void diag_products(const float2* W, float2 (&w)[N], const SubX<GP_NB>& xs, int first,
                                               dfl& s0, dfl& s1) {
-    dfl a0 = {0.f, 0.f}, a1 = {0.f, 0.f}, b0 = {0.f, 0.f}, b1 = {0.f, 0.f};
+    df2 even = {f2_pack(0.f, 0.f), f2_pack(0.f, 0.f)}, odd = even;
 #pragma unroll 1
     for (int c0 = 0; c0 < GP_NB / 2; c0 += N) {
         float2 next[N];
         if (c0 + N < GP_NB / 2) diag_load(W + (size_t)(c0 + N) * GP_NB, next);
 #pragma unroll
         for (int j = 0; j < N; j += 2) {
-            const dfl w0 = {w[j].x, w[j].y}, w1 = {w[j + 1].x, w[j + 1].y};
-            a0 = df_fma(w0, xs0[c0 + j], a0);
-            b0 = df_fma(w0, xs1[c0 + j], b0);
-            a1 = df_fma(w1, xs0[c0 + j + 1], a1);
-            b1 = df_fma(w1, xs1[c0 + j + 1], b1);
+            even = xs.fma(dfl{w[j].x, w[j].y}, first + c0 + j, even);
+            odd = xs.fma(dfl{w[j + 1].x, w[j + 1].y}, first + c0 + j + 1, odd);
         }
 #pragma unroll
         for (int j = 0; j < N; ++j) w[j] = next[j];
     }
-    s0 = df_add(a0, a1);
-    s1 = df_add(b0, b1);
+    s0 = df_add(df2_first(even), df2_first(odd));
+    s1 = df_add(df2_second(even), df2_second(odd));
 }
 
 // forward, block J: z_J <- W_J (z_J - sum_{K<J} L_JK z_K), W_J = L_JJ^-1.
@@ -975,7 +995,7 @@ __device__ __forceinline__ void diag_products(const float2* W, float2 (&w)[N], c
 // fixed order.  W is zero above its diagonal; a fixed trip count.
 // part: 2 x 2 x 128 scratch.
 template <typename V>
-__device__ __forceinline__ void fwd_diag_step(const MixedBatch& b, int t, int c0, int J, dfl (*rhs)[GP_NB],
+__device__ __forceinline__ void fwd_diag_step(const MixedBatch& b, int t, int c0, int J, SubX<GP_NB>& rhs,
                                               dfl (*part)[2][GP_NB]) {
     const int r = threadIdx.x & 127, h = threadIdx.x >> 7;
     float2* zr = zcol(b, t, c0 + h) + (size_t)J * GP_NB + r;     // half h finishes right-hand side h
@@ -988,10 +1008,10 @@ __device__ __forceinline__ void fwd_diag_step(const MixedBatch& b, int t, int c0
     part[h][0][r] = p0;
     part[h][1][r] = p1;
     __syncthreads();
-    rhs[h][r] = df_sub(z, df_add(part[0][h][r], part[1][h][r]));
+    rhs.set(r, h, df_sub(z, df_add(part[0][h][r], part[1][h][r])));
     __syncthreads();
     dfl s0, s1;
-    diag_products(W, w, rhs[0] + 64 * h, rhs[1] + 64 * h, s0, s1);
+    diag_products(W, w, rhs, 64 * h, s0, s1);
     part[h][0][r] = s0;
     part[h][1][r] = s1;
     __syncthreads();
@@ -1000,7 +1020,7 @@ __device__ __forceinline__ void fwd_diag_step(const MixedBatch& b, int t, int c0
 
 __global__ void __launch_bounds__(kSubThreads) k_fwd_diag(MixedBatch b, int c0, int J) {
     grid_dependency();
-    __shared__ dfl rhs[2][GP_NB];
+    __shared__ SubX<GP_NB> rhs;
     __shared__ dfl part[2][2][GP_NB];
     const int t = blockIdx.x;
     if (!sub_active(b, t)) return;
@@ -1013,9 +1033,9 @@ __global__ void __launch_bounds__(kSubThreads) k_fwd_diag(MixedBatch b, int c0, 
 template <typename V>
 __global__ void __launch_bounds__(kSubThreads, V::kFwd) k_fwd_tiles(MixedBatch b, int c0, int J) {
     grid_dependency();
-    __shared__ dfl xs[2][GP_NB / 2];
+    __shared__ SubX<GP_NB / 2> xs;
     __shared__ dfl part[2][2][GP_NB];
-    __shared__ dfl rhs[2][GP_NB];
+    __shared__ SubX<GP_NB> rhs;
     const int t = blockIdx.x;
     if (!sub_active(b, t)) return;
     const int I = J + 1 + (blockIdx.y >> 1), h = blockIdx.y & 1;
@@ -1028,9 +1048,10 @@ __global__ void __launch_bounds__(kSubThreads, V::kFwd) k_fwd_tiles(MixedBatch b
     float2 l[V::kL];
 #pragma unroll
     for (int c = 0; c < V::kL; ++c) l[c] = __ldg(L + (size_t)c * GP_NB);
-    if (tid < GP_NB) xs[tid >> 6][tid & 63] = df_load(zcol(b, t, c0 + (tid >> 6)) + (size_t)J * GP_NB + 64 * h + (tid & 63));
+    if (tid < GP_NB)
+        xs.set(tid & 63, tid >> 6, df_load(zcol(b, t, c0 + (tid >> 6)) + (size_t)J * GP_NB + 64 * h + (tid & 63)));
     __syncthreads();
-    dfl u0 = {0.f, 0.f}, u1 = {0.f, 0.f};
+    df2 u = {f2_pack(0.f, 0.f), f2_pack(0.f, 0.f)};
 #pragma unroll 1
     for (int q = 0; q < 32; q += V::kL) {
         float2 next[V::kL];
@@ -1039,16 +1060,12 @@ __global__ void __launch_bounds__(kSubThreads, V::kFwd) k_fwd_tiles(MixedBatch b
             for (int c = 0; c < V::kL; ++c) next[c] = __ldg(L + (size_t)(q + V::kL + c) * GP_NB);
         }
 #pragma unroll
-        for (int c = 0; c < V::kL; ++c) {
-            const dfl ld = {l[c].x, l[c].y};
-            u0 = df_fma(ld, xs[0][32 * g + q + c], u0);
-            u1 = df_fma(ld, xs[1][32 * g + q + c], u1);
-        }
+        for (int c = 0; c < V::kL; ++c) u = xs.fma(dfl{l[c].x, l[c].y}, 32 * g + q + c, u);
 #pragma unroll
         for (int c = 0; c < V::kL; ++c) l[c] = next[c];
     }
-    part[g][0][r] = u0;
-    part[g][1][r] = u1;
+    part[g][0][r] = df2_first(u);
+    part[g][1][r] = df2_second(u);
     __syncthreads();
     const int k = tid >> 7;
     df_store(rp_part(b, t, I, J) + (h * 2 + k) * GP_NB + r, df_add(part[0][k][r], part[1][k][r]));
@@ -1062,7 +1079,7 @@ __global__ void __launch_bounds__(kSubThreads, V::kFwd) k_fwd_tiles(MixedBatch b
 // With add_to >= 0 the result is also added into (add_to, add_to + 1).
 template <typename V>
 __device__ __forceinline__ void bwd_diag_step(const MixedBatch& b, int t, int c0, int K, int add_to,
-                                              dfl (*rhs)[GP_NB], dfl (*part)[2][GP_NB]) {
+                                              SubX<GP_NB>& rhs, dfl (*part)[2][GP_NB]) {
     const int c = threadIdx.x & 127, h = threadIdx.x >> 7;
     float2* zc = zcol(b, t, c0 + h) + (size_t)K * GP_NB + c;     // half h finishes right-hand side h
     float2* acc = add_to >= 0 ? zcol(b, t, add_to + h) + (size_t)K * GP_NB + c : nullptr;
@@ -1077,10 +1094,10 @@ __device__ __forceinline__ void bwd_diag_step(const MixedBatch& b, int t, int c0
     part[h][0][c] = p0;
     part[h][1][c] = p1;
     __syncthreads();
-    rhs[h][c] = df_sub(z, df_add(part[0][h][c], part[1][h][c]));
+    rhs.set(c, h, df_sub(z, df_add(part[0][h][c], part[1][h][c])));
     __syncthreads();
     dfl s0, s1;
-    diag_products(W, w, rhs[0] + 64 * h, rhs[1] + 64 * h, s0, s1);
+    diag_products(W, w, rhs, 64 * h, s0, s1);
     part[h][0][c] = s0;
     part[h][1][c] = s1;
     __syncthreads();
@@ -1091,7 +1108,7 @@ __device__ __forceinline__ void bwd_diag_step(const MixedBatch& b, int t, int c0
 
 __global__ void __launch_bounds__(kSubThreads) k_bwd_diag(MixedBatch b, int c0, int K, int add_to) {
     grid_dependency();
-    __shared__ dfl rhs[2][GP_NB];
+    __shared__ SubX<GP_NB> rhs;
     __shared__ dfl part[2][2][GP_NB];
     const int t = blockIdx.x;
     if (!sub_active(b, t)) return;
@@ -1107,9 +1124,9 @@ template <typename V>
 __global__ void __launch_bounds__(kSubThreads, V::kBwd) k_bwd_tiles(MixedBatch b, int c0, int K, int add_to) {
     grid_dependency();
     extern __shared__ dfl T[];                  // GP_NB x kBwdTs
-    __shared__ dfl xs[2][GP_NB / 2];
+    __shared__ SubX<GP_NB / 2> xs;
     __shared__ dfl part[2][2][GP_NB];
-    __shared__ dfl rhs[2][GP_NB];
+    __shared__ SubX<GP_NB> rhs;
     const int t = blockIdx.x;
     if (!sub_active(b, t)) return;
     const int I = K - 1 - (blockIdx.y >> 1), h = blockIdx.y & 1;
@@ -1117,7 +1134,8 @@ __global__ void __launch_bounds__(kSubThreads, V::kBwd) k_bwd_tiles(MixedBatch b
     // W_{K-1} (row-major) heads for L2 for the next diagonal step
     if (tid == 0 && I == K - 1 && h == 0)
         prefetch_l2(b.WR + (size_t)t * b.wt_stride + (size_t)(K - 1) * GP_TILE_ELEMS, GP_TILE_ELEMS * sizeof(float2));
-    if (tid < GP_NB) xs[tid >> 6][tid & 63] = df_load(zcol(b, t, c0 + (tid >> 6)) + (size_t)K * GP_NB + 64 * h + (tid & 63));
+    if (tid < GP_NB)
+        xs.set(tid & 63, tid >> 6, df_load(zcol(b, t, c0 + (tid >> 6)) + (size_t)K * GP_NB + 64 * h + (tid & 63)));
     const float2* L = df_tile(b, b.A, t, K, I) + 64 * h;
 #pragma unroll
     for (int e = tid; e < 64 * GP_NB; e += kSubThreads) {
@@ -1128,14 +1146,11 @@ __global__ void __launch_bounds__(kSubThreads, V::kBwd) k_bwd_tiles(MixedBatch b
     __syncthreads();
     const int c = tid & 127, g = tid >> 7;
     const dfl* col = T + c * kBwdTs;
-    dfl s0 = {0.f, 0.f}, s1 = {0.f, 0.f};
+    df2 sum = {f2_pack(0.f, 0.f), f2_pack(0.f, 0.f)};
 #pragma unroll 8
-    for (int rr = 32 * g; rr < 32 * g + 32; ++rr) {
-        s0 = df_fma(col[rr], xs[0][rr], s0);
-        s1 = df_fma(col[rr], xs[1][rr], s1);
-    }
-    part[g][0][c] = s0;
-    part[g][1][c] = s1;
+    for (int rr = 32 * g; rr < 32 * g + 32; ++rr) sum = xs.fma(col[rr], rr, sum);
+    part[g][0][c] = df2_first(sum);
+    part[g][1][c] = df2_second(sum);
     __syncthreads();
     const int k = tid >> 7;
     df_store(rp_part(b, t, K, I) + (h * 2 + k) * GP_NB + c, df_add(part[0][k][c], part[1][k][c]));
@@ -1159,8 +1174,8 @@ static_assert(kRpTile == 2 * 2 * GP_NB + 2 * 2 * kResCols, "residual partial lay
 __global__ void __launch_bounds__(kResThreads) k_resid_tiles(MixedBatch b) {
     grid_dependency();
     extern __shared__ dfl T[];                  // kResCols x kTs
-    __shared__ dfl xa[2][kResCols];             // x_J on this half's columns
-    __shared__ dfl xb[2][GP_NB];                // x_I
+    __shared__ SubX<kResCols> xa;               // x_J on this half's columns
+    __shared__ SubX<GP_NB> xb;                  // x_I
     __shared__ dfl part[2 * 2 * GP_NB];           // U: [2][2][128], then V: [4][2][64]
     const int t = blockIdx.y;
     if (b.st[t].status != GP_OK || b.st[t].refine_done) return;
@@ -1173,8 +1188,9 @@ __global__ void __launch_bounds__(kResThreads) k_resid_tiles(MixedBatch b) {
     }
     const int I = J + rem;
     const int tid = threadIdx.x;
-    if (tid < 2 * kResCols) xa[tid >> 6][tid & 63] = df_load(zcol(b, t, tid >> 6) + J * GP_NB + hc * kResCols + (tid & 63));
-    xb[tid >> 7][tid & 127] = df_load(zcol(b, t, tid >> 7) + I * GP_NB + (tid & 127));
+    if (tid < 2 * kResCols)
+        xa.set(tid & 63, tid >> 6, df_load(zcol(b, t, tid >> 6) + J * GP_NB + hc * kResCols + (tid & 63)));
+    xb.set(tid & 127, tid >> 7, df_load(zcol(b, t, tid >> 7) + I * GP_NB + (tid & 127)));
     const float2* src = df_tile(b, b.Rc, t, I, J) + (size_t)hc * kResCols * GP_NB;
 #pragma unroll
     for (int e = tid; e < kResCols * GP_NB; e += kResThreads) cp_async8(T + (e >> 7) * kTs + (e & 127), src + e);
@@ -1184,15 +1200,11 @@ __global__ void __launch_bounds__(kResThreads) k_resid_tiles(MixedBatch b) {
     {
         // U: thread (r, h) takes the columns 32h .. 32h + 31 of the half
         const int r = tid & 127, h = tid >> 7;
-        dfl u0 = {0.f, 0.f}, u1 = {0.f, 0.f};
-#pragma unroll 4
-        for (int c = 32 * h; c < 32 * h + 32; ++c) {
-            const dfl v = T[c * kTs + r];
-            u0 = df_fma(v, xa[0][c], u0);
-            u1 = df_fma(v, xa[1][c], u1);
-        }
-        part[(h * 2 + 0) * GP_NB + r] = u0;
-        part[(h * 2 + 1) * GP_NB + r] = u1;
+        df2 u = {f2_pack(0.f, 0.f), f2_pack(0.f, 0.f)};
+#pragma unroll 8
+        for (int c = 32 * h; c < 32 * h + 32; ++c) u = xa.fma(T[c * kTs + r], c, u);
+        part[(h * 2 + 0) * GP_NB + r] = df2_first(u);
+        part[(h * 2 + 1) * GP_NB + r] = df2_second(u);
     }
     __syncthreads();
     {
@@ -1205,14 +1217,11 @@ __global__ void __launch_bounds__(kResThreads) k_resid_tiles(MixedBatch b) {
         // V: thread (c, h) takes the rows 32h .. 32h + 31 of column c
         const int c = tid & 63, h = tid >> 6;
         const dfl* col = T + c * kTs;
-        dfl s0 = {0.f, 0.f}, s1 = {0.f, 0.f};
-#pragma unroll 4
-        for (int r = 32 * h; r < 32 * h + 32; ++r) {
-            s0 = df_fma(col[r], xb[0][r], s0);
-            s1 = df_fma(col[r], xb[1][r], s1);
-        }
-        part[(h * 2 + 0) * kResCols + c] = s0;
-        part[(h * 2 + 1) * kResCols + c] = s1;
+        df2 sum = {f2_pack(0.f, 0.f), f2_pack(0.f, 0.f)};
+#pragma unroll 8
+        for (int r = 32 * h; r < 32 * h + 32; ++r) sum = xb.fma(col[r], r, sum);
+        part[(h * 2 + 0) * kResCols + c] = df2_first(sum);
+        part[(h * 2 + 1) * kResCols + c] = df2_second(sum);
     }
     __syncthreads();
     if (tid < 2 * kResCols) {
