@@ -214,13 +214,14 @@ __global__ void __launch_bounds__(ER ? kGemmThreadsER : kGemmThreads, 1)
         }
     };
 
-    // The diagonal step of a later block column may run beside kind 4 and fail a
-    // candidate: its warps must agree on the tiles they skip, so they go by
-    // what the CTA read at its start.
+    // In a look-ahead a diagonal step may fail a candidate beside this kernel, or
+    // another of these kernels give one up: the warps must agree on the tiles
+    // they skip, so they go by what the CTA read at its start.
     __shared__ uint8_t live[kLookaheadMixedMax];
-    if (MODE == 1 && kind == 4)
+    const bool snapshot = b.lookahead > 0;
+    if (snapshot)
         for (int i = threadIdx.x; i < b.count; i += blockDim.x) live[i] = b.st[i].status == GP_OK;
-    auto alive = [&](int t) { return (MODE == 1 && kind == 4) ? live[t] != 0 : b.st[t].status == GP_OK; };
+    auto alive = [&](int t) { return snapshot ? live[t] != 0 : b.st[t].status == GP_OK; };
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {

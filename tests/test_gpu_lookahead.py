@@ -50,3 +50,27 @@ def test_lookahead_gives_the_batch_bits(gp, n, few, tile):
         for k in KEYS:
             assert np.array_equal(out[k].cpu().numpy(), whole[k][:few], equal_nan=True), k
     plan.free()
+
+
+def test_timeout_under_lookahead_reports_and_recovers(gp):
+    """A wait that nothing ends (the 5 ms hook) in the split GEMMs of a factor
+    with look-ahead: the candidates it gives up come back GP_ETIMEOUT, the
+    others with their bits, and the next call is normal."""
+    ctx = gp.Context(0)
+    g = np.random.default_rng(11)
+    x = dev(inputs.random_lhd(g, 1500, 3))
+    y = dev(inputs.y_sinsum(x.cpu().numpy()))
+    th = dev(inputs.log_uniform_thetas(g, 8, 3, lo=0.0, hi=1.0))
+    good = ctx.nll_batch(x, y, th, 1.95, 1e-6, "mixed")
+    try:
+        ctx.set_options(inject_timeout=1)
+        bad = ctx.nll_batch(x, y, th, 1.95, 1e-6, "mixed")
+        st = bad["status"].cpu().numpy()
+    finally:
+        ctx.set_options(inject_timeout=0)
+    assert (st == -5).any() and np.isin(st, (0, -5)).all()
+    assert np.isnan(bad["nll"].cpu().numpy()[st == -5]).all()
+    assert np.array_equal(bad["nll"].cpu().numpy()[st == 0], good["nll"].cpu().numpy()[st == 0])
+    again = ctx.nll_batch(x, y, th, 1.95, 1e-6, "mixed")
+    for k in KEYS:
+        assert np.array_equal(again[k].cpu().numpy(), good[k].cpu().numpy()), k
