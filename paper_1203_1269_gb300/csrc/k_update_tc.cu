@@ -12,8 +12,9 @@
 // (balanced digits), each digit exact in fp16.  The product groups S_g =
 // sum_{a+b=g} q_a q_b', g = 0 .. 7, summed over the panel's 128 columns in fp32
 // are integers below 2^24, hence exact (at most 2^21 for a pair of lower
-// digits, of which a group has six at most, and less than 2^20 by
-// Cauchy-Schwarz for a pair with q_0, since the rows of L have norm 1); what
+// digits, of which a group has six at most, and less than 2^18.6 by
+// Cauchy-Schwarz for a pair with q_0, since the rows of L have norm 1; the
+// inverse's operands, which have no such norm: at combine() below); what
 // is left out, a + b >= 8, is below 2^-66 of 1 per term.  The dropped part of l
 // is at most 2^-56, so all panels together leave an error of about 2^-56 in
 // an entry of A, where each IEEE subtraction from A rounds to 2^-53 of it:
@@ -141,18 +142,30 @@ __device__ __forceinline__ void tmem_ld4(uint32_t taddr, float* v) {
 }
 
 // sum_g S_g 256^(5 - g), groups 6 and 7 rounded: the product of the two rows
-// in units of 2^-56.  Groups 0 .. 2 (below 2^22) and 6, 7 (as one rounded
-// float) turn into integers by an addition; only 3 .. 5 need the conversion
-// instruction, an eighth of an addition's rate.
+// in units of 2^-56 (below 2^63 for 128 terms under 1; the high word wraps on
+// the way).  A group turns into an integer by the conversion instruction, or, an
+// eighth of its cost, by adding 1.5 2^23, which is exact up to 2^22.  Groups 6 and 7
+// go as one rounded float, |S_6 + S_7 / 256| 2^-8 < 2^17.  The others:
+//
+//   L L' (FACTOR)  both operands' rows have norm 1, so by Cauchy-Schwarz a pair
+//                  with q_0 stays below 2^18.6 and a pair of lower digits below
+//                  2^21: S_0 .. S_2 < 2^21.5, S_3 .. S_5 < 2^23.2.
+//   W S, L X, X'X  (the inverse) only |q_0| <= 256, |q_a| <= 128 hold, and they
+//                  are reached: a column of L^-1 next to a dominant nugget is
+//                  nearly constant over a block, so that S_0 of X'X comes
+//                  close to 128 2^16 = 2^23.  S_1 <= 2^23, S_2 <= 2^23.4,
+//                  S_3 .. S_5 <= 2^24, so groups 0 .. 5 by the instruction; S_6 <=
+//                  2^24.2, rounded in any case.
+template <bool FACTOR>
 __device__ __forceinline__ long long combine(const float (&s)[kNG]) {
     constexpr float kRound = 12582912.f;                  // 1.5 2^23, unit 1
     constexpr int kBits = 0x4b400000;
-    const int t0 = __float_as_int(__fadd_rn(s[0], kRound)) - kBits;
-    const int t1 = __float_as_int(__fadd_rn(s[1], kRound)) - kBits;
-    const int t2 = __float_as_int(__fadd_rn(s[2], kRound)) - kBits;
+    auto whole = [](float v) { return FACTOR ? __float_as_int(__fadd_rn(v, kRound)) - kBits : __float2int_rn(v); };
+    const unsigned t0 = whole(s[0]), t1 = whole(s[1]);
+    const int t2 = whole(s[2]);
     const float low = __fmaf_rn(s[7], 0x1p-8f, s[6]);
     const int t6 = __float_as_int(__fmaf_rn(low, 0x1p-8f, kRound)) - kBits;
-    long long v = (long long)(t0 * 256 + t1) << 32;
+    long long v = (long long)((unsigned long long)(t0 * 256u + t1) << 32);
     v += (long long)t2 * (1 << 24);
     v += (long long)__float2int_rn(s[3]) * (1 << 16);
     v += (long long)__float2int_rn(s[4]) * (1 << 8);
@@ -318,7 +331,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     float u[kNG];
 #pragma unroll
                     for (int g = 0; g < kNG; ++g) u[g] = s[g][j];
-                    v[c + j] = combine(u);
+                    v[c + j] = combine<!kInv>(u);
                 }
             }
             tc_fence_before();
