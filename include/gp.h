@@ -132,9 +132,11 @@ typedef struct {
                              (128-wide tiles, the last group rounded) or 7 (64-wide
                              tiles, every group exact) */
     int inject_timeout;   /* test hook, default 0, bits: 1 = the first CTA of the first
-                             trailing-update launch of each GP_MIXED batch waits 5 ms on
-                             a barrier nothing signals, gives up, and the instances it
-                             would have updated come back GP_ETIMEOUT; 2 = the first CTA
+                             trailing-update launch of each GP_MIXED batch, of each
+                             double-precision one from three block columns on, and of a
+                             gradient's inverse waits 5 ms on a barrier nothing signals,
+                             gives up, and the instances it would have updated come back
+                             GP_ETIMEOUT; 2 = the first CTA
                              of each tensor-core variance pass of gp_predict does the
                              same and its points' s2 come back NaN (the bounded-wait
                              failure paths, exercised without faulting the GPU) */

@@ -602,6 +602,7 @@ int fp64_nll_batch(gp_ctx* ctx, int n, int d, const double* x, const double* y, 
         b.n = n; b.d = d; b.nt = nt; b.count = cnt; b.corr = ctx->opt.correlation;
         b.p = p; b.delta = delta; b.x = x; b.y = y; b.theta = theta + (size_t)c0 * d;
         b.A = A; b.inst_stride = a_bytes / sizeof(double); b.st = st;
+        b.inject_timeout = ctx->opt.inject_timeout & 1;
         {
             PhaseScope ps(ctx, GP_PHASE_ASSEMBLE, 2);
             GP_CUDA(ctx, gp::launch_validate_theta(b, ctx->stream));
@@ -1324,6 +1325,7 @@ int gp_cholesky(gp_ctx* ctx, int n, int d, const double* x, const double* theta,
         gp::Batch b{};
         b.n = n; b.d = d; b.nt = nt; b.count = 1; b.p = p; b.delta = delta; b.corr = ctx->opt.correlation;
         b.x = x; b.y = nullptr; b.theta = theta; b.A = L; b.inst_stride = gp::packed_elems(n); b.st = st;
+        b.inject_timeout = ctx->opt.inject_timeout & 1;
         {
             PhaseScope ps(ctx, GP_PHASE_ASSEMBLE, 2);
             GP_CUDA(ctx, gp::launch_validate_theta(b, ctx->stream));
@@ -1403,6 +1405,7 @@ int gp_nll_grad_batch(gp_ctx* ctx, int n, int d, const double* x, const double* 
         b.n = n; b.d = d; b.nt = nt; b.count = cnt; b.corr = ctx->opt.correlation;
         b.p = p; b.delta = delta; b.x = x; b.y = y; b.theta = theta + (size_t)c0 * d;
         b.A = A; b.inst_stride = a_bytes / sizeof(double); b.st = st;
+        b.inject_timeout = ctx->opt.inject_timeout & 1;
         {
             PhaseScope ps(ctx, GP_PHASE_ASSEMBLE, 2);
             GP_CUDA(ctx, gp::launch_validate_theta(b, ctx->stream));
@@ -1418,8 +1421,8 @@ int gp_nll_grad_batch(gp_ctx* ctx, int n, int d, const double* x, const double* 
                                              ctx->stream));
         }
         int kernels = 0;
-        cudaError_t e = gp::launch_grad(b, Z, zs, X, Ri, status + c0, grad + (size_t)c0 * d,
-                                        ctx->stream, &kernels);
+        cudaError_t e = gp::launch_grad(b, Z, zs, X, Ri, status + c0, nll + c0,
+                                        grad + (size_t)c0 * d, ctx->stream, &kernels);
         ctx->launches += kernels;
         ctx->phase_launches[GP_PHASE_SOLVE] += kernels;
         if (e != cudaSuccess) return fail(ctx, GP_ECUDA, "gradient launch: %s", cudaGetErrorString(e));
@@ -1714,6 +1717,7 @@ int gp_fit(gp_ctx* ctx, int n, int d, const double* x, const double* y, const do
     b.n = n; b.d = d; b.nt = m->nt; b.count = 1; b.p = p; b.delta = delta; b.corr = m->corr;
     b.x = x; b.y = y; b.theta = m->theta; b.A = m->L; b.inst_stride = gp::packed_elems(n);
     b.st = m->st;
+    b.inject_timeout = ctx->opt.inject_timeout & 1;
     {
         PhaseScope ps(ctx, GP_PHASE_ASSEMBLE, 2);
         if (gp::launch_validate_theta(b, ctx->stream) || gp::launch_assemble_tiles(b, ctx->stream))

@@ -93,6 +93,7 @@ struct Batch {
     InstState* st;                // count
     int asm_cols;                 // double-float assembly: tile columns per CTA (16 or 32)
     int corr;                     // gp_correlation
+    int inject_timeout;           // test hook: one tensor-core CTA waits on a barrier nothing signals
 };
 
 // Split-precision path: per-instance buffers (double-float tiles, bf16
@@ -368,7 +369,7 @@ cudaError_t launch_df_forward(const MixedBatch& b, int c0, int init, cudaStream_
 cudaError_t launch_rhs_init(const MixedBatch& b, cudaStream_t s);
 cudaError_t launch_df_backward(const MixedBatch& b, int c0, int add_to, cudaStream_t s);
 cudaError_t launch_df_residual(const MixedBatch& b, cudaStream_t s);
-cudaError_t launch_grad(const Batch& b, double* Z, size_t zs, double* X, double* Ri, const int* status,
+cudaError_t launch_grad(const Batch& b, double* Z, size_t zs, double* X, double* Ri, int* status, double* nll,
                         double* grad, cudaStream_t s, int* kernels);
 cudaError_t launch_norm1(const MixedBatch& b, cudaStream_t s);
 cudaError_t launch_hager(const MixedBatch& b, int phase, double* cond, cudaStream_t s);

@@ -243,14 +243,20 @@ __global__ void __launch_bounds__(kThreads) k_grad_tiles(Batch b, const double* 
 
 // grad[t][k] = the sum of the tile parts' sums, in a fixed order (a warp per k);
 // NaN where the likelihood itself failed (status: the finalize kernel's, which
-// also flags Q = 0)
-__global__ void k_grad_reduce(Batch b, int parts, const int* status, double* grad) {
+// also flags Q = 0).  A candidate that a kernel of the inverse gave up after
+// finalize has its status and -2logL corrected here.
+__global__ void k_grad_reduce(Batch b, int parts, int* status, double* nll, double* grad) {
     grid_dependency();
     const int t = blockIdx.x, d = b.d;
     const int k = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (k >= d) return;
     if (b.st[t].status != GP_OK || status[t] != GP_OK) {
-        if (lane == 0) grad[(size_t)t * d + k] = __longlong_as_double(0x7ff8000000000000LL);
+        const double nan = __longlong_as_double(0x7ff8000000000000LL);
+        if (lane == 0) grad[(size_t)t * d + k] = nan;
+        if (threadIdx.x == 0 && b.st[t].status == GP_ETIMEOUT && status[t] != GP_ETIMEOUT) {
+            status[t] = GP_ETIMEOUT;
+            nll[t] = nan;
+        }
         return;
     }
     const double* partial = b.A + (size_t)t * b.inst_stride;
@@ -262,7 +268,7 @@ __global__ void k_grad_reduce(Batch b, int parts, const int* status, double* gra
 
 }  // namespace
 
-cudaError_t launch_grad(const Batch& b, double* Z, size_t zs, double* X, double* Ri, const int* status,
+cudaError_t launch_grad(const Batch& b, double* Z, size_t zs, double* X, double* Ri, int* status, double* nll,
                         double* grad, cudaStream_t s, int* kernels) {
     const int nt = b.nt;
     int k = 0;
@@ -307,7 +313,7 @@ cudaError_t launch_grad(const Batch& b, double* Z, size_t zs, double* X, double*
     else               GP_GRAD_TILES(16);
 #undef GP_GRAD_TILES
     ++k;
-    launch_chained(ahead_f64(b), k_grad_reduce, b.count, 32 * 16, 0, s, b, parts, status, grad);
+    launch_chained(ahead_f64(b), k_grad_reduce, b.count, 32 * 16, 0, s, b, parts, status, nll, grad);
     ++k;
     if (kernels) *kernels = k;
     return cudaGetLastError();

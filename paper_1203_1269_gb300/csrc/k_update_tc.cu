@@ -212,6 +212,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     __shared__ __align__(8) uint64_t full_bar[2];
     __shared__ __align__(8) uint64_t empty_bar[2];
     __shared__ __align__(8) uint64_t tfull_bar, tempty_bar, drain_bar;
+    __shared__ __align__(8) uint64_t never_bar;   // never signalled: the timeout test waits on it
     __shared__ uint32_t tmem_base;
     __shared__ volatile int abort_flag;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -231,6 +232,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         mbar_init(&tfull_bar, 1);
         mbar_init(&tempty_bar, 32 * kEpiWarps);
         mbar_init(&drain_bar, 1);
+        mbar_init(&never_bar, 1);
         abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -442,6 +444,12 @@ __global__ void __launch_bounds__(kThreads, 1)
             int g = 0, i = 0;
             for (int w = next_live(blockIdx.x); w < total && !abort_flag; w = next_live(w + gridDim.x), ++i) {
                 if (i >= 1 && !mbar_wait(&tempty_bar, (i - 1) & 1, &abort_flag)) {
+                    abort_flag = 1;
+                    break;
+                }
+                // test hook: a wait that nothing ends, limited to 5 ms
+                if ((MODE == kFactorMode || MODE == kInvUpdate) && b.inject_timeout && J == 0 && blockIdx.x == 0 &&
+                    i == 0 && !mbar_wait(&never_bar, 0, &abort_flag, 5000000ull)) {
                     abort_flag = 1;
                     break;
                 }
