@@ -296,6 +296,10 @@ inline cudaError_t launch_chained(bool ahead, void (*kernel)(P...), dim3 grid, d
     return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
+// What the launch directly before has written is read by ordinary loads, after
+// this: that kernel may still run when this one starts, and __ldg wants data that
+// nothing writes while the kernel lives.  Older data may go through __ldg: the
+// launch before lets this one start only after its own wait.
 __device__ __forceinline__ void grid_dependency() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

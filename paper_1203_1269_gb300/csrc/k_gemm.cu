@@ -350,13 +350,16 @@ __global__ void __launch_bounds__(ER ? kGemmThreadsER : kGemmThreads, 1)
 #pragma unroll
             for (int cb = 0; cb < kPartCols; cb += CB2) {
                 float2 cv[CB2];
+                int eb[CB2];
+#pragma unroll
+                for (int j = 0; j < CB2; ++j) eb[j] = eBp[cb + j];
                 if (MODE == 1) {
 #pragma unroll
                     for (int j = 0; j < CB2; ++j) cv[j] = C[(size_t)(cbase + cb + j) * GP_NB + r];
                 }
 #pragma unroll
                 for (int j = 0; j < CB2; ++j) {
-                    const int e = eA + __ldg(eBp + cb + j) - 14;
+                    const int e = eA + eb[j] - 14;
                     const float sc = (e < -126) ? 0.f : __int_as_float((e + 127) << 23);
                     const float h = __fmul_rn(hv[cb + j], sc);
                     const float l = __fmul_rn(lv[cb + j], sc);
@@ -498,6 +501,9 @@ __global__ void __launch_bounds__(ER ? kGemmThreadsER : kGemmThreads, 1)
             const int eA = eAp[r];
             for (int c0 = part * kPartCols; c0 < (part + 1) * kPartCols; c0 += CB) {
                 float2 cv[CB];
+                int eb[CB];
+#pragma unroll
+                for (int j = 0; j < CB; ++j) eb[j] = eBp[c0 + j];
                 if (MODE == 1) {
 #pragma unroll
                     for (int j = 0; j < CB; ++j) cv[j] = C[(size_t)(c0 + j) * GP_NB + r];
@@ -538,7 +544,7 @@ __global__ void __launch_bounds__(ER ? kGemmThreadsER : kGemmThreads, 1)
                     } else {
                         sum_panel_groups<NG>(d, j, h, l);
                     }
-                    const int e = eA + __ldg(eBp + c) - 14;
+                    const int e = eA + eb[j] - 14;
                     const float sc = (e < -126) ? 0.f : __int_as_float((e + 127) << 23);
                     h = __fmul_rn(h, sc);
                     l = __fmul_rn(l, sc);

@@ -337,7 +337,7 @@ __global__ void __launch_bounds__(kInnerThreads) k_trailing_f64(Batch b) {
     __syncthreads();
 #pragma unroll 16
     for (int c = 0; c < GP_NB; ++c) {
-        const double lr = __ldg(L + (size_t)c * GP_NB);
+        const double lr = L[(size_t)c * GP_NB];
 #pragma unroll
         for (int j = 0; j < kInnerCols; ++j) acc[j] = fma(lr, Lk[c][warp + 8 * j], acc[j]);
     }
