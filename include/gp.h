@@ -201,7 +201,8 @@ size_t gp_workspace_bytes(const gp_ctx* ctx);
 enum {
     GP_PHASE_ASSEMBLE = 0,   /* theta checks + correlation assembly        */
     GP_PHASE_POTRF = 1,      /* diagonal-tile factorisation (and inverse)  */
-    GP_PHASE_TRSM = 2,       /* panel solve                                */
+    GP_PHASE_TRSM = 2,       /* panel solve (double: and the products inside
+                                the block column)                          */
     GP_PHASE_UPDATE = 3,     /* trailing update                            */
     GP_PHASE_SOLVE = 4,      /* triangular solves, refinement, reductions  */
     GP_PHASE_SPLIT = 5,      /* bf16 slicing of panels (GP_MIXED)          */

@@ -7,6 +7,7 @@
 #include <cstdio>
 #include <cstring>
 #include <cmath>
+#include <optional>
 #include <string>
 #include <utility>
 #include <vector>
@@ -104,6 +105,15 @@ struct PhaseScope {
             ctx->ev_open.push_back({phase, {e0, e1}});
         }
     }
+};
+
+// A scope of one kernel around each launch of the functions that mix phases.
+struct PhaseLog final : gp::LaunchLog {
+    gp_ctx* ctx;
+    std::optional<PhaseScope> scope;
+    explicit PhaseLog(gp_ctx* c) : ctx(c) {}
+    void begin(int phase, cudaStream_t s) override { scope.emplace(ctx, phase, 1, s); }
+    void end() override { scope.reset(); }
 };
 
 int fail(gp_ctx* ctx, int code, const char* fmt, ...) {
@@ -213,18 +223,14 @@ constexpr int kLookaheadMax = 16;
 // as without.
 int run_factor_f64(gp_ctx* ctx, const gp::Batch& b) {
     const int nt = b.nt;
+    PhaseLog log(ctx);
     if (nt < gp::kUpdateTcTiles) {
-        int k = 0;
-        PhaseScope ps(ctx, GP_PHASE_POTRF, 0);
-        const cudaError_t e = gp::launch_factor_small_f64(b, ctx->stream, &k);
-        ps.kernels += k;
-        GP_CUDA(ctx, e);
+        GP_CUDA(ctx, gp::launch_factor_small_f64(b, ctx->stream, &log));
         return GP_OK;
     }
     // block column J finished: factored and solved
     auto panel = [&](int J, cudaStream_t st) -> int {
-        PhaseScope ps(ctx, GP_PHASE_POTRF, gp::panel_f64_launches(nt, J), st);
-        GP_CUDA(ctx, gp::launch_panel_f64(b, J, st));
+        GP_CUDA(ctx, gp::launch_panel_f64(b, J, st, &log));
         return GP_OK;
     };
     auto update = [&](int J, int which) -> int {

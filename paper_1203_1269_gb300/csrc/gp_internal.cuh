@@ -211,17 +211,22 @@ enum : int { kUpdateAll = 0, kUpdateColumn = 1, kUpdateRest = 2 };
 cudaError_t launch_update_f64_tc(const Batch& b, int J, cudaStream_t s, int which = kUpdateAll);
 // columns 32 step .. 32 step + 31 of block column J, less the products of its columns before them
 cudaError_t launch_update_f64_inner(const Batch& b, int J, int step, cudaStream_t s);
-// block column J factored and solved (kUpdateTcTiles block columns and more), and the
-// log-determinant once they all are
 // steps of X = L^-1 and R^-1 = X'X by rows of X (k_grad.cu, k_update_tc.cu)
 cudaError_t launch_inverse_apply(const Batch& b, int J, double* X, double* S, cudaStream_t s);
 cudaError_t launch_inverse_update(const Batch& b, int J, double* X, double* S, cudaStream_t s);
+// What a caller that accounts for phases (GP_PHASE_*) is told around each launch
+// of the functions that mix them
+struct LaunchLog {
+    virtual void begin(int phase, cudaStream_t s) = 0;
+    virtual void end() = 0;
+};
 constexpr int kPanelStep = 32;
-int panel_f64_launches(int nt, int J);
-cudaError_t launch_panel_f64(const Batch& b, int J, cudaStream_t s);
+// block column J factored and solved (kUpdateTcTiles block columns and more), and the
+// log-determinant once they all are
+cudaError_t launch_panel_f64(const Batch& b, int J, cudaStream_t s, LaunchLog* log = nullptr);
 cudaError_t launch_logdet_f64(const Batch& b, cudaStream_t s);
 // the whole factorisation and log-determinant of fewer block columns
-cudaError_t launch_factor_small_f64(const Batch& b, cudaStream_t s, int* kernels);
+cudaError_t launch_factor_small_f64(const Batch& b, cudaStream_t s, LaunchLog* log = nullptr);
 // Block columns from which the double path's products run on the tensor cores
 // (k_update_tc.cu), whatever the batch.  They are faster from the first tile on
 // (a tile's update is 0.55 ms of one SM's FP64 pipe, 22 us as digits); up to 256 points the factor keeps IEEE operations

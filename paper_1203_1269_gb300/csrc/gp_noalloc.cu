@@ -85,7 +85,7 @@ extern "C" int gp_nll_batch_noalloc(gp_ctx* ctx, int n, int d, const double* x, 
         e = gp::launch_validate_theta(b, stream);
         if (e == cudaSuccess) e = gp::launch_assemble_tiles(b, stream);
         if (nt < gp::kUpdateTcTiles) {
-            if (e == cudaSuccess) e = gp::launch_factor_small_f64(b, stream, nullptr);
+            if (e == cudaSuccess) e = gp::launch_factor_small_f64(b, stream);
         } else {
             for (int J = 0; J < nt && e == cudaSuccess; ++J) {
                 e = gp::launch_panel_f64(b, J, stream);

@@ -273,6 +273,17 @@ __global__ void __launch_bounds__(kThreads) k_solve32_f64(Batch b, int J, int s,
     }
 }
 
+// LaunchLog around one launch
+struct Logged {
+    LaunchLog* log;
+    Logged(LaunchLog* l, int phase, cudaStream_t st) : log(l) {
+        if (log) log->begin(phase, st);
+    }
+    ~Logged() {
+        if (log) log->end();
+    }
+};
+
 template <int LANES>
 void launch_solve32(const Batch& b, int J, int s, int rows, int sms, cudaStream_t st) {
     const int units = rows / (32 / LANES);
@@ -393,51 +404,56 @@ __global__ void __launch_bounds__(256) k_logdet_f64(Batch b) {
 // as they are (the identity).  Every position takes its operations in the
 // order of the unblocked loops: the same bits as one CTA per tile and instance
 // on the FP64 pipe gave (n = 200, T = 64: 1.59 -> 0.52 ms).
-cudaError_t launch_factor_small_f64(const Batch& b, cudaStream_t st, int* kernels) {
+cudaError_t launch_factor_small_f64(const Batch& b, cudaStream_t st, LaunchLog* log) {
     const int sms = device_sms();
-    int k = 0;
     for (int J = 0; J < b.nt; ++J) {
         const int left = b.n - J * GP_NB;                    // real rows from block column J on
         for (int s = 0; s < GP_NB / kB && kB * s < left; ++s) {
-            launch_chained(ahead_f64(b), k_diag32_f64<true>, b.count, kThreads, 0, st, b, J, s);
-            ++k;
+            {
+                Logged l(log, GP_PHASE_POTRF, st);
+                launch_chained(ahead_f64(b), k_diag32_f64<true>, b.count, kThreads, 0, st, b, J, s);
+            }
             const int rows = (left - kB * (s + 1) + 7) / 8 * 8;
             if (rows <= 0) continue;
-            if ((long long)rows * b.count <= 4 * 4LL * sms) launch_solve32<8>(b, J, s, rows, sms, st);
-            else                                            launch_solve32<4>(b, J, s, rows, sms, st);
-            ++k;
+            {
+                Logged l(log, GP_PHASE_TRSM, st);
+                if ((long long)rows * b.count <= 4 * 4LL * sms) launch_solve32<8>(b, J, s, rows, sms, st);
+                else                                            launch_solve32<4>(b, J, s, rows, sms, st);
+            }
             const int cols = GP_NB / kB - 1 - s, groups = (left + kB - 1) / kB - 1 - s;
             if (cols > 0 && groups > 0) {
+                Logged l(log, GP_PHASE_TRSM, st);
                 launch_chained(ahead_f64(b), k_inner_f64, dim3(groups, cols < groups ? cols : groups, b.count),
                                kInnerThreads, 0, st, b, J, s);
-                ++k;
             }
         }
         if (J + 1 < b.nt) {
             const int groups = (left - GP_NB + kB - 1) / kB;
+            Logged l(log, GP_PHASE_UPDATE, st);
             launch_chained(ahead_f64(b), k_trailing_f64, dim3(groups * (groups + 1) / 2, b.count),
                            kInnerThreads, 0, st, b);
-            ++k;
         }
     }
+    Logged l(log, GP_PHASE_POTRF, st);
     launch_chained(ahead_f64(b), k_logdet_small_f64, b.count, GP_NB, 0, st, b);
-    if (kernels) *kernels = k + 1;
     return cudaGetLastError();
 }
 
-// Kernels of launch_panel_f64.
-int panel_f64_launches(int nt, int J) { return J + 1 < nt ? 11 : 10; }
-
-cudaError_t launch_panel_f64(const Batch& b, int J, cudaStream_t st) {
+cudaError_t launch_panel_f64(const Batch& b, int J, cudaStream_t st, LaunchLog* log) {
     const int sms = device_sms();
     for (int s = 0; s < GP_NB / kB; ++s) {
         if (s > 0) {
+            Logged l(log, GP_PHASE_TRSM, st);
             cudaError_t e = launch_update_f64_inner(b, J, s, st);
             if (e != cudaSuccess) return e;
         }
-        launch_chained(s > 0 && ahead_f64(b), k_diag32_f64<false>, b.count, kThreads, 0, st, b, J, s);
+        {
+            Logged l(log, GP_PHASE_POTRF, st);
+            launch_chained(s > 0 && ahead_f64(b), k_diag32_f64<false>, b.count, kThreads, 0, st, b, J, s);
+        }
         const int rows = (b.nt - J) * GP_NB - kB * (s + 1);
         if (rows > 0) {
+            Logged l(log, GP_PHASE_TRSM, st);
             if ((long long)rows * b.count <= 4 * 4LL * sms) launch_solve32<8>(b, J, s, rows, sms, st);
             else                                            launch_solve32<4>(b, J, s, rows, sms, st);
         }
