@@ -55,11 +55,13 @@ typedef struct gp_plan gp_plan;
 
 /* Arithmetic of the factorisation.
  * GP_FP64:  double precision throughout: assembly, pivots, row solves and
- *           substitutions in IEEE double; from three block columns (n > 256)
- *           on, the products of the Cholesky factorisation as exact digit
- *           products on the tensor cores (7 digits of 8 bits per entry),
- *           subtracted in double: the factor's backward error is that of
- *           IEEE multiply-adds or smaller.
+ *           substitutions in double; from three block columns (n > 256) on,
+ *           the products of the Cholesky factorisation as exact digit
+ *           products on the tensor cores (7 digits of 8 bits per entry, an
+ *           absolute unit of 2^-56), subtracted in double, and pivots to an
+ *           ulp (below, correctly rounded).  The largest entry of R - LL' is
+ *           0.1 to 0.7 times that of IEEE multiply-adds, measured for n = 300
+ *           to 5000; the bound holds for the matrix, not entry by entry.
  * GP_MIXED: the panel solves and trailing updates of the blocked Cholesky
  *           on the tensor cores: operands split into bf16 slices, exact fp32
  *           accumulation of the product groups (Ozaki-style), recombined in

@@ -8,17 +8,23 @@
 // sum_{k<i} l_ik^2 = 1 + delta - l_ii^2 and l_ii^2 >= delta for a positive
 // semidefinite R.  So every entry is cut at one fixed scale, with no row
 // exponents:
-//   X = floor(l 2^56) = sum_{a=0..6} q_a 256^(6-a),  |q_a| <= 128 (a > 0), |q_0| <= 256
+//   X = round(l 2^56) = sum_{a=0..6} q_a 256^(6-a),  |q_a| <= 128 (a > 0), |q_0| <= 256
 // (balanced digits), each digit exact in fp16.  The product groups S_g =
 // sum_{a+b=g} q_a q_b', g = 0 .. 7, summed over the panel's 128 columns in fp32
 // are integers below 2^24, hence exact (at most 2^21 for a pair of lower
 // digits, of which a group has six at most, and less than 2^18.6 by
 // Cauchy-Schwarz for a pair with q_0, since the rows of L have norm 1; the
 // inverse's operands, which have no such norm: at combine() below); what
-// is left out, a + b >= 8, is below 2^-66 of 1 per term.  The dropped part of l
-// is at most 2^-56, so all panels together leave an error of about 2^-56 in
-// an entry of A, where each IEEE subtraction from A rounds to 2^-53 of it:
-// the factor is as accurate as with double multiply-adds.
+// is left out, a + b >= 8, is below 2^-66 of 1 per term.  Rounding moves l by at
+// most 2^-57, so that all panels together leave sum_k (|l_ik| + |l_jk|) 2^-57 in an
+// entry of A at most, and about 2^-57 as a root mean square, where IEEE
+// multiply-adds leave up to 2^-53 of the entry per panel column.  The unit is
+// absolute: entries of L below 2^-3 keep fewer than 53 bits in the products,
+// so the bound holds for the matrix, not entry by entry.  R - L L' over 50
+// matrices (n = 300 .. 5000, d = 2 .. 12, p = 1 .. 2, delta = 0 .. 1) against IEEE
+// multiply-adds: its largest entry 0.08 to 0.67 times, its root mean square 0.10
+// to 1.0 times in 46 of them and up to 1.5 times (1.0e-17) in the four whose
+// entries of R are smallest.
 //
 // The digits are cut on the way into shared memory by eight converter
 // warps, from the double tiles themselves: no workspace, so the callers'
@@ -28,7 +34,7 @@
 // cycles here (its operands' shared-memory reads), so a half tile's 272 take
 // 22 k cycles, then the groups' sum in front of the next tile 3 k (5 k with
 // every group through the conversion instruction).  The cutting runs beside
-// it since it costs 13 integer instructions an entry and 2 a digit (38 in
+// it since it costs 15 integer instructions an entry and 2 a digit (38 in
 // all, where it set the pace: 19.9 -> 15 us a half tile).
 // Measured, max |R - L L'| at n = 900, d = 2: 1.3e-16 (1.6e-15 with double
 // multiply-adds on the FP64 pipe).  Twelve candidates at n = 4064: 270 ms with
@@ -56,21 +62,25 @@ constexpr int kMmaRegs = 56, kConvRegs = 96, kEpiRegs = 112;
 static_assert(128 * kMmaRegs + 32 * kConvWarps * kConvRegs + 32 * kEpiWarps * kEpiRegs <= kThreads * 96,
               "register split exceeds the launch's registers");
 
-// X = floor(l 2^(56 - E)) plus the digits' bias: byte 6 - a of the result is q_a +
-// 128 (a >= 1), the 16 bits from 48 up q_0 + 512.  |l| >= 2^E (possible only on
-// the way to a failed factorisation) is cut to its significand, in [1, 2) 2^E.
-// 13 integer instructions, which this GPU issues at half the FP32 rate: the
-// converters' rate is what they cost.
+// X = l 2^(56 - E) rounded to the nearest integer, plus the digits' bias: byte 6 - a
+// of the result is q_a + 128 (a >= 1), the 16 bits from 48 up q_0 + 512.  |l| >= 2^E
+// (possible only on the way to a failed factorisation) is cut to its
+// significand, in [1, 2) 2^E.  15 integer instructions, which this GPU issues at
+// half the FP32 rate: the converters' rate is what they cost.  Two of them are the
+// rounding's (cut down without it, the sums' errors had one sign: mean of R - L L'
+// -3e-17 at n = 4064, d = 12, and a root mean square up to three times that of
+// IEEE multiply-adds where the entries of R are small).
 __device__ __forceinline__ uint2 biased_digits(double l, int E) {
     const unsigned hi = (unsigned)__double2hiint(l), lo = (unsigned)__double2loint(l);
-    // r = 1023 + E - e in [0, 63]: l 2^(56 - E) = (m << 4) >> r for the 53-bit significand m
+    // r = 1023 + E - e in [0, 63]: l 2^(57 - E) = (m << 5) >> r for the 53-bit significand m
     const int r = __viaddmin_s32_relu((int)((~hi & 0x7ff00000u) >> 20), 1023 + E - 2047, 63);
     const unsigned long long m = (unsigned long long)((hi & 0xfffffu) | 0x100000u) << 32 | lo;
-    const unsigned long long w = (m << 4) >> r;
-    // -1 - w for a negative l: the floor
+    const unsigned long long w = (m << 5) >> r;
+    // -1 - w for a negative l, so that what is cut off below the half lies on the
+    // same side of it for either sign
     const unsigned s = (unsigned)((int)hi >> 31);
     const unsigned long long x = (unsigned long long)((unsigned)(w >> 32) ^ s) << 32 | ((unsigned)w ^ s);
-    const unsigned long long y = x + 0x0200808080808080ull;
+    const unsigned long long y = (x + (2 * 0x0200808080808080ull + 1)) >> 1;
     return make_uint2((unsigned)y, (unsigned)(y >> 32));
 }
 
