@@ -64,7 +64,7 @@ __device__ __forceinline__ df2 matern_q_df2(df2 h, int corr, df2 third, f32x2 nt
 // 15 (1989)): an FP64 instruction is worth 64 FP32 ones here, so what counts is
 // their number, 11 against about 20.
 // exp(-S) = 2^(k/128) exp(r), k = round(-128 S / ln 2), r = -S - k ln2/128
-// (two fmas against ln2/128 as 32 + 53 bits), exp(r) - 1 = r + r^2 (1/2 + r/6 +
+// (two fmas against ln2/128 as 33 + 53 bits), exp(r) - 1 = r + r^2 (1/2 + r/6 +
 // r^2/24 + r^3/120) (the next term is below 2^-60), times the table's 2^(j/128)
 // as a double-double, scaled by its exponent bits: 11 double operations.  S
 // above 700 takes exp.

@@ -259,7 +259,7 @@ constexpr int kExpTab = 1 << kExpTabBits;
 // q < 6e-8 is needed to float precision only, so past the reduction the
 // only double-float steps are 1 - r and the product with the table.  S may
 // be negative down to -83 (the logarithms of df_log's Newton step).
-// tab[j] = 2^(-j/N) as double-float (filled by fill_exp2_table).  Results
+// tab[j] = 2^(-j/N) as double-float (load_exp2_table).  Results
 // below 2^-125 (S > 86.6) are returned as zero.
 __device__ __forceinline__ dfl df_exp_neg(dfl S, const dfl* tab) {
     constexpr double kLn2OverN = 0.693147180559945309417232121458176568 / kExpTab;

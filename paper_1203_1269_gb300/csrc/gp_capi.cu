@@ -354,7 +354,8 @@ int ensure_aux(gp_ctx* ctx) {
 // measured costs: a tile of the rest kTile us of one SM; a block column of the
 // pair kLatency us in which only the candidates' diagonal steps run, then
 // kFront us of one SM per tile (slices, panel solve, column update), on the SMs
-// left and, once the rest has ended, on all.
+// left and, once the rest has ended, on all.  The costs are those of five slices and
+// 128-column tiles; with other options the split may be a poorer one.
 int lookahead_sms(int m, int count) {
     constexpr double kTile = 13.4, kFront = 90.0, kLatency = 140.0;
     const int sms = gp::device_sms();

@@ -866,6 +866,7 @@ __global__ void k_rhs_init(MixedBatch b) {
 // 35 -> 24 backward; the solve phase there .82 -> .56 ms, 32 x 1448 1.07 ->
 // .64, 8 x 16384 17.4 -> 10.7, 256 x 4000 15.5 -> 14.4 (2.4 a pass is what the
 // factor's bytes take).
+
 // N entries of both right-hand sides side by side, for the paired FP32
 // instructions: hl = {hi of both, lo of both}, and the negated high words.  A
 // product with L then takes half the issue slots of two scalar ones (the

@@ -38,8 +38,8 @@
 // all, where it set the pace: 19.9 -> 15 us a half tile).
 // Measured, max |R - L L'| at n = 900, d = 2: 1.3e-16 (1.6e-15 with double
 // multiply-adds on the FP64 pipe).  Twelve candidates at n = 4064: 270 ms with
-// the updates on the FP64 pipe (256 of them), 28.8 ms now (updates 19); the
-// double fit at n = 4064 54.6 -> 10.5 ms (9.6 with its launches set up ahead).
+// the updates on the FP64 pipe (256 of them), 28.9 ms now (updates 19); the
+// double fit at n = 4064 54.6 -> 10.5 ms (9.65 with its launches set up ahead).
 #include "mixed_common.cuh"
 
 namespace gp {
@@ -503,9 +503,9 @@ cudaError_t launch(const Batch& b, int J, cudaStream_t s, int which, int per_ins
     const long long total = (long long)per_inst * b.count;
     // the rest of an update runs beside the next block column's panel, whose
     // kernels cannot share an SM with this one: a third of the SMs stay free
-    // for them (n = 4064, one candidate: 14.25 ms without the look-ahead, 14.4
-    // with every SM taken, 13.55 with a third or a half free; twelve: 38.6,
-    // 38.5, 37.3 and 44.2 ms)
+    // for them (ms, without the look-ahead / every SM taken / a third free / half
+    // free; candidates x n: 1x4064 8.59 / 9.08 / 8.23 / 8.23, 4x2048 4.79 / 5.13 / 4.72 /
+    // 4.65, 16x1024 2.81 / 3.07 / 2.84 / 2.81, 12x4064 28.57 / 29.65 / 28.85 / 32.77)
     const int cap = which == kUpdateRest ? device_sms() - device_sms() / 3 : device_sms();
     const int grid = (int)(total < cap ? total : cap);
     launch_chained(which != kUpdateColumn && ahead_f64(b), k_update_f64_tc<NT, MODE>, grid, kThreads, smem, s, b, J,
